@@ -237,44 +237,56 @@ __global__ void __launch_bounds__(kRsThreads) rescore_partial_kernel(
   }
 }
 
-__global__ void rescore_final_kernel(const double* __restrict__ part, int m, int nchunk, int r,
-                                     const int64_t* __restrict__ idx, int64_t S, double* __restrict__ f_out,
-                                     int64_t* __restrict__ best_out, double* __restrict__ best_f_out) {
+// f of every candidate: one warp per candidate and one candidate per block, so
+// that the candidates spread over the SMs.  What bounds it is FP64: a warp-wide
+// FP64 add holds an SM's FP64 unit (two lanes wide) for 16 cycles, and the
+// shuffle trees take 2r x 5 of them; on one block of eight warps the m
+// candidates queued for one SM's unit (77.6 us at m = 64, 107.5 us at m = 164;
+// now 3-4 us).  The chunk sums keep their order: lanes sum fixed subsets of
+// the chunks, then a fixed shuffle tree adds the lanes.
+__global__ void __launch_bounds__(32) rescore_sum_kernel(const double* __restrict__ part, int nchunk, int r,
+                                                         const int64_t* __restrict__ idx, int64_t S,
+                                                         double* __restrict__ f_out) {
+  const int lane = threadIdx.x, t = blockIdx.x;
+  double a[2 * kMaxRank];
+#pragma unroll
+  for (int j = 0; j < 2 * kMaxRank; ++j) a[j] = 0.0;
+  for (int c = lane; c < nchunk; c += 32) {
+    const double* pc = part + (static_cast<int64_t>(t) * nchunk + c) * (2 * kMaxRank);
+#pragma unroll
+    for (int j = 0; j < 2 * kMaxRank; ++j)
+      if (j < 2 * r) a[j] += pc[j];
+  }
+  double f = 0.0;
+#pragma unroll
+  for (int j = 0; j < 2 * kMaxRank; ++j) {
+    if (j < 2 * r) {
+      double v = a[j];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+      f += v * v;  // meaningful in lane 0
+    }
+  }
+  if (lane == 0) {
+    const int64_t s = idx[t];
+    f_out[t] = (s < 0 || s >= S) ? -1.0 : f;
+  }
+}
+
+// the best of the m candidates (largest f, ties to the earlier position)
+__global__ void __launch_bounds__(256) rescore_best_kernel(const double* __restrict__ f_out, int m,
+                                                           const int64_t* __restrict__ idx,
+                                                           int64_t* __restrict__ best_out,
+                                                           double* __restrict__ best_f_out) {
   __shared__ double bf[256];
   __shared__ int bt[256];
   double my_best = -1.0;
   int my_t = 0x7fffffff;
-  // one warp per candidate: lanes sum fixed subsets of the chunks, then a
-  // fixed shuffle tree adds the lanes (deterministic order)
-  const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-  for (int t = threadIdx.x >> 5; t < m; t += nwarp) {
-    double a[2 * kMaxRank];
-#pragma unroll
-    for (int j = 0; j < 2 * kMaxRank; ++j) a[j] = 0.0;
-    for (int c = lane; c < nchunk; c += 32) {
-      const double* pc = part + (static_cast<int64_t>(t) * nchunk + c) * (2 * kMaxRank);
-#pragma unroll
-      for (int j = 0; j < 2 * kMaxRank; ++j)
-        if (j < 2 * r) a[j] += pc[j];
-    }
-    double f = 0.0;
-#pragma unroll
-    for (int j = 0; j < 2 * kMaxRank; ++j) {
-      if (j < 2 * r) {
-        double v = a[j];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        f += v * v;  // meaningful in lane 0
-      }
-    }
-    if (lane == 0) {
-      const int64_t s = idx[t];
-      if (s < 0 || s >= S) f = -1.0;
-      f_out[t] = f;
-      if (f > my_best || (f == my_best && t < my_t)) {
-        my_best = f;
-        my_t = t;
-      }
+  for (int t = threadIdx.x; t < m; t += blockDim.x) {
+    const double f = f_out[t];
+    if (f > my_best || (f == my_best && t < my_t)) {
+      my_best = f;
+      my_t = t;
     }
   }
   bf[threadIdx.x] = my_best;
@@ -354,9 +366,10 @@ int launch_rescore(const RescorePlan& p, const Alphabet& a, const float2* V, con
   count_launch();
   int e = cuda_check(cudaGetLastError(), "rescore_partial_kernel");
   if (e) return e;
-  rescore_final_kernel<<<1, 256, 0, st>>>(part, p.m, p.nchunk, p.r, idx, S, f_out, best_out, best_f_out);
-  count_launch();
-  return cuda_check(cudaGetLastError(), "rescore_final_kernel");
+  rescore_sum_kernel<<<static_cast<unsigned>(p.m), 32, 0, st>>>(part, p.nchunk, p.r, idx, S, f_out);
+  rescore_best_kernel<<<1, 256, 0, st>>>(f_out, p.m, idx, best_out, best_f_out);
+  count_launch(2);
+  return cuda_check(cudaGetLastError(), "rescore_sum_kernel");
 }
 
 }  // namespace lrq
