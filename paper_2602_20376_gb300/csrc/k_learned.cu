@@ -11,6 +11,7 @@
 // every GEMM operand is rounded to bfloat16 (round to nearest even) as it is
 // staged in shared memory and the products accumulate in FP32, on the tensor
 // cores (k_mlp_tc.cu); FP32 mode runs the CUDA-core GEMM below.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -22,6 +23,8 @@
 #include "lrq_internal.h"
 
 namespace lrq {
+
+namespace cg = cooperative_groups;
 
 constexpr int kWidth = 256;
 constexpr int kComp = 16;
@@ -219,25 +222,42 @@ __global__ void colsum_f32_kernel(const float* __restrict__ G, int B, int N, flo
 // vMF normaliser on S^7 (FP64): log I_nu by its power series for kappa <= 30
 // and by the large-argument expansion above
 // ---------------------------------------------------------------------------
-__device__ double log_bessel_i_dev(int nu, double kappa) {
+// 1 / ((k + 1)(k + 1 + nu)), the ratio of consecutive series terms without
+// (kappa / 2)^2: at kappa = 30 the terms fall below 1e-18 of the sum before
+// k = 64, so 96 entries always suffice
+constexpr int kBesselTerms = 96;
+struct BesselTable {
+  double v[2][kBesselTerms];  // nu = 3, 4
+};
+constexpr BesselTable make_bessel_table() {
+  BesselTable t{};
+  for (int h = 0; h < 2; ++h)
+    for (int k = 0; k < kBesselTerms; ++k)
+      t.v[h][k] = 1.0 / (static_cast<double>(k + 1) * static_cast<double>(k + 1 + 3 + h));
+  return t;
+}
+__constant__ BesselTable c_bessel = make_bessel_table();
+
+// log I_nu(kappa), nu = 3 + h
+__device__ __forceinline__ double log_bessel_i_dev(int h, double kappa) {
   if (kappa <= 30.0) {
-    const double half = 0.5 * kappa;
-    double fact = 1.0;
-    for (int k = 2; k <= nu; ++k) fact *= k;
-    double t = pow(half, static_cast<double>(nu)) / fact;
+    const double half = 0.5 * kappa, h2 = half * half;
+    double t = h == 0 ? h2 * half * (1.0 / 6.0) : h2 * h2 * (1.0 / 24.0);
     double s = t;
-    for (int k = 0; k < 500; ++k) {
-      t *= half * half / (static_cast<double>(k + 1) * static_cast<double>(k + 1 + nu));
+    for (int k = 0; k < kBesselTerms; ++k) {
+      t *= h2 * c_bessel.v[h][k];
       s += t;
       if (t < 1e-18 * s) break;
     }
     return log(s);
   }
+  const int nu = 3 + h;
   const double mu = 4.0 * nu * nu;
+  const double ik = 1.0 / (8.0 * kappa);
   double s = 1.0, t = 1.0;
   for (int j = 1; j < 12; ++j) {
     const double o = 2.0 * j - 1.0;
-    t *= -(mu - o * o) / (j * 8.0 * kappa);
+    t *= -(mu - o * o) / j * ik;
     s += t;
   }
   return kappa - 0.5 * log(2.0 * kPi * kappa) + log(s);
@@ -254,79 +274,180 @@ struct CompParams {
   double a8[kComp];
 };
 
-// threads 0..15 fill one component each; thread 0 normalises the weights
+// Fills cp from one instance's outputs; every thread of the block calls it.
+// One warp does the work: an SM's FP64 unit is two lanes wide, so a warp-wide
+// FP64 instruction takes 16 cycles and what counts is how few of them there
+// are.  Lanes m and m + 16 share component m (I_3 and I_4, half of mu each);
+// the series multiply by tabulated reciprocals instead of dividing, and the
+// weights are normalised across lanes instead of by one thread in turn
+// (vmf_sample_kernel, which runs it once a block: 3092 -> 2298 us at B = 16,
+// S = 65520).
 __device__ void head_params(const float* __restrict__ O, CompParams& cp) {
-  const int m = threadIdx.x;
-  if (m < kComp) {
+  if (threadIdx.x < 32) {
+    const int m = threadIdx.x & (kComp - 1), h = threadIdx.x >> 4;
     const float* o = O + m * kHead;
     double nrm = 0.0;
     for (int d = 0; d < kDim; ++d) nrm += static_cast<double>(o[d]) * o[d];
     nrm = sqrt(nrm);
-    cp.unorm[m] = nrm;
-    for (int d = 0; d < kDim; ++d) cp.mu[m][d] = nrm > 0.0 ? o[d] / nrm : (d == 0 ? 1.0 : 0.0);
+    for (int d = h * (kDim / 2); d < (h + 1) * (kDim / 2); ++d)
+      cp.mu[m][d] = nrm > 0.0 ? o[d] / nrm : (d == 0 ? 1.0 : 0.0);
     const double x = o[kDim];
     const double kap = x > 20.0 ? x : log1p(exp(x));
-    cp.kappa[m] = kap;
-    cp.sig[m] = 1.0 / (1.0 + exp(-x));
-    const double li3 = log_bessel_i_dev(3, kap), li4 = log_bessel_i_dev(4, kap);
-    cp.logc[m] = 3.0 * log(kap) - 4.0 * log(2.0 * kPi) - li3;
-    cp.a8[m] = exp(li4 - li3);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double mx = -INFINITY;
-    for (int k = 0; k < kComp; ++k) mx = fmax(mx, static_cast<double>(O[k * kHead + kDim + 1]));
-    double s = 0.0;
-    for (int k = 0; k < kComp; ++k) s += exp(static_cast<double>(O[k * kHead + kDim + 1]) - mx);
-    const double lse = mx + log(s);
-    for (int k = 0; k < kComp; ++k) {
-      cp.logpi[k] = O[k * kHead + kDim + 1] - lse;
-      cp.pi[k] = exp(cp.logpi[k]);
+    const double li = log_bessel_i_dev(h, kap);
+    const double li4 = __shfl_down_sync(0xffffffffu, li, 16);
+    const double lg = o[kDim + 1];
+    double mx = lg;
+#pragma unroll
+    for (int q = kComp / 2; q > 0; q >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, q));
+    double s = exp(lg - mx);
+#pragma unroll
+    for (int q = kComp / 2; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+    if (h == 0) {
+      cp.unorm[m] = nrm;
+      cp.kappa[m] = kap;
+      cp.sig[m] = 1.0 / (1.0 + exp(-x));
+      cp.logc[m] = 3.0 * log(kap) - 4.0 * log(2.0 * kPi) - li;
+      cp.a8[m] = exp(li4 - li);
+      const double lp = lg - (mx + log(s));
+      cp.logpi[m] = lp;
+      cp.pi[m] = exp(lp);
     }
   }
   __syncthreads();
 }
 
-// Loss and gradient of the mean negative log-likelihood, one block per
-// instance; gradient contributions summed in shared memory (FP64).
-__global__ void __launch_bounds__(128) vmf_nll_kernel(const float* __restrict__ O, int B, const float* __restrict__ X,
-                                                      int T, double* __restrict__ loss, float* __restrict__ dO) {
+// Loss and gradient of the mean negative log-likelihood.  A cluster of NB
+// blocks per instance, each taking every NB-th group of targets; a lane owns
+// one component and half a warp one target, so that the 11 sums a component
+// needs (of its responsibility gamma, gamma (mu.x - A_8), gamma mu.x and
+// gamma x) stay in FP64 registers over all targets.  Bound: FP64 (about 60
+// warp instructions of 16 cycles per 32 (target, component) pairs; 16 us of
+// the whole chip at B = 64, T = 164).  The first version let every thread
+// take a target and added 160 gradient terms per target into shared memory
+// with FP64 atomics, all threads on the same address: 841 us at that size,
+// now about 52.  The blocks' sums meet in shared memory (across the cluster) in a
+// fixed order; the loss keeps its one atomic per block.
+constexpr int kNllThreads = 128;
+constexpr int kNllSums = 11;
+
+// x's bits as an integer that orders like it: maxima run on the integer pipe
+// (and the same map takes the integer back)
+__device__ __forceinline__ long long order64(long long bits) {
+  return bits >= 0 ? bits : bits ^ 0x7fffffffffffffffll;
+}
+
+__global__ void __launch_bounds__(kNllThreads) vmf_nll_kernel(const float* __restrict__ O, int B,
+                                                              const float* __restrict__ X, int T,
+                                                              double* __restrict__ loss, float* __restrict__ dO) {
   __shared__ CompParams cp;
-  __shared__ double g[kOut];
-  __shared__ double lred[4];
-  const int b = blockIdx.x;
+  __shared__ double part[kNllThreads / 32][kNllSums][kComp];
+  __shared__ double g[kNllSums][kComp];
+  __shared__ double lred[kNllThreads / 16];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int nb = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
+  const int b = blockIdx.x / nb;
   const float* Ob = O + static_cast<int64_t>(b) * kOut;
-  for (int k = threadIdx.x; k < kOut; k += blockDim.x) g[k] = 0.0;
   head_params(Ob, cp);
-  double lsum = 0.0;
-  for (int t = threadIdx.x; t < T; t += blockDim.x) {
-    const float* x = X + (static_cast<int64_t>(b) * T + t) * kDim;
-    double xv[kDim];
-    for (int d = 0; d < kDim; ++d) xv[d] = x[d];
-    double dots[kComp], ell[kComp], mx = -INFINITY;
-    for (int m = 0; m < kComp; ++m) {
-      double s = 0.0;
-      for (int d = 0; d < kDim; ++d) s += cp.mu[m][d] * xv[d];
-      dots[m] = s;
-      ell[m] = cp.logpi[m] + cp.logc[m] + cp.kappa[m] * s;
-      mx = fmax(mx, ell[m]);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, m = lane & (kComp - 1), half = threadIdx.x >> 4;
+  constexpr int kHalves = kNllThreads / 16;
+  double mu[kDim], sum[kNllSums];
+#pragma unroll
+  for (int d = 0; d < kDim; ++d) mu[d] = cp.mu[m][d];
+#pragma unroll
+  for (int q = 0; q < kNllSums; ++q) sum[q] = 0.0;
+  const double base = cp.logpi[m] + cp.logc[m], kap = cp.kappa[m], a8 = cp.a8[m];
+  // -sum_t (shift_t + log se_t), the logarithm taken of products of se_t in
+  // [1, 16]: 64 of them stay far inside the range
+  double lsum = 0.0, prod = 1.0;
+  int nprod = 0;
+  const int groups = (T + kHalves - 1) / kHalves;
+  const bool vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0;  // rows are 32 bytes
+  for (int gr = rank; gr < groups; gr += nb) {  // the same trips for every thread
+    const int t = gr * kHalves + half;
+    const bool act = t < T;
+    const float4* x4 = reinterpret_cast<const float4*>(X + (static_cast<int64_t>(b) * T + (act ? t : T - 1)) * kDim);
+    float xf[kDim];
+    if (vec) {
+      const float4 u = x4[0], w = x4[1];
+      xf[0] = u.x, xf[1] = u.y, xf[2] = u.z, xf[3] = u.w, xf[4] = w.x, xf[5] = w.y, xf[6] = w.z, xf[7] = w.w;
+    } else {
+#pragma unroll
+      for (int d = 0; d < kDim; ++d) xf[d] = reinterpret_cast<const float*>(x4)[d];
     }
-    double se = 0.0;
-    for (int m = 0; m < kComp; ++m) se += exp(ell[m] - mx);
-    lsum += -(mx + log(se));
-    for (int m = 0; m < kComp; ++m) {
-      const double gam = exp(ell[m] - mx) / se;
-      atomicAdd(&g[m * kHead + kDim + 1], cp.pi[m] - gam);
-      atomicAdd(&g[m * kHead + kDim], -gam * (dots[m] - cp.a8[m]) * cp.sig[m]);
-      const double c = -gam * cp.kappa[m] / cp.unorm[m];
-      for (int d = 0; d < kDim; ++d) atomicAdd(&g[m * kHead + d], c * (xv[d] - dots[m] * cp.mu[m][d]));
+    double xv[kDim], dot = 0.0;
+#pragma unroll
+    for (int d = 0; d < kDim; ++d) {
+      xv[d] = xf[d];
+      dot = fma(mu[d], xv[d], dot);
+    }
+    const double ell = fma(kap, dot, base);
+    long long key = order64(__double_as_longlong(ell));
+#pragma unroll
+    for (int q = kComp / 2; q > 0; q >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, q));
+    const double shift = __longlong_as_double(order64(key));
+    const double e = exp(ell - shift);
+    double se = e;
+#pragma unroll
+    for (int q = kComp / 2; q > 0; q >>= 1) se += __shfl_xor_sync(0xffffffffu, se, q);
+    const double gam = act ? e / se : 0.0;
+    if (act) {
+      lsum -= shift;
+      prod *= se;
+    }
+    if (++nprod == 64) {
+      lsum -= log(prod);
+      prod = 1.0;
+      nprod = 0;
+    }
+    sum[0] += gam;
+    sum[1] = fma(gam, dot - a8, sum[1]);
+    sum[2] = fma(gam, dot, sum[2]);
+#pragma unroll
+    for (int d = 0; d < kDim; ++d) sum[3 + d] = fma(gam, xv[d], sum[3 + d]);
+  }
+  lsum -= log(prod);
+  // the two halves of a warp, then the warps, then the blocks of the cluster
+#pragma unroll
+  for (int q = 0; q < kNllSums; ++q) {
+    sum[q] += __shfl_xor_sync(0xffffffffu, sum[q], 16);
+    if (lane < kComp) part[warp][q][m] = sum[q];
+  }
+  if (m == 0) lred[half] = lsum;
+  __syncthreads();
+  for (int k = threadIdx.x; k < kNllSums * kComp; k += kNllThreads) {
+    double v = 0.0;
+    for (int w = 0; w < kNllThreads / 32; ++w) v += part[w][k / kComp][k % kComp];
+    g[k / kComp][k % kComp] = v;
+  }
+  const double inv = 1.0 / (static_cast<double>(B) * T);
+  if (threadIdx.x == 0) {
+    double ls = 0.0;
+    for (int k = 0; k < kHalves; ++k) ls += lred[k];
+    atomicAdd(loss, ls * inv);
+  }
+  cluster.sync();
+  if (rank == 0) {
+    for (int k = threadIdx.x; k < kNllSums * kComp; k += kNllThreads) {
+      double v = g[k / kComp][k % kComp];
+      for (int q = 1; q < nb; ++q) v += cluster.map_shared_rank(&g[0][0], q)[k];
+      part[0][k / kComp][k % kComp] = v;
+    }
+    __syncthreads();
+    // d/d logit = sum (pi - gamma), d/d kappa' = -softplus' sum gamma (mu.x - A_8),
+    // d/d u = -(kappa / ||u||) (sum gamma x - mu sum gamma mu.x)
+    for (int k = threadIdx.x; k < kOut; k += kNllThreads) {
+      const int c = k / kHead, d = k % kHead;
+      double v;
+      if (d == kDim + 1)
+        v = T * cp.pi[c] - part[0][0][c];
+      else if (d == kDim)
+        v = -cp.sig[c] * part[0][1][c];
+      else
+        v = -(cp.kappa[c] / cp.unorm[c]) * (part[0][3 + d][c] - cp.mu[c][d] * part[0][2][c]);
+      dO[static_cast<int64_t>(b) * kOut + k] = static_cast<float>(v * inv);
     }
   }
-  const double ls = block_sum_f64(lsum, lred);
-  __syncthreads();
-  const double inv = 1.0 / (static_cast<double>(B) * T);
-  for (int k = threadIdx.x; k < kOut; k += blockDim.x) dO[static_cast<int64_t>(b) * kOut + k] = static_cast<float>(g[k] * inv);
-  if (threadIdx.x == 0) atomicAdd(loss, ls * inv);
+  cluster.sync();  // the other blocks' sums stay until block 0 has read them
 }
 
 // ---------------------------------------------------------------------------
@@ -541,9 +662,24 @@ int launch_mlp_backward(const float* params, int F, int B, const float* X, const
 int launch_vmf_nll(const float* O, int B, const float* X, int T, double* loss, float* dO, cudaStream_t st) {
   int e = cuda_check(cudaMemsetAsync(loss, 0, sizeof(double), st), "reset loss");
   if (e) return e;
-  vmf_nll_kernel<<<B, 128, 0, st>>>(O, B, X, T, loss, dO);
+  // blocks per instance: up to two per SM over all instances, at least two
+  // groups of targets each, at most the portable cluster size
+  int nb = 1;
+  while (nb < 8 && static_cast<int64_t>(B) * nb * 2 <= 2 * 152 && T >= 4 * nb * (kNllThreads / 16)) nb *= 2;
+  if (B > 0x7fffffff / nb) return fail(LRQ_EUNSUPPORTED, "vmf_nll: batch too large");
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(B) * nb);
+  cfg.blockDim = dim3(kNllThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = nb;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  e = cuda_check(cudaLaunchKernelEx(&cfg, vmf_nll_kernel, O, B, X, T, loss, dO), "vmf_nll_kernel");
   count_launch();
-  return cuda_check(cudaGetLastError(), "vmf_nll_kernel");
+  return e;
 }
 
 int launch_vmf_sample(const float* O, int B, int S, int K, uint64_t seed, float2* C, int32_t* status,
