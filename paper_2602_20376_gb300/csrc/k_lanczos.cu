@@ -13,9 +13,10 @@
 //     Gram-Schmidt pass over components of rounding size); alpha_j =
 //     u_j^H Q u_j is the sum of the two projections onto u_j, and
 //     beta_j = ||w||.  The tridiagonal T_J is real for Hermitian Q.
-//   * Convergence: eigenvalues of T_J by multisection on Sturm counts, their
-//     eigenvectors by inverse iteration (Gaussian elimination with partial
-//     pivoting), residual ||Q y - theta y|| = beta_{J-1} |x_{J-1}|.
+//   * Convergence, on the host beside the next GPU steps: eigenvalues of T_J
+//     by multisection on Sturm counts, their eigenvectors by inverse
+//     iteration (Gaussian elimination with partial pivoting), residual
+//     ||Q y - theta y|| = beta_{J-1} |x_{J-1}|.
 //   * Locking: converged Ritz vectors are stored in front of the Krylov
 //     basis and every later vector is orthogonalised against them, so that a
 //     new run (fresh random start) sees only the rest of the spectrum.  A
@@ -25,7 +26,10 @@
 //     that belongs to the top r.
 // Vectors are stored column-major (each basis vector contiguous, n doubles
 // or complex doubles); the projections are tall-skinny GEMV pairs over
-// row chunks with a fixed-order reduction (deterministic).
+// row chunks with a fixed-order reduction (deterministic).  A step is five
+// launches: operator (with the projections on the last two vectors),
+// three-term step, projections, their subtraction (with the norm, alpha and
+// beta), scaling; the last block of a kernel to finish adds its block sums.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -33,6 +37,7 @@
 #include <cfloat>
 #include <cmath>
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "lrq_device.cuh"
@@ -41,8 +46,11 @@
 namespace lrq {
 
 constexpr int kLzThreads = 256;
-constexpr int kLzChunkMax = 4096;  // rows per block in the projection kernels (at most)
-constexpr int kLzGroup = 8;        // basis vectors per block in the projection kernels
+constexpr int kLzChunkMax = 4096;  // rows per block in lz_dots (at most; at least four a thread)
+constexpr int kLzDotThreads = 128;
+constexpr int kLzGroup = 8;        // basis vectors per block in lz_dots
+constexpr int kLzMvThreads = 64;   // lz_matvec_dense
+constexpr int kLzMaxBlocks = 152 * 16;  // blocks that leave a partial sum (matvec, three-term step, update)
 constexpr int kLzWant = kMaxRank;  // at most 8 wanted pairs per run
 constexpr int kLzMaxIter = 4096;
 constexpr int kLzDefaultIter = 500;
@@ -51,11 +59,6 @@ constexpr int kLzLag = 2;          // Lanczos steps run while a convergence chec
 // ---------------------------------------------------------------------------
 // scalar helpers: real (graph Laplacian) and complex (dense Hermitian) paths
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double lz_cdot(double a, double b) { return a * b; }
-__device__ __forceinline__ double2 lz_cdot(double2 a, double2 b) {  // conj(a) b
-  return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.x, b.y, -a.y * b.x));
-}
-__device__ __forceinline__ double lz_mul(double a, double b) { return a * b; }
 __device__ __forceinline__ double2 lz_mul(double2 a, double2 b) {
   return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
@@ -71,8 +74,6 @@ __device__ __forceinline__ void lz_sub(double2& a, double2 b) {
   a.x -= b.x;
   a.y -= b.y;
 }
-__device__ __forceinline__ double lz_abs2(double a) { return a * a; }
-__device__ __forceinline__ double lz_abs2(double2 a) { return a.x * a.x + a.y * a.y; }
 __device__ __forceinline__ double lz_re(double a) { return a; }
 __device__ __forceinline__ double lz_re(double2 a) { return a.x; }
 template <typename T>
@@ -96,15 +97,95 @@ __device__ __forceinline__ double2 lz_as_complex(double2 a) { return a; }
 __device__ __forceinline__ double lz_real_or_gauss(double, double g0, double) { return g0; }
 __device__ __forceinline__ double2 lz_real_or_gauss(double2, double g0, double g1) { return make_double2(g0, g1); }
 
+__device__ __forceinline__ double lz_neg(double a) { return -a; }
+__device__ __forceinline__ double2 lz_neg(double2 a) { return make_double2(-a.x, -a.y); }
+__device__ __forceinline__ double lz_scale_fma(double a, double s, double c) { return fma(a, s, c); }
+__device__ __forceinline__ double2 lz_scale_fma(double2 a, double s, double2 c) {
+  return make_double2(fma(a.x, s, c.x), fma(a.y, s, c.y));
+}
+__device__ __forceinline__ double lz_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double2 lz_fma(double2 a, double2 b, double2 c) {  // a b + c, four FMAs
+  return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
+}
+__device__ __forceinline__ double lz_cfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double2 lz_cfma(double2 a, double2 b, double2 c) {  // conj(a) b + c
+  return make_double2(fma(a.x, b.x, fma(a.y, b.y, c.x)), fma(a.x, b.y, fma(-a.y, b.x, c.y)));
+}
+__device__ __forceinline__ double lz_abs2_fma(double a, double c) { return fma(a, a, c); }
+__device__ __forceinline__ double lz_abs2_fma(double2 a, double c) { return fma(a.x, a.x, fma(a.y, a.y, c)); }
+
+// Sums N values over the warp: at each step half of the values change lanes,
+// so that N + log2(32 / N) additions a lane do what a butterfly per value
+// does with 5 N (an FP64 addition of a warp holds the SM's two-lane FP64 unit
+// for 16 cycles).  The total of value v ends in the lanes whose upper
+// log2(N) bits, read from the top, are v; `mine` tells which one a lane has.
+template <int N, typename T>
+__device__ __forceinline__ T lz_warp_sums(T (&v)[N], int* mine) {
+  const int lane = threadIdx.x & 31;
+  int id = 0, m = 16;
+#pragma unroll
+  for (int k = N / 2; k > 0; k >>= 1, m >>= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int q = 0; q < k; ++q) {
+      const T give = up ? v[q] : v[k + q];
+      T keep = up ? v[k + q] : v[q];
+      lz_add(keep, lz_shfl_xor(give, m));
+      v[q] = keep;
+    }
+    id = 2 * id + (up ? 1 : 0);
+  }
+#pragma unroll
+  for (int q = 16; q > 0; q >>= 1)
+    if (q <= m) lz_add(v[0], lz_shfl_xor(v[0], q));
+  *mine = id;
+  return v[0];
+}
+
+// Whether this block is the last of `count` to arrive at the counter (which
+// returns to zero): every block's earlier global writes are then visible to
+// it.  All threads of the block call it.
+__device__ __forceinline__ bool lz_last_block(unsigned* counter, unsigned count) {
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicInc(counter, count - 1) == count - 1;
+  __syncthreads();
+  if (last) __threadfence();
+  return last != 0;
+}
+
+// Sum of part[0..count) by the whole block in a fixed order (every thread
+// gets it); NT threads.
+template <int NT, typename T>
+__device__ __forceinline__ T lz_block_total(const T* part, int count) {
+  __shared__ T red[NT / 32];
+  T s = lz_zero<T>();
+  for (int k = threadIdx.x; k < count; k += NT) lz_add(s, __ldcg(part + k));  // other blocks' writes: from L2
+  s = lz_warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  T t = red[0];
+  for (int k = 1; k < NT / 32; ++k) lz_add(t, red[k]);
+  __syncthreads();
+  return t;
+}
+
 // Device state of one Lanczos run.
 struct LzState {
   int stop;        // set on breakdown (invariant subspace reached)
   int jdone;       // Lanczos vectors whose alpha and beta are known
   double tnorm;    // running estimate of ||T||
   double inv_beta;
+  double wnorm2;   // ||w||^2 after the three-term step (lz_threeterm)
 };
 
-// Result of a convergence check (copied to the host).
+// What a convergence check needs (lz_snapshot), in front of alpha and beta.
+struct LzSnap {
+  int stop, jdone, status, pad;
+};
+
+// Verdict of a convergence check (host).
 struct LzCheck {
   int J;
   int converged;
@@ -118,19 +199,43 @@ struct LzCheck {
 // ---------------------------------------------------------------------------
 // operators
 // ---------------------------------------------------------------------------
+// Every operator also leaves the projections of y on the last two basis
+// vectors, h1[0] = u_prev^H y (when there is one) and h1[1] = x^H y: the
+// block sums meet in the last block to finish, in block order.
+template <int NT, typename T>
+__device__ __forceinline__ void lz_two_dots(T d0, T d1, T* __restrict__ part, unsigned* counter, int has_prev,
+                                            T* __restrict__ h1) {
+  __shared__ T red[2][NT / 32];
+  T v[2] = {d0, d1};
+  int mine;
+  const T t = lz_warp_sums<2>(v, &mine);
+  if ((threadIdx.x & 15) == 0) red[mine][threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    T s = red[threadIdx.x][0];
+    for (int k = 1; k < NT / 32; ++k) lz_add(s, red[threadIdx.x][k]);
+    part[threadIdx.x * kLzMaxBlocks + blockIdx.x] = s;
+  }
+  if (!lz_last_block(counter, gridDim.x)) return;
+  for (int q = has_prev ? 0 : 1; q < 2; ++q) {
+    const T s = lz_block_total<NT>(part + q * kLzMaxBlocks, static_cast<int>(gridDim.x));
+    if (threadIdx.x == 0) h1[q] = s;
+  }
+}
+
 // y = L x = D x - A x for the graph Laplacian, a thread per row: the
 // weighted degrees D are precomputed (lz_degree), so a row costs one FP64
 // add or FMA per stored edge (GB300's FP64 rate, not memory, bounds this
 // operator).  Self loops are skipped, out-of-range columns ignored (they are
 // reported by lz_check_csr).
-__global__ void __launch_bounds__(kLzThreads) lz_matvec_laplacian(const int32_t* __restrict__ rowptr,
-                                                                  const int32_t* __restrict__ colidx,
-                                                                  const double* __restrict__ wts,
-                                                                  const double* __restrict__ deg, int64_t n,
-                                                                  int64_t nnz, const double* __restrict__ x,
-                                                                  double* __restrict__ y, const LzState* st) {
+__global__ void __launch_bounds__(kLzThreads) lz_matvec_laplacian(
+    const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx, const double* __restrict__ wts,
+    const double* __restrict__ deg, int64_t n, int64_t nnz, const double* __restrict__ x, double* __restrict__ y,
+    const double* __restrict__ uprev, double* __restrict__ part, unsigned* counter, double* __restrict__ h1,
+    const LzState* st) {
   if (st->stop) return;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  double d0 = 0.0, d1 = 0.0;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
     int64_t k0 = rowptr[i], k1 = rowptr[i + 1];
     k0 = k0 < 0 ? 0 : (k0 > nnz ? nnz : k0);
@@ -141,8 +246,12 @@ __global__ void __launch_bounds__(kLzThreads) lz_matvec_laplacian(const int32_t*
       if (j < 0 || j >= n || j == i) continue;
       acc = wts ? fma(wts[k], x[j], acc) : acc + x[j];
     }
-    y[i] = fma(deg[i], x[i], -acc);
+    const double xi = x[i], yi = fma(deg[i], xi, -acc);
+    y[i] = yi;
+    if (uprev) d0 = fma(uprev[i], yi, d0);
+    d1 = fma(xi, yi, d1);
   }
+  lz_two_dots<kLzThreads>(d0, d1, part, counter, uprev != nullptr, h1);
 }
 
 // deg[i] = sum of the row's edge weights (self loops and invalid columns
@@ -167,39 +276,98 @@ __global__ void __launch_bounds__(kLzThreads) lz_degree(const int32_t* __restric
 }
 
 // y = Q x for dense Hermitian Q (row-major, leading dimension ld): a warp
-// per row.
-__global__ void __launch_bounds__(kLzThreads) lz_matvec_dense(const double2* __restrict__ Q, int64_t n, int64_t ld,
-                                                              const double2* __restrict__ x, double2* __restrict__ y,
-                                                              const LzState* st) {
+// takes ROWS rows at a time, so that one load of x serves ROWS of them.
+// Bound: FP64 (four FMAs an entry, 16 cycles a warp instruction: 108 us at
+// n = 4096 with all SMs equally loaded; the 268 MB take 40).  Two rows a warp
+// and two warps a block: 4096 rows are 1024 blocks, 6.7 an SM, so the fullest
+// SM has 28 rows where the average has 27 (blocks of sixteen rows: 32).
+// n = 4096: 143 us with the two projections; 230 us without them before (a row
+// per warp, six FP64 instructions an entry).
+template <int ROWS>
+__global__ void __launch_bounds__(kLzMvThreads) lz_matvec_dense(
+    const double2* __restrict__ Q, int64_t n, int64_t ld, const double2* __restrict__ x, double2* __restrict__ y,
+    const double2* __restrict__ uprev, double2* __restrict__ part, unsigned* counter, double2* __restrict__ h1,
+    const LzState* st) {
   if (st->stop) return;
   const int lane = threadIdx.x & 31;
-  const int64_t nwarps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
-  for (int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; i < n; i += nwarps) {
-    const double2* row = Q + i * ld;
-    double2 a0 = make_double2(0.0, 0.0), a1 = a0;
-    int64_t j = lane;
-    for (; j + 32 < n; j += 64) {
-      lz_add(a0, lz_mul(row[j], x[j]));
-      lz_add(a1, lz_mul(row[j + 32], x[j + 32]));
+  const int64_t nwarps = static_cast<int64_t>(gridDim.x) * (kLzMvThreads / 32);
+  double2 d0 = make_double2(0.0, 0.0), d1 = d0;
+  for (int64_t i0 = ((static_cast<int64_t>(blockIdx.x) * kLzMvThreads + threadIdx.x) >> 5) * ROWS; i0 < n;
+       i0 += nwarps * ROWS) {
+    const double2* row[ROWS];
+    double2 acc[ROWS];
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+      row[q] = Q + min(i0 + q, n - 1) * ld;
+      acc[q] = make_double2(0.0, 0.0);
     }
-    if (j < n) lz_add(a0, lz_mul(row[j], x[j]));
-    lz_add(a0, a1);
-    a0 = lz_warp_sum(a0);
-    if (lane == 0) y[i] = a0;
+#pragma unroll(ROWS == 1 ? 2 : 4)
+    for (int64_t j = lane; j < n; j += 32) {
+      const double2 xj = x[j];
+#pragma unroll
+      for (int q = 0; q < ROWS; ++q) acc[q] = lz_fma(row[q][j], xj, acc[q]);
+    }
+    int mine = 0;
+    double2 v = lz_warp_sums<ROWS>(acc, &mine);
+    // row `mine`'s total is in this lane; one lane per row goes on
+    const int64_t i = i0 + mine;
+    if ((lane & (32 / ROWS - 1)) == 0 && i < n) {
+      y[i] = v;
+      if (uprev) d0 = lz_cfma(uprev[i], v, d0);
+      d1 = lz_cfma(x[i], v, d1);
+    }
   }
+  lz_two_dots<kLzMvThreads>(d0, d1, part, counter, uprev != nullptr, h1);
 }
 
 // ---------------------------------------------------------------------------
 // projections
 // ---------------------------------------------------------------------------
-// partial[c * nch + chunk] = sum over the chunk's rows of conj(U_c) w, for
-// basis vectors c in [0, nc).  grid = (nch, ceil(nc / 8)).
+// The three-term step, w -= u_prev h1[0] + u h1[1] (uprev NULL: the second
+// only), and ||w||^2 after it.
 template <typename T>
-__global__ void __launch_bounds__(kLzThreads) lz_dots(const T* __restrict__ U, int64_t n, int nc,
-                                                      const T* __restrict__ w, T* __restrict__ partial, int nch,
-                                                      int chunk_rows, const LzState* st) {
+__global__ void __launch_bounds__(kLzThreads) lz_threeterm(T* __restrict__ w, int64_t n, const T* __restrict__ uprev,
+                                                           const T* __restrict__ u, const T* __restrict__ h1,
+                                                           double* __restrict__ npart, unsigned* counter,
+                                                           LzState* st) {
   if (st->stop) return;
-  __shared__ T red[kLzGroup][kLzThreads / 32];
+  __shared__ double red[kLzThreads / 32];
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * kLzThreads;
+  const T h0 = uprev ? lz_neg(h1[0]) : lz_zero<T>(), hc = lz_neg(h1[1]);
+  double s = 0.0;
+  for (int64_t i = static_cast<int64_t>(blockIdx.x) * kLzThreads + threadIdx.x; i < n; i += stride) {
+    T v = w[i];
+    if (uprev) v = lz_fma(uprev[i], h0, v);
+    v = lz_fma(u[i], hc, v);
+    w[i] = v;
+    s = lz_abs2_fma(v, s);
+  }
+  s = lz_warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = red[0];
+    for (int k = 1; k < kLzThreads / 32; ++k) t += red[k];
+    npart[blockIdx.x] = t;
+  }
+  if (!lz_last_block(counter, gridDim.x)) return;
+  const double t = lz_block_total<kLzThreads>(npart, static_cast<int>(gridDim.x));
+  if (threadIdx.x == 0) st->wnorm2 = t;
+}
+
+// h[c] = U_c^H w for basis vectors c in [0, nc): a block takes one row chunk
+// and 8 vectors, and the last block of a group of vectors adds the group's
+// chunk sums in chunk order.  grid = (nch, ceil(nc / 8)).  Bound: FP64 (one
+// FMA per entry for real vectors, four for complex).  Per thread 26 rows x 8
+// FMAs and 9 additions at n = 10^6; a butterfly per vector cost 40.  n = 10^6,
+// 80 vectors: 176 us, 241 before.
+template <typename T>
+__global__ void __launch_bounds__(kLzDotThreads) lz_dots(const T* __restrict__ U, int64_t n, int nc,
+                                                         const T* __restrict__ w, T* __restrict__ partial, int nch,
+                                                         int chunk_rows, unsigned* counter, T* __restrict__ h,
+                                                         const LzState* st) {
+  if (st->stop) return;
+  __shared__ T red[kLzGroup][kLzDotThreads / 32];
   const int chunk = blockIdx.x;
   const int cg = blockIdx.y * kLzGroup;
   const int64_t i0 = static_cast<int64_t>(chunk) * chunk_rows;
@@ -208,110 +376,97 @@ __global__ void __launch_bounds__(kLzThreads) lz_dots(const T* __restrict__ U, i
 #pragma unroll
   for (int q = 0; q < kLzGroup; ++q) acc[q] = lz_zero<T>();
   const int ncols = min(kLzGroup, nc - cg);
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    const T wi = w[i];
+  const T* Ug = U + static_cast<int64_t>(cg) * n;
+  if (ncols == kLzGroup) {
+#pragma unroll 2
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += kLzDotThreads) {
+      const T wi = w[i];
 #pragma unroll
-    for (int q = 0; q < kLzGroup; ++q)
-      if (q < ncols) lz_add(acc[q], lz_cdot(U[static_cast<int64_t>(cg + q) * n + i], wi));
+      for (int q = 0; q < kLzGroup; ++q) acc[q] = lz_cfma(Ug[static_cast<int64_t>(q) * n + i], wi, acc[q]);
+    }
+  } else {
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += kLzDotThreads) {
+      const T wi = w[i];
+#pragma unroll
+      for (int q = 0; q < kLzGroup; ++q)
+        if (q < ncols) acc[q] = lz_cfma(Ug[static_cast<int64_t>(q) * n + i], wi, acc[q]);
+    }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < kLzGroup; ++q) {
-    T v = lz_warp_sum(acc[q]);
-    if (lane == 0) red[q][warp] = v;
-  }
+  int mine;
+  const T v = lz_warp_sums<kLzGroup>(acc, &mine);
+  if ((lane & 3) == 0) red[mine][warp] = v;
   __syncthreads();
   if (threadIdx.x < ncols) {
-    T s = lz_zero<T>();
-    for (int k = 0; k < kLzThreads / 32; ++k) lz_add(s, red[threadIdx.x][k]);
+    T s = red[threadIdx.x][0];
+    for (int k = 1; k < kLzDotThreads / 32; ++k) lz_add(s, red[threadIdx.x][k]);
     partial[static_cast<int64_t>(cg + threadIdx.x) * nch + chunk] = s;
   }
-}
-
-// h[c] = sum_chunk partial[c * nch + chunk] in chunk order (a warp per c).
-template <typename T>
-__global__ void lz_reduce(const T* __restrict__ partial, int nc, int nch, T* __restrict__ h, const LzState* st) {
-  if (st->stop) return;
-  const int lane = threadIdx.x & 31;
-  const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (c >= nc) return;  // whole warps leave together
-  T s = lz_zero<T>();
-  for (int k = lane; k < nch; k += 32) lz_add(s, partial[static_cast<int64_t>(c) * nch + k]);
-  s = lz_warp_sum(s);
-  if (lane == 0) h[c] = s;
-}
-
-// w -= sum_c U_c h[c]: a block takes 32 rows, its 8 warps take every 8th
-// basis vector (coalesced 32-row loads), and the 8 partial sums of a row are
-// added in warp order (deterministic).
-template <typename T>
-__global__ void __launch_bounds__(kLzThreads) lz_update(const T* __restrict__ U, int64_t n, int nc,
-                                                        const T* __restrict__ h, T* __restrict__ w,
-                                                        const LzState* st) {
-  if (st->stop) return;
-  __shared__ T part[kLzThreads / 32][32];
-  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
-  constexpr int NS = kLzThreads / 32;
-  for (int64_t r0 = static_cast<int64_t>(blockIdx.x) * 32; r0 < n; r0 += static_cast<int64_t>(gridDim.x) * 32) {
-    const int64_t i = r0 + lane;
-    T s0 = lz_zero<T>(), s1 = lz_zero<T>();
-    if (i < n) {
-      int c = slice;
-      for (; c + NS < nc; c += 2 * NS) {
-        lz_add(s0, lz_mul(U[static_cast<int64_t>(c) * n + i], h[c]));
-        lz_add(s1, lz_mul(U[static_cast<int64_t>(c + NS) * n + i], h[c + NS]));
-      }
-      if (c < nc) lz_add(s0, lz_mul(U[static_cast<int64_t>(c) * n + i], h[c]));
-    }
-    lz_add(s0, s1);
-    part[slice][lane] = s0;
-    __syncthreads();
-    if (slice == 0 && i < n) {
-      T t = part[0][lane];
-      for (int k = 1; k < NS; ++k) lz_add(t, part[k][lane]);
-      T v = w[i];
-      lz_sub(v, t);
-      w[i] = v;
-    }
-    __syncthreads();
+  if (!lz_last_block(counter + blockIdx.y, gridDim.x)) return;
+  for (int q = warp; q < ncols; q += kLzDotThreads / 32) {
+    const T* pc = partial + static_cast<int64_t>(cg + q) * nch;
+    T s = lz_zero<T>();
+    for (int k = lane; k < nch; k += 32) lz_add(s, __ldcg(pc + k));
+    s = lz_warp_sum(s);
+    if (lane == 0) h[cg + q] = s;
   }
 }
 
-// npart[chunk] = sum over the chunk of |w_i|^2
-template <typename T>
-__global__ void __launch_bounds__(kLzThreads) lz_norm_partial(const T* __restrict__ w, int64_t n,
-                                                              double* __restrict__ npart, int chunk_rows,
-                                                              const LzState* st) {
-  if (st->stop) return;
-  __shared__ double red[kLzThreads / 32];
-  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * chunk_rows;
-  const int64_t i1 = min(n, i0 + chunk_rows);
-  double s = 0.0;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) s += lz_abs2(w[i]);
-  s = lz_warp_sum(s);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int k = 0; k < kLzThreads / 32; ++k) t += red[k];
-    npart[blockIdx.x] = t;
-  }
+// x rounded towards zero to FP32 by integer operations (a conversion
+// instruction runs on the slow FP64 unit); 0 below the FP32 normal range.
+// For |x| < 2^127: the entries of unit vectors.
+__device__ __forceinline__ float lz_to_float(double x) {
+  const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+  const uint32_t mag = (__funnelshift_l(lo, hi, 3) + 0x40000000u) & 0x7fffffffu;
+  const bool tiny = (hi & 0x7fffffffu) < (897u << 20);
+  return __uint_as_float(tiny ? 0u : ((hi & 0x80000000u) | mag));
 }
-
-// Close step j: beta_j = ||w||, alpha_j = Re(h1[c] + h2[c]) (c = column of
-// u_j), breakdown test.  mode 1 = normalising a start vector (no alpha).
+// the same for any x: infinite from 2^127 on and for NaN
+__device__ __forceinline__ float lz_to_float_sat(double x) {
+  return (__double2hiint(x) & 0x7fffffff) >= (1150 << 20) ? INFINITY : lz_to_float(x);
+}
+__device__ __forceinline__ float2 lz_to_float_sat(double2 x) {
+  return make_float2(lz_to_float_sat(x.x), lz_to_float_sat(x.y));
+}
+__device__ __forceinline__ float2 lz_to_float(double2 x) { return make_float2(lz_to_float(x.x), lz_to_float(x.y)); }
+__device__ __forceinline__ float lz_fma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float2 lz_fma(float2 a, float2 b, float2 c) {
+  return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(a.y, b.x, c.y)));
+}
+__device__ __forceinline__ float lz_abs1(float a) { return fabsf(a); }
+__device__ __forceinline__ float lz_abs1(float2 a) { return fabsf(a.x) + fabsf(a.y); }
+__device__ __forceinline__ void lz_add(float& a, float b) { a += b; }
+__device__ __forceinline__ void lz_add(float2& a, float2 b) {
+  a.x += b.x;
+  a.y += b.y;
+}
+// w + neg s
+__device__ __forceinline__ double lz_add_scaled(double w, float s, double neg) {
+  return fma(neg, static_cast<double>(s), w);
+}
+__device__ __forceinline__ double2 lz_add_scaled(double2 w, float2 s, double neg) {
+  return make_double2(fma(neg, static_cast<double>(s.x), w.x), fma(neg, static_cast<double>(s.y), w.y));
+}
 template <typename T>
-__global__ void lz_finish(const double* __restrict__ npart, int nch, const T* __restrict__ h1,
-                          const T* __restrict__ h2, int c, int j, int mode, double* __restrict__ alpha,
-                          double* __restrict__ beta, LzState* st) {
-  if (blockIdx.x != 0 || st->stop) return;
-  // the chunk norms, lane-strided then a fixed shuffle tree (deterministic)
-  double s = 0.0;
-  for (int k = threadIdx.x; k < nch; k += 32) s += npart[k];
-#pragma unroll
-  for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
-  if (threadIdx.x != 0) return;
-  const double b = sqrt(s);
+struct LzFloat;
+template <>
+struct LzFloat<double> {
+  using type = float;
+  __device__ static float zero() { return 0.f; }
+};
+template <>
+struct LzFloat<double2> {
+  using type = float2;
+  __device__ static float2 zero() { return make_float2(0.f, 0.f); }
+};
+
+// One thread closes step j: beta_j = ||w||, alpha_j = Re(h1[1] + h2[c]) (c =
+// column of u_j), breakdown test.  mode 1 = normalising a start vector (no
+// alpha).
+template <typename T>
+__device__ void lz_finish(double nrm2, const T* __restrict__ h1, const T* __restrict__ h2, int c, int j, int mode,
+                          double* __restrict__ alpha, double* __restrict__ beta, LzState* st) {
+  const double b = sqrt(nrm2);
   if (mode == 1) {
     // start vector: b is its norm after projection; a zero vector means the
     // locked vectors already span the space
@@ -322,7 +477,7 @@ __global__ void lz_finish(const double* __restrict__ npart, int nch, const T* __
     st->inv_beta = 1.0 / b;
     return;
   }
-  const double a = lz_re(h1[c]) + lz_re(h2[c]);
+  const double a = lz_re(h1[1]) + lz_re(h2[c]);
   alpha[j] = a;
   beta[j] = b;
   const double bprev = j > 0 ? beta[j - 1] : 0.0;
@@ -335,6 +490,126 @@ __global__ void lz_finish(const double* __restrict__ npart, int nch, const T* __
   st->inv_beta = 1.0 / b;
 }
 
+// w -= sum_c U_c h[c], then the norm of w and (in the last block to finish)
+// what lz_finish does with it: mode 0 closes step j (h1 and h2 = h: the two
+// projections, c the column of u_j), mode 1 prepares a start vector, mode 2
+// only subtracts.
+//
+// SL warps of a block share a tile of 256 / SL rows, each taking every SL-th
+// vector: SL = 8 gives a small n enough warps (n = 4096: 128 tiles), SL = 1
+// needs no exchange.
+//
+// After the three-term step w is orthogonal to every stored vector up to
+// rounding, so h is of rounding size and the correction sum_c U_c h[c] needs
+// no more than FP32: with sum |h_c| <= 2^-30 ||w|| (checked here, ||w|| from
+// lz_threeterm; h is taken relative to the power of two below ||w||, so that
+// the operator's scale does not matter), its relative error of 2^-22 moves w
+// by less than 2^-52 ||w||, within the rounding of w itself.  U is then read through lz_to_float and the
+// kernel is bound by HBM instead of FP64 (n = 10^6, 80 vectors: 121 us, 206 in
+// FP64).  Larger h (a start vector against
+// locked vectors, a vector close to the span) takes the FP64 sum.
+template <int SL, typename T>
+__global__ void __launch_bounds__(kLzThreads) lz_update(const T* __restrict__ U, int64_t n, int nc,
+                                                        const T* __restrict__ h, T* __restrict__ w,
+                                                        double* __restrict__ npart, unsigned* counter, int mode,
+                                                        int allow32, const T* __restrict__ h1,
+                                                        int c, int j, double* __restrict__ alpha,
+                                                        double* __restrict__ beta, LzState* st) {
+  if (st->stop) return;
+  using F = typename LzFloat<T>::type;
+  extern __shared__ __align__(16) uint8_t lz_smem[];
+  T* hs = reinterpret_cast<T*>(lz_smem);
+  F* hf = reinterpret_cast<F*>(lz_smem + static_cast<size_t>(nc) * sizeof(T));
+  __shared__ T part[SL][32];
+  __shared__ double red[kLzThreads / 32];
+  __shared__ float fred[kLzThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // 2^-floor(log2 ||w||) and its inverse; 0 outside the comfortable range
+  double scale = 0.0, unscale = 0.0;
+  if (allow32) {
+    const double wn2 = st->wnorm2;
+    if (wn2 > 0x1p-900 && wn2 < 0x1p900) {
+      const int e = (__double2hiint(sqrt(wn2)) >> 20) - 1023;
+      scale = __hiloint2double((1023 - e) << 20, 0);
+      unscale = __hiloint2double((1023 + e) << 20, 0);
+    }
+  }
+  float ha = 0.f;
+  for (int q = threadIdx.x; q < nc; q += kLzThreads) {
+    const T v = h[q];
+    hs[q] = v;
+    const F f = lz_to_float_sat(lz_scale(v, scale));
+    hf[q] = f;
+    ha += lz_abs1(f);
+  }
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) ha += __shfl_xor_sync(0xffffffffu, ha, m);
+  if (lane == 0) fred[warp] = ha;
+  __syncthreads();
+  bool f32 = false;
+  if (scale > 0.0) {
+    float t = 0.f;
+    for (int k = 0; k < kLzThreads / 32; ++k) t += fred[k];
+    f32 = t <= 0x1p-30f;
+  }
+  const int slice = SL == 1 ? 0 : warp;
+  constexpr int TILE = kLzThreads / SL;
+  const int rowin = SL == 1 ? static_cast<int>(threadIdx.x) : lane;
+  double s2 = 0.0;
+  for (int64_t r0 = static_cast<int64_t>(blockIdx.x) * TILE; r0 < n; r0 += static_cast<int64_t>(gridDim.x) * TILE) {
+    const int64_t i = r0 + rowin;
+    T t = lz_zero<T>();
+    F tf = LzFloat<T>::zero();
+    if (i < n) {
+      const T* ui = U + i;
+      if (f32) {
+#pragma unroll 8
+        for (int q = slice; q < nc; q += SL) tf = lz_fma(lz_to_float(ui[static_cast<int64_t>(q) * n]), hf[q], tf);
+      } else {
+#pragma unroll 4
+        for (int q = slice; q < nc; q += SL) t = lz_fma(ui[static_cast<int64_t>(q) * n], hs[q], t);
+      }
+    }
+    if constexpr (SL > 1) {
+      if (f32)
+        reinterpret_cast<F&>(part[slice][lane]) = tf;
+      else
+        part[slice][lane] = t;
+      __syncthreads();
+      if (slice == 0) {
+        for (int k = 1; k < SL; ++k) {
+          if (f32)
+            lz_add(tf, reinterpret_cast<F&>(part[k][lane]));
+          else
+            lz_add(t, part[k][lane]);
+        }
+      }
+    }
+    if (slice == 0 && i < n) {
+      T v = w[i];
+      if (f32)
+        v = lz_add_scaled(v, tf, -unscale);
+      else
+        lz_sub(v, t);
+      w[i] = v;
+      s2 = lz_abs2_fma(v, s2);
+    }
+    if constexpr (SL > 1) __syncthreads();
+  }
+  if (mode == 2) return;
+  s2 = lz_warp_sum(s2);
+  if (lane == 0) red[warp] = s2;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = red[0];
+    for (int k = 1; k < kLzThreads / 32; ++k) t += red[k];
+    npart[blockIdx.x] = t;
+  }
+  if (!lz_last_block(counter, gridDim.x)) return;
+  const double nrm2 = lz_block_total<kLzThreads>(npart, static_cast<int>(gridDim.x));
+  if (threadIdx.x == 0) lz_finish(nrm2, h1, h, c, j, mode, alpha, beta, st);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kLzThreads) lz_scale_into(const T* __restrict__ w, int64_t n, T* __restrict__ u,
                                                             const LzState* st) {
@@ -343,6 +618,23 @@ __global__ void __launch_bounds__(kLzThreads) lz_scale_into(const T* __restrict_
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride)
     u[i] = lz_scale(w[i], s);
+}
+
+// What a convergence check reads, in one piece: the state of the step just
+// enqueued, alpha and beta of its J entries, the call's status.
+__global__ void lz_snapshot(const LzState* __restrict__ st, const double* __restrict__ alpha,
+                            const double* __restrict__ beta, int J, const int32_t* __restrict__ status,
+                            LzSnap* __restrict__ out) {
+  if (threadIdx.x == 0) {
+    out->stop = st->stop;
+    out->jdone = st->jdone;
+    out->status = *status;
+  }
+  double* v = reinterpret_cast<double*>(out + 1);
+  for (int i = threadIdx.x; i < J; i += blockDim.x) {
+    v[i] = alpha[i];
+    v[J + i] = beta[i];
+  }
 }
 
 // Gaussian start vector from Philox4x32-10: key = seed, counter =
@@ -365,73 +657,88 @@ __global__ void __launch_bounds__(kLzThreads) lz_start(T* __restrict__ w, int64_
 }
 
 // ---------------------------------------------------------------------------
-// tridiagonal eigenproblem of T_J (one block)
+// tridiagonal eigenproblem of T_J, on the host: the problem is a chain of a
+// few hundred dependent divisions per shift, which one SM's FP64 unit takes
+// milliseconds for (1.2 ms a check on average over n = 4096, up to 3.4 ms)
+// and a host core tens of microseconds, while the GPU runs the next steps.
 // ---------------------------------------------------------------------------
-// Number of eigenvalues of T_J below x (Sturm sequence of the LDL^T pivots).
-__device__ int lz_sturm(const double* __restrict__ a, const double* __restrict__ b, int J, double x, double pivmin) {
-  int cnt = 0;
-  double d = a[0] - x;
-  if (fabs(d) < pivmin) d = -pivmin;
-  cnt += d < 0.0;
+namespace {
+
+constexpr int kLzShifts = 8;  // shifts counted side by side (independent division chains)
+
+// Number of eigenvalues of T_J below each of the shifts (Sturm sequence of
+// the LDL^T pivots; b2 = squared off-diagonals).
+void lz_sturm(const double* a, const double* b2, int J, const double* x, double pivmin, int* cnt) {
+  double d[kLzShifts];
+  int c[kLzShifts];
+  for (int q = 0; q < kLzShifts; ++q) {
+    d[q] = a[0] - x[q];
+    if (std::fabs(d[q]) < pivmin) d[q] = -pivmin;
+    c[q] = d[q] < 0.0;
+  }
   for (int i = 1; i < J; ++i) {
-    d = (a[i] - x) - b[i - 1] * b[i - 1] / d;
-    if (fabs(d) < pivmin) d = -pivmin;
-    cnt += d < 0.0;
+    const double ai = a[i], bi = b2[i - 1];
+    for (int q = 0; q < kLzShifts; ++q) {
+      double v = (ai - x[q]) - bi / d[q];
+      v = std::fabs(v) < pivmin ? -pivmin : v;
+      c[q] += v < 0.0;
+      d[q] = v;
+    }
   }
-  return cnt;
+  for (int q = 0; q < kLzShifts; ++q) cnt[q] = c[q];
 }
 
-// One solve of (T - theta I) x = rhs by Gaussian elimination with partial
-// pivoting; x overwrites rhs.  Work arrays D, DL, DU, DU2, PV of length J.
-__device__ void lz_tri_solve(const double* __restrict__ a, const double* __restrict__ b, int J, double theta,
-                             double pivtol, double* D, double* DL, double* DU, double* DU2, double* PV,
-                             double* x) {
-  for (int i = 0; i < J; ++i) {
-    D[i] = a[i] - theta;
-    if (i + 1 < J) {
-      DL[i] = b[i];
-      DU[i] = b[i];
+// (T - theta I) = P L U by Gaussian elimination with partial pivoting, then
+// solves with it.
+struct LzTriLu {
+  std::vector<double> D, DL, DU, DU2;
+  std::vector<char> swapped;
+  void factor(const double* a, const double* b, int J, double theta, double pivtol) {
+    D.assign(J, 0.0);
+    DL.assign(J, 0.0);
+    DU.assign(J, 0.0);
+    DU2.assign(J, 0.0);
+    swapped.assign(J, 0);
+    for (int i = 0; i < J; ++i) {
+      D[i] = a[i] - theta;
+      if (i + 1 < J) DL[i] = DU[i] = b[i];
     }
-    DU2[i] = 0.0;
-  }
-  for (int i = 0; i + 1 < J; ++i) {
-    if (fabs(D[i]) >= fabs(DL[i])) {
-      if (fabs(D[i]) < pivtol) D[i] = D[i] < 0.0 ? -pivtol : pivtol;
-      const double f = DL[i] / D[i];
-      DL[i] = f;
-      D[i + 1] -= f * DU[i];
-      PV[i] = 0.0;
-    } else {
-      const double f = D[i] / DL[i];
-      D[i] = DL[i];
-      DL[i] = f;
-      const double t = DU[i];
-      DU[i] = D[i + 1];
-      D[i + 1] = t - f * D[i + 1];
-      if (i + 2 < J) {
-        DU2[i] = DU[i + 1];
-        DU[i + 1] = -f * DU[i + 1];
+    for (int i = 0; i + 1 < J; ++i) {
+      if (std::fabs(D[i]) >= std::fabs(DL[i])) {
+        if (std::fabs(D[i]) < pivtol) D[i] = D[i] < 0.0 ? -pivtol : pivtol;
+        const double f = DL[i] / D[i];
+        DL[i] = f;
+        D[i + 1] -= f * DU[i];
+      } else {
+        const double f = D[i] / DL[i];
+        D[i] = DL[i];
+        DL[i] = f;
+        const double t = DU[i];
+        DU[i] = D[i + 1];
+        D[i + 1] = t - f * D[i + 1];
+        if (i + 2 < J) {
+          DU2[i] = DU[i + 1];
+          DU[i + 1] = -f * DU[i + 1];
+        }
+        swapped[i] = 1;
       }
-      PV[i] = 1.0;
     }
+    if (std::fabs(D[J - 1]) < pivtol) D[J - 1] = D[J - 1] < 0.0 ? -pivtol : pivtol;
   }
-  if (fabs(D[J - 1]) < pivtol) D[J - 1] = D[J - 1] < 0.0 ? -pivtol : pivtol;
-  for (int i = 0; i + 1 < J; ++i) {
-    if (PV[i] != 0.0) {
-      const double t = x[i];
-      x[i] = x[i + 1];
-      x[i + 1] = t;
+  void solve(int J, double* x) const {
+    for (int i = 0; i + 1 < J; ++i) {
+      if (swapped[i]) std::swap(x[i], x[i + 1]);
+      x[i + 1] -= DL[i] * x[i];
     }
-    x[i + 1] -= DL[i] * x[i];
+    x[J - 1] /= D[J - 1];
+    if (J > 1) x[J - 2] = (x[J - 2] - DU[J - 2] * x[J - 1]) / D[J - 2];
+    for (int i = J - 3; i >= 0; --i) x[i] = (x[i] - DU[i] * x[i + 1] - DU2[i] * x[i + 2]) / D[i];
   }
-  x[J - 1] /= D[J - 1];
-  if (J > 1) x[J - 2] = (x[J - 2] - DU[J - 2] * x[J - 1]) / D[J - 2];
-  for (int i = J - 3; i >= 0; --i) x[i] = (x[i] - DU[i] * x[i + 1] - DU2[i] * x[i + 2]) / D[i];
-}
+};
 
-__device__ void lz_normalize(double* x, int J) {
+void lz_normalize(double* x, int J) {
   double s = 0.0, mx = 0.0;
-  for (int i = 0; i < J; ++i) mx = fmax(mx, fabs(x[i]));
+  for (int i = 0; i < J; ++i) mx = std::max(mx, std::fabs(x[i]));
   if (!(mx > 0.0)) {
     x[0] = 1.0;
     return;
@@ -440,142 +747,133 @@ __device__ void lz_normalize(double* x, int J) {
     x[i] /= mx;
     s += x[i] * x[i];
   }
-  s = 1.0 / sqrt(s);
+  s = 1.0 / std::sqrt(s);
   for (int i = 0; i < J; ++i) x[i] *= s;
 }
 
-// p largest eigenvalues of T_J, their eigenvectors X[w * ldx + k], residual
-// bounds and the convergence verdict.  256 threads; warp w < p bisects the
-// w-th largest eigenvalue with 32-point multisection.
-__global__ void __launch_bounds__(256) lz_tridiag(const double* __restrict__ alpha, const double* __restrict__ beta,
-                                                  int p, double tol, int ldx, double* __restrict__ X,
-                                                  double* __restrict__ work, const LzState* st,
-                                                  LzCheck* __restrict__ out) {
-  __shared__ double s_lo, s_hi, s_theta[kLzWant];
-  __shared__ double red_lo[8], red_hi[8];
-  const int J = st->jdone;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (J <= 0) {
-    if (tid == 0) {
-      out->J = 0;
-      out->converged = 0;
-      out->breakdown = st->stop;
-      out->nvalid = 0;
-    }
-    return;
+// The p largest eigenvalues of T_J (multisection on Sturm counts), their
+// eigenvectors X[w * J + k] (three rounds of inverse iteration, Gram-Schmidt
+// inside clusters), residual bounds and the convergence verdict.  `out` holds
+// the previous check of the same run on entry (nvalid = 0 at its first): its
+// Ritz values and residuals give the first shifts, which narrows the interval
+// but decides nothing.
+void lz_tridiag(const double* a, const double* b, int J, int p, double tol, std::vector<double>* Xout,
+                LzCheck* out) {
+  const LzCheck prev = *out;
+  double lo = INFINITY, hi = -INFINITY;  // Gershgorin interval
+  std::vector<double> b2(J);
+  for (int i = 0; i < J; ++i) {
+    const double r = (i > 0 ? std::fabs(b[i - 1]) : 0.0) + (i + 1 < J ? std::fabs(b[i]) : 0.0);
+    lo = std::min(lo, a[i] - r);
+    hi = std::max(hi, a[i] + r);
+    b2[i] = b[i] * b[i];
   }
-  // Gershgorin interval of T_J
-  double lo = INFINITY, hi = -INFINITY;
-  for (int i = tid; i < J; i += blockDim.x) {
-    const double r = (i > 0 ? fabs(beta[i - 1]) : 0.0) + (i + 1 < J ? fabs(beta[i]) : 0.0);
-    lo = fmin(lo, alpha[i] - r);
-    hi = fmax(hi, alpha[i] + r);
-  }
-  for (int m = 16; m > 0; m >>= 1) {
-    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, m));
-    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, m));
-  }
-  if (lane == 0) {
-    red_lo[warp] = lo;
-    red_hi[warp] = hi;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    double a = red_lo[0], c = red_hi[0];
-    for (int k = 1; k < 8; ++k) {
-      a = fmin(a, red_lo[k]);
-      c = fmax(c, red_hi[k]);
-    }
-    s_lo = a;
-    s_hi = c;
-  }
-  __syncthreads();
-  const double tn = fmax(fmax(fabs(s_lo), fabs(s_hi)), DBL_MIN);
-  const double pivmin = DBL_MIN * fmax(1.0, tn * tn);
-  const int nwant = min(p, J);
-  if (warp < nwant) {
-    const int k = J - 1 - warp;  // 0-based ascending index
-    double l = s_lo - 1e-12 * tn - pivmin, h = s_hi + 1e-12 * tn + pivmin;
+  const double tn = std::max(std::max(std::fabs(lo), std::fabs(hi)), DBL_MIN);
+  const double pivmin = DBL_MIN * std::max(1.0, tn * tn);
+  const int nwant = std::min(p, J);
+  double theta[kLzWant];
+  for (int w = 0; w < nwant; ++w) {
+    const int k = J - 1 - w;  // 0-based ascending index
+    double l = lo - 1e-12 * tn - pivmin, h = hi + 1e-12 * tn + pivmin;
     for (int round = 0; round < 64; ++round) {
-      if (h - l <= 4.0 * DBL_EPSILON * fmax(fabs(l), fabs(h)) + pivmin) break;
-      const double x = l + (h - l) * static_cast<double>(lane + 1) / 33.0;
-      const int cnt = lz_sturm(alpha, beta, J, x, pivmin);
-      double nl = cnt <= k ? x : -INFINITY;
-      double nh = cnt >= k + 1 ? x : INFINITY;
-      for (int m = 16; m > 0; m >>= 1) {
-        nl = fmax(nl, __shfl_xor_sync(0xffffffffu, nl, m));
-        nh = fmin(nh, __shfl_xor_sync(0xffffffffu, nh, m));
+      if (h - l <= 4.0 * DBL_EPSILON * std::max(std::fabs(l), std::fabs(h)) + pivmin) break;
+      double x[kLzShifts];
+      int cnt[kLzShifts];
+      if (round == 0 && w < prev.nvalid) {
+        double step = 1.1 * prev.res[w] + 8.0 * DBL_EPSILON * tn;
+        x[0] = prev.theta[w] - 8.0 * DBL_EPSILON * tn;
+        for (int q = 1; q < kLzShifts; ++q, step *= 16.0) x[q] = prev.theta[w] + step;
+        for (int q = 0; q < kLzShifts; ++q) x[q] = std::min(std::max(x[q], l), h);
+      } else {
+        for (int q = 0; q < kLzShifts; ++q) x[q] = l + (h - l) * static_cast<double>(q + 1) / (kLzShifts + 1.0);
       }
-      if (nl > l) l = nl;
-      if (nh < h) h = nh;
+      lz_sturm(a, b2.data(), J, x, pivmin, cnt);
+      for (int q = 0; q < kLzShifts; ++q) {
+        if (cnt[q] <= k)
+          l = std::max(l, x[q]);
+        else
+          h = std::min(h, x[q]);
+      }
     }
-    if (lane == 0) s_theta[warp] = 0.5 * (l + h);
+    theta[w] = 0.5 * (l + h);
   }
-  __syncthreads();
-  // inverse iteration, three rounds, with Gram-Schmidt inside clusters
   const double pivtol = DBL_EPSILON * tn;
+  std::vector<double>& X = *Xout;
+  X.assign(static_cast<size_t>(nwant) * J, 0.0);
+  std::vector<LzTriLu> lu(nwant);
   for (int it = 0; it < 3; ++it) {
-    if (tid < nwant) {
-      double* x = X + static_cast<int64_t>(tid) * ldx;
-      double* wk = work + static_cast<int64_t>(tid) * 5 * ldx;
-      if (it == 0)
-        for (int i = 0; i < J; ++i) x[i] = 1.0 + 0.01 * static_cast<double>((i * 7 + tid * 3) % 11);
-      const double shift = s_theta[tid] + 2.0 * DBL_EPSILON * tn;
-      lz_tri_solve(alpha, beta, J, shift, pivtol, wk, wk + ldx, wk + 2 * ldx, wk + 3 * ldx, wk + 4 * ldx, x);
+    for (int w = 0; w < nwant; ++w) {
+      double* x = X.data() + static_cast<size_t>(w) * J;
+      if (it == 0) {
+        for (int i = 0; i < J; ++i) x[i] = 1.0 + 0.01 * static_cast<double>((i * 7 + w * 3) % 11);
+        lu[w].factor(a, b, J, theta[w] + 2.0 * DBL_EPSILON * tn, pivtol);
+      }
+      lu[w].solve(J, x);
       lz_normalize(x, J);
     }
-    __syncthreads();
-    if (tid == 0) {
-      for (int a = 1; a < nwant; ++a)
-        for (int c = 0; c < a; ++c) {
-          if (fabs(s_theta[a] - s_theta[c]) > 1e-3 * tn) continue;
-          double* xa = X + static_cast<int64_t>(a) * ldx;
-          const double* xc = X + static_cast<int64_t>(c) * ldx;
-          double d = 0.0;
-          for (int i = 0; i < J; ++i) d += xa[i] * xc[i];
-          for (int i = 0; i < J; ++i) xa[i] -= d * xc[i];
-          lz_normalize(xa, J);
-        }
-    }
-    __syncthreads();
+    for (int w = 1; w < nwant; ++w)
+      for (int c = 0; c < w; ++c) {
+        if (std::fabs(theta[w] - theta[c]) > 1e-3 * tn) continue;
+        double* xa = X.data() + static_cast<size_t>(w) * J;
+        const double* xc = X.data() + static_cast<size_t>(c) * J;
+        double d = 0.0;
+        for (int i = 0; i < J; ++i) d += xa[i] * xc[i];
+        for (int i = 0; i < J; ++i) xa[i] -= d * xc[i];
+        lz_normalize(xa, J);
+      }
   }
-  if (tid == 0) {
-    const double bJ = beta[J - 1];
-    int conv = 1;
-    for (int a = 0; a < nwant; ++a) {
-      const double r = fabs(bJ) * fabs(X[static_cast<int64_t>(a) * ldx + J - 1]);
-      out->theta[a] = s_theta[a];
-      out->res[a] = r;
-      if (!(r <= tol * tn)) conv = 0;
+  int conv = 1;
+  for (int w = 0; w < nwant; ++w) {
+    const double r = std::fabs(b[J - 1]) * std::fabs(X[static_cast<size_t>(w) * J + J - 1]);
+    out->theta[w] = theta[w];
+    out->res[w] = r;
+    if (!(r <= tol * tn)) conv = 0;
+  }
+  out->J = J;
+  out->nvalid = nwant;
+  out->converged = conv && nwant == p;
+  out->tnorm = tn;
+}
+
+}  // namespace
+
+// Y[a] = sum_k U_{c0+k} X[a][k] for a < P (Ritz vectors), a thread per row;
+// P is a template argument so that a row costs P FMAs a basis vector and the
+// loads of four vectors are in flight (n = 10^6, P = 3, J = 78: 0.49 ms, 1.36 ms with
+// P <= 8 predicated).
+template <int P, typename T>
+__global__ void __launch_bounds__(kLzThreads) lz_ritz(const T* __restrict__ U, int64_t n, int c0, int J,
+                                                      const double* __restrict__ X, T* __restrict__ Y) {
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
+    T acc[P];
+#pragma unroll
+    for (int a = 0; a < P; ++a) acc[a] = lz_zero<T>();
+    const T* u0 = U + static_cast<int64_t>(c0) * n + i;
+#pragma unroll 4
+    for (int k = 0; k < J; ++k) {
+      const T u = u0[static_cast<int64_t>(k) * n];
+#pragma unroll
+      for (int a = 0; a < P; ++a) acc[a] = lz_scale_fma(u, X[static_cast<int64_t>(a) * J + k], acc[a]);
     }
-    out->J = J;
-    out->nvalid = nwant;
-    out->breakdown = st->stop;
-    out->converged = conv && nwant == p;
-    out->tnorm = tn;
+#pragma unroll
+    for (int a = 0; a < P; ++a) Y[static_cast<int64_t>(a) * n + i] = acc[a];
   }
 }
 
-// Y[a] = sum_k U_{c0+k} X[a][k] for a < p (Ritz vectors), a thread per row.
 template <typename T>
-__global__ void __launch_bounds__(kLzThreads) lz_ritz(const T* __restrict__ U, int64_t n, int c0, int J,
-                                                      const double* __restrict__ X, int ldx, int p,
-                                                      T* __restrict__ Y) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
-    T acc[kLzWant];
-#pragma unroll
-    for (int a = 0; a < kLzWant; ++a) acc[a] = lz_zero<T>();
-    for (int k = 0; k < J; ++k) {
-      const T u = U[static_cast<int64_t>(c0 + k) * n + i];
-#pragma unroll
-      for (int a = 0; a < kLzWant; ++a)
-        if (a < p) lz_add(acc[a], lz_scale(u, X[static_cast<int64_t>(a) * ldx + k]));
-    }
-#pragma unroll
-    for (int a = 0; a < kLzWant; ++a)
-      if (a < p) Y[static_cast<int64_t>(a) * n + i] = acc[a];
+void lz_launch_ritz(int p, int blocks, cudaStream_t st, const T* U, int64_t n, int c0, int J, const double* X, T* Y) {
+  switch (p) {
+    case 1: lz_ritz<1, T><<<blocks, kLzThreads, 0, st>>>(U, n, c0, J, X, Y); break;
+    case 2: lz_ritz<2, T><<<blocks, kLzThreads, 0, st>>>(U, n, c0, J, X, Y); break;
+    case 3: lz_ritz<3, T><<<blocks, kLzThreads, 0, st>>>(U, n, c0, J, X, Y); break;
+    case 4: lz_ritz<4, T><<<blocks, kLzThreads, 0, st>>>(U, n, c0, J, X, Y); break;
+    case 5: lz_ritz<5, T><<<blocks, kLzThreads, 0, st>>>(U, n, c0, J, X, Y); break;
+    case 6: lz_ritz<6, T><<<blocks, kLzThreads, 0, st>>>(U, n, c0, J, X, Y); break;
+    case 7: lz_ritz<7, T><<<blocks, kLzThreads, 0, st>>>(U, n, c0, J, X, Y); break;
+    default: lz_ritz<8, T><<<blocks, kLzThreads, 0, st>>>(U, n, c0, J, X, Y); break;
   }
+  count_launch();
 }
 
 struct LzOutput {
@@ -640,8 +938,8 @@ struct LzPlan {
   int64_t n;
   int r, maxit, lmax, cap, nch, chunk, ldx;
   size_t esz;
-  size_t off_U, off_w, off_Y, off_part, off_h1, off_h2, off_npart, off_alpha, off_beta, off_state, off_check, off_X,
-      off_work, off_deg, off_snap, total;
+  size_t off_U, off_w, off_Y, off_part, off_h1, off_h2, off_npart, off_alpha, off_beta, off_state, off_X, off_deg,
+      off_snap, off_count, off_two, total;
 };
 
 size_t lz_take(size_t& cur, size_t bytes) {
@@ -656,9 +954,11 @@ void lz_plan(int64_t n, int r, int maxit, bool cplx, LzPlan* p) {
   p->maxit = maxit;
   p->lmax = 2 * r + 8;                    // locked vectors (repeated eigenvalues need extra slots)
   p->cap = p->lmax + maxit + 1;           // basis columns
-  // about two row chunks per SM, 256 to 4096 rows each
+  // about two row chunks per SM, 512 (four rows a thread, which pay for the
+  // block's sums) to 4096 rows each
   p->chunk = static_cast<int>(std::min<int64_t>(
-      kLzChunkMax, std::max<int64_t>(256, static_cast<int64_t>(align_up(ceil_div(n, 2 * 152), 256)))));
+      kLzChunkMax,
+      std::max<int64_t>(4 * kLzDotThreads, static_cast<int64_t>(align_up(ceil_div(n, 2 * 152), kLzDotThreads)))));
   p->nch = static_cast<int>(ceil_div(n, p->chunk));
   p->ldx = maxit + 1;
   p->esz = cplx ? sizeof(double2) : sizeof(double);
@@ -669,15 +969,16 @@ void lz_plan(int64_t n, int r, int maxit, bool cplx, LzPlan* p) {
   p->off_part = lz_take(cur, static_cast<size_t>(p->cap) * p->nch * p->esz);
   p->off_h1 = lz_take(cur, static_cast<size_t>(p->cap) * p->esz);
   p->off_h2 = lz_take(cur, static_cast<size_t>(p->cap) * p->esz);
-  p->off_npart = lz_take(cur, static_cast<size_t>(p->nch) * sizeof(double));
+  p->off_npart = lz_take(cur, static_cast<size_t>(kLzMaxBlocks) * sizeof(double));
   p->off_alpha = lz_take(cur, static_cast<size_t>(p->ldx) * sizeof(double));
   p->off_beta = lz_take(cur, static_cast<size_t>(p->ldx) * sizeof(double));
   p->off_state = lz_take(cur, sizeof(LzState));
-  p->off_check = lz_take(cur, sizeof(LzCheck));
   p->off_X = lz_take(cur, static_cast<size_t>(kLzWant) * p->ldx * sizeof(double));
-  p->off_work = lz_take(cur, static_cast<size_t>(kLzWant) * 5 * p->ldx * sizeof(double));
   p->off_deg = lz_take(cur, cplx ? 0 : static_cast<size_t>(n) * sizeof(double));  // Laplacian degrees
-  p->off_snap = lz_take(cur, sizeof(LzState));  // the state a convergence check reads
+  p->off_snap = lz_take(cur, sizeof(LzSnap) + 2 * static_cast<size_t>(p->ldx) * sizeof(double));
+  // arrival counters: matvec, three-term step, update, then one per vector group of lz_dots
+  p->off_count = lz_take(cur, (3 + static_cast<size_t>(ceil_div(p->cap, kLzGroup))) * sizeof(unsigned));
+  p->off_two = lz_take(cur, 2 * static_cast<size_t>(kLzMaxBlocks) * p->esz);  // the operator's block sums
   p->total = cur;
 }
 
@@ -703,7 +1004,6 @@ struct LzRun {
   cudaStream_t st;
   cudaStream_t side;  // convergence checks run here, beside the next Lanczos steps
   cudaEvent_t ev;     // step done (the check waits for it)
-  cudaEvent_t done;   // check done (the host polls it)
 
   T* U() const { return reinterpret_cast<T*>(ws + p.off_U); }
   T* col(int c) const { return U() + static_cast<int64_t>(c) * n; }
@@ -716,81 +1016,100 @@ struct LzRun {
   double* alpha() const { return reinterpret_cast<double*>(ws + p.off_alpha); }
   double* beta() const { return reinterpret_cast<double*>(ws + p.off_beta); }
   LzState* state() const { return reinterpret_cast<LzState*>(ws + p.off_state); }
-  LzCheck* check() const { return reinterpret_cast<LzCheck*>(ws + p.off_check); }
   double* X() const { return reinterpret_cast<double*>(ws + p.off_X); }
-  double* work() const { return reinterpret_cast<double*>(ws + p.off_work); }
   double* deg() const { return reinterpret_cast<double*>(ws + p.off_deg); }
-  LzState* snap() const { return reinterpret_cast<LzState*>(ws + p.off_snap); }
+  LzSnap* snap() const { return reinterpret_cast<LzSnap*>(ws + p.off_snap); }
+  unsigned* counter(int i) const { return reinterpret_cast<unsigned*>(ws + p.off_count) + i; }
+  T* two() const { return reinterpret_cast<T*>(ws + p.off_two); }
 
-  void matvec(const T* x, T* y) const;
+  // y = Q x, h1()[0] = uprev^H y (uprev may be NULL), h1()[1] = x^H y
+  void matvec(const T* x, T* y, const T* uprev) const;
   void prepare() const;  // operator set-up once per truncation (Laplacian degrees)
 
-  // w -= U[:, first:first+nc] (U[:, first:first+nc]^H w), projections into
-  // h[first:first+nc]
-  void project(int first, int nc, T* h) const {
-    if (nc <= 0) return;
-    dim3 g(p.nch, static_cast<unsigned>(ceil_div(nc, kLzGroup)));
-    lz_dots<T><<<g, kLzThreads, 0, st>>>(col(first), n, nc, w(), part(), p.nch, p.chunk, state());
-    lz_reduce<T><<<static_cast<unsigned>(ceil_div(static_cast<int64_t>(nc) * 32, 256)), 256, 0, st>>>(
-        part(), nc, p.nch, h + first, state());
-    lz_update<T><<<static_cast<unsigned>(std::min<int64_t>(ceil_div(n, 32), 152 * 16)), kLzThreads, 0, st>>>(
-        col(first), n, nc, h + first, w(), state());
-    count_launch(3);
+  // h2() = U[:, :nc]^H w, w -= U[:, :nc] h2(), then by mode (lz_update): 0
+  // closes Lanczos step j (column nc - 1), 1 normalises a start vector, 2
+  // nothing more.
+  int project(int nc, int j, int mode) const {
+    if (nc > 0) {
+      dim3 g(p.nch, static_cast<unsigned>(ceil_div(nc, kLzGroup)));
+      lz_dots<T><<<g, kLzDotThreads, 0, st>>>(U(), n, nc, w(), part(), p.nch, p.chunk, counter(3), h2(), state());
+      count_launch();
+    }
+    using F = typename LzFloat<T>::type;
+    const size_t smem = static_cast<size_t>(nc) * (sizeof(T) + sizeof(F));
+    // eight warps a tile of 32 rows until the rows fill the chip by themselves
+    const bool wide = n >= static_cast<int64_t>(152) * 4 * kLzThreads;
+    const auto kern = wide ? lz_update<1, T> : lz_update<8, T>;
+    const int tile = wide ? kLzThreads : 32;
+    if (smem > 40 * 1024) {
+      int e = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              static_cast<int>(smem)),
+                         "lz_update shared memory");
+      if (e) return e;
+    }
+    const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(n, tile), 152 * 8));
+    kern<<<blocks, kLzThreads, smem, st>>>(U(), n, nc, h2(), w(), npart(), counter(2), mode, mode == 0 ? 1 : 0, h1(),
+                                           nc - 1, j, alpha(), beta(), state());
+    count_launch();
+    return LRQ_OK;
   }
-  // normalise w into column c; mode 0 closes Lanczos step j (column c - 1)
-  void close(int c, int j, int mode) const {
-    lz_norm_partial<T><<<p.nch, kLzThreads, 0, st>>>(w(), n, npart(), p.chunk, state());
-    lz_finish<T><<<1, 32, 0, st>>>(npart(), p.nch, h1(), h2(), c - 1, j, mode, alpha(), beta(), state());
+  void scale(int c) const {  // column c = w / ||w||
     lz_scale_into<T><<<lz_rows_grid(n), kLzThreads, 0, st>>>(w(), n, col(c), state());
-    count_launch(3);
+    count_launch();
   }
-  // A convergence check reads alpha, beta and a snapshot of the state of
-  // step J and runs on the side stream, so the next Lanczos steps (which
-  // only append to alpha, beta and the basis) proceed meanwhile; its verdict
-  // is read kLzLag steps later: the host waits for it with those steps
-  // queued, so the GPU is not left idle and at most kLzLag steps run past
-  // convergence.
-  int launch_check(int p_want) const {
-    int e = cuda_check(cudaMemcpyAsync(snap(), state(), sizeof(LzState), cudaMemcpyDeviceToDevice, st),
-                       "snapshot state");
+  // A convergence check takes alpha, beta and the state as they are after
+  // step J (lz_snapshot) to the host, on the side stream, so the next Lanczos
+  // steps proceed meanwhile; its verdict is worked out kLzLag steps later: the
+  // host waits for the copy with those steps queued, so the GPU is not left
+  // idle and at most kLzLag steps run past convergence.
+  int launch_check(int J) const {
+    lz_snapshot<<<1, 256, 0, st>>>(state(), alpha(), beta(), J, status, snap());
+    count_launch();
+    int e = cuda_check(cudaGetLastError(), "lanczos step kernels");
     if (e) return e;
     if ((e = cuda_check(cudaEventRecord(ev, st), "record step event"))) return e;
-    if ((e = cuda_check(cudaStreamWaitEvent(side, ev, 0), "order check after step"))) return e;
-    lz_tridiag<<<1, 256, 0, side>>>(alpha(), beta(), p_want, tol, p.ldx, X(), work(), snap(), check());
-    count_launch();
-    if ((e = cuda_check(cudaGetLastError(), "lz_tridiag"))) return e;
-    return cuda_check(cudaEventRecord(done, side), "record check event");
+    return cuda_check(cudaStreamWaitEvent(side, ev, 0), "order check after step");
   }
-  int finish_check(LzCheck* hc) const {
-    int32_t hs = 0;
-    int e = cuda_check(cudaEventSynchronize(done), "wait for the check");
+  int finish_check(int J, int p_want, std::vector<double>* buf, std::vector<double>* x, LzCheck* hc) const {
+    buf->resize(sizeof(LzSnap) / sizeof(double) + 2 * static_cast<size_t>(J));
+    int e = cuda_check(cudaMemcpyAsync(buf->data(), snap(), buf->size() * sizeof(double), cudaMemcpyDeviceToHost,
+                                       side),
+                       "copy check");
     if (e) return e;
-    if ((e = cuda_check(cudaMemcpyAsync(hc, check(), sizeof(LzCheck), cudaMemcpyDeviceToHost, side), "copy check")))
-      return e;
-    if (e) return e;
-    if ((e = cuda_check(cudaMemcpyAsync(&hs, status, sizeof(int32_t), cudaMemcpyDeviceToHost, side),
-                        "copy status")))
-      return e;
     if ((e = cuda_check(cudaStreamSynchronize(side), "lanczos sync"))) return e;
-    if (hs != 0) return fail(hs, "lrq_truncate: the device reported an invalid input or error");
+    LzSnap hs;
+    std::memcpy(&hs, buf->data(), sizeof(hs));
+    if (hs.status != 0) return fail(hs.status, "lrq_truncate: the device reported an invalid input or error");
+    const double* a = buf->data() + sizeof(LzSnap) / sizeof(double);
+    if (hs.jdone > 0) {
+      lz_tridiag(a, a + J, std::min(hs.jdone, J), p_want, tol, x, hc);
+    } else {
+      hc->J = hc->converged = hc->nvalid = 0;
+    }
+    hc->breakdown = hs.stop;
     return LRQ_OK;
   }
 
   // One Lanczos run against the L locked vectors; wants the p largest
   // eigenpairs of the deflated operator.
-  int run(int L, int p_want, int run_id, LzCheck* hc, int64_t* steps) const {
+  int run(int L, int p_want, int run_id, LzCheck* hc, std::vector<double>* x, int64_t* steps) const {
     int e = cuda_check(cudaMemsetAsync(state(), 0, sizeof(LzState), st), "memset state");
     if (e) return e;
+    if ((e = cuda_check(cudaMemsetAsync(counter(0), 0, (3 + ceil_div(p.cap, kLzGroup)) * sizeof(unsigned), st),
+                        "memset counters")))
+      return e;
+    std::memset(hc, 0, sizeof(*hc));
+    std::vector<double> buf;
     lz_start<T><<<lz_rows_grid(n), kLzThreads, 0, st>>>(w(), n, seed, run_id, state());
     count_launch();
-    project(0, L, h1());
-    project(0, L, h2());
-    close(L, 0, 1);
+    if (L > 0 && (e = project(L, 0, 2))) return e;
+    if ((e = project(L, 0, 1))) return e;
+    scale(L);
     int pending = 0, since = 0;  // a check in flight, and steps taken since it started
     // the verdict of the check in flight: 1 = this run is over, 0 = go on
     auto verdict = [&](int* over) -> int {
+      const int e2 = finish_check(pending, p_want, &buf, x, hc);
       pending = 0;
-      int e2 = finish_check(hc);
       if (e2) return e2;
       if (hc->breakdown == 2) hc->nvalid = 0;  // the start vector had no part outside the locked space
       *over = hc->breakdown || hc->converged || L + hc->J >= n;
@@ -798,17 +1117,17 @@ struct LzRun {
     };
     for (int j = 0; j < p.maxit && L + j < n; ++j) {
       const int c = L + j;
-      matvec(col(c), w());
+      const T* uprev = j > 0 ? col(c - 1) : nullptr;
+      matvec(col(c), w(), uprev);
       // the three-term step: the large components of w = Q u_j lie along u_j
       // and u_{j-1}; taking them out first leaves components of rounding size
       // along every other stored vector, which one full Gram-Schmidt pass then
-      // removes (alpha_j = h1[c] + h2[c])
-      if (j > 0)
-        project(c - 1, 2, h1());
-      else
-        project(c, 1, h1());
-      project(0, c + 1, h2());
-      close(c + 1, j, 0);
+      // removes (alpha_j = h1[1] + h2[c])
+      lz_threeterm<T><<<lz_rows_grid(n), kLzThreads, 0, st>>>(w(), n, uprev, col(c), h1(), npart(), counter(1),
+                                                              state());
+      count_launch();
+      if ((e = project(c + 1, j, 0))) return e;
+      scale(c + 1);
       ++*steps;
       ++since;
       const int J = j + 1;
@@ -821,7 +1140,7 @@ struct LzRun {
         if (over) return LRQ_OK;
       }
       if (due || last) {
-        if ((e = launch_check(p_want))) return e;
+        if ((e = launch_check(J))) return e;
         pending = J;
         since = 0;
       }
@@ -846,7 +1165,8 @@ struct LzRun {
       if (!verify && L >= r) verify = true;
       const int p_want = verify ? 1 : static_cast<int>(std::min<int64_t>(r - L, n - L));
       LzCheck hc;
-      if ((e = run(L, p_want, run_id++, &hc, &steps))) return e;
+      std::vector<double> x;  // the wanted eigenvectors of T
+      if ((e = run(L, p_want, run_id++, &hc, &x, &steps))) return e;
       if (hc.nvalid <= 0) break;
       tn = std::max(tn, hc.tnorm);
       if (verify) {
@@ -859,8 +1179,11 @@ struct LzRun {
       }
       const int q = verify ? 1 : hc.nvalid;
       if (L + q > p.lmax) return fail(LRQ_ENOCONV, "lrq_truncate: more repeated eigenvalues than locking slots");
-      lz_ritz<T><<<lz_rows_grid(n), kLzThreads, 0, st>>>(U(), n, L, hc.J, X(), p.ldx, q, Y());
-      count_launch();
+      if ((e = cuda_check(cudaMemcpyAsync(X(), x.data(), static_cast<size_t>(q) * hc.J * sizeof(double),
+                                          cudaMemcpyHostToDevice, st),
+                          "copy eigenvectors of T")))
+        return e;
+      lz_launch_ritz<T>(q, lz_rows_grid(n), st, U(), n, L, hc.J, X(), Y());
       if ((e = cuda_check(cudaMemcpyAsync(col(L), Y(), static_cast<size_t>(q) * n * sizeof(T),
                                           cudaMemcpyDeviceToDevice, st),
                           "copy Ritz vectors")))
@@ -900,8 +1223,9 @@ struct LzRun {
 };
 
 template <>
-void LzRun<double>::matvec(const double* x, double* y) const {
-  lz_matvec_laplacian<<<lz_rows_grid(n), kLzThreads, 0, st>>>(rowptr, colidx, wts, deg(), n, nnz, x, y, state());
+void LzRun<double>::matvec(const double* x, double* y, const double* uprev) const {
+  lz_matvec_laplacian<<<lz_rows_grid(n), kLzThreads, 0, st>>>(rowptr, colidx, wts, deg(), n, nnz, x, y, uprev, two(),
+                                                              counter(0), h1(), state());
   count_launch();
 }
 
@@ -915,9 +1239,14 @@ template <>
 void LzRun<double2>::prepare() const {}
 
 template <>
-void LzRun<double2>::matvec(const double2* x, double2* y) const {
-  const int blocks = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 8), 152 * 16)));
-  lz_matvec_dense<<<blocks, kLzThreads, 0, st>>>(Q, n, ld, x, y, state());
+void LzRun<double2>::matvec(const double2* x, double2* y, const double2* uprev) const {
+  // two rows a warp once every SM has a few warps that way
+  const int rows = n >= 152 * 4 ? 2 : 1;
+  const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(n, rows * (kLzMvThreads / 32)), kLzMaxBlocks));
+  if (rows == 2)
+    lz_matvec_dense<2><<<blocks, kLzMvThreads, 0, st>>>(Q, n, ld, x, y, uprev, two(), counter(0), h1(), state());
+  else
+    lz_matvec_dense<1><<<blocks, kLzMvThreads, 0, st>>>(Q, n, ld, x, y, uprev, two(), counter(0), h1(), state());
   count_launch();
 }
 
@@ -953,16 +1282,14 @@ namespace {
 // the side stream and event of one truncation call, released on every path
 struct LzSide {
   cudaStream_t side = nullptr;
-  cudaEvent_t ev = nullptr, done = nullptr;
+  cudaEvent_t ev = nullptr;
   int init() {
     int e = cuda_check(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking), "create check stream");
     if (e) return e;
-    if ((e = cuda_check(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "create step event"))) return e;
-    return cuda_check(cudaEventCreateWithFlags(&done, cudaEventDisableTiming), "create check event");
+    return cuda_check(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "create step event");
   }
   ~LzSide() {
     if (side) cudaStreamSynchronize(side);
-    if (done) cudaEventDestroy(done);
     if (ev) cudaEventDestroy(ev);
     if (side) cudaStreamDestroy(side);
   }
@@ -994,7 +1321,6 @@ int launch_truncate(const lrq_matrix* Q, int r, double tol, int max_iter, uint64
     R.st = st;
     R.side = sd.side;
     R.ev = sd.ev;
-    R.done = sd.done;
     lz_check_dense<<<lz_rows_grid(Q->n * Q->n), kLzThreads, 0, st>>>(R.Q, Q->n, Q->ld, status);
     count_launch();
     return R.solve(r, lambda_out, V, V32, iters_out);
@@ -1016,7 +1342,6 @@ int launch_truncate(const lrq_matrix* Q, int r, double tol, int max_iter, uint64
   R.st = st;
   R.side = sd.side;
   R.ev = sd.ev;
-  R.done = sd.done;
   lz_check_csr<<<lz_rows_grid(std::max<int64_t>(Q->n, Q->nnz)), kLzThreads, 0, st>>>(Q->rowptr, Q->colidx,
                                                                                      Q->weights, Q->n, Q->nnz,
                                                                                      status);
