@@ -11,26 +11,59 @@
 
 namespace lrq {
 
-__global__ void cut_count_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
-                                 int64_t n, const uint8_t* __restrict__ z, unsigned long long* __restrict__ out) {
-  __shared__ unsigned long long red[256];
+// A thread takes a row of up to kCutRowMax entries with four label gathers in
+// flight (they bound it), the warp longer rows together.
+constexpr int kCutRowMax = 64;
+
+__global__ void __launch_bounds__(256) cut_count_kernel(const int32_t* __restrict__ rowptr,
+                                                        const int32_t* __restrict__ colidx, int64_t n,
+                                                        const uint8_t* __restrict__ z,
+                                                        unsigned long long* __restrict__ out) {
+  __shared__ unsigned long long red[8];
+  const int lane = threadIdx.x & 31;
   unsigned long long cnt = 0;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const uint8_t zi = z[i];
-    const int32_t e1 = rowptr[i + 1];
-    for (int32_t e = rowptr[i]; e < e1; ++e) {
-      const int32_t j = colidx[e];
-      cnt += (j > i && z[j] != zi) ? 1ull : 0ull;
+  for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + (threadIdx.x & ~31); i0 < n; i0 += stride) {
+    const int64_t i = i0 + lane;  // warp-uniform trips
+    uint8_t zi = 0;
+    int32_t e0 = 0, e1 = 0;
+    if (i < n) {
+      zi = z[i];
+      e0 = rowptr[i];
+      e1 = rowptr[i + 1];
+    }
+    const bool big = e1 > e0 && static_cast<int64_t>(e1) - e0 > kCutRowMax;
+    if (!big) {
+      for (int64_t e = e0; e < e1; e += 4) {
+        int32_t j[4];
+        uint8_t zj[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          j[u] = e1 - e > u ? colidx[e + u] : -1;
+          zj[u] = j[u] > i ? z[j[u]] : zi;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) cnt += zj[u] != zi ? 1ull : 0ull;
+      }
+    }
+    for (unsigned m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const int64_t ib = i0 + src, b1 = __shfl_sync(0xffffffffu, e1, src);
+      const uint8_t zb = static_cast<uint8_t>(__shfl_sync(0xffffffffu, static_cast<int>(zi), src));
+      for (int64_t e = static_cast<int64_t>(__shfl_sync(0xffffffffu, e0, src)) + lane; e < b1; e += 32) {
+        const int32_t j = colidx[e];
+        cnt += (j > ib && z[j] != zb) ? 1ull : 0ull;
+      }
     }
   }
-  red[threadIdx.x] = cnt;
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, m);
+  if (lane == 0) red[threadIdx.x >> 5] = cnt;
   __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) cnt += red[k];
+    atomicAdd(out, cnt);
   }
-  if (threadIdx.x == 0) atomicAdd(out, red[0]);
 }
 
 int launch_cut_count(const int32_t* rowptr, const int32_t* colidx, int64_t n, const uint8_t* z, int64_t* cut_out,
