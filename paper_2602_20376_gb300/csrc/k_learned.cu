@@ -607,15 +607,13 @@ int launch_features(const float2* V, int B, int64_t n, int r, const double* lamb
 }
 
 // BF16 mode on the tensor cores (k_mlp_tc.cu); FP32 mode on the CUDA cores
-static void gemm(cudaStream_t st, int M, int N, int K, const float* A, int lda, int ta, const float* Bm, int ldb,
-                 int tb, const float* bias, int relu, const float* mask, float* C, int ldc, int bf16) {
-  if (bf16) {
-    launch_mlp_gemm_tc(st, M, N, K, A, lda, ta, Bm, ldb, tb, bias, relu, mask, C, ldc);
-    return;
-  }
+static int gemm(cudaStream_t st, int M, int N, int K, const float* A, int lda, int ta, const float* Bm, int ldb,
+                int tb, const float* bias, int relu, const float* mask, float* C, int ldc, int bf16) {
+  if (bf16) return launch_mlp_gemm_tc(st, M, N, K, A, lda, ta, Bm, ldb, tb, bias, relu, mask, C, ldc);
   dim3 grid(static_cast<unsigned>(ceil_div(N, 32)), static_cast<unsigned>(ceil_div(M, 32)));
   mlp_gemm_kernel<<<grid, 256, 0, st>>>(M, N, K, A, lda, ta, Bm, ldb, tb, bias, relu, mask, C, ldc, 0);
   count_launch();
+  return LRQ_OK;
 }
 
 int launch_mlp_forward(const float* params, int F, int B, const float* X, float* H1, float* H2, float* O, int bf16,
@@ -626,9 +624,10 @@ int launch_mlp_forward(const float* params, int F, int B, const float* X, float*
   const float* b2 = W2 + kWidth * kWidth;
   const float* W3 = b2 + kWidth;
   const float* b3 = W3 + kWidth * kOut;
-  gemm(st, B, kWidth, F, X, F, 0, W1, kWidth, 0, b1, 1, nullptr, H1, kWidth, bf16);
-  gemm(st, B, kWidth, kWidth, H1, kWidth, 0, W2, kWidth, 0, b2, 1, nullptr, H2, kWidth, bf16);
-  gemm(st, B, kOut, kWidth, H2, kWidth, 0, W3, kOut, 0, b3, 0, nullptr, O, kOut, bf16);
+  int e;
+  if ((e = gemm(st, B, kWidth, F, X, F, 0, W1, kWidth, 0, b1, 1, nullptr, H1, kWidth, bf16))) return e;
+  if ((e = gemm(st, B, kWidth, kWidth, H1, kWidth, 0, W2, kWidth, 0, b2, 1, nullptr, H2, kWidth, bf16))) return e;
+  if ((e = gemm(st, B, kOut, kWidth, H2, kWidth, 0, W3, kOut, 0, b3, 0, nullptr, O, kOut, bf16))) return e;
   return cuda_check(cudaGetLastError(), "mlp forward");
 }
 
@@ -644,16 +643,18 @@ int launch_mlp_backward(const float* params, int F, int B, const float* X, const
   float* db3 = dW3 + kWidth * kOut;
   float* dH2 = scratch;
   float* dH1 = scratch + static_cast<int64_t>(B) * kWidth;
+  int e;
   // layer 3
-  gemm(st, kWidth, kOut, B, H2, kWidth, 1, dO, kOut, 0, nullptr, 0, nullptr, dW3, kOut, bf16);
+  if ((e = gemm(st, kWidth, kOut, B, H2, kWidth, 1, dO, kOut, 0, nullptr, 0, nullptr, dW3, kOut, bf16))) return e;
   colsum_f32_kernel<<<1, 256, 0, st>>>(dO, B, kOut, db3);
-  gemm(st, B, kWidth, kOut, dO, kOut, 0, W3, kOut, 1, nullptr, 0, H2, dH2, kWidth, bf16);
+  if ((e = gemm(st, B, kWidth, kOut, dO, kOut, 0, W3, kOut, 1, nullptr, 0, H2, dH2, kWidth, bf16))) return e;
   // layer 2
-  gemm(st, kWidth, kWidth, B, H1, kWidth, 1, dH2, kWidth, 0, nullptr, 0, nullptr, dW2, kWidth, bf16);
+  if ((e = gemm(st, kWidth, kWidth, B, H1, kWidth, 1, dH2, kWidth, 0, nullptr, 0, nullptr, dW2, kWidth, bf16)))
+    return e;
   colsum_f32_kernel<<<1, 256, 0, st>>>(dH2, B, kWidth, db2);
-  gemm(st, B, kWidth, kWidth, dH2, kWidth, 0, W2, kWidth, 1, nullptr, 0, H1, dH1, kWidth, bf16);
+  if ((e = gemm(st, B, kWidth, kWidth, dH2, kWidth, 0, W2, kWidth, 1, nullptr, 0, H1, dH1, kWidth, bf16))) return e;
   // layer 1
-  gemm(st, F, kWidth, B, X, F, 1, dH1, kWidth, 0, nullptr, 0, nullptr, dW1, kWidth, bf16);
+  if ((e = gemm(st, F, kWidth, B, X, F, 1, dH1, kWidth, 0, nullptr, 0, nullptr, dW1, kWidth, bf16))) return e;
   colsum_f32_kernel<<<1, 256, 0, st>>>(dH1, B, kWidth, db1);
   count_launch(3);
   return cuda_check(cudaGetLastError(), "mlp backward");
