@@ -4,11 +4,11 @@
 //
 // Work decomposition: an item is (problem p, a tile of T consecutive
 // candidates); it scores those T directions against all n_p coordinates, so
-// items are independent and need no cross-item reduction.  A block of 256
-// threads holds T candidates x (256 / T) row groups; the row groups split the
-// coordinates of each shared-memory stage and are combined in FP64 at the end
-// of the item.  Items are sorted by cost (n_p T) longest first and pulled by
-// the persistent blocks from an atomic counter.
+// items are independent and need no cross-item reduction.  A block of 64
+// threads holds T candidates (four per thread) x (256 / T) row groups; the row
+// groups split the coordinates of each shared-memory stage and are combined in
+// FP64 at the end of the item.  Items are sorted by cost (n_p T) longest first
+// and pulled by the persistent blocks from an atomic counter.
 //
 // Per problem the launch sequence is: input checks, direction sampling
 // (Philox, when the caller passes no directions), the persistent scoring
@@ -39,10 +39,14 @@
 #include "gauss_df32.cuh"
 #include "lrq_device.cuh"
 #include "lrq_internal.h"
+#include "score_f32x2.cuh"
 
 namespace lrq {
 
-constexpr int kBThreads = 256;
+constexpr int kBThreads = 64;
+constexpr int kBSlots = 256;      // candidate x row group slots of a block, four per thread
+constexpr int kBPerThread = kBSlots / kBThreads;
+constexpr int kBSelThreads = 256; // selection kernel
 constexpr int kBRows = 128;       // V rows per shared-memory stage
 constexpr int kBMaxS = 8192;      // candidates per problem
 constexpr int kBMaxTopM = 16;
@@ -111,98 +115,118 @@ __global__ void batched_check_kernel(const BProb* __restrict__ probs, int32_t* s
 // ---------------------------------------------------------------------------
 // persistent scoring kernel
 // ---------------------------------------------------------------------------
+// The slots' FP64 sums: while a thread takes its four slots at once (r <= 4,
+// where the first 24 KB hold sums and staged rows) they stay in shared memory
+// over the stages; for larger r they take the staged rows' place at the end.
 struct BShared {
-  float2 vs[kBRows * kMaxRank];
-  float2 zt[kMaxK];
-  double comb[kBThreads * 2 * kMaxRank];
+  union {
+    struct {
+      double sums[kBSlots * 8];             // r <= 4: [2 r][slot]
+      float4 vs[kBRows * 4];                // {re, re, im, im} per entry (score_f32x2.cuh)
+    } small;
+    float4 vs[kBRows * kMaxRank];
+    double comb[kBSlots * 2 * kMaxRank];    // [slot][2 r]
+  };
+  float2 zt[kMaxK];                         // z table: 16 sign patterns at most, or a code each
   int next;
 };
 
-// Sector of w = x + i y: boundary signs for K <= 8 (KC = K), the angle for
-// larger K (KC = 0).
-template <int KC>
-__device__ __forceinline__ int b_decide(float x, float y, const float* bc, const float* bs, int K) {
-  if constexpr (KC > 0) {
-    return decide_fp32<KC>(x, y, bc, bs);
-  } else {
-    if (K <= 8) {
-      const int BK = (K % 2 == 0) ? K / 2 : K;
-      uint32_t sb = 0;
-#pragma unroll
-      for (int m = 0; m < 8; ++m)
-        if (m < BK) sb |= (fmaf(y, bc[m], -x * bs[m]) > 0.0f ? 1u : 0u) << m;
-      if (K % 2 == 0) {
-        const int c = __popc(sb);
-        return (sb & 1u) ? c : (c == 0 ? 0 : K - c);
-      }
-      const uint32_t t = sb & ~(sb >> 1) & ((1u << (K - 1)) - 1u);
-      return t ? __ffs(t) : 0;
-    }
-    return decide_fp32_generic(x, y, K);
-  }
-}
-
+// A thread scores candidates s0 + cl + q T / 4, q < 4, on row group g: all on
+// every row it reads (r <= 4), or a part of them at a time on the staged rows
+// (their directions re-read, their FP64 sums in local memory).
+// Bound: FP32 FMAs and shared-memory reads, as score_fp32_kernel; 512 uneven
+// instances of up to 8192 directions: 11.1 ms, 15.3 with one candidate per thread
+// and scalar FMAs, 11.7 with two.
 template <int R, int KC>
 __device__ void b_score_item(const BProb& pb, int s0, BShared& sh, uint64_t* __restrict__ keys) {
-  const int T = pb.tile, RS = kBThreads / T;
-  const int tid = threadIdx.x, cl = tid % T, g = tid / T;
-  const int s = s0 + cl;
-  const bool act = s < pb.S;
+  constexpr int P = R <= 4 ? kBPerThread : (R <= 6 ? 2 : 1);  // candidates at once
+  constexpr bool kShared = P == kBPerThread;
+  const int T = pb.tile, H = T / kBPerThread, RS = kBSlots / T;
+  const int tid = threadIdx.x, cl = tid % H, g = tid / H;
   const BTable& tb = g_btab[pb.K];
-  float cr[R], ci[R], bc[8], bs[8];
+  float4* const vs = kShared ? sh.small.vs : sh.vs;
+  Dir2<R> d[P];
+  auto load_dirs = [&](int q0) {
 #pragma unroll
-  for (int j = 0; j < R; ++j) {
-    const float2 c = act ? pb.C[static_cast<int64_t>(s) * R + j] : make_float2(0.f, 0.f);
-    cr[j] = c.x;
-    ci[j] = c.y;
+    for (int q = 0; q < P; ++q) {
+      const int s = s0 + cl + (q0 + q) * H;
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+        d[q].set(j, s < pb.S ? pb.C[static_cast<int64_t>(s) * R + j] : make_float2(0.f, 0.f));
+    }
+  };
+  double acc64[kShared ? 1 : kBPerThread][2 * R];
+  auto slot = [&](int q) { return g * T + cl + q * H; };
+  if constexpr (kShared) {
+    load_dirs(0);
+#pragma unroll
+    for (int q = 0; q < P; ++q)
+#pragma unroll
+      for (int j = 0; j < 2 * R; ++j) sh.small.sums[j * kBSlots + slot(q)] = 0.0;
+  } else {
+    for (int q = 0; q < kBPerThread; ++q)
+#pragma unroll
+      for (int j = 0; j < 2 * R; ++j) acc64[q][j] = 0.0;
   }
-#pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    bc[m] = tb.bcos[m];
-    bs[m] = tb.bsin[m];
-  }
-  for (int k = tid; k < pb.K; k += kBThreads) sh.zt[k] = make_float2(tb.zr[k], tb.zi[k]);
-  double acc64[2 * R];
-#pragma unroll
-  for (int j = 0; j < 2 * R; ++j) acc64[j] = 0.0;
+  fill_ztable<KC>(sh.zt, tb.zr, tb.zi, pb.K);
   for (int64_t b0 = 0; b0 < pb.n; b0 += kBRows) {
     const int rows = static_cast<int>(min(static_cast<int64_t>(kBRows), pb.n - b0));
     __syncthreads();
-    for (int t = tid; t < rows * R; t += kBThreads) sh.vs[t] = pb.V[b0 * R + t];
-    __syncthreads();
-    float acc[2 * R];
-#pragma unroll
-    for (int j = 0; j < 2 * R; ++j) acc[j] = 0.f;
-    for (int i = g; i < rows; i += RS) {
-      float vr[R], vi[R], x = 0.f, y = 0.f;
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        const float2 v = sh.vs[i * R + j];
-        vr[j] = v.x;
-        vi[j] = v.y;
-        x = fmaf(vr[j], cr[j], fmaf(-vi[j], ci[j], x));
-        y = fmaf(vr[j], ci[j], fmaf(vi[j], cr[j], y));
-      }
-      const float2 z = sh.zt[b_decide<KC>(x, y, bc, bs, pb.K)];
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        acc[2 * j] = fmaf(vr[j], z.x, fmaf(vi[j], z.y, acc[2 * j]));
-        acc[2 * j + 1] = fmaf(vr[j], z.y, fmaf(-vi[j], z.x, acc[2 * j + 1]));
-      }
+#pragma unroll 4
+    for (int t = tid; t < rows * R; t += kBThreads) {
+      const float2 v = pb.V[b0 * R + t];
+      vs[t] = make_float4(v.x, v.x, v.y, v.y);
     }
+    __syncthreads();
+#pragma unroll 1
+    for (int q0 = 0; q0 < kBPerThread; q0 += P) {
+      if constexpr (!kShared) load_dirs(q0);
+      f32x2 acc[P][R];
 #pragma unroll
-    for (int j = 0; j < 2 * R; ++j) acc64[j] += static_cast<double>(acc[j]);
+      for (int q = 0; q < P; ++q)
+#pragma unroll
+        for (int j = 0; j < R; ++j) acc[q][j] = 0;
+#pragma unroll 1
+      for (int i = g; i < rows; i += RS) {
+        ulonglong2 v[R];
+#pragma unroll
+        for (int j = 0; j < R; ++j) v[j] = reinterpret_cast<const ulonglong2*>(vs)[i * R + j];
+#pragma unroll
+        for (int q = 0; q < P; ++q)
+          score_row<KC, R, false>(v, d[q], sh.zt, pb.K, tb.bcos, tb.bsin, acc[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < P; ++q)
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          float re, im;
+          unpack2(acc[q][j], re, im);
+          if constexpr (kShared) {
+            sh.small.sums[2 * j * kBSlots + slot(q)] += static_cast<double>(re);
+            sh.small.sums[(2 * j + 1) * kBSlots + slot(q)] += static_cast<double>(im);
+          } else {
+            acc64[q0 + q][2 * j] += static_cast<double>(re);
+            acc64[q0 + q][2 * j + 1] += static_cast<double>(im);
+          }
+        }
+    }
   }
   __syncthreads();
+  if constexpr (!kShared) {
+    for (int q = 0; q < kBPerThread; ++q)
 #pragma unroll
-  for (int j = 0; j < 2 * R; ++j) sh.comb[(g * T + cl) * (2 * R) + j] = acc64[j];
-  __syncthreads();
-  if (g == 0 && act) {
+      for (int j = 0; j < 2 * R; ++j) sh.comb[slot(q) * (2 * R) + j] = acc64[q][j];
+    __syncthreads();
+  }
+  for (int c = tid; c < T; c += kBThreads) {
+    const int s = s0 + c;
+    if (s >= pb.S) break;
     double f = 0.0;
 #pragma unroll
     for (int j = 0; j < 2 * R; ++j) {
       double v = 0.0;
-      for (int gg = 0; gg < RS; ++gg) v += sh.comb[(gg * T + cl) * (2 * R) + j];
+      for (int gg = 0; gg < RS; ++gg)
+        v += kShared ? sh.small.sums[j * kBSlots + gg * T + c] : sh.comb[(gg * T + c) * (2 * R) + j];
       f += v * v;
     }
     const uint32_t fb = __float_as_uint(static_cast<float>(f));
@@ -268,7 +292,7 @@ __device__ __noinline__ void b_enum_item(const BProb& pb, int chunk, BShared& sh
     }
     q = base + l1;
   }
-  EnumBest* sb = reinterpret_cast<EnumBest*>(sh.comb);
+  EnumBest* sb = reinterpret_cast<EnumBest*>(sh.comb);  // kBThreads entries
   __syncthreads();
   sb[threadIdx.x] = best;
   __syncthreads();
@@ -280,7 +304,7 @@ __device__ __noinline__ void b_enum_item(const BProb& pb, int chunk, BShared& sh
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(kBThreads) batched_score_kernel(const BProb* __restrict__ probs,
+__global__ void __launch_bounds__(kBThreads, 6) batched_score_kernel(const BProb* __restrict__ probs,
                                                                   const BItem* __restrict__ items, int nitems,
                                                                   int* __restrict__ counter,
                                                                   uint64_t* __restrict__ keys,
@@ -325,7 +349,7 @@ __device__ __forceinline__ uint64_t b_block_max(uint64_t v, uint64_t* red) {
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   uint64_t b = red[0];
-  for (int k = 1; k < kBThreads / 32; ++k) b = red[k] > b ? red[k] : b;
+  for (int k = 1; k < kBSelThreads / 32; ++k) b = red[k] > b ? red[k] : b;
   return b;
 }
 
@@ -340,7 +364,7 @@ __device__ double b_rescore(const BProb& pb, int s, double* red) {
     acc[2 * j] = acc[2 * j + 1] = 0.0;
   }
   const BTable& tb = g_btab[pb.K];
-  for (int64_t i = threadIdx.x; i < pb.n; i += kBThreads) {
+  for (int64_t i = threadIdx.x; i < pb.n; i += kBSelThreads) {
     double vr[R], vi[R], x = 0.0, y = 0.0;
 #pragma unroll
     for (int j = 0; j < R; ++j) {
@@ -368,7 +392,7 @@ __device__ double b_rescore(const BProb& pb, int s, double* red) {
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     double t = 0.0;
-    for (int k = 0; k < kBThreads / 32; ++k) t += red[k];
+    for (int k = 0; k < kBSelThreads / 32; ++k) t += red[k];
     f += t * t;
   }
   return f;
@@ -377,18 +401,18 @@ __device__ double b_rescore(const BProb& pb, int s, double* red) {
 // Exact problem: the best of its chunk results, in the solver's order.
 __device__ void b_select_exact(const BProb& pb, const EnumBest* __restrict__ ebest, double* best_f, int64_t* best_idx,
                                int32_t* status) {
-  __shared__ EnumBest sb[kBThreads];
+  __shared__ EnumBest sb[kBSelThreads];
   EnumBest best;
   best.f = -1.0;
   best.level = 0;
   best.sign = 1;
   best.rank = 0;
   best.choice = 0;
-  for (int c = threadIdx.x; c < pb.nchunks; c += kBThreads)
+  for (int c = threadIdx.x; c < pb.nchunks; c += kBSelThreads)
     if (enum_better(ebest[pb.eb_off + c], best)) best = ebest[pb.eb_off + c];
   sb[threadIdx.x] = best;
   __syncthreads();
-  for (int h = kBThreads / 2; h > 0; h >>= 1) {
+  for (int h = kBSelThreads / 2; h > 0; h >>= 1) {
     if (threadIdx.x < h && enum_better(sb[threadIdx.x + h], sb[threadIdx.x])) sb[threadIdx.x] = sb[threadIdx.x + h];
     __syncthreads();
   }
@@ -400,15 +424,15 @@ __device__ void b_select_exact(const BProb& pb, const EnumBest* __restrict__ ebe
   }
 }
 
-__global__ void __launch_bounds__(kBThreads) batched_select_kernel(const BProb* __restrict__ probs,
+__global__ void __launch_bounds__(kBSelThreads) batched_select_kernel(const BProb* __restrict__ probs,
                                                                    const uint64_t* __restrict__ keys, int top_m,
                                                                    const EnumBest* __restrict__ ebest,
                                                                    double* __restrict__ best_f,
                                                                    int64_t* __restrict__ best_idx,
                                                                    int64_t* __restrict__ epoch,
                                                                    int32_t* __restrict__ status) {
-  __shared__ uint64_t redk[kBThreads / 32];
-  __shared__ double redd[kBThreads / 32];
+  __shared__ uint64_t redk[kBSelThreads / 32];
+  __shared__ double redd[kBSelThreads / 32];
   const BProb pb = probs[blockIdx.x];
   if (blockIdx.x == 0 && threadIdx.x == 0) *epoch += 1;  // the next call draws fresh directions
   if (pb.exact) {
@@ -422,7 +446,7 @@ __global__ void __launch_bounds__(kBThreads) batched_select_kernel(const BProb* 
   uint64_t prev = ~0ull;
   for (int q = 0; q < m; ++q) {
     uint64_t v = 0;
-    for (int s = threadIdx.x; s < pb.S; s += kBThreads) {
+    for (int s = threadIdx.x; s < pb.S; s += kBSelThreads) {
       const uint64_t k = kp[s];
       if (k < prev && k > v) v = k;
     }
@@ -621,7 +645,7 @@ int upload(lrq_batched_plan_impl* pl, uint8_t* ws, const std::vector<int>& subse
   // vertices of about n_p (4 d + 24) FP64 operations, weighted 32x
   auto cost = [&](const BItem& it) {
     const BProb& b = hp[it.p];
-    if (b.exact) return static_cast<double>(b.n) * kBEnumChunk * 2.0 * (4.0 * b.r + 24.0) * 32.0 / kBThreads;
+    if (b.exact) return static_cast<double>(b.n) * kBEnumChunk * 2.0 * (4.0 * b.r + 24.0) * 32.0 / kBSlots;
     return static_cast<double>(b.n) * b.tile * (b.r + 1);
   };
   std::stable_sort(items.begin(), items.end(), [&](const BItem& a, const BItem& b) { return cost(a) > cost(b); });
@@ -663,7 +687,7 @@ int launch_sequence(const lrq_batched_plan_impl* pl, uint8_t* ws, int nitems, bo
   timing_stop(st);
   count_launch();
   if (select) {
-    batched_select_kernel<<<P, kBThreads, 0, st>>>(probs, keys, pl->top_m, ebest, best_f, best_idx, epoch, status);
+    batched_select_kernel<<<P, kBSelThreads, 0, st>>>(probs, keys, pl->top_m, ebest, best_f, best_idx, epoch, status);
     count_launch();
   }
   return cuda_check(cudaGetLastError(), "batched kernels");

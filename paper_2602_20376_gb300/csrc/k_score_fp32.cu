@@ -12,6 +12,7 @@
 #include "gauss_df32.cuh"
 #include "lrq_device.cuh"
 #include "lrq_internal.h"
+#include "score_f32x2.cuh"
 
 namespace lrq {
 
@@ -103,98 +104,95 @@ int launch_colsum(const float2* V, int64_t n, int r, double* Tpart, double* T, i
 
 // ---------------------------------------------------------------------------
 // FP32 CUDA-core scoring.
-// Block: 256 candidates (one per thread) x one coordinate chunk (blockIdx.y).
-// Coordinates are staged through shared memory 256 rows at a time and read
-// back as broadcasts.  Per coordinate: w = V_i c (FP32 FMA), decision from
-// the boundary-line signs, V^H z += conj(V_i) omega^k.  The FP32 running sum
+// Block: 256 candidates x one coordinate chunk (blockIdx.y).  Coordinates are
+// staged through shared memory 256 rows at a time and read back as broadcasts.
+// Per coordinate: w = V_i c (packed FP32 FMAs), decision from the boundary-line
+// signs, V^H z += conj(V_i) omega^k (score_f32x2.cuh).  The FP32 running sum
 // covers one 256-row batch and is then added into FP64 (blocked partials, so
 // the FP32 error is that of a 256-term sum).
+// Bound: the FMA pipe (38 cycles an evaluation at r = 4, K = 8) and the
+// shared-memory reads.  The scalar form with one candidate a thread issued
+// about 81 instructions an evaluation.  n = 4096, S = 2^14, r = 4, K = 8: 112
+// us, 145 before (same bits).  Two candidates a thread while that leaves 16
+// warps an SM; four halve the reads again but leave 12 warps here: 133 us.
 // Output: partial[chunk][s][2r] doubles = (Re, Im) of sum_{i in chunk} conj(V_i) z_i.
 // ---------------------------------------------------------------------------
 struct Fp32Tables {
-  float bcos[8], bsin[8];
   float zr[kMaxK], zi[kMaxK];
 };
 
-constexpr int kFp32Block = 256;
+constexpr int kFp32Block = 256;    // candidates
 constexpr int kFp32Batch = 256;
+template <int R>
+struct Fp32Shape {
+  static constexpr int kCpt = R <= 5 ? 2 : 1;  // candidates per thread
+  static constexpr int kThreads = kFp32Block / kCpt;
+};
 
 template <int K, int R>
-__global__ void __launch_bounds__(kFp32Block) score_fp32_kernel(const float2* __restrict__ V, int64_t n,
-                                                                const float2* __restrict__ C, int64_t S,
-                                                                int64_t S_pad, int64_t rows_per_chunk,
-                                                                int Kdyn, const __grid_constant__ Fp32Tables tab,
-                                                                double* __restrict__ partial) {
-  __shared__ float2 vs[kFp32Batch * R];
-  __shared__ float2 ztab[kMaxK];
-  const int Kr = (K > 0) ? K : Kdyn;
-  for (int k = threadIdx.x; k < Kr; k += blockDim.x) ztab[k] = make_float2(tab.zr[k], tab.zi[k]);
+__global__ void __launch_bounds__(Fp32Shape<R>::kThreads) score_fp32_kernel(const float2* __restrict__ V, int64_t n,
+                                                                  const float2* __restrict__ C, int64_t S,
+                                                                  int64_t S_pad, int64_t rows_per_chunk, int Kdyn,
+                                                                  const __grid_constant__ Fp32Tables tab,
+                                                                  double* __restrict__ partial) {
+  constexpr int kFp32Cpt = Fp32Shape<R>::kCpt, kFp32Threads = Fp32Shape<R>::kThreads;
+  __shared__ __align__(16) float4 vs[kFp32Batch * R];
+  __shared__ float2 zt[ZTable<K>::kEntries];
+  fill_ztable<K>(zt, tab.zr, tab.zi, Kdyn);
 
-  const int64_t s = static_cast<int64_t>(blockIdx.x) * kFp32Block + threadIdx.x;
-  const bool active = s < S;
-  float cr[R], ci[R];
+  const int64_t s0 = static_cast<int64_t>(blockIdx.x) * kFp32Block + threadIdx.x;
+  Dir2<R> d[kFp32Cpt];
+  double acc64[kFp32Cpt][2 * R];
 #pragma unroll
-  for (int j = 0; j < R; ++j) {
-    float2 c = active ? C[s * R + j] : make_float2(0.f, 0.f);
-    cr[j] = c.x;
-    ci[j] = c.y;
+  for (int q = 0; q < kFp32Cpt; ++q) {
+    const int64_t s = s0 + q * kFp32Threads;
+#pragma unroll
+    for (int j = 0; j < R; ++j) d[q].set(j, s < S ? C[s * R + j] : make_float2(0.f, 0.f));
+#pragma unroll
+    for (int j = 0; j < 2 * R; ++j) acc64[q][j] = 0.0;
   }
-  float bc[8], bs[8];
-#pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    bc[m] = tab.bcos[m];
-    bs[m] = tab.bsin[m];
-  }
-  double acc64[2 * R];
-#pragma unroll
-  for (int j = 0; j < 2 * R; ++j) acc64[j] = 0.0;
 
   const int64_t i_begin = static_cast<int64_t>(blockIdx.y) * rows_per_chunk;
   const int64_t i_end = min(n, i_begin + rows_per_chunk);
   for (int64_t b0 = i_begin; b0 < i_end; b0 += kFp32Batch) {
     const int rows = static_cast<int>(min(static_cast<int64_t>(kFp32Batch), i_end - b0));
     __syncthreads();
-    for (int t = threadIdx.x; t < rows * R; t += blockDim.x) vs[t] = V[b0 * R + t];
+#pragma unroll 4
+    for (int t = threadIdx.x; t < rows * R; t += kFp32Threads) {
+      const float2 v = V[b0 * R + t];
+      vs[t] = make_float4(v.x, v.x, v.y, v.y);
+    }
     __syncthreads();
-    float acc[2 * R];
+    f32x2 acc[kFp32Cpt][R];
 #pragma unroll
-    for (int j = 0; j < 2 * R; ++j) acc[j] = 0.f;
+    for (int q = 0; q < kFp32Cpt; ++q)
+#pragma unroll
+      for (int j = 0; j < R; ++j) acc[q][j] = 0;
     for (int i = 0; i < rows; ++i) {
-      float vr[R], vi[R];
+      ulonglong2 v[R];
 #pragma unroll
-      for (int j = 0; j < R; ++j) {
-        float2 v = vs[i * R + j];
-        vr[j] = v.x;
-        vi[j] = v.y;
-      }
-      float x = 0.f, y = 0.f;
+      for (int j = 0; j < R; ++j) v[j] = reinterpret_cast<const ulonglong2*>(vs)[i * R + j];
 #pragma unroll
-      for (int j = 0; j < R; ++j) {
-        x = fmaf(vr[j], cr[j], x);
-        x = fmaf(-vi[j], ci[j], x);
-        y = fmaf(vr[j], ci[j], y);
-        y = fmaf(vi[j], cr[j], y);
-      }
-      int k;
-      if constexpr (K > 0)
-        k = decide_fp32<K>(x, y, bc, bs);
-      else
-        k = decide_fp32_generic(x, y, Kr);
-      float2 z = ztab[k];
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        // conj(V_ij) z = (vr zr + vi zi) + i (vr zi - vi zr)
-        acc[2 * j] = fmaf(vr[j], z.x, fmaf(vi[j], z.y, acc[2 * j]));
-        acc[2 * j + 1] = fmaf(vr[j], z.y, fmaf(-vi[j], z.x, acc[2 * j + 1]));
-      }
+      for (int q = 0; q < kFp32Cpt; ++q) score_row<K, R, true>(v, d[q], zt, Kdyn, nullptr, nullptr, acc[q]);
     }
 #pragma unroll
-    for (int j = 0; j < 2 * R; ++j) acc64[j] += static_cast<double>(acc[j]);
-  }
-  if (active) {
-    double* out = partial + (static_cast<int64_t>(blockIdx.y) * S_pad + s) * (2 * R);
+    for (int q = 0; q < kFp32Cpt; ++q)
 #pragma unroll
-    for (int j = 0; j < 2 * R; ++j) out[j] = acc64[j];
+      for (int j = 0; j < R; ++j) {
+        float re, im;
+        unpack2(acc[q][j], re, im);
+        acc64[q][2 * j] += static_cast<double>(re);
+        acc64[q][2 * j + 1] += static_cast<double>(im);
+      }
+  }
+#pragma unroll
+  for (int q = 0; q < kFp32Cpt; ++q) {
+    const int64_t s = s0 + q * kFp32Threads;
+    if (s < S) {
+      double* out = partial + (static_cast<int64_t>(blockIdx.y) * S_pad + s) * (2 * R);
+#pragma unroll
+      for (int j = 0; j < 2 * R; ++j) out[j] = acc64[q][j];
+    }
   }
 }
 
@@ -204,12 +202,11 @@ static int launch_fp32_r(const ScorePlan& p, const Fp32Tables& tab, const float2
   dim3 grid(static_cast<unsigned>(ceil_div(p.S, kFp32Block)), static_cast<unsigned>(p.nsplit));
   int64_t S_pad = p.c_tiles * 128;
   switch (p.r) {
-#define LRQ_FP32_CASE(RR)                                                                            \
-  case RR:                                                                                           \
-    score_fp32_kernel<K, RR><<<grid, kFp32Block, 0, st>>>(V, p.n, C, p.S, S_pad,                     \
-                                                          p.fp32_rows_per_chunk, p.K, tab, partial); \
+#define LRQ_FP32_CASE(RR)                                                                              \
+  case RR:                                                                                             \
+    score_fp32_kernel<K, RR><<<grid, Fp32Shape<RR>::kThreads, 0, st>>>(                                \
+        V, p.n, C, p.S, S_pad, p.fp32_rows_per_chunk, p.K, tab, partial);                              \
     break;
-    count_launch();
     LRQ_FP32_CASE(1)
     LRQ_FP32_CASE(2)
     LRQ_FP32_CASE(3)
@@ -222,16 +219,13 @@ static int launch_fp32_r(const ScorePlan& p, const Fp32Tables& tab, const float2
     default:
       return fail(LRQ_EUNSUPPORTED, "score_fp32: r out of range");
   }
+  count_launch();
   return cuda_check(cudaGetLastError(), "score_fp32_kernel");
 }
 
 int launch_score_fp32(const ScorePlan& p, const Alphabet& a, const float2* V, const float2* C,
                       double* partial, cudaStream_t st) {
   Fp32Tables tab;
-  for (int m = 0; m < 8; ++m) {
-    tab.bcos[m] = m < a.BK ? a.bcos[m] : 0.f;
-    tab.bsin[m] = m < a.BK ? a.bsin[m] : 0.f;
-  }
   for (int k = 0; k < kMaxK; ++k) {
     tab.zr[k] = k < a.K ? a.zr[k] : 0.f;
     tab.zi[k] = k < a.K ? a.zi[k] : 0.f;

@@ -1,0 +1,209 @@
+// score_f32x2.cuh -- the FP32 scoring step of one coordinate with packed
+// FP32 instructions, shared by the CUDA-core scoring kernel and the batched
+// kernel.
+//
+// sm_103a's fma.rn.f32x2 does two FP32 FMAs a lane in one instruction, each
+// rounded like fmaf.  Real and imaginary part are the two halves, so that the
+// projection w = V_i c and the update V^H z += conj(V_i) omega^k keep the
+// operations and the order of the scalar form (same bits) in half the
+// instructions; a row's V is staged as {re, re, im, im} per entry and read
+// back as one 16-byte broadcast.  The boundary signs form the byte offset of
+// omega^k in a table with one entry per sign pattern, so no code is computed.
+// What binds next are the shared-memory reads: an SM returns 128 bytes a cycle,
+// 4 cycles for a 16-byte read of a warp whatever it broadcasts, so a row's
+// entries are read once for several candidates of a thread and the table entry
+// is 8 bytes.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "lrq_device.cuh"
+
+namespace lrq {
+
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Decision boundaries theta_m = pi(2m+1)/K in FP32, the first (B_K + 1) / 2 of
+// them: the others are mirror images (odd K: m and K-1-m share cos and have
+// opposite sin; even K: m and K/2-1-m share sin and have opposite cos).  The
+// same values as make_alphabet's FP32 tables.
+template <int K>
+__host__ __device__ constexpr float boundary_cos(int m) {
+  if (K == 2) {
+    constexpr float t[] = {0.f};
+    return t[m];
+  }
+  if (K == 3) {
+    constexpr float t[] = {0x1p-1f, -1.f};
+    return t[m];
+  }
+  if (K == 4) {
+    constexpr float t[] = {0x1.6a09e6p-1f};
+    return t[m];
+  }
+  if (K == 5) {
+    constexpr float t[] = {0x1.9e377ap-1f, -0x1.3c6ef4p-2f, -1.f};
+    return t[m];
+  }
+  if (K == 6) {
+    constexpr float t[] = {0x1.bb67aep-1f, 0.f};
+    return t[m];
+  }
+  if (K == 7) {
+    constexpr float t[] = {0x1.cd4bcap-1f, 0x1.c7b90ep-3f, -0x1.3f3a0ep-1f, -1.f};
+    return t[m];
+  }
+  if (K == 8) {
+    constexpr float t[] = {0x1.d906bcp-1f, 0x1.87de2ap-2f};
+    return t[m];
+  }
+  return 0.f;
+}
+template <int K>
+__host__ __device__ constexpr float boundary_sin(int m) {
+  if (K == 2) {
+    constexpr float t[] = {1.f};
+    return t[m];
+  }
+  if (K == 3) {
+    constexpr float t[] = {0x1.bb67aep-1f, 0.f};
+    return t[m];
+  }
+  if (K == 4) {
+    constexpr float t[] = {0x1.6a09e6p-1f};
+    return t[m];
+  }
+  if (K == 5) {
+    constexpr float t[] = {0x1.2cf23p-1f, 0x1.e6f0e2p-1f, 0.f};
+    return t[m];
+  }
+  if (K == 6) {
+    constexpr float t[] = {0x1p-1f, 1.f};
+    return t[m];
+  }
+  if (K == 7) {
+    constexpr float t[] = {0x1.bc4c04p-2f, 0x1.f329cp-1f, 0x1.904c38p-1f, 0.f};
+    return t[m];
+  }
+  if (K == 8) {
+    constexpr float t[] = {0x1.87de2ap-2f, 0x1.d906bcp-1f};
+    return t[m];
+  }
+  return 0.f;
+}
+
+// Sign pattern of the boundary projections p_m = y cos - x sin > 0 (the same
+// roundings as decide_fp32), times 8: a byte offset into the z table.
+template <int K>
+__device__ __forceinline__ uint32_t sign_offset(float x, float y) {
+  constexpr int BK = (K % 2 == 0) ? K / 2 : K;
+  uint32_t off = 0;
+#pragma unroll
+  for (int m = 0; m < (BK + 1) / 2; ++m) {
+    const float c = boundary_cos<K>(m), s = boundary_sin<K>(m);
+    const int mm = BK - 1 - m;
+    float p, q;
+    if (s == 0.f) {  // the boundary on the negative real axis
+      p = q = -y;
+    } else if (c == 0.f) {  // the boundary on the imaginary axis
+      p = q = -x;
+    } else {
+      const float t = x * s;
+      p = fmaf(y, c, -t);
+      q = K % 2 == 1 ? fmaf(y, c, t) : fmaf(y, -c, -t);
+    }
+    if (p > 0.f) off |= 8u << m;
+    if (mm != m && q > 0.f) off |= 8u << mm;
+  }
+  return off;
+}
+
+// entries of the z table (sign patterns; codes for K > 8) and its filling by
+// a block's threads
+template <int K>
+struct ZTable {
+  static constexpr int kEntries = K == 0 ? kMaxK : 1 << ((K % 2 == 0) ? K / 2 : K);
+};
+template <int K>
+__device__ __forceinline__ void fill_ztable(float2* zt, const float* zr, const float* zi, int Kdyn) {
+  const int count = K == 0 ? Kdyn : ZTable<K>::kEntries;
+  for (int t = threadIdx.x; t < count; t += blockDim.x) {
+    int k = t;
+    if constexpr (K > 0) k = decide_from_signs<K>(static_cast<uint32_t>(t));
+    zt[t] = make_float2(zr[k], zi[k]);
+  }
+}
+
+// One candidate's direction: {cr, ci} and {-ci, cr} per component.
+template <int R>
+struct Dir2 {
+  f32x2 a[R], b[R];
+  __device__ __forceinline__ void set(int j, float2 c) {
+    a[j] = pack2(c.x, c.y);
+    b[j] = pack2(-c.y, c.x);
+  }
+};
+
+// K known at run time only: the sign rule of decide_fp32 for K <= 8 (bc, bs:
+// its boundaries), the angle above.
+__device__ __forceinline__ int decide_any(float x, float y, int K, const float* bc, const float* bs) {
+  if (K > 8) return decide_fp32_generic(x, y, K);
+  const int BK = (K % 2 == 0) ? K / 2 : K;
+  uint32_t sb = 0;
+  for (int m = 0; m < BK; ++m) sb |= (fmaf(y, bc[m], -x * bs[m]) > 0.0f ? 1u : 0u) << m;
+  if (K % 2 == 0) {
+    const int c = __popc(sb);
+    return (sb & 1u) ? c : (c == 0 ? 0 : K - c);
+  }
+  const uint32_t t = sb & ~(sb >> 1) & ((1u << (K - 1)) - 1u);
+  return t ? __ffs(t) : 0;
+}
+
+// acc[j] += conj(V_ij) z_i for one candidate; v: the row's {re, re, im, im}.
+// K = 0: any alphabet, Kdyn.  VFIRST: the order of the two products of w (each caller's own).
+template <int K, int R, bool VFIRST>
+__device__ __forceinline__ void score_row(const ulonglong2 (&v)[R], const Dir2<R>& d, const float2* zt, int Kdyn,
+                                          const float* bc, const float* bs, f32x2 (&acc)[R]) {
+  f32x2 w = 0;  // {0, 0}
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    if constexpr (VFIRST) {
+      w = fma2(v[j].x, d.a[j], w);
+      w = fma2(v[j].y, d.b[j], w);
+    } else {
+      w = fma2(v[j].y, d.b[j], w);
+      w = fma2(v[j].x, d.a[j], w);
+    }
+  }
+  float x, y;
+  unpack2(w, x, y);
+  uint32_t off;
+  if constexpr (K > 0)
+    off = sign_offset<K>(x, y);
+  else
+    off = 8u * static_cast<uint32_t>(decide_any(x, y, Kdyn, bc, bs));
+  const float2 z = *reinterpret_cast<const float2*>(reinterpret_cast<const char*>(zt) + off);
+  const f32x2 za = pack2(z.x, z.y), zb = pack2(z.y, -z.x);
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    acc[j] = fma2(v[j].y, zb, acc[j]);
+    acc[j] = fma2(v[j].x, za, acc[j]);
+  }
+}
+
+}  // namespace lrq
