@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "gauss_df32.cuh"
 #include "lrq_device.cuh"
 #include "lrq_internal.h"
 
@@ -35,120 +36,189 @@ constexpr int kDim = 8;              // S^7 in R^8 = C^4
 // ---------------------------------------------------------------------------
 // features (FP64): gauge, then eigenvalue shares and moments
 // ---------------------------------------------------------------------------
-__device__ double block_sum_f64(double v, double* red) {
-  for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double s = 0.0;
-  for (int k = 0; k < static_cast<int>(blockDim.x >> 5); ++k) s += red[k];
-  return s;
+__device__ __forceinline__ df32 df_from(double x) {
+  const float h = static_cast<float>(x);
+  return df32{h, static_cast<float>(x - static_cast<double>(h))};
 }
 
-// one block (256 threads) per instance
-__global__ void __launch_bounds__(256) features_kernel(const float2* __restrict__ V, int64_t n, int r,
-                                                       const double* __restrict__ lambda, float2* __restrict__ Vg,
-                                                       float* __restrict__ feat, int32_t* status) {
-  __shared__ double red[8];
-  __shared__ unsigned long long red_key[8];
-  __shared__ double s_ph_re[kMaxRank], s_ph_im[kMaxRank];
-  const int b = blockIdx.x;
+// A cluster of blocks per instance, each with every NB-th group of 256 rows.
+// Two passes over V: the entries of largest modulus and the sums of the row
+// norms and column moduli; then the gauge-fixed copy and the central moments
+// of all r + 1 populations at once (q = 0: a_i = ||V_i||^2 n / total, q = 1 + j:
+// b_ij = |V_ij|^2 n / lambda_j).  Bound: FP64 (about 60 warp instructions of 16
+// cycles per 32 rows at r = 4); the gauge product is double-float.  One block
+// per instance with eleven passes took 247 us at B = 16, n = 4096; 77 now.
+constexpr int kFeatThreads = 256;
+constexpr int kFeatSums = 3 * (kMaxRank + 1);
+
+struct FeatShared {
+  double part[kFeatThreads / 32][kFeatSums];
+  double sum[kFeatSums];            // the block's sums, then the cluster's
+  long long best[kMaxRank];         // bits of the largest |V_ij|^2 (non-negative doubles order like their bits)
+  long long row[kMaxRank];
+  long long wbest[kFeatThreads / 32][kMaxRank], wrow[kFeatThreads / 32][kMaxRank];
+  df32 ph_re[kMaxRank], ph_im[kMaxRank];
+};
+
+// the cluster's sums of `count` values per thread, in a fixed order
+__device__ __forceinline__ void feat_sums(cg::cluster_group& cluster, FeatShared& sh, const double* v, int count) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int q = 0; q < count; ++q) {
+    double s = v[q];
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+    if (lane == 0) sh.part[warp][q] = s;
+  }
+  __syncthreads();
+  double mine = 0.0;
+  if (threadIdx.x < count)
+    for (int w = 0; w < kFeatThreads / 32; ++w) mine += sh.part[w][threadIdx.x];
+  if (threadIdx.x < count) sh.sum[threadIdx.x] = mine;
+  cluster.sync();
+  double total = 0.0;
+  if (threadIdx.x < count)
+    for (int b = 0; b < static_cast<int>(cluster.num_blocks()); ++b)
+      total += cluster.map_shared_rank(&sh.sum[0], b)[threadIdx.x];
+  cluster.sync();  // every block has read the others' sums
+  if (threadIdx.x < count) sh.sum[threadIdx.x] = total;
+  __syncthreads();
+}
+
+__device__ __forceinline__ double feat_mod2(float2 v) {
+  return fma(static_cast<double>(v.x), static_cast<double>(v.x), static_cast<double>(v.y) * static_cast<double>(v.y));
+}
+
+__global__ void __launch_bounds__(kFeatThreads) features_kernel(const float2* __restrict__ V, int64_t n, int r,
+                                                                const double* __restrict__ lambda,
+                                                                float2* __restrict__ Vg, float* __restrict__ feat,
+                                                                int32_t* status) {
+  __shared__ FeatShared sh;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int nb = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
+  const int b = blockIdx.x / nb;
   const float2* Vb = V + static_cast<int64_t>(b) * n * r;
   const double* lam = lambda + static_cast<int64_t>(b) * r;
   const int F = 5 * r + 4;
   float* fo = feat + static_cast<int64_t>(b) * F;
   double total = 0.0;
   for (int j = 0; j < r; ++j) total += lam[j];
-  if (!(total > 0.0)) {
-    if (threadIdx.x == 0) dev_fail(status, LRQ_EINVAL);
+  if (!(total > 0.0)) {  // the same for every block of the cluster
+    if (threadIdx.x == 0 && rank == 0) dev_fail(status, LRQ_EINVAL);
     return;
   }
-  // gauge: per column the entry of largest modulus (lowest row on ties)
-  for (int j = 0; j < r; ++j) {
-    // argmax of |V_ij|^2 with ties to the lower row
-    double best = -1.0;
-    int64_t brow = n;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-      const float2 v = Vb[i * r + j];
-      const double m2 = static_cast<double>(v.x) * v.x + static_cast<double>(v.y) * v.y;
-      if (m2 > best) {
-        best = m2;
-        brow = i;
-      }
-    }
-    for (int m = 16; m > 0; m >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, m);
-      const int64_t orow = __shfl_xor_sync(0xffffffffu, brow, m);
-      if (ob > best || (ob == best && orow < brow)) {
-        best = ob;
-        brow = orow;
-      }
-    }
-    if ((threadIdx.x & 31) == 0) {
-      red[threadIdx.x >> 5] = best;
-      red_key[threadIdx.x >> 5] = static_cast<unsigned long long>(brow);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double bb = red[0];
-      int64_t br = static_cast<int64_t>(red_key[0]);
-      for (int k = 1; k < static_cast<int>(blockDim.x >> 5); ++k) {
-        const int64_t rr = static_cast<int64_t>(red_key[k]);
-        if (red[k] > bb || (red[k] == bb && rr < br)) {
-          bb = red[k];
-          br = rr;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i0 = static_cast<int64_t>(rank) * kFeatThreads + threadIdx.x, stride = static_cast<int64_t>(nb) * kFeatThreads;
+  double scale[kMaxRank + 1], acc[kFeatSums];
+  scale[0] = static_cast<double>(n) / total;
+#pragma unroll
+  for (int j = 0; j < kMaxRank; ++j) scale[1 + j] = j < r ? static_cast<double>(n) / lam[j] : 0.0;
+#pragma unroll
+  for (int q = 0; q < kFeatSums; ++q) acc[q] = 0.0;
+  // pass 1: per column the entry of largest modulus (lowest row on ties), sums
+  long long best[kMaxRank], brow[kMaxRank];
+#pragma unroll
+  for (int j = 0; j < kMaxRank; ++j) {
+    best[j] = -1;
+    brow[j] = n;
+  }
+  for (int64_t i = i0; i < n; i += stride) {
+    double a = 0.0;
+#pragma unroll
+    for (int j = 0; j < kMaxRank; ++j) {
+      if (j < r) {
+        const double m2 = feat_mod2(Vb[i * r + j]);
+        const long long bits = __double_as_longlong(m2);
+        if (m2 == m2 && bits > best[j]) {
+          best[j] = bits;
+          brow[j] = i;
         }
+        a += m2;
+        acc[1 + j] = fma(m2, scale[1 + j], acc[1 + j]);
       }
-      const float2 a = Vb[br * r + j];
-      const double am = sqrt(static_cast<double>(a.x) * a.x + static_cast<double>(a.y) * a.y);
-      // multiply the column by |a| / a = conj(a) / |a|
-      s_ph_re[j] = am > 0.0 ? a.x / am : 1.0;
-      s_ph_im[j] = am > 0.0 ? -a.y / am : 0.0;
     }
-    __syncthreads();
+    acc[0] = fma(a, scale[0], acc[0]);
   }
-  // gauge-fixed copy
+  auto better = [](long long& v, long long& row, long long o, long long orow) {
+    if (o > v || (o == v && orow < row)) {
+      v = o;
+      row = orow;
+    }
+  };
+#pragma unroll
+  for (int j = 0; j < kMaxRank; ++j) {
+    if (j < r) {
+#pragma unroll
+      for (int m = 16; m > 0; m >>= 1)
+        better(best[j], brow[j], __shfl_xor_sync(0xffffffffu, best[j], m), __shfl_xor_sync(0xffffffffu, brow[j], m));
+      if (lane == 0) {
+        sh.wbest[warp][j] = best[j];
+        sh.wrow[warp][j] = brow[j];
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < r) {
+    long long v = sh.wbest[0][threadIdx.x], row = sh.wrow[0][threadIdx.x];
+    for (int w = 1; w < kFeatThreads / 32; ++w) better(v, row, sh.wbest[w][threadIdx.x], sh.wrow[w][threadIdx.x]);
+    sh.best[threadIdx.x] = v;
+    sh.row[threadIdx.x] = row;
+  }
+  cluster.sync();
+  if (threadIdx.x < r) {
+    const int j = threadIdx.x;
+    long long v = -1, row = n;
+    for (int q = 0; q < nb; ++q)
+      better(v, row, cluster.map_shared_rank(&sh.best[0], q)[j], cluster.map_shared_rank(&sh.row[0], q)[j]);
+    const float2 a = Vb[min(row, static_cast<long long>(n - 1)) * r + j];
+    const double am = sqrt(static_cast<double>(a.x) * a.x + static_cast<double>(a.y) * a.y);
+    // multiply the column by |a| / a = conj(a) / |a|
+    sh.ph_re[j] = df_from(am > 0.0 ? a.x / am : 1.0);
+    sh.ph_im[j] = df_from(am > 0.0 ? -a.y / am : 0.0);
+  }
+  feat_sums(cluster, sh, acc, r + 1);  // its barriers also publish the phases
+  double mean[kMaxRank + 1];
+#pragma unroll
+  for (int q = 0; q <= kMaxRank; ++q) mean[q] = q <= r ? sh.sum[q] / static_cast<double>(n) : 0.0;
+#pragma unroll
+  for (int q = 0; q < kFeatSums; ++q) acc[q] = 0.0;
+  // pass 2: gauge-fixed copy, central moments
   float2* Vo = Vg + static_cast<int64_t>(b) * n * r;
-  for (int64_t t = threadIdx.x; t < n * r; t += blockDim.x) {
-    const int j = static_cast<int>(t % r);
-    const float2 v = Vb[t];
-    const double re = v.x * s_ph_re[j] - v.y * s_ph_im[j];
-    const double im = v.x * s_ph_im[j] + v.y * s_ph_re[j];
-    Vo[t] = make_float2(static_cast<float>(re), static_cast<float>(im));
+  auto moments = [&](int q, double x) {
+    const double d = fma(x, scale[q], -mean[q]), d2 = d * d;
+    acc[3 * q] += d2;
+    acc[3 * q + 1] = fma(d2, d, acc[3 * q + 1]);
+    acc[3 * q + 2] = fma(d2, d2, acc[3 * q + 2]);
+  };
+  for (int64_t i = i0; i < n; i += stride) {
+    double a = 0.0;
+#pragma unroll
+    for (int j = 0; j < kMaxRank; ++j) {
+      if (j < r) {
+        const float2 v = Vb[i * r + j];
+        const df32 pr = sh.ph_re[j], pi = sh.ph_im[j];
+        const df32 x = df_times(df32{v.x, 0.f}, pr), y = df_times(df32{v.y, 0.f}, pi);
+        const df32 z = df_times(df32{v.x, 0.f}, pi), w = df_times(df32{v.y, 0.f}, pr);
+        Vo[i * r + j] = make_float2(df_sum(x, df32{-y.h, -y.l}).h, df_sum(z, w).h);
+        const double m2 = feat_mod2(v);
+        a += m2;
+        moments(1 + j, m2);
+      }
+    }
+    moments(0, a);
   }
-  if (threadIdx.x < r) fo[threadIdx.x] = static_cast<float>(lam[threadIdx.x] / total);
-  // moments of a_i = ||V_i||^2 n / total and b_ij = |V_ij|^2 n / lambda_j:
-  // q = 0 is a, q = 1 + j is column j
-  for (int q = 0; q <= r; ++q) {
-    const double scale = q == 0 ? static_cast<double>(n) / total : static_cast<double>(n) / lam[q - 1];
-    double s1 = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-      double a = 0.0;
-      for (int j = (q == 0 ? 0 : q - 1); j < (q == 0 ? r : q); ++j) {
-        const float2 v = Vb[i * r + j];
-        a += static_cast<double>(v.x) * v.x + static_cast<double>(v.y) * v.y;
-      }
-      s1 += a * scale;
-    }
-    const double mean = block_sum_f64(s1, red) / static_cast<double>(n);
-    double s2 = 0.0, s3 = 0.0, s4 = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-      double a = 0.0;
-      for (int j = (q == 0 ? 0 : q - 1); j < (q == 0 ? r : q); ++j) {
-        const float2 v = Vb[i * r + j];
-        a += static_cast<double>(v.x) * v.x + static_cast<double>(v.y) * v.y;
-      }
-      const double d = a * scale - mean;
-      s2 += d * d;
-      s3 += d * d * d;
-      s4 += d * d * d * d;
-    }
-    const double var = block_sum_f64(s2, red) / static_cast<double>(n);
-    const double m3 = block_sum_f64(s3, red) / static_cast<double>(n);
-    const double m4 = block_sum_f64(s4, red) / static_cast<double>(n);
-    if (threadIdx.x == 0) {
+  feat_sums(cluster, sh, acc, 3 * (r + 1));
+  if (rank == 0) {
+    if (threadIdx.x < r) fo[threadIdx.x] = static_cast<float>(lam[threadIdx.x] / total);
+    if (threadIdx.x <= r) {
+      const int q = threadIdx.x;
+      const double dn = static_cast<double>(n);
+      const double var = sh.sum[3 * q] / dn, m3 = sh.sum[3 * q + 1] / dn, m4 = sh.sum[3 * q + 2] / dn;
+      double mq = 0.0;
+#pragma unroll
+      for (int k = 0; k <= kMaxRank; ++k)
+        if (k == q) mq = mean[k];
       float* o = fo + r + 4 * q;
-      o[0] = static_cast<float>(mean);
+      o[0] = static_cast<float>(mq);
       o[1] = static_cast<float>(var);
       o[2] = var > 0.0 ? static_cast<float>(m3 / (var * sqrt(var))) : 0.f;
       o[3] = var > 0.0 ? static_cast<float>(m4 / (var * var) - 3.0) : 0.f;
@@ -453,34 +523,72 @@ __global__ void __launch_bounds__(kNllThreads) vmf_nll_kernel(const float* __res
 // ---------------------------------------------------------------------------
 // sampling: component by its weight, Wood's rejection step for the cosine
 // to mu, a uniform direction orthogonal to mu, then a random omega^k
+//
+// With G1, G2 the two Gamma(7/2) variates, b Wood's constant and
+// Q = G2 + b G1 the candidate is w = (G2 - b G1) / Q, sqrt(1 - w^2) =
+// 2 sqrt(b G1 G2) / Q (no cancellation at large kappa), and the acceptance test
+//   kappa w + 7 log(1 - x0 w) - (kappa x0 + 7 log(1 - x0^2)) >= log u
+// is 2 kappa b / (1 + b) (G2 - G1) / Q + 7 log((1 + b)(G1 + G2) / (2 Q)) >= log u.
+// The test runs in FP32 with a margin; inside the margin (about one try in
+// 10^4) it is repeated in FP64 as first written, so every draw is accepted or
+// not as in FP64.  Logs, Gaussians and the vectors are double-float
+// (gauss_df32.cuh): FP64 runs at 1/64 of the FP32 rate and took about 800
+// instructions a sample (16 x 65520 draws: 2298 us, 361 now).
 // ---------------------------------------------------------------------------
+constexpr int kVmfThreads = 128;
+
 struct VmfRng {
   uint64_t seed;
   uint32_t s, b, ctr;
+  // the two uniforms' 2 x + 1 over 2^54 (x: 53 bits)
+  __device__ __forceinline__ void bits2(uint64_t* u, uint64_t* v) {
+    const PhiloxOut o =
+        philox4x32_10(s, b, ctr++, 0x564D46u, static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32));
+    *u = ((((static_cast<uint64_t>(o.w[0]) << 32) | o.w[1]) >> 11) << 1) | 1ull;
+    *v = ((((static_cast<uint64_t>(o.w[2]) << 32) | o.w[3]) >> 11) << 1) | 1ull;
+  }
   __device__ double2 uniform2() {  // two 53-bit uniforms in (0, 1)
     PhiloxOut o = philox4x32_10(s, b, ctr++, 0x564D46u, static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32));
     return make_double2(uniform53(o.w[0], o.w[1]), uniform53(o.w[2], o.w[3]));
   }
-  __device__ double2 normal2() {
-    const double2 u = uniform2();
+  // Gamma(7/2) = Gamma(3) + Gamma(1/2): -log(u1 u2 u3) + n^2 / 2 with
+  // n^2 / 2 = -log(u) cos^2
+  __device__ __forceinline__ df32 gamma35() {
+    uint64_t a, b2, c, d, e, f;
+    bits2(&a, &b2);
+    bits2(&c, &d);
+    bits2(&e, &f);
+    df32 sn, cs;
+    df_sincos(f, GaussTab(), &sn, &cs);
+    return df_sum(df_neg_log3(a, b2, c, GaussTab()), df_times(df_neg_log(e, GaussTab()), df_times(cs, cs)));
+  }
+  __device__ double gamma35_fp64() {
+    const double2 a = uniform2(), c = uniform2(), u = uniform2();
     const double rad = sqrt(-2.0 * log(u.x));
     double sn, cs;
     sincospi(2.0 * u.y, &sn, &cs);
-    return make_double2(rad * cs, rad * sn);
-  }
-  // Gamma(7/2) = Gamma(3) + Gamma(1/2): -log(u1 u2 u3) + n^2 / 2
-  __device__ double gamma35() {
-    const double2 a = uniform2(), c = uniform2();
-    const double2 nn = normal2();
-    return -log(a.x * a.y * c.x) + 0.5 * nn.x * nn.x;
+    return -log(a.x * a.y * c.x) + 0.5 * (rad * cs) * (rad * cs);
   }
 };
 
-__global__ void __launch_bounds__(128) vmf_sample_kernel(const float* __restrict__ O, int B, int S, int K,
-                                                         uint64_t seed, float2* __restrict__ C,
-                                                         int32_t* status) {
+// the acceptance test in FP64 for the try whose first counter is rng.ctr
+__device__ __noinline__ bool vmf_accept_fp64(VmfRng rng, double kap, double bb, double x0, double cc) {
+  const double g1 = rng.gamma35_fp64(), g2 = rng.gamma35_fp64();
+  const double z = g1 / (g1 + g2);  // Beta(7/2, 7/2)
+  const double w = (1.0 - (1.0 + bb) * z) / (1.0 - (1.0 - bb) * z);
+  const double u = rng.uniform2().x;
+  return kap * w + (kDim - 1.0) * log(1.0 - x0 * w) - cc >= log(u);
+}
+
+__global__ void __launch_bounds__(kVmfThreads) vmf_sample_kernel(const float* __restrict__ O, int B, int S, int K,
+                                                                 uint64_t seed, float2* __restrict__ C,
+                                                                 int32_t* status) {
   __shared__ CompParams cp;
-  __shared__ double wb[kComp], wx0[kComp], wc[kComp], cdf[kComp];
+  __shared__ double wb[kComp], wx0[kComp], wc[kComp];
+  __shared__ long long cdf[kComp];  // bits of the cumulative weights (positive doubles order like their bits)
+  __shared__ double total;
+  __shared__ df32 smu[kComp][kDim], sb[kComp], root_c[kMaxK], root_s[kMaxK];
+  __shared__ float sa[kComp], shalf[kComp];
   const int b = blockIdx.y;
   head_params(O + static_cast<int64_t>(b) * kOut, cp);
   if (threadIdx.x < kComp) {
@@ -492,60 +600,92 @@ __global__ void __launch_bounds__(128) vmf_sample_kernel(const float* __restrict
     wb[m] = bb;
     wx0[m] = x0;
     wc[m] = kap * x0 + p1 * log(1.0 - x0 * x0);
+    sb[m] = df_from(bb);
+    sa[m] = static_cast<float>(2.0 * kap * bb / (1.0 + bb));
+    shalf[m] = static_cast<float>(0.5 * (1.0 + bb));
+  }
+  for (int t = threadIdx.x; t < kComp * kDim; t += kVmfThreads) smu[t / kDim][t % kDim] = df_from(cp.mu[t / kDim][t % kDim]);
+  if (threadIdx.x < K) {
+    double sn, cs;
+    sincospi(2.0 * threadIdx.x / static_cast<double>(K), &sn, &cs);
+    root_c[threadIdx.x] = df_from(cs);
+    root_s[threadIdx.x] = df_from(sn);
   }
   if (threadIdx.x == 0) {
     double s = 0.0;
     for (int m = 0; m < kComp; ++m) {
       s += cp.pi[m];
-      cdf[m] = s;
+      cdf[m] = __double_as_longlong(s);
     }
+    total = s;
   }
   __syncthreads();
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= S) return;
-  VmfRng rng{seed, static_cast<uint32_t>(s), static_cast<uint32_t>(b), 0u};
-  const double2 u0 = rng.uniform2();
-  int m = 0;
-  const double target = u0.x * cdf[kComp - 1];
-  while (m < kComp - 1 && cdf[m] < target) ++m;
-  const double kap = cp.kappa[m], bb = wb[m], x0 = wx0[m], cc = wc[m];
-  double w = 1.0;
-  bool ok = false;
-  for (int tries = 0; tries < 1000; ++tries) {
-    const double g1 = rng.gamma35(), g2 = rng.gamma35();
-    const double z = g1 / (g1 + g2);  // Beta(7/2, 7/2)
-    w = (1.0 - (1.0 + bb) * z) / (1.0 - (1.0 - bb) * z);
-    const double u = rng.uniform2().x;
-    if (kap * w + (kDim - 1.0) * log(1.0 - x0 * w) - cc >= log(u)) {
-      ok = true;
-      break;
+  for (int s = blockIdx.x * kVmfThreads + threadIdx.x; s < S; s += gridDim.x * kVmfThreads) {
+    VmfRng rng{seed, static_cast<uint32_t>(s), static_cast<uint32_t>(b), 0u};
+    uint64_t ux, uy;
+    rng.bits2(&ux, &uy);
+    // the component and the member of the K-fold equivalence class
+    const long long target = __double_as_longlong((static_cast<double>(ux >> 1) + 0.5) * (1.0 / 9007199254740992.0) * total);
+    int m = 0;
+    while (m < kComp - 1 && cdf[m] < target) ++m;
+    const int k = min(K - 1, static_cast<int>(__umul64hi(uy << 10, static_cast<uint64_t>(K))));
+    const float a = sa[m], half = shalf[m];
+    const df32 bb = sb[m];
+    df32 w{1.f, 0.f}, sw{0.f, 0.f};
+    bool ok = false;
+    for (int tries = 0; tries < 1000 && !ok; ++tries) {
+      const VmfRng at = rng;
+      const df32 g1 = rng.gamma35(), g2 = rng.gamma35();
+      uint64_t u, unused;
+      rng.bits2(&u, &unused);
+      const df32 bg = df_times(bb, g1), q = df_sum(g2, bg);
+      const float rq = 1.0f / q.h;
+      const float t1 = a * ((g2.h - g1.h) + (g2.l - g1.l)) * rq;
+      const float t2 = (kDim - 1.0f) * logf(half * (g1.h + g2.h) * rq);
+      const float lu = -df_neg_log(u, GaussTab()).h;
+      const float d = t1 + t2 - lu;
+      // FP32 rounding of terms of size |t1|, |t2|, |lu|: below 16 * 2^-24 each
+      const float margin = 1e-5f * (1.0f + fabsf(t1) + fabsf(t2) + fabsf(lu));
+      ok = d >= 0.0f;
+      if (fabsf(d) <= margin) ok = vmf_accept_fp64(at, cp.kappa[m], wb[m], wx0[m], wc[m]);
+      const df32 r = df_recip(q);
+      w = df_times(df_sum(g2, df32{-bg.h, -bg.l}), r);
+      const df32 root = df_times(df_sqrt(df_times(bg, g2)), r);
+      sw = df32{2.0f * root.h, 2.0f * root.l};
     }
-  }
-  if (!ok) dev_fail(status, LRQ_ETIMEOUT);
-  double v[kDim], dot = 0.0;
-  for (int d = 0; d < kDim; d += 2) {
-    const double2 nn = rng.normal2();
-    v[d] = nn.x;
-    v[d + 1] = nn.y;
-  }
-  for (int d = 0; d < kDim; ++d) dot += v[d] * cp.mu[m][d];
-  double nv = 0.0;
-  for (int d = 0; d < kDim; ++d) {
-    v[d] -= dot * cp.mu[m][d];
-    nv += v[d] * v[d];
-  }
-  nv = nv > 0.0 ? 1.0 / sqrt(nv) : 0.0;
-  const double sw = sqrt(fmax(0.0, 1.0 - w * w));
-  double x[kDim];
-  for (int d = 0; d < kDim; ++d) x[d] = w * cp.mu[m][d] + sw * v[d] * nv;
-  // random member of the K-fold equivalence class
-  const int k = min(K - 1, static_cast<int>(u0.y * K));
-  double sn, cs;
-  sincospi(2.0 * k / static_cast<double>(K), &sn, &cs);
-  float2* out = C + (static_cast<int64_t>(b) * S + s) * (kDim / 2);
-  for (int j = 0; j < kDim / 2; ++j) {
-    const double re = x[2 * j], im = x[2 * j + 1];
-    out[j] = make_float2(static_cast<float>(re * cs - im * sn), static_cast<float>(re * sn + im * cs));
+    if (!ok) dev_fail(status, LRQ_ETIMEOUT);
+    // a Gaussian vector (up to its scale) made orthogonal to mu
+    df32 v[kDim], dot{0.f, 0.f};
+#pragma unroll
+    for (int d = 0; d < kDim; d += 2) {
+      uint64_t e, f;
+      rng.bits2(&e, &f);
+      const df32 rad = df_sqrt(df_neg_log(e, GaussTab()));
+      df32 sn, cs;
+      df_sincos(f, GaussTab(), &sn, &cs);
+      v[d] = df_times(rad, cs);
+      v[d + 1] = df_times(rad, sn);
+    }
+#pragma unroll
+    for (int d = 0; d < kDim; ++d) dot = df_sum(dot, df_times(v[d], smu[m][d]));
+    df32 nv{0.f, 0.f};
+#pragma unroll
+    for (int d = 0; d < kDim; ++d) {
+      const df32 t = df_times(dot, smu[m][d]);
+      v[d] = df_sum(v[d], df32{-t.h, -t.l});
+      nv = df_sum(nv, df_times(v[d], v[d]));
+    }
+    const df32 scale = nv.h > 0.f ? df_times(sw, df_recip(df_sqrt(nv))) : df32{0.f, 0.f};
+    const df32 cs = root_c[k], sn = root_s[k];
+    float2* out = C + (static_cast<int64_t>(b) * S + s) * (kDim / 2);
+#pragma unroll
+    for (int j = 0; j < kDim / 2; ++j) {
+      const df32 re = df_sum(df_times(w, smu[m][2 * j]), df_times(scale, v[2 * j]));
+      const df32 im = df_sum(df_times(w, smu[m][2 * j + 1]), df_times(scale, v[2 * j + 1]));
+      const df32 p = df_times(im, sn), q = df_times(im, cs);
+      const df32 x = df_sum(df_times(re, cs), df32{-p.h, -p.l}), y = df_sum(df_times(re, sn), q);
+      out[j] = make_float2(x.h, y.h);
+    }
   }
 }
 
@@ -601,9 +741,25 @@ int64_t proposal_num_params(int F) {
 
 int launch_features(const float2* V, int B, int64_t n, int r, const double* lambda, float2* Vg, float* feat,
                     int32_t* status, cudaStream_t st) {
-  features_kernel<<<B, 256, 0, st>>>(V, n, r, lambda, Vg, feat, status);
+  // blocks per instance: about two per SM over all instances, a group of rows
+  // each at least, at most the portable cluster size
+  int nb = 1;
+  while (nb < 8 && static_cast<int64_t>(B) * nb * 2 <= 2 * num_sms_current() && n > static_cast<int64_t>(nb) * kFeatThreads)
+    nb *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(B) * nb);
+  cfg.blockDim = dim3(kFeatThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = nb;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const int e = cuda_check(cudaLaunchKernelEx(&cfg, features_kernel, V, n, r, lambda, Vg, feat, status),
+                           "features_kernel");
   count_launch();
-  return cuda_check(cudaGetLastError(), "features_kernel");
+  return e;
 }
 
 // BF16 mode on the tensor cores (k_mlp_tc.cu); FP32 mode on the CUDA cores
@@ -685,8 +841,11 @@ int launch_vmf_nll(const float* O, int B, const float* X, int T, double* loss, f
 
 int launch_vmf_sample(const float* O, int B, int S, int K, uint64_t seed, float2* C, int32_t* status,
                       cudaStream_t st) {
-  dim3 grid(static_cast<unsigned>(ceil_div(S, 128)), static_cast<unsigned>(B));
-  vmf_sample_kernel<<<grid, 128, 0, st>>>(O, B, S, K, seed, C, status);
+  // about eight blocks per SM over all instances: a block works out its
+  // instance's parameters once (a few us of FP64) and then loops over samples
+  const int64_t per = std::max<int64_t>(1, ceil_div(static_cast<int64_t>(8) * num_sms_current(), B));
+  dim3 grid(static_cast<unsigned>(std::min<int64_t>(ceil_div(S, kVmfThreads), per)), static_cast<unsigned>(B));
+  vmf_sample_kernel<<<grid, kVmfThreads, 0, st>>>(O, B, S, K, seed, C, status);
   count_launch();
   return cuda_check(cudaGetLastError(), "vmf_sample_kernel");
 }
