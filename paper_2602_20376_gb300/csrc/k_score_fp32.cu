@@ -52,54 +52,121 @@ int launch_check_finite(const float* x, int64_t count, int32_t* status, cudaStre
 }
 
 // ---------------------------------------------------------------------------
-// T = sum_i conj(V_i) in FP64 (the class-0 base of the odd-K indicator form).
-// Stage 1: each block sums a contiguous row range; stage 2 adds the blocks in
-// order (deterministic).
+// One pass over V for the tensor-core mode: the finiteness check, each block's
+// largest |component| and (sums) each block's part of T = sum_i conj(V_i) in
+// FP64 (the class-0 base of the odd-K indicator form).  The packing kernel
+// reduces the parts (in block order: deterministic).  Bound: FP64 (2r
+// additions a row; the conversions from FP32 are integer operations, since a
+// conversion instruction runs on the FP64 unit too).
 // ---------------------------------------------------------------------------
-__global__ void colsum_stage1(const float2* __restrict__ V, int64_t n, int r, double* __restrict__ Tpart) {
-  __shared__ double red[256][2 * kMaxRank];
-  int64_t rows_per_block = ceil_div(n, gridDim.x);
-  int64_t i0 = static_cast<int64_t>(blockIdx.x) * rows_per_block;
-  int64_t i1 = min(n, i0 + rows_per_block);
+__device__ __forceinline__ double exact_double(float x) {
+  const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  if (e == 0u || e == 0xffu) return static_cast<double>(x);  // zero, subnormal, infinite, NaN
+  return __hiloint2double(static_cast<int>((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3)) + (896 << 20),
+                          static_cast<int>(b << 29));
+}
+
+// Sums 16 doubles over the warp, halving the values at every step (16 additions
+// a lane instead of 80): lane l ends with the total of value l >> 1.
+__device__ __forceinline__ double warp_sums16(double (&v)[16]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 8, m = 16; k > 0; k >>= 1, m >>= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int q = 0; q < k; ++q) {
+      const double give = up ? v[q] : v[k + q], keep = up ? v[k + q] : v[q];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, give, m);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+template <int R, bool SUMS>
+__global__ void __launch_bounds__(kVScanThreads) v_scan_kernel(const float2* __restrict__ V, int64_t n,
+                                                               float* __restrict__ amax_part,
+                                                               double* __restrict__ Tpart, int32_t* status) {
+  constexpr int NW = kVScanThreads / 32, kRows = R <= 4 ? 4 : 2;  // rows in flight per thread
+  __shared__ double red[NW][2 * kMaxRank];
+  __shared__ float wmax[NW];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double acc[2 * kMaxRank];
 #pragma unroll
   for (int j = 0; j < 2 * kMaxRank; ++j) acc[j] = 0.0;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+  float mx = 0.f;
+  bool bad = false;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * kVScanThreads;
+  for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * kVScanThreads + threadIdx.x; i0 < n; i0 += kRows * stride) {
+    float2 v[kRows][R];
 #pragma unroll
-    for (int j = 0; j < kMaxRank; ++j)
-      if (j < r) {
-        float2 v = V[i * r + j];
-        acc[2 * j] += v.x;
-        acc[2 * j + 1] -= v.y;
+    for (int q = 0; q < kRows; ++q)
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+        v[q][j] = i0 + q * stride < n ? V[(i0 + q * stride) * R + j] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < kRows; ++q)
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        bad |= !isfinite(v[q][j].x) || !isfinite(v[q][j].y);
+        mx = fmaxf(mx, fmaxf(fabsf(v[q][j].x), fabsf(v[q][j].y)));
+        if (SUMS && i0 + q * stride < n) {
+          acc[2 * j] += exact_double(v[q][j].x);
+          acc[2 * j + 1] -= exact_double(v[q][j].y);
+        }
       }
   }
+  if (__any_sync(0xffffffffu, bad) && lane == 0) dev_fail(status, LRQ_EINVAL);
 #pragma unroll
-  for (int j = 0; j < 2 * kMaxRank; ++j) red[threadIdx.x][j] = acc[j];
-  __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h)
-      for (int j = 0; j < 2 * r; ++j) red[threadIdx.x][j] += red[threadIdx.x + h][j];
-    __syncthreads();
+  for (int m = 16; m > 0; m >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, m));
+  if (lane == 0) wmax[warp] = mx;
+  if (SUMS) {
+    const double v = warp_sums16(acc);
+    if ((lane & 1) == 0) red[warp][lane >> 1] = v;
   }
-  if (threadIdx.x < 2 * r) Tpart[blockIdx.x * 2 * kMaxRank + threadIdx.x] = red[0][threadIdx.x];
+  __syncthreads();
+  if (SUMS && threadIdx.x < 2 * R) {
+    double v = red[0][threadIdx.x];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) v += red[w][threadIdx.x];
+    Tpart[static_cast<int64_t>(blockIdx.x) * 2 * kMaxRank + threadIdx.x] = v;
+  }
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < NW; ++w) mx = fmaxf(mx, wmax[w]);
+    amax_part[blockIdx.x] = mx;
+  }
 }
 
-__global__ void colsum_stage2(const double* __restrict__ Tpart, int nblocks, int r, double* __restrict__ T) {
-  int j = threadIdx.x;
-  if (j >= 2 * r) return;
-  double a = 0.0;
-  for (int b = 0; b < nblocks; ++b) a += Tpart[b * 2 * kMaxRank + j];
-  T[j] = a;
+// At most one block per SM; few rows a thread while that spreads them over more
+// SMs (n = 20000, r = 4: 4.4 us, 15.1 with 2048 rows a block).
+int v_scan_blocks(int64_t n) {
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kVScanMaxBlocks, ceil_div(n, kVScanThreads))));
 }
 
-int launch_colsum(const float2* V, int64_t n, int r, double* Tpart, double* T, int nblocks, cudaStream_t st) {
-  colsum_stage1<<<nblocks, 256, 0, st>>>(V, n, r, Tpart);
+int launch_v_scan(const float2* V, int64_t n, int r, bool sums, float* amax_part, double* Tpart, int32_t* status,
+                  cudaStream_t st) {
+  const int blocks = v_scan_blocks(n);
+  switch (r) {
+#define LRQ_VSCAN_CASE(RR)                                                                            \
+  case RR:                                                                                            \
+    if (sums)                                                                                         \
+      v_scan_kernel<RR, true><<<blocks, kVScanThreads, 0, st>>>(V, n, amax_part, Tpart, status);      \
+    else                                                                                              \
+      v_scan_kernel<RR, false><<<blocks, kVScanThreads, 0, st>>>(V, n, amax_part, Tpart, status);     \
+    break;
+    LRQ_VSCAN_CASE(1)
+    LRQ_VSCAN_CASE(2)
+    LRQ_VSCAN_CASE(3)
+    LRQ_VSCAN_CASE(4)
+    LRQ_VSCAN_CASE(5)
+    LRQ_VSCAN_CASE(6)
+    LRQ_VSCAN_CASE(7)
+    LRQ_VSCAN_CASE(8)
+#undef LRQ_VSCAN_CASE
+    default:
+      return fail(LRQ_EUNSUPPORTED, "v_scan: r out of range");
+  }
   count_launch();
-  int e = cuda_check(cudaGetLastError(), "colsum_stage1");
-  if (e) return e;
-  colsum_stage2<<<1, 32, 0, st>>>(Tpart, nblocks, r, T);
-  count_launch();
-  return cuda_check(cudaGetLastError(), "colsum_stage2");
+  return cuda_check(cudaGetLastError(), "v_scan_kernel");
 }
 
 // ---------------------------------------------------------------------------
@@ -248,37 +315,48 @@ int launch_score_fp32(const ScorePlan& p, const Alphabet& a, const float2* V, co
 // selection key (score bits above the complemented index: larger key = larger
 // f, ties to the smaller index).
 // ---------------------------------------------------------------------------
-__global__ void finalize_kernel(const double* __restrict__ partial, int nsplit, int64_t S, int64_t S_pad, int r,
-                                const double* __restrict__ T, float* __restrict__ scores,
-                                uint64_t* __restrict__ keys) {
-  int64_t s = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (s >= S) return;
-  double v[2 * kMaxRank];
-#pragma unroll
-  for (int j = 0; j < 2 * kMaxRank; ++j) v[j] = (T && j < 2 * r) ? T[j] : 0.0;
-  for (int c = 0; c < nsplit; ++c) {
-    const double* src = partial + (static_cast<int64_t>(c) * S_pad + s) * (2 * r);
-#pragma unroll
-    for (int j = 0; j < 2 * kMaxRank; ++j)
-      if (j < 2 * r) v[j] += src[j];
+// A thread per (candidate, component) adds the chunk partials (coalesced
+// reads, 2r times as many threads as candidates), then one per candidate forms
+// f.  A thread per candidate took 14.5 us at S = 2^14, 16 chunks, r = 4, 7.6
+// now; same additions in the same order.
+constexpr int kFinThreads = 256;
+
+__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const double* __restrict__ partial, int nsplit,
+                                                               int64_t S, int64_t S_pad, int r2,
+                                                               const double* __restrict__ T,
+                                                               float* __restrict__ scores, uint64_t* __restrict__ keys) {
+  __shared__ double vj[kFinThreads];
+  const int per = kFinThreads / r2;  // candidates per block
+  const int c = threadIdx.x / r2, j = threadIdx.x - c * r2;
+  const int64_t s0 = static_cast<int64_t>(blockIdx.x) * per;
+  double v = 0.0;
+  if (c < per && s0 + c < S) {
+    v = T ? T[j] : 0.0;
+    const double* src = partial + (s0 + c) * r2 + j;
+#pragma unroll 4
+    for (int k = 0; k < nsplit; ++k) v += src[static_cast<int64_t>(k) * S_pad * r2];
   }
+  vj[threadIdx.x] = v;
+  __syncthreads();
+  const int64_t s = s0 + threadIdx.x;
+  if (static_cast<int>(threadIdx.x) >= per || s >= S) return;
   double f = 0.0;
-#pragma unroll
-  for (int j = 0; j < 2 * kMaxRank; ++j)
-    if (j < 2 * r) f += v[j] * v[j];
-  float ff = static_cast<float>(f);
+  for (int q = 0; q < r2; ++q) {
+    const double x = vj[threadIdx.x * r2 + q];
+    f += x * x;
+  }
+  const float ff = static_cast<float>(f);
   if (scores) scores[s] = ff;
   if (keys)
     keys[s] = (static_cast<uint64_t>(__float_as_uint(ff)) << 32) |
               static_cast<uint64_t>(0xFFFFFFFFu - static_cast<uint32_t>(s));
 }
 
-int launch_finalize(const ScorePlan& p, const Alphabet& a, const double* partial, const double* T,
-                    float* scores, uint64_t* keys, cudaStream_t st) {
-  (void)a;
-  int64_t S_pad = p.c_tiles * 128;
-  finalize_kernel<<<static_cast<unsigned>(ceil_div(p.S, 256)), 256, 0, st>>>(partial, p.npart, p.S, S_pad, p.r,
-                                                                             T, scores, keys);
+int launch_finalize(const ScorePlan& p, const double* partial, const double* T, float* scores, uint64_t* keys,
+                    cudaStream_t st) {
+  const int per = kFinThreads / (2 * p.r);
+  finalize_kernel<<<static_cast<unsigned>(ceil_div(p.S, per)), kFinThreads, 0, st>>>(
+      partial, p.npart, p.S, p.c_tiles * 128, 2 * p.r, T, scores, keys);
   count_launch();
   return cuda_check(cudaGetLastError(), "finalize_kernel");
 }

@@ -90,6 +90,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "lrq_device.cuh"
@@ -744,50 +745,6 @@ struct PackTables {
   float beta_r[8], beta_i[8];  // per-indicator coefficients
 };
 
-// augmented rows: tile t, chunk ch, row (b*ROWS + i) for boundary line
-// line(b), 8 slots
-template <int K, int KCH>
-__global__ void pack_vaug_kernel(const float2* __restrict__ V, int64_t n, int r, int64_t n_tiles, PackTables tb,
-                                 uint8_t* __restrict__ tiles) {
-  using Sh = TcShape<K, KCH>;
-  using L = TcLayout<K, KCH>;
-  const int64_t total = n_tiles * Sh::N1;
-  int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (q >= total) return;
-  const int64_t t = q / Sh::N1;
-  const int rowin = static_cast<int>(q % Sh::N1);
-  const int m = Sh::line(rowin / Sh::ROWS), i = rowin % Sh::ROWS;
-  const int64_t ig = t * Sh::ROWS + i;
-  float slot[16];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) slot[k] = 0.f;
-  if (ig < n) {
-    // a row's signs do not change under a positive scale: a power of two
-    // brings its largest component into [1, 2), so every product and the F16
-    // accumulator stay far inside the F16 range and keep its precision
-    float mx = 0.f;
-    for (int jj = 0; jj < r; ++jj) {
-      const float2 v = V[ig * r + jj];
-      mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
-    }
-    const int sh = (mx > 0.f && isfinite(mx)) ? -ilogbf(mx) : 0;
-    const float bc = tb.bcos[m], bs = tb.bsin[m];
-    for (int jj = 0; jj < r; ++jj) {
-      const float2 v = V[ig * r + jj];
-      // rho_m V = (bc - i bs)(vr + i vi)
-      slot[jj] = ldexpf(fmaf(bc, v.y, -bs * v.x), sh);     // Im(rho_m V_ij)
-      slot[r + jj] = ldexpf(fmaf(bc, v.x, bs * v.y), sh);  // Re(rho_m V_ij)
-    }
-  }
-#pragma unroll
-  for (int ch = 0; ch < KCH; ++ch) {
-    __align__(16) __half h[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) h[k] = __float2half_rn(slot[ch * 8 + k]);
-    *reinterpret_cast<uint4*>(tiles + t * L::TILE_BYTES + (ch * Sh::N1 + rowin) * 16) = *reinterpret_cast<uint4*>(h);
-  }
-}
-
 // Scales of the GEMM2 operands.  B2 entries are components of
 // beta conj(V_i) with |beta| <= 2, so |B2| < 3 m_i, m_i = max |V_i component|.
 // Coordinate i is scaled by 2^e_i, e_i = 5 - ilogb(m_i), which moves m_i into
@@ -797,122 +754,158 @@ __global__ void pack_vaug_kernel(const float2* __restrict__ V, int64_t n, int r,
 // entry times 2^g, one global power of two (g = 5 - ilogb(max_i m_i)) that the
 // epilogue removes.  2^(g - e_i) must be an E4M3 number (down to 2^-9), so
 // e_i <= g + 9: rows more than 2^9 below the largest lose relative precision
-// (their share of the sums is as small).  scale = {2^g, 2^-g, max m_i bits}.
-__global__ void b2_amax_kernel(const float2* __restrict__ V, int64_t count, float* __restrict__ scale) {
-  float m = 0.f;
-  for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < count;
-       q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const float2 v = V[q];
-    m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  // non-negative floats order like their bit patterns
-  if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(reinterpret_cast<unsigned*>(scale + 2), __float_as_uint(m));
+// (their share of the sums is as small).  scale = {2^g, 2^-g, max m_i}.
+__device__ __forceinline__ int b2_global_exp(float amax) {
+  return 5 - ((amax > 0.f && isfinite(amax)) ? ilogbf(amax) : 5);
 }
 
-__device__ __forceinline__ int b2_global_exp(const float* scale) {
-  const float a = scale[2];
-  return 5 - ((a > 0.f && isfinite(a)) ? ilogbf(a) : 5);
+// 2^e, |e| <= 252, as two normal factors: a value times both is ldexpf(value, e)
+// but for roundings below 2^-126, which the F16 and E4M3 operands do not have.
+__device__ __forceinline__ float2 pow2_pair(int e) {
+  const int h = e >> 1;
+  return make_float2(__int_as_float((h + 127) << 23), __int_as_float((e - h + 127) << 23));
 }
 
-__global__ void b2_scale_kernel(float* scale) {
-  if (threadIdx.x != 0) return;
-  const int g = b2_global_exp(scale);
-  scale[0] = ldexpf(1.f, g);
-  scale[1] = ldexpf(1.f, -g);
-}
-
-// e_i of coordinate ig (see above); g for a zero row
-__device__ __forceinline__ int b2_coord_exp(const float2* __restrict__ V, int64_t ig, int r, int g) {
-  float m = 0.f;
-  for (int jj = 0; jj < r; ++jj) {
-    const float2 v = V[ig * r + jj];
-    m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
-  }
-  const int e = (m > 0.f && isfinite(m)) ? 5 - ilogbf(m) : g;
-  return e < g ? g : (e > g + 9 ? g + 9 : e);
-}
-
-// GEMM2 B rows (FP8 E4M3): tile t, K-chunk kc (16 reduction entries), row nr:
-// output column nr (hi part) for nr < NOUT, output column nr - NOUT (lo part,
-// the rounding remainder of hi) above
-// e_i from the coordinate's indicator magnitude byte 2^(g - e_i) (written by
-// pack_indicator_scale_kernel, below): d = g - e_i in [-9, 0]
-__device__ __forceinline__ int b2_exp_from_code(uint32_t code, int g) {
-  const int d = code >= 8u ? static_cast<int>(code >> 3) - 7 : (code == 4u ? -7 : (code == 2u ? -8 : -9));
-  return g - d;
-}
+// Packs whole tiles from V: the augmented rows of GEMM1 (tile, chunk ch, row
+// b * ROWS + i for boundary line line(b), 8 F16 slots), the FP8 class rows of
+// GEMM2 (K-chunk of 16 reduction entries, output column nc: hi parts, then
+// NOUT rows on the remainders, lo) and the indicator magnitudes 2^(g - e_i) as
+// E4M3 bytes (0 past n).  A block keeps the tile's rows of V and each
+// coordinate's exponents in shared memory; the first block also finishes what
+// v_scan_kernel left in per-block parts: the scale and (odd K) the column sums
+// T of conj(V).  Bound: the conversions and the writes of the packed tiles (2.1
+// times V's bytes).  n = 10^6, r = 3, K = 3: one pass here 48 us after
+// v_scan's 28; seven passes over V took 225 (column sums 105, augmented rows
+// 23, largest entry 10, exponents 7, class rows 78).
+constexpr int kPackThreads = 256;
 
 template <int K, int KCH>
-__global__ void pack_b2_kernel(const float2* __restrict__ V, int64_t n, int r, int64_t n_tiles, PackTables tb,
-                               const float* __restrict__ scale, const uint8_t* __restrict__ iwb,
-                               uint8_t* __restrict__ tiles) {
+__global__ void __launch_bounds__(kPackThreads) pack_tiles_kernel(const float2* __restrict__ V, int64_t n, int r,
+                                                                  int64_t n_tiles,
+                                                                  const __grid_constant__ PackTables tb,
+                                                                  const float* __restrict__ amax_part,
+                                                                  const double* __restrict__ Tpart, int nparts,
+                                                                  float* __restrict__ scale, double* __restrict__ T,
+                                                                  uint8_t* __restrict__ tiles) {
   using Sh = TcShape<K, KCH>;
   using L = TcLayout<K, KCH>;
-  const int64_t total = n_tiles * L::B2ROWS;
-  int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (q >= total) return;
-  const int64_t t = q / L::B2ROWS;
-  const int within = static_cast<int>(q % L::B2ROWS);
-  const int kc = within / L::N2R, nr = within % L::N2R;
-  const bool lo = nr >= Sh::NOUT;
-  const int nc = lo ? nr - Sh::NOUT : nr;
-  const int g = b2_global_exp(scale);
-  __align__(16) uint8_t h[16];
+  static_assert(Sh::ROWS <= kPackThreads && Sh::ROWS % 4 == 0 && L::N2R == 2 * Sh::NOUT, "a thread per coordinate");
+  __shared__ float2 vs[Sh::ROWS * kMaxRank];
+  __shared__ float wmax[kPackThreads / 32];
+  __shared__ float2 sc1[Sh::ROWS], sc2[Sh::ROWS];  // 2^e as two factors (|e| up to 149)
+  __shared__ __align__(4) uint8_t mag[Sh::ROWS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float amax = 0.f;
+  for (int b = threadIdx.x; b < nparts; b += kPackThreads) amax = fmaxf(amax, amax_part[b]);
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const int kk = kc * 16 + k;
-    const int gc = kk / Sh::ROWS, i = kk % Sh::ROWS;
-    const int64_t ig = t * Sh::ROWS + i;
-    const int jj = nc >> 1;
-    float val = 0.f;
-    if (ig < n && jj < r) {
-      float2 v = V[ig * r + jj];
-      const float br = tb.beta_r[gc], bi = tb.beta_i[gc];
-      // beta conj(V) = (br vr + bi vi) + i (bi vr - br vi)
-      val = ldexpf((nc & 1) ? fmaf(bi, v.x, -br * v.y) : fmaf(br, v.x, bi * v.y), b2_exp_from_code(iwb[ig], g));
+  for (int m = 16; m > 0; m >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, m));
+  if (lane == 0) wmax[warp] = amax;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kPackThreads / 32; ++w) amax = fmaxf(amax, wmax[w]);
+  const int g = b2_global_exp(amax);
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) {
+      scale[0] = ldexpf(1.f, g);
+      scale[1] = ldexpf(1.f, -g);
+      scale[2] = amax;
     }
-    const __nv_fp8_e4m3 hi(val);
-    h[k] = lo ? __nv_fp8_e4m3(val - static_cast<float>(hi)).__x : hi.__x;
+    if (K % 2 == 1) {
+      for (int j = warp; j < 2 * r; j += kPackThreads / 32) {
+        double a = 0.0;
+        for (int b = lane; b < nparts; b += 32) a += Tpart[static_cast<int64_t>(b) * 2 * kMaxRank + j];
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) a += __shfl_xor_sync(0xffffffffu, a, m);
+        if (lane == 0) T[j] = a;
+      }
+    }
   }
-  *reinterpret_cast<uint4*>(tiles + t * L::TILE_BYTES + L::B2_OFF_IN_STAGE + within * 16) =
-      *reinterpret_cast<uint4*>(h);
-}
-
-// Indicator magnitudes 2^(g - e_i) as E4M3 bytes, four coordinates per word
-// (lowest coordinate in the lowest byte), R / 4 words per tile; 0 past n.
-// Written twice: into `iw` (read back by the GEMM2 row packing) and into the
-// magnitude row of each packed tile (read by the scoring kernel's rounding
-// threads from the tile's stage).
-template <int K, int KCH>
-__global__ void pack_indicator_scale_kernel(const float2* __restrict__ V, int64_t n, int r, int64_t words,
-                                            const float* __restrict__ scale, uint32_t* __restrict__ iw,
-                                            uint8_t* __restrict__ tiles) {
-  using Sh = TcShape<K, KCH>;
-  using L = TcLayout<K, KCH>;
-  const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (q >= words) return;
-  const int g = b2_global_exp(scale);
-  uint32_t w = 0;
-  for (int c = 0; c < 4; ++c) {
-    const int64_t ig = q * 4 + c;
-    if (ig >= n) continue;
-    const int d = g - b2_coord_exp(V, ig, r, g);  // in [-9, 0]
-    // E4M3 2^d: normal ((d + 7) << 3) down to 2^-6, subnormal 0x4 >> (-7 - d) below
-    const uint32_t code = d >= -6 ? static_cast<uint32_t>(d + 7) << 3 : (0x4u >> (-7 - d));
-    w |= code << (8 * c);
+  for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+    const int64_t i0 = t * Sh::ROWS;
+    const int rows = static_cast<int>(min(static_cast<int64_t>(Sh::ROWS), n - i0));
+    uint8_t* const tile = tiles + t * L::TILE_BYTES;
+    __syncthreads();  // the previous tile has been packed
+    for (int q = threadIdx.x; q < rows * r; q += kPackThreads) vs[q] = V[i0 * r + q];
+    __syncthreads();
+    if (threadIdx.x < Sh::ROWS) {
+      const int i = threadIdx.x;
+      float mx = 0.f;
+      if (i < rows)
+        for (int jj = 0; jj < r; ++jj) mx = fmaxf(mx, fmaxf(fabsf(vs[i * r + jj].x), fabsf(vs[i * r + jj].y)));
+      const bool fin = mx > 0.f && isfinite(mx);
+      const int lb = fin ? ilogbf(mx) : 0;
+      // a row's signs do not change under a positive scale: a power of two
+      // brings its largest component into [1, 2), so every product and the F16
+      // accumulator stay far inside the F16 range and keep its precision
+      sc1[i] = pow2_pair(fin ? -lb : 0);
+      int e = fin ? 5 - lb : g;
+      e = e < g ? g : (e > g + 9 ? g + 9 : e);
+      sc2[i] = pow2_pair(e);
+      const int d = g - e;  // in [-9, 0]
+      // E4M3 2^d: normal ((d + 7) << 3) down to 2^-6, subnormal 0x4 >> (-7 - d) below
+      mag[i] = i < rows ? static_cast<uint8_t>(d >= -6 ? (d + 7) << 3 : 0x4 >> (-7 - d)) : 0;
+    }
+    __syncthreads();
+    // N1 rows of GEMM1, then the class rows, four entries (one word) an item
+    for (int q = threadIdx.x; q < Sh::N1 + Sh::KD2 / 4 * Sh::NOUT; q += kPackThreads) {
+      if (q < Sh::N1) {
+        const int m = Sh::line(q / Sh::ROWS), i = q % Sh::ROWS;
+        const float bc = tb.bcos[m], bs = tb.bsin[m];
+        const float2 sc = sc1[i];
+#pragma unroll
+        for (int ch = 0; ch < KCH; ++ch) {
+          __align__(16) __half2 h[4];
+#pragma unroll
+          for (int k2 = 0; k2 < 4; ++k2) {
+            float x[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              // slots: Im(rho_m V_ij), j < r, then Re; rho_m V = (bc - i bs)(vr + i vi)
+              const int k = ch * 8 + 2 * k2 + e;
+              x[e] = 0.f;
+              if (i < rows && k < 2 * r) {
+                const float2 v = vs[i * r + (k < r ? k : k - r)];
+                x[e] = (k < r ? fmaf(bc, v.y, -bs * v.x) : fmaf(bc, v.x, bs * v.y)) * sc.x * sc.y;
+              }
+            }
+            h[k2] = __floats2half2_rn(x[0], x[1]);
+          }
+          *reinterpret_cast<uint4*>(tile + (ch * Sh::N1 + q) * 16) = *reinterpret_cast<const uint4*>(h);
+        }
+      } else {
+        const int it = q - Sh::N1, k4 = it / (4 * Sh::NOUT) * 4 + (it & 3), nc = (it >> 2) % Sh::NOUT, jj = nc >> 1;
+        const int gc = k4 * 4 / Sh::ROWS, i0 = k4 * 4 % Sh::ROWS;  // ROWS is a multiple of 16
+        const float br = tb.beta_r[gc], bi = tb.beta_i[gc];
+        uint32_t hi = 0, lo = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int i = i0 + k;
+          float val = 0.f;
+          if (i < rows && jj < r) {
+            const float2 v = vs[i * r + jj], sc = sc2[i];
+            // beta conj(V) = (br vr + bi vi) + i (bi vr - br vi)
+            val = ((nc & 1) ? fmaf(bi, v.x, -br * v.y) : fmaf(br, v.x, bi * v.y)) * sc.x * sc.y;
+          }
+          const __nv_fp8_e4m3 h(val);
+          hi |= static_cast<uint32_t>(h.__x) << (8 * k);
+          lo |= static_cast<uint32_t>(__nv_fp8_e4m3(val - static_cast<float>(h)).__x) << (8 * k);
+        }
+        uint32_t* const row =
+            reinterpret_cast<uint32_t*>(tile + L::B2_OFF_IN_STAGE + (k4 / 4 * L::N2R + nc) * 16) + (k4 & 3);
+        row[0] = hi;
+        row[Sh::NOUT * 4] = lo;
+      }
+    }
+    if (threadIdx.x < Sh::ROWS / 4)
+      reinterpret_cast<uint32_t*>(tile + L::MAG_OFF_IN_STAGE)[threadIdx.x] = reinterpret_cast<const uint32_t*>(mag)[threadIdx.x];
   }
-  iw[q] = w;
-  const int64_t t = q / (Sh::ROWS / 4);
-  const int wi = static_cast<int>(q % (Sh::ROWS / 4));
-  *reinterpret_cast<uint32_t*>(tiles + t * L::TILE_BYTES + L::MAG_OFF_IN_STAGE + 4 * wi) = w;
 }
 
 // directions: candidate tile ct, chunk ch, row s: slots [Re c, Im c, 0...]
+// (and the input check of C)
 template <int KCH>
 __global__ void pack_dirs_kernel(const float2* __restrict__ C, int64_t S, int r, int64_t c_tiles,
-                                 __half* __restrict__ ctp) {
+                                 __half* __restrict__ ctp, int32_t* status) {
   const int64_t total = c_tiles * kTcM;
   int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (q >= total) return;
@@ -925,10 +918,13 @@ __global__ void pack_dirs_kernel(const float2* __restrict__ C, int64_t S, int r,
     // a positive power-of-two scale (the largest component into [1, 2))
     // changes no decision and keeps the F16 products in range
     float mx = 0.f;
+    bool bad = false;
     for (int jj = 0; jj < r; ++jj) {
       const float2 c = C[q * r + jj];
       mx = fmaxf(mx, fmaxf(fabsf(c.x), fabsf(c.y)));
+      bad |= !isfinite(c.x) || !isfinite(c.y);
     }
+    if (bad) dev_fail(status, LRQ_EINVAL);
     const int sh = (mx > 0.f && isfinite(mx)) ? -ilogbf(mx) : 0;
     for (int jj = 0; jj < r; ++jj) {
       const float2 c = C[q * r + jj];
@@ -956,42 +952,23 @@ static PackTables make_pack_tables(const Alphabet& a) {
   return tb;
 }
 
-// The instance's operands (depend on V only): augmented rows, the GEMM2
-// scale, the per-coordinate indicator magnitudes and the class rows.
+// The instance's operands (depend on V only), from V and v_scan_kernel's parts.
 template <int K, int KCH>
 static int pack_v_impl(const ScorePlan& p, const Alphabet& a, const float2* V, void* tiles, float* scale,
-                       uint32_t* iw, cudaStream_t st) {
-  using Sh = TcShape<K, KCH>;
-  using L = TcLayout<K, KCH>;
-  PackTables tb = make_pack_tables(a);
-  int64_t nv = p.n_tiles * Sh::N1;
-  pack_vaug_kernel<K, KCH><<<static_cast<unsigned>(ceil_div(nv, 256)), 256, 0, st>>>(
-      V, p.n, p.r, p.n_tiles, tb, static_cast<uint8_t*>(tiles));
+                       const float* amax_part, const double* Tpart, int nparts, double* T, cudaStream_t st) {
+  const unsigned blocks = static_cast<unsigned>(std::min<int64_t>(p.n_tiles, static_cast<int64_t>(8) * num_sms_current()));
+  pack_tiles_kernel<K, KCH><<<blocks, kPackThreads, 0, st>>>(V, p.n, p.r, p.n_tiles, make_pack_tables(a), amax_part,
+                                                             Tpart, nparts, scale, T, static_cast<uint8_t*>(tiles));
   count_launch();
-  int e = cuda_check(cudaMemsetAsync(scale + 2, 0, sizeof(float), st), "cudaMemsetAsync(scale)");
-  if (e) return e;
-  const int64_t nvr = p.n * p.r;
-  b2_amax_kernel<<<static_cast<unsigned>(std::min<int64_t>(ceil_div(nvr, 256), 152 * 8)), 256, 0, st>>>(V, nvr,
-                                                                                                           scale);
-  b2_scale_kernel<<<1, 32, 0, st>>>(scale);
-  count_launch(2);
-  // the per-coordinate exponents first: the GEMM2 rows read them back
-  const int64_t words = p.n_tiles * (Sh::ROWS / 4);
-  pack_indicator_scale_kernel<K, KCH><<<static_cast<unsigned>(ceil_div(words, 256)), 256, 0, st>>>(
-      V, p.n, p.r, words, scale, iw, static_cast<uint8_t*>(tiles));
-  int64_t nb = p.n_tiles * L::B2ROWS;
-  pack_b2_kernel<K, KCH><<<static_cast<unsigned>(ceil_div(nb, 256)), 256, 0, st>>>(
-      V, p.n, p.r, p.n_tiles, tb, scale, reinterpret_cast<const uint8_t*>(iw), static_cast<uint8_t*>(tiles));
-  count_launch(2);
-  return cuda_check(cudaGetLastError(), "tc operand packing");
+  return cuda_check(cudaGetLastError(), "pack_tiles_kernel");
 }
 
 // The directions (depend on C only).
 template <int KCH>
-static int pack_dirs_impl(const ScorePlan& p, const float2* C, void* ct, cudaStream_t st) {
+static int pack_dirs_impl(const ScorePlan& p, const float2* C, void* ct, int32_t* status, cudaStream_t st) {
   int64_t nc = p.c_tiles * kTcM;
   pack_dirs_kernel<KCH><<<static_cast<unsigned>(ceil_div(nc, 256)), 256, 0, st>>>(C, p.S, p.r, p.c_tiles,
-                                                                                  static_cast<__half*>(ct));
+                                                                                  static_cast<__half*>(ct), status);
   count_launch();
   return cuda_check(cudaGetLastError(), "pack_dirs_kernel");
 }
@@ -1100,10 +1077,6 @@ size_t tc_bytes_tiles(int K, int r, int64_t n_tiles) {
 #undef LRQ_TILE
 }
 
-size_t tc_bytes_indicator_scale(int K, int r, int64_t n_tiles) {
-  return static_cast<size_t>(n_tiles) * static_cast<size_t>(tc_rows_per_tile(K, r));  // one byte per coordinate
-}
-
 size_t tc_bytes_dirs(int r, int64_t c_tiles) {
   int kch = r <= 4 ? 1 : 2;
   return static_cast<size_t>(c_tiles) * kch * kTcM * 16;
@@ -1124,20 +1097,18 @@ size_t tc_bytes_dirs(int r, int64_t c_tiles) {
     }                                                                   \
   } while (0)
 
-int launch_tc_pack_v(const ScorePlan& p, const Alphabet& a, const float2* V, void* tiles, void* scale, void* iw,
-                     cudaStream_t st) {
-  LRQ_TC_DISPATCH(pack_v_impl, p, a, V, tiles, static_cast<float*>(scale), static_cast<uint32_t*>(iw), st);
+int launch_tc_pack_v(const ScorePlan& p, const Alphabet& a, const float2* V, void* tiles, float* scale,
+                     const float* amax_part, const double* Tpart, int nparts, double* T, cudaStream_t st) {
+  LRQ_TC_DISPATCH(pack_v_impl, p, a, V, tiles, scale, amax_part, Tpart, nparts, T, st);
 }
 
-int launch_tc_pack_dirs(const ScorePlan& p, const float2* C, void* ct, cudaStream_t st) {
-  return p.r > 4 ? pack_dirs_impl<2>(p, C, ct, st) : pack_dirs_impl<1>(p, C, ct, st);
+int launch_tc_pack_dirs(const ScorePlan& p, const float2* C, void* ct, int32_t* status, cudaStream_t st) {
+  return p.r > 4 ? pack_dirs_impl<2>(p, C, ct, status, st) : pack_dirs_impl<1>(p, C, ct, status, st);
 }
 
-int launch_score_tc(const ScorePlan& p, const Alphabet& a, const void* tiles, const void* ct, const void* scale,
-                    const void* iw, double* partial, int32_t* status, cudaStream_t st) {
-  (void)a;
-  (void)iw;  // the magnitudes travel inside the packed tiles
-  LRQ_TC_DISPATCH(score_impl, p, tiles, ct, static_cast<const float*>(scale), partial, status, st);
+int launch_score_tc(const ScorePlan& p, const void* tiles, const void* ct, const float* scale, double* partial,
+                    int32_t* status, cudaStream_t st) {
+  LRQ_TC_DISPATCH(score_impl, p, tiles, ct, scale, partial, status, st);
 }
 
 }  // namespace lrq

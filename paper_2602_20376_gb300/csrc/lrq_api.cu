@@ -21,7 +21,6 @@ namespace lrq {
 int tc_rows_per_tile(int K, int r);
 int tc_workers_per_cta(int K, int r);
 size_t tc_bytes_tiles(int K, int r, int64_t n_tiles);
-size_t tc_bytes_indicator_scale(int K, int r, int64_t n_tiles);
 size_t tc_bytes_dirs(int r, int64_t c_tiles);
 
 static thread_local char g_last_error[512] = {0};
@@ -163,8 +162,10 @@ int plan_score(int64_t n, int r, int K, int64_t S, int mode, int top_m, int num_
   if (with_prep) {
     p->sz_T = 2 * kMaxRank * sizeof(double);
     p->off_T = take(cur, p->sz_T);
-    p->sz_Tpart = 256 * 2 * kMaxRank * sizeof(double);
+    p->sz_Tpart = kVScanMaxBlocks * 2 * kMaxRank * sizeof(double);
     p->off_Tpart = take(cur, p->sz_Tpart);
+    p->sz_amax = kVScanMaxBlocks * sizeof(float);
+    p->off_amax = take(cur, p->sz_amax);
   }
   if (mode == LRQ_MODE_BF16_TC) {
     if (with_prep) {
@@ -176,8 +177,6 @@ int plan_score(int64_t n, int r, int K, int64_t S, int mode, int top_m, int num_
     if (with_prep) {
       p->sz_scale = 4 * sizeof(float);
       p->off_scale = take(cur, p->sz_scale);
-      p->sz_iw = tc_bytes_indicator_scale(K, r, p->n_tiles);
-      p->off_iw = take(cur, p->sz_iw);
     }
   }
   p->sz_scores = static_cast<size_t>(S) * sizeof(float);
@@ -194,10 +193,10 @@ int plan_prepare(int64_t n, int r, int K, int mode, PrepLayout* L) {
   L->n_tiles = ceil_div(n, tc_rows_per_tile(K, r));
   size_t cur = 0;
   L->off_T = take(cur, 2 * kMaxRank * sizeof(double));
-  L->off_Tpart = take(cur, 256 * 2 * kMaxRank * sizeof(double));
+  L->off_Tpart = take(cur, kVScanMaxBlocks * 2 * kMaxRank * sizeof(double));
+  L->off_amax = take(cur, kVScanMaxBlocks * sizeof(float));
   L->off_tiles = take(cur, tc_bytes_tiles(K, r, L->n_tiles));
   L->off_scale = take(cur, 4 * sizeof(float));
-  L->off_iw = take(cur, tc_bytes_indicator_scale(K, r, L->n_tiles));
   L->total = cur;
   return LRQ_OK;
 }
@@ -252,21 +251,27 @@ struct InstanceOperands {
   const float2* V;
   uint8_t* tiles;   // packed coordinate tiles (tensor-core mode)
   float* scale;     // GEMM2 operand scale
-  uint8_t* iw;      // indicator magnitudes
   double* T;        // column sums of conj(V) (odd K, tensor-core mode)
-  double* Tpart;    // their per-block partials
+  double* Tpart;    // their per-block parts
+  float* amax;      // per-block largest |component|
 };
+
+static InstanceOperands prepared_operands(const PrepLayout& L, const float2* V, uint8_t* b) {
+  return InstanceOperands{V,
+                          b + L.off_tiles,
+                          reinterpret_cast<float*>(b + L.off_scale),
+                          reinterpret_cast<double*>(b + L.off_T),
+                          reinterpret_cast<double*>(b + L.off_Tpart),
+                          reinterpret_cast<float*>(b + L.off_amax)};
+}
 
 static int prepare_operands(const ScorePlan& p, const Alphabet& a, const InstanceOperands& io, int32_t* dev_status,
                             cudaStream_t st) {
-  int e;
-  if ((e = launch_check_finite(reinterpret_cast<const float*>(io.V), 2 * p.n * p.r, dev_status, st))) return e;
-  if (p.mode != LRQ_MODE_BF16_TC) return LRQ_OK;
-  if (p.K % 2 == 1) {
-    int nb = static_cast<int>(std::min<int64_t>(256, std::max<int64_t>(1, ceil_div(p.n, 4096))));
-    if ((e = launch_colsum(io.V, p.n, p.r, io.Tpart, io.T, nb, st))) return e;
-  }
-  return launch_tc_pack_v(p, a, io.V, io.tiles, io.scale, io.iw, st);
+  if (p.mode != LRQ_MODE_BF16_TC)
+    return launch_check_finite(reinterpret_cast<const float*>(io.V), 2 * p.n * p.r, dev_status, st);
+  const int e = launch_v_scan(io.V, p.n, p.r, p.K % 2 == 1, io.amax, io.Tpart, dev_status, st);
+  if (e) return e;
+  return launch_tc_pack_v(p, a, io.V, io.tiles, io.scale, io.amax, io.Tpart, v_scan_blocks(p.n), io.T, st);
 }
 
 // Directions -> scores -> top-m, on prepared operands; w is the per-call
@@ -280,20 +285,23 @@ static int score_directions(const ScorePlan& p, const Alphabet& a, const Instanc
   uint64_t* keys = reinterpret_cast<uint64_t*>(w + p.off_keys);
   uint64_t* keys_scratch = keys + p.S;
   if (generate && (e = launch_sample_directions(seed, p.S, p.r, Cf, st))) return e;
-  if ((e = launch_check_finite(reinterpret_cast<const float*>(Cf), 2 * p.S * p.r, dev_status, st))) return e;
   const double* Tuse = nullptr;
   if (p.mode == LRQ_MODE_BF16_TC) {
     if (p.K % 2 == 1) Tuse = io.T;
-    if ((e = launch_tc_pack_dirs(p, Cf, w + p.off_ct, st))) return e;
+    if ((e = launch_tc_pack_dirs(p, Cf, w + p.off_ct, dev_status, st))) return e;  // checks C too
     timing_start(st);
-    if ((e = launch_score_tc(p, a, io.tiles, w + p.off_ct, io.scale, io.iw, partial, dev_status, st))) return e;
+    if ((e = launch_score_tc(p, io.tiles, w + p.off_ct, io.scale, partial, dev_status, st))) return e;
     timing_stop(st);
   } else {
+    // directions drawn here are finite
+    if (!generate &&
+        (e = launch_check_finite(reinterpret_cast<const float*>(Cf), 2 * p.S * p.r, dev_status, st)))
+      return e;
     timing_start(st);
     if ((e = launch_score_fp32(p, a, io.V, Cf, partial, st))) return e;
     timing_stop(st);
   }
-  if ((e = launch_finalize(p, a, partial, Tuse, scores, keys, st))) return e;
+  if ((e = launch_finalize(p, partial, Tuse, scores, keys, st))) return e;
   return launch_topm(keys, p.S, p.top_m, keys_scratch, top_idx_out, top_f_out, st);
 }
 
@@ -358,8 +366,12 @@ int lrq_sample_score(const void* V, int64_t n, int r, int K, void* C, int genera
   if ((e = check_ws(ws, ws_bytes, p.total))) return e;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t* w = static_cast<uint8_t*>(ws);
-  InstanceOperands io{static_cast<const float2*>(V), w + p.off_tiles, reinterpret_cast<float*>(w + p.off_scale),
-                      w + p.off_iw, reinterpret_cast<double*>(w + p.off_T), reinterpret_cast<double*>(w + p.off_Tpart)};
+  InstanceOperands io{static_cast<const float2*>(V),
+                      w + p.off_tiles,
+                      reinterpret_cast<float*>(w + p.off_scale),
+                      reinterpret_cast<double*>(w + p.off_T),
+                      reinterpret_cast<double*>(w + p.off_Tpart),
+                      reinterpret_cast<float*>(w + p.off_amax)};
   const Alphabet a = make_alphabet(K);
   if ((e = prepare_operands(p, a, io, dev_status, st))) return e;
   return score_directions(p, a, io, static_cast<float2*>(C), generate_C != 0, seed, w, scores_out, top_idx_out,
@@ -401,9 +413,7 @@ int lrq_prepare(lrq_prepared_v* h, const void* V, void* buf, size_t buf_bytes, i
   ScorePlan p;
   plan_score(h->n, h->r, h->K, 1, h->mode, 1, num_sms_current(), &p, false);
   uint8_t* b = static_cast<uint8_t*>(buf);
-  InstanceOperands io{static_cast<const float2*>(V), b + h->L.off_tiles, reinterpret_cast<float*>(b + h->L.off_scale),
-                      b + h->L.off_iw, reinterpret_cast<double*>(b + h->L.off_T),
-                      reinterpret_cast<double*>(b + h->L.off_Tpart)};
+  InstanceOperands io = prepared_operands(h->L, static_cast<const float2*>(V), b);
   if ((e = prepare_operands(p, make_alphabet(h->K), io, dev_status, static_cast<cudaStream_t>(stream)))) return e;
   h->V = static_cast<const float2*>(V);
   h->buf = b;
@@ -433,8 +443,7 @@ int lrq_sample_score_prepared(const lrq_prepared_v* h, void* C, int generate_C, 
   plan_score(h->n, h->r, h->K, S, h->mode, top_m, num_sms_current(), &p, false);
   if ((e = check_ws(ws, ws_bytes, p.total))) return e;
   uint8_t* b = h->buf;
-  InstanceOperands io{h->V, b + h->L.off_tiles, reinterpret_cast<float*>(b + h->L.off_scale), b + h->L.off_iw,
-                      reinterpret_cast<double*>(b + h->L.off_T), reinterpret_cast<double*>(b + h->L.off_Tpart)};
+  InstanceOperands io = prepared_operands(h->L, h->V, b);
   return score_directions(p, make_alphabet(h->K), io, static_cast<float2*>(C), generate_C != 0, seed,
                           static_cast<uint8_t*>(ws), scores_out, top_idx_out, top_f_out, dev_status,
                           static_cast<cudaStream_t>(stream));

@@ -63,10 +63,10 @@ struct ScorePlan {
   size_t off_partial, sz_partial;   // npart x S_pad x 2r doubles
   size_t off_T, sz_T;               // 2r doubles (column sums of conj(V), odd K)
   size_t off_Tpart, sz_Tpart;       // per-block partial column sums
+  size_t off_amax, sz_amax;         // per-block largest |component|
   size_t off_tiles, sz_tiles;       // packed coordinate tiles: augmented rows (bf16) | class rows (FP8 hi | lo)
   size_t off_ct, sz_ct;             // packed directions (bf16)
   size_t off_scale, sz_scale;       // GEMM2 operand scale {2^g, 2^-g, max|V component|}
-  size_t off_iw, sz_iw;             // per-coordinate indicator magnitudes (E4M3, 1 byte per coordinate)
   size_t off_scores, sz_scores;     // S floats (when the caller passes none)
   size_t off_keys, sz_keys;         // selection keys
   size_t total;
@@ -80,7 +80,7 @@ int plan_score(int64_t n, int r, int K, int64_t S, int mode, int top_m, int num_
 // that does not depend on the directions.
 struct PrepLayout {
   int64_t n_tiles;
-  size_t off_T, off_Tpart, off_tiles, off_scale, off_iw;
+  size_t off_T, off_Tpart, off_amax, off_tiles, off_scale;
   size_t total;
 };
 int plan_prepare(int64_t n, int r, int K, int mode, PrepLayout* L);
@@ -105,12 +105,15 @@ void timing_stop(cudaStream_t st);
 // ---- launch helpers (return lrq_status; never synchronise) -----------------
 int launch_sample_directions(uint64_t seed, int64_t S, int r, float2* C, cudaStream_t st);
 int launch_check_finite(const float* x, int64_t count, int32_t* status, cudaStream_t st);
-int launch_colsum(const float2* V, int64_t n, int r, double* Tpart, double* T, int nblocks,
+constexpr int kVScanThreads = 256;
+constexpr int kVScanMaxBlocks = 152;
+int v_scan_blocks(int64_t n);
+int launch_v_scan(const float2* V, int64_t n, int r, bool sums, float* amax_part, double* Tpart, int32_t* status,
                   cudaStream_t st);
 int launch_score_fp32(const ScorePlan& p, const Alphabet& a, const float2* V, const float2* C,
                       double* partial, cudaStream_t st);
-int launch_finalize(const ScorePlan& p, const Alphabet& a, const double* partial, const double* T,
-                    float* scores, uint64_t* keys, cudaStream_t st);
+int launch_finalize(const ScorePlan& p, const double* partial, const double* T, float* scores, uint64_t* keys,
+                    cudaStream_t st);
 int launch_topm(const uint64_t* keys_in, int64_t count, int m, uint64_t* scratch, int64_t* top_idx,
                 float* top_f, cudaStream_t st);
 size_t topm_scratch_keys(int64_t count, int m);
@@ -169,11 +172,11 @@ size_t enum_workspace_bytes(int64_t n, int r);
 int launch_enumerate(const double2* V, int64_t n, int r, int K, uint8_t* z_out, double* f_out, int64_t* n_sets_out,
                      void* ws, int32_t* status, cudaStream_t st);
 // tensor-core path
-int launch_tc_pack_v(const ScorePlan& p, const Alphabet& a, const float2* V, void* tiles, void* scale, void* iw,
-                     cudaStream_t st);
-int launch_tc_pack_dirs(const ScorePlan& p, const float2* C, void* ct, cudaStream_t st);
-int launch_score_tc(const ScorePlan& p, const Alphabet& a, const void* tiles, const void* ct, const void* scale,
-                    const void* iw, double* partial, int32_t* status, cudaStream_t st);
+int launch_tc_pack_v(const ScorePlan& p, const Alphabet& a, const float2* V, void* tiles, float* scale,
+                     const float* amax_part, const double* Tpart, int nparts, double* T, cudaStream_t st);
+int launch_tc_pack_dirs(const ScorePlan& p, const float2* C, void* ct, int32_t* status, cudaStream_t st);
+int launch_score_tc(const ScorePlan& p, const void* tiles, const void* ct, const float* scale, double* partial,
+                    int32_t* status, cudaStream_t st);
 
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
