@@ -475,7 +475,6 @@ int lrq_rescore(const void* V, int64_t n, int r, int K, const void* C, int64_t S
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t* w = static_cast<uint8_t*>(ws);
   Alphabet a = make_alphabet(K);
-  if ((e = launch_check_finite(reinterpret_cast<const float*>(V), 2 * n * r, dev_status, st))) return e;
   return launch_rescore(p, a, static_cast<const float2*>(V), static_cast<const float2*>(C), S, idx,
                         reinterpret_cast<double*>(w + p.off_part), f_out, z_out, best_out, best_f_out, dev_status,
                         st);

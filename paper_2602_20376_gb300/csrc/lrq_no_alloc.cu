@@ -122,7 +122,6 @@ extern "C" int lrq_rescore_no_alloc(const void* V, int64_t n, int r, int K, cons
   if (e) return e;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Alphabet a = make_alphabet(K);
-  if ((e = launch_check_finite(reinterpret_cast<const float*>(V), 2 * n * r, dev_status, st))) return e;
   return launch_rescore(p, a, static_cast<const float2*>(V), static_cast<const float2*>(C), S, idx,
                         reinterpret_cast<double*>(static_cast<uint8_t*>(scratch) + p.off_part), f_out, z_out,
                         best_out, best_f_out, dev_status, st);

@@ -133,6 +133,50 @@ __device__ __forceinline__ uint32_t sign_offset(float x, float y) {
   return off;
 }
 
+// Sign pattern [p_m > 0] (bit m) and the smallest |p_m|, with the roundings of
+// decide_fp32.
+template <int K>
+__device__ __forceinline__ uint32_t sign_lines(float x, float y, float* pmin) {
+  constexpr int BK = (K % 2 == 0) ? K / 2 : K;
+  uint32_t bits = 0;
+  float mn = INFINITY;
+#pragma unroll
+  for (int m = 0; m < (BK + 1) / 2; ++m) {
+    const float c = boundary_cos<K>(m), s = boundary_sin<K>(m);
+    const int mm = BK - 1 - m;
+    float p, q;
+    if (s == 0.f) {
+      p = q = -y;
+    } else if (c == 0.f) {
+      p = q = -x;
+    } else {
+      const float t = x * s;
+      p = fmaf(y, c, -t);
+      q = K % 2 == 1 ? fmaf(y, c, t) : fmaf(y, -c, -t);
+    }
+    if (p > 0.f) bits |= 1u << m;
+    mn = fminf(mn, fabsf(p));
+    if (mm != m) {
+      if (q > 0.f) bits |= 1u << mm;
+      mn = fminf(mn, fabsf(q));
+    }
+  }
+  *pmin = mn;
+  return bits;
+}
+
+// A sign pattern whose code is k.
+template <int K>
+__device__ __forceinline__ uint32_t pattern_of(int k) {
+  if constexpr (K % 2 == 0) {
+    // w in sector k lies beyond boundaries 0..k-1 (mod K/2, the other side past half a turn)
+    constexpr int H = K / 2;
+    return k <= H ? (1u << k) - 1u : ((1u << H) - 1u) ^ ((1u << (k - H)) - 1u);
+  } else {
+    return k == 0 ? 0u : 1u << (k - 1);
+  }
+}
+
 // entries of the z table (sign patterns; codes for K > 8) and its filling by
 // a block's threads
 template <int K>
