@@ -161,6 +161,7 @@ template <int NT, typename T>
 __device__ __forceinline__ T lz_block_total(const T* part, int count) {
   __shared__ T red[NT / 32];
   T s = lz_zero<T>();
+#pragma unroll 8
   for (int k = threadIdx.x; k < count; k += NT) lz_add(s, __ldcg(part + k));  // other blocks' writes: from L2
   s = lz_warp_sum(s);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -281,7 +282,8 @@ __global__ void __launch_bounds__(kLzThreads) lz_degree(const int32_t* __restric
 // n = 4096 with all SMs equally loaded; the 268 MB take 40).  Two rows a warp
 // and two warps a block: 4096 rows are 1024 blocks, 6.7 an SM, so the fullest
 // SM has 28 rows where the average has 27 (blocks of sixteen rows: 32).
-// n = 4096: 143 us with the two projections; 230 us without them before (a row
+// Runs for n < 1024 and n > 32768 (lz_matvec_fixed between).  n = 4096: 143 us with
+// the two projections; 230 us without them before (a row
 // per warp, six FP64 instructions an entry).
 template <int ROWS>
 __global__ void __launch_bounds__(kLzMvThreads) lz_matvec_dense(
@@ -318,6 +320,239 @@ __global__ void __launch_bounds__(kLzMvThreads) lz_matvec_dense(
     }
   }
   lz_two_dots<kLzMvThreads>(d0, d1, part, counter, uprev != nullptr, h1);
+}
+
+// ---------------------------------------------------------------------------
+// the dense operator in fixed point
+// ---------------------------------------------------------------------------
+// Four FP64 FMAs an entry keep the dense operator (141 us at n = 4096) well
+// above its bytes (40 us).  Here Q's entries are 55-bit integers relative to
+// their row's largest component (off by 2^-55 of it at most) and the unit
+// vector's are 63-bit integers, both cut into signed bytes (seven and eight
+// base-256 digits d and j, the most significant first).  The digit products with
+// d + j <= 7 are summed exactly by 4-way byte dot products, by d + j; the others
+// are below 2^-59 of the largest product.  FP64 only joins a row's sums.
+// Against exact arithmetic the result is at least as close as that of FP64
+// FMAs, whose partial sums round at every entry.  Q's digits are laid out once
+// per truncation (14 bytes an entry for 16), a vector's by the kernel that
+// normalises it.  (The 8-bit matrix instruction has the rate of the byte dot
+// products here and takes all 56 digit pairs: 91 us.)
+constexpr int kLzQDigits = 7, kLzXDigits = 8;
+constexpr int kLzFixThreads = 256;  // laying out
+constexpr int kLzFixRows = 4;       // rows a warp
+// Smaller matrices leave SMs without rows; the sums of 8 digit pairs of 2 n
+// products of at most 2^14, times 2^24, have to stay below 2^63, and the digits
+// take as much memory as Q.
+constexpr int64_t kLzFixMin = 1024, kLzFixMax = 32768;
+
+struct LzFixed {
+  int64_t units, steps;  // of four rows, of 128 columns
+  size_t qbytes, xbytes;
+};
+inline LzFixed lz_fixed(int64_t n) {
+  LzFixed f;
+  f.units = ceil_div(n, kLzFixRows);
+  f.steps = ceil_div(n, 128);
+  f.qbytes = static_cast<size_t>(f.units * f.steps) * 2 * kLzQDigits * 512;
+  f.xbytes = static_cast<size_t>(f.steps) * 3 * kLzXDigits * 128;
+  return f;
+}
+inline bool lz_use_fixed(int64_t n) { return n >= kLzFixMin && n <= kLzFixMax; }
+
+// rowexp[i]: biased exponent of the row's largest component (0 for padding),
+// and the input check; a warp per row.
+__global__ void __launch_bounds__(kLzFixThreads) lz_row_exponents(const double2* __restrict__ Q, int64_t n, int64_t ld,
+                                                                  int64_t rows, int32_t* __restrict__ rowexp,
+                                                                  int32_t* status) {
+  const int lane = threadIdx.x & 31;
+  const int64_t i = (static_cast<int64_t>(blockIdx.x) * kLzFixThreads + threadIdx.x) >> 5;
+  uint32_t mx = 0;
+  if (i < n) {
+#pragma unroll 4
+    for (int64_t j = lane; j < n; j += 32) {
+      const double2 q = Q[i * ld + j];
+      mx = max(mx, max(static_cast<uint32_t>(__double2hiint(q.x)) & 0x7fffffffu,
+                       static_cast<uint32_t>(__double2hiint(q.y)) & 0x7fffffffu));
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane != 0 || i >= rows) return;
+  if ((mx >> 20) == 0x7ffu) dev_fail(status, LRQ_EINVAL);
+  rowexp[i] = static_cast<int32_t>(mx >> 20);
+}
+
+// digits of x 2^(1076 - E) to the nearest integer, |x| < 2^(E - 1022): the bytes
+// of the result are signed, the most significant in byte 6
+__device__ __forceinline__ uint64_t lz_q_digits(double x, int E) {
+  const uint64_t b = static_cast<uint64_t>(__double_as_longlong(x));
+  const int ex = static_cast<int>(b >> 52) & 0x7ff;
+  uint64_t m = (b & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
+  const int s = max(ex, 1) + 1 - E;  // value = m 2^s, s <= 2
+  if (s >= 0)
+    m <<= min(s, 2);
+  else
+    m = s < -54 ? 0ull : (m + (1ull << (-s - 1))) >> -s;
+  const int64_t v = (b >> 63) ? -static_cast<int64_t>(m) : static_cast<int64_t>(m);
+  return static_cast<uint64_t>(v + 0x0080808080808080ll) ^ 0x0080808080808080ull;
+}
+
+// byte k of four values
+__device__ __forceinline__ uint32_t lz_byte4(const uint64_t (&u)[4], int k) {
+  const int sh = 32 * (k >> 2), sel = (k & 3) * 0x11 + 0x40;
+  const uint32_t a = __byte_perm(static_cast<uint32_t>(u[0] >> sh), static_cast<uint32_t>(u[1] >> sh), sel);
+  const uint32_t c = __byte_perm(static_cast<uint32_t>(u[2] >> sh), static_cast<uint32_t>(u[3] >> sh), sel);
+  return __byte_perm(a, c, 0x5410);
+}
+
+// Q's digits: [4 rows][128 columns][re, im][digit][lane] 16 bytes, a word (the
+// lane's four columns) per row.  A thread per lane.
+__global__ void __launch_bounds__(kLzFixThreads) lz_dense_digits(const double2* __restrict__ Q, int64_t n, int64_t ld,
+                                                                 int64_t units, int64_t steps,
+                                                                 const int32_t* __restrict__ rowexp,
+                                                                 uint4* __restrict__ out) {
+  const int64_t id = static_cast<int64_t>(blockIdx.x) * kLzFixThreads + threadIdx.x;
+  const int64_t tile = id >> 5;
+  if (tile >= units * steps) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t i0 = tile / steps * kLzFixRows, j0 = tile % steps * 128 + lane * 4;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    uint64_t u[kLzFixRows][4];
+#pragma unroll
+    for (int q = 0; q < kLzFixRows; ++q) {
+      const int64_t i = i0 + q;
+      const int E = rowexp[i];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        double x = 0.0;
+        if (i < n && j0 + e < n) x = c == 0 ? Q[i * ld + j0 + e].x : Q[i * ld + j0 + e].y;
+        u[q][e] = lz_q_digits(x, E);
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < kLzQDigits; ++d)
+      out[(tile * 2 * kLzQDigits + c * kLzQDigits + d) * 32 + lane] =
+          make_uint4(lz_byte4(u[0], kLzQDigits - 1 - d), lz_byte4(u[1], kLzQDigits - 1 - d),
+                     lz_byte4(u[2], kLzQDigits - 1 - d), lz_byte4(u[3], kLzQDigits - 1 - d));
+  }
+}
+
+// Digits of entry i of a unit vector, |x| <= 1: x 2^62 to the nearest integer.
+// Per 128 entries, 24 words a lane (its four entries), six 16-byte groups of 32
+// lanes: the digits of re, of im, of -im.
+__device__ __forceinline__ void lz_store_digits(uint8_t* xs, int64_t i, double2 x) {
+  const double two62 = 4611686018427387904.0;
+  const int64_t v[3] = {__double2ll_rn(x.x * two62), __double2ll_rn(x.y * two62), __double2ll_rn(x.y * -two62)};
+  uint8_t* p = xs + (i >> 7) * (3 * kLzXDigits * 128) + ((i & 127) >> 2) * 16 + (i & 3);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const uint64_t u = (static_cast<uint64_t>(v[c]) + 0x8080808080808080ull) ^ 0x8080808080808080ull;
+#pragma unroll
+    for (int j = 0; j < kLzXDigits; ++j) {
+      const int w = c * kLzXDigits + j;
+      p[(w >> 2) * 512 + (w & 3) * 4] = static_cast<uint8_t>(u >> (8 * (kLzXDigits - 1 - j)));
+    }
+  }
+}
+__device__ __forceinline__ void lz_store_digits(uint8_t*, int64_t, double) {}
+
+// Sums 16 integers over the warp, halving the values at every step: lane l ends
+// with the total of value l >> 1.
+__device__ __forceinline__ int64_t lz_warp_sums16(int64_t (&v)[16]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 8, m = 16; k > 0; k >>= 1, m >>= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int q = 0; q < k; ++q) {
+      const int64_t give = up ? v[q] : v[k + q], keep = up ? v[k + q] : v[q];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, give, m);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// y = Q x from the digits, four rows a warp and one warp a block (n = 4096: 1024
+// blocks, at most seven an SM where the average is 6.7).  Per step of 128
+// columns 7 KB of Q (the next step's loads in flight) and 560 byte dot products,
+// which take two cycles each.  Bound: these (31 us at n = 4096) and the 14 bytes
+// an entry (35 us).  n = 4096: 61 us, 141 in FP64; n = 1024: 15, 18.5.
+__global__ void __launch_bounds__(32) lz_matvec_fixed(
+    const uint4* __restrict__ Qd, const int32_t* __restrict__ rowexp, int64_t n, int units, int steps,
+    const uint4* __restrict__ xs, const double2* __restrict__ x, double2* __restrict__ y,
+    const double2* __restrict__ uprev, double2* __restrict__ part, unsigned* counter, double2* __restrict__ h1,
+    const LzState* st) {
+  if (st->stop) return;
+  constexpr int ND = kLzQDigits, NX = kLzXDigits, NR = kLzFixRows;
+  const int lane = threadIdx.x;
+  double2 d0 = make_double2(0.0, 0.0), d1 = d0;
+  for (int un = blockIdx.x; un < units; un += gridDim.x) {
+    int acc[NR][2][NX];  // re, im by d + j
+#pragma unroll
+    for (int q = 0; q < NR; ++q)
+#pragma unroll
+      for (int g = 0; g < NX; ++g) acc[q][0][g] = acc[q][1][g] = 0;
+    const uint4* qa = Qd + static_cast<int64_t>(un) * steps * (2 * ND * 32) + lane;
+    uint4 a[2 * ND];
+#pragma unroll
+    for (int d = 0; d < 2 * ND; ++d) a[d] = __ldcs(qa + d * 32);
+#pragma unroll 1
+    for (int s = 0; s < steps; ++s) {
+      uint32_t xw[3][NX];
+#pragma unroll
+      for (int g = 0; g < 6; ++g) {
+        const uint4 v = xs[(s * 6 + g) * 32 + lane];
+        xw[g >> 1][(g & 1) * 4] = v.x;
+        xw[g >> 1][(g & 1) * 4 + 1] = v.y;
+        xw[g >> 1][(g & 1) * 4 + 2] = v.z;
+        xw[g >> 1][(g & 1) * 4 + 3] = v.w;
+      }
+      uint4 an[2 * ND];
+      const uint4* qn = qa + static_cast<int64_t>(s + 1 < steps ? s + 1 : s) * (2 * ND * 32);
+#pragma unroll
+      for (int d = 0; d < 2 * ND; ++d) an[d] = __ldcs(qn + d * 32);
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {
+        const uint32_t re[NR] = {a[d].x, a[d].y, a[d].z, a[d].w};
+        const uint32_t im[NR] = {a[ND + d].x, a[ND + d].y, a[ND + d].z, a[ND + d].w};
+#pragma unroll
+        for (int j = 0; j + d < NX; ++j)
+#pragma unroll
+          for (int q = 0; q < NR; ++q) {
+            acc[q][0][d + j] = __dp4a(static_cast<int>(re[q]), static_cast<int>(xw[0][j]), acc[q][0][d + j]);
+            acc[q][1][d + j] = __dp4a(static_cast<int>(re[q]), static_cast<int>(xw[1][j]), acc[q][1][d + j]);
+            acc[q][0][d + j] = __dp4a(static_cast<int>(im[q]), static_cast<int>(xw[2][j]), acc[q][0][d + j]);
+            acc[q][1][d + j] = __dp4a(static_cast<int>(im[q]), static_cast<int>(xw[0][j]), acc[q][1][d + j]);
+          }
+      }
+#pragma unroll
+      for (int d = 0; d < 2 * ND; ++d) a[d] = an[d];
+    }
+    // sum_g acc_g 256^(13 - g), in two halves
+    int64_t v[16];
+#pragma unroll
+    for (int q = 0; q < NR; ++q)
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          v[q * 4 + c * 2 + h] = static_cast<int64_t>(acc[q][c][4 * h]) * 16777216 +
+                                 static_cast<int64_t>(acc[q][c][4 * h + 1]) * 65536 +
+                                 static_cast<int64_t>(acc[q][c][4 * h + 2]) * 256 + acc[q][c][4 * h + 3];
+    double t = static_cast<double>(lz_warp_sums16(v));  // lane: row lane / 8, re or im (bit 2), half (bit 1)
+    t = fma(t, 4294967296.0, __shfl_xor_sync(0xffffffffu, t, 2));  // meaningful in the upper half's lanes
+    const int64_t i = static_cast<int64_t>(un) * NR + (lane >> 3);
+    // 256^6 2^(E - 1076) 2^-62
+    t = scalbn(t, rowexp[i] - 1090);
+    const double im = __shfl_xor_sync(0xffffffffu, t, 4);
+    if ((lane & 7) == 0 && i < n) {
+      const double2 yi = make_double2(t, im);
+      y[i] = yi;
+      if (uprev) d0 = lz_cfma(uprev[i], yi, d0);
+      d1 = lz_cfma(x[i], yi, d1);
+    }
+  }
+  lz_two_dots<32>(d0, d1, part, counter, uprev != nullptr, h1);
 }
 
 // ---------------------------------------------------------------------------
@@ -612,12 +847,15 @@ __global__ void __launch_bounds__(kLzThreads) lz_update(const T* __restrict__ U,
 
 template <typename T>
 __global__ void __launch_bounds__(kLzThreads) lz_scale_into(const T* __restrict__ w, int64_t n, T* __restrict__ u,
-                                                            const LzState* st) {
+                                                            uint8_t* __restrict__ digits, const LzState* st) {
   if (st->stop) return;
   const double s = st->inv_beta;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride)
-    u[i] = lz_scale(w[i], s);
+  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const T v = lz_scale(w[i], s);
+    u[i] = v;
+    if (digits) lz_store_digits(digits, i, v);  // for lz_matvec_fixed
+  }
 }
 
 // What a convergence check reads, in one piece: the state of the step just
@@ -939,7 +1177,7 @@ struct LzPlan {
   int r, maxit, lmax, cap, nch, chunk, ldx;
   size_t esz;
   size_t off_U, off_w, off_Y, off_part, off_h1, off_h2, off_npart, off_alpha, off_beta, off_state, off_X, off_deg,
-      off_snap, off_count, off_two, total;
+      off_snap, off_count, off_two, off_qdig, off_xdig, off_rowexp, total;
 };
 
 size_t lz_take(size_t& cur, size_t bytes) {
@@ -979,6 +1217,11 @@ void lz_plan(int64_t n, int r, int maxit, bool cplx, LzPlan* p) {
   // arrival counters: matvec, three-term step, update, then one per vector group of lz_dots
   p->off_count = lz_take(cur, (3 + static_cast<size_t>(ceil_div(p->cap, kLzGroup))) * sizeof(unsigned));
   p->off_two = lz_take(cur, 2 * static_cast<size_t>(kLzMaxBlocks) * p->esz);  // the operator's block sums
+  const bool fixed = cplx && lz_use_fixed(n);  // the dense operator's digits
+  const LzFixed f = lz_fixed(n);
+  p->off_qdig = lz_take(cur, fixed ? f.qbytes : 0);
+  p->off_xdig = lz_take(cur, fixed ? f.xbytes : 0);
+  p->off_rowexp = lz_take(cur, fixed ? static_cast<size_t>(f.units) * kLzFixRows * sizeof(int32_t) : 0);
   p->total = cur;
 }
 
@@ -1021,10 +1264,13 @@ struct LzRun {
   LzSnap* snap() const { return reinterpret_cast<LzSnap*>(ws + p.off_snap); }
   unsigned* counter(int i) const { return reinterpret_cast<unsigned*>(ws + p.off_count) + i; }
   T* two() const { return reinterpret_cast<T*>(ws + p.off_two); }
+  uint4* qdig() const { return reinterpret_cast<uint4*>(ws + p.off_qdig); }
+  uint8_t* xdig() const { return dense && lz_use_fixed(n) ? ws + p.off_xdig : nullptr; }
+  int32_t* rowexp() const { return reinterpret_cast<int32_t*>(ws + p.off_rowexp); }
 
   // y = Q x, h1()[0] = uprev^H y (uprev may be NULL), h1()[1] = x^H y
   void matvec(const T* x, T* y, const T* uprev) const;
-  void prepare() const;  // operator set-up once per truncation (Laplacian degrees)
+  int prepare() const;  // operator set-up once per truncation (Laplacian degrees, dense digits)
 
   // h2() = U[:, :nc]^H w, w -= U[:, :nc] h2(), then by mode (lz_update): 0
   // closes Lanczos step j (column nc - 1), 1 normalises a start vector, 2
@@ -1054,7 +1300,7 @@ struct LzRun {
     return LRQ_OK;
   }
   void scale(int c) const {  // column c = w / ||w||
-    lz_scale_into<T><<<lz_rows_grid(n), kLzThreads, 0, st>>>(w(), n, col(c), state());
+    lz_scale_into<T><<<lz_rows_grid(n), kLzThreads, 0, st>>>(w(), n, col(c), xdig(), state());
     count_launch();
   }
   // A convergence check takes alpha, beta and the state as they are after
@@ -1160,7 +1406,7 @@ struct LzRun {
     bool verify = false;
     double tn = 0.0;
     int e;
-    prepare();
+    if ((e = prepare())) return e;
     while (L < n) {
       if (!verify && L >= r) verify = true;
       const int p_want = verify ? 1 : static_cast<int>(std::min<int64_t>(r - L, n - L));
@@ -1230,16 +1476,41 @@ void LzRun<double>::matvec(const double* x, double* y, const double* uprev) cons
 }
 
 template <>
-void LzRun<double>::prepare() const {
+int LzRun<double>::prepare() const {
   lz_degree<<<lz_rows_grid(n), kLzThreads, 0, st>>>(rowptr, colidx, wts, n, nnz, deg());
   count_launch();
+  return LRQ_OK;
 }
 
 template <>
-void LzRun<double2>::prepare() const {}
+int LzRun<double2>::prepare() const {
+  if (!lz_use_fixed(n)) {
+    lz_check_dense<<<lz_rows_grid(n * n), kLzThreads, 0, st>>>(Q, n, ld, status);
+    count_launch();
+    return LRQ_OK;
+  }
+  const LzFixed f = lz_fixed(n);
+  int e = cuda_check(cudaMemsetAsync(xdig(), 0, f.xbytes, st), "clear the digits past n");
+  if (e) return e;
+  lz_row_exponents<<<static_cast<unsigned>(ceil_div(f.units * kLzFixRows, kLzFixThreads / 32)), kLzFixThreads, 0,
+                     st>>>(Q, n, ld, f.units * kLzFixRows, rowexp(), status);
+  lz_dense_digits<<<static_cast<unsigned>(ceil_div(f.units * f.steps * 32, kLzFixThreads)), kLzFixThreads, 0, st>>>(
+      Q, n, ld, f.units, f.steps, rowexp(), qdig());
+  count_launch(2);
+  return cuda_check(cudaGetLastError(), "lz_dense_digits");
+}
 
 template <>
 void LzRun<double2>::matvec(const double2* x, double2* y, const double2* uprev) const {
+  if (lz_use_fixed(n)) {  // x is the column that scale() wrote last: its digits are in xdig()
+    const LzFixed f = lz_fixed(n);
+    const int blocks = static_cast<int>(std::min<int64_t>(f.units, kLzMaxBlocks));
+    lz_matvec_fixed<<<blocks, 32, 0, st>>>(qdig(), rowexp(), n, static_cast<int>(f.units), static_cast<int>(f.steps),
+                                           reinterpret_cast<const uint4*>(xdig()), x, y, uprev, two(), counter(0),
+                                           h1(), state());
+    count_launch();
+    return;
+  }
   // two rows a warp once every SM has a few warps that way
   const int rows = n >= 152 * 4 ? 2 : 1;
   const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(n, rows * (kLzMvThreads / 32)), kLzMaxBlocks));
@@ -1321,8 +1592,6 @@ int launch_truncate(const lrq_matrix* Q, int r, double tol, int max_iter, uint64
     R.st = st;
     R.side = sd.side;
     R.ev = sd.ev;
-    lz_check_dense<<<lz_rows_grid(Q->n * Q->n), kLzThreads, 0, st>>>(R.Q, Q->n, Q->ld, status);
-    count_launch();
     return R.solve(r, lambda_out, V, V32, iters_out);
   }
   LzRun<double> R;
