@@ -533,9 +533,14 @@ __global__ void __launch_bounds__(kNllThreads) vmf_nll_kernel(const float* __res
 // 10^4) it is repeated in FP64 as first written, so every draw is accepted or
 // not as in FP64.  Logs, Gaussians and the vectors are double-float
 // (gauss_df32.cuh): FP64 runs at 1/64 of the FP32 rate and took about 800
-// instructions a sample (16 x 65520 draws: 2298 us, 361 now).
+// instructions a sample (16 x 65520 draws: 2298 us, 361 with one sample a thread
+// at a time).  A warp's tries run until its unluckiest lane is done, about four
+// times where the mean is 1.5, so a thread takes kVmfPer samples through the
+// tries one after the other and the warp then finishes all of them together:
+// 262 us.
 // ---------------------------------------------------------------------------
 constexpr int kVmfThreads = 128;
+constexpr int kVmfPer = 8;  // samples of a thread at a time
 
 struct VmfRng {
   uint64_t seed;
@@ -581,7 +586,7 @@ __device__ __noinline__ bool vmf_accept_fp64(VmfRng rng, double kap, double bb, 
 }
 
 __global__ void __launch_bounds__(kVmfThreads) vmf_sample_kernel(const float* __restrict__ O, int B, int S, int K,
-                                                                 uint64_t seed, float2* __restrict__ C,
+                                                                 int nper, uint64_t seed, float2* __restrict__ C,
                                                                  int32_t* status) {
   __shared__ CompParams cp;
   __shared__ double wb[kComp], wx0[kComp], wc[kComp];
@@ -589,6 +594,9 @@ __global__ void __launch_bounds__(kVmfThreads) vmf_sample_kernel(const float* __
   __shared__ double total;
   __shared__ df32 smu[kComp][kDim], sb[kComp], root_c[kMaxK], root_s[kMaxK];
   __shared__ float sa[kComp], shalf[kComp];
+  __shared__ float4 sw4[kVmfPer][kVmfThreads];    // w and sqrt(1 - w^2)
+  __shared__ uint32_t smk[kVmfPer][kVmfThreads];  // component, power of omega
+  __shared__ uint32_t sctr[kVmfPer][kVmfThreads]; // random numbers used
   const int b = blockIdx.y;
   head_params(O + static_cast<int64_t>(b) * kOut, cp);
   if (threadIdx.x < kComp) {
@@ -620,71 +628,88 @@ __global__ void __launch_bounds__(kVmfThreads) vmf_sample_kernel(const float* __
     total = s;
   }
   __syncthreads();
-  for (int s = blockIdx.x * kVmfThreads + threadIdx.x; s < S; s += gridDim.x * kVmfThreads) {
-    VmfRng rng{seed, static_cast<uint32_t>(s), static_cast<uint32_t>(b), 0u};
-    uint64_t ux, uy;
-    rng.bits2(&ux, &uy);
-    // the component and the member of the K-fold equivalence class
-    const long long target = __double_as_longlong((static_cast<double>(ux >> 1) + 0.5) * (1.0 / 9007199254740992.0) * total);
-    int m = 0;
-    while (m < kComp - 1 && cdf[m] < target) ++m;
-    const int k = min(K - 1, static_cast<int>(__umul64hi(uy << 10, static_cast<uint64_t>(K))));
-    const float a = sa[m], half = shalf[m];
-    const df32 bb = sb[m];
-    df32 w{1.f, 0.f}, sw{0.f, 0.f};
-    bool ok = false;
-    for (int tries = 0; tries < 1000 && !ok; ++tries) {
+  const int tid = threadIdx.x;
+  for (int64_t b0 = static_cast<int64_t>(blockIdx.x) * kVmfThreads * nper; b0 < S;
+       b0 += static_cast<int64_t>(gridDim.x) * kVmfThreads * nper) {
+    const int base = static_cast<int>(b0) + tid;
+    const int count = base < S ? min(nper, (S - 1 - base) / kVmfThreads + 1) : 0;
+    for (int q = 0; q < count; ++q) {
+      VmfRng rng{seed, static_cast<uint32_t>(base + q * kVmfThreads), static_cast<uint32_t>(b), 0u};
+      uint64_t ux, uy;
+      rng.bits2(&ux, &uy);
+      // the component and the member of the K-fold equivalence class
+      const long long target = __double_as_longlong((static_cast<double>(ux >> 1) + 0.5) * (1.0 / 9007199254740992.0) * total);
+      int m = 0;
+      while (m < kComp - 1 && cdf[m] < target) ++m;
+      const int k = min(K - 1, static_cast<int>(__umul64hi(uy << 10, static_cast<uint64_t>(K))));
+      smk[q][tid] = static_cast<uint32_t>(m) | static_cast<uint32_t>(k) << 8;
+    }
+    for (int q = 0, tries = 0, ctr = 1; q < count;) {
+      VmfRng rng{seed, static_cast<uint32_t>(base + q * kVmfThreads), static_cast<uint32_t>(b), static_cast<uint32_t>(ctr)};
+      const int m = smk[q][tid] & 0xffu;
       const VmfRng at = rng;
-      const df32 g1 = rng.gamma35(), g2 = rng.gamma35();
+      const df32 bb = sb[m], g1 = rng.gamma35(), g2 = rng.gamma35();
       uint64_t u, unused;
       rng.bits2(&u, &unused);
-      const df32 bg = df_times(bb, g1), q = df_sum(g2, bg);
-      const float rq = 1.0f / q.h;
-      const float t1 = a * ((g2.h - g1.h) + (g2.l - g1.l)) * rq;
-      const float t2 = (kDim - 1.0f) * logf(half * (g1.h + g2.h) * rq);
+      const df32 bg = df_times(bb, g1), sum = df_sum(g2, bg);
+      const float rq = 1.0f / sum.h;
+      const float t1 = sa[m] * ((g2.h - g1.h) + (g2.l - g1.l)) * rq;
+      const float t2 = (kDim - 1.0f) * logf(shalf[m] * (g1.h + g2.h) * rq);
       const float lu = -df_neg_log(u, GaussTab()).h;
       const float d = t1 + t2 - lu;
       // FP32 rounding of terms of size |t1|, |t2|, |lu|: below 16 * 2^-24 each
       const float margin = 1e-5f * (1.0f + fabsf(t1) + fabsf(t2) + fabsf(lu));
-      ok = d >= 0.0f;
+      bool ok = d >= 0.0f;
       if (fabsf(d) <= margin) ok = vmf_accept_fp64(at, cp.kappa[m], wb[m], wx0[m], wc[m]);
-      const df32 r = df_recip(q);
-      w = df_times(df_sum(g2, df32{-bg.h, -bg.l}), r);
+      ctr = static_cast<int>(rng.ctr);
+      if (!ok && ++tries < 1000) continue;
+      if (!ok) dev_fail(status, LRQ_ETIMEOUT);
+      const df32 r = df_recip(sum), w = df_times(df_sum(g2, df32{-bg.h, -bg.l}), r);
       const df32 root = df_times(df_sqrt(df_times(bg, g2)), r);
-      sw = df32{2.0f * root.h, 2.0f * root.l};
+      sw4[q][tid] = make_float4(w.h, w.l, 2.0f * root.h, 2.0f * root.l);
+      sctr[q][tid] = rng.ctr;
+      ++q;
+      tries = 0;
+      ctr = 1;
     }
-    if (!ok) dev_fail(status, LRQ_ETIMEOUT);
-    // a Gaussian vector (up to its scale) made orthogonal to mu
-    df32 v[kDim], dot{0.f, 0.f};
-#pragma unroll
-    for (int d = 0; d < kDim; d += 2) {
-      uint64_t e, f;
-      rng.bits2(&e, &f);
-      const df32 rad = df_sqrt(df_neg_log(e, GaussTab()));
-      df32 sn, cs;
-      df_sincos(f, GaussTab(), &sn, &cs);
-      v[d] = df_times(rad, cs);
-      v[d + 1] = df_times(rad, sn);
-    }
-#pragma unroll
-    for (int d = 0; d < kDim; ++d) dot = df_sum(dot, df_times(v[d], smu[m][d]));
-    df32 nv{0.f, 0.f};
-#pragma unroll
-    for (int d = 0; d < kDim; ++d) {
-      const df32 t = df_times(dot, smu[m][d]);
-      v[d] = df_sum(v[d], df32{-t.h, -t.l});
-      nv = df_sum(nv, df_times(v[d], v[d]));
-    }
-    const df32 scale = nv.h > 0.f ? df_times(sw, df_recip(df_sqrt(nv))) : df32{0.f, 0.f};
-    const df32 cs = root_c[k], sn = root_s[k];
-    float2* out = C + (static_cast<int64_t>(b) * S + s) * (kDim / 2);
-#pragma unroll
-    for (int j = 0; j < kDim / 2; ++j) {
-      const df32 re = df_sum(df_times(w, smu[m][2 * j]), df_times(scale, v[2 * j]));
-      const df32 im = df_sum(df_times(w, smu[m][2 * j + 1]), df_times(scale, v[2 * j + 1]));
-      const df32 p = df_times(im, sn), q = df_times(im, cs);
-      const df32 x = df_sum(df_times(re, cs), df32{-p.h, -p.l}), y = df_sum(df_times(re, sn), q);
-      out[j] = make_float2(x.h, y.h);
+    __syncwarp();  // a thread reads its own entries; the warp goes on together
+    for (int q = 0; q < count; ++q) {
+      const int s = base + q * kVmfThreads, m = smk[q][tid] & 0xffu, k = smk[q][tid] >> 8;
+      const float4 ws = sw4[q][tid];
+      const df32 w{ws.x, ws.y}, sw{ws.z, ws.w};
+      VmfRng rng{seed, static_cast<uint32_t>(s), static_cast<uint32_t>(b), sctr[q][tid]};
+      // a Gaussian vector (up to its scale) made orthogonal to mu
+      df32 v[kDim], dot{0.f, 0.f};
+  #pragma unroll
+      for (int d = 0; d < kDim; d += 2) {
+        uint64_t e, f;
+        rng.bits2(&e, &f);
+        const df32 rad = df_sqrt(df_neg_log(e, GaussTab()));
+        df32 sn, cs;
+        df_sincos(f, GaussTab(), &sn, &cs);
+        v[d] = df_times(rad, cs);
+        v[d + 1] = df_times(rad, sn);
+      }
+  #pragma unroll
+      for (int d = 0; d < kDim; ++d) dot = df_sum(dot, df_times(v[d], smu[m][d]));
+      df32 nv{0.f, 0.f};
+  #pragma unroll
+      for (int d = 0; d < kDim; ++d) {
+        const df32 t = df_times(dot, smu[m][d]);
+        v[d] = df_sum(v[d], df32{-t.h, -t.l});
+        nv = df_sum(nv, df_times(v[d], v[d]));
+      }
+      const df32 scale = nv.h > 0.f ? df_times(sw, df_recip(df_sqrt(nv))) : df32{0.f, 0.f};
+      const df32 cs = root_c[k], sn = root_s[k];
+      float2* out = C + (static_cast<int64_t>(b) * S + s) * (kDim / 2);
+  #pragma unroll
+      for (int j = 0; j < kDim / 2; ++j) {
+        const df32 re = df_sum(df_times(w, smu[m][2 * j]), df_times(scale, v[2 * j]));
+        const df32 im = df_sum(df_times(w, smu[m][2 * j + 1]), df_times(scale, v[2 * j + 1]));
+        const df32 p = df_times(im, sn), q = df_times(im, cs);
+        const df32 x = df_sum(df_times(re, cs), df32{-p.h, -p.l}), y = df_sum(df_times(re, sn), q);
+        out[j] = make_float2(x.h, y.h);
+      }
     }
   }
 }
@@ -841,11 +866,14 @@ int launch_vmf_nll(const float* O, int B, const float* X, int T, double* loss, f
 
 int launch_vmf_sample(const float* O, int B, int S, int K, uint64_t seed, float2* C, int32_t* status,
                       cudaStream_t st) {
-  // about eight blocks per SM over all instances: a block works out its
-  // instance's parameters once (a few us of FP64) and then loops over samples
-  const int64_t per = std::max<int64_t>(1, ceil_div(static_cast<int64_t>(8) * num_sms_current(), B));
-  dim3 grid(static_cast<unsigned>(std::min<int64_t>(ceil_div(S, kVmfThreads), per)), static_cast<unsigned>(B));
-  vmf_sample_kernel<<<grid, kVmfThreads, 0, st>>>(O, B, S, K, seed, C, status);
+  // about eight blocks per SM over all instances (a block works out its
+  // instance's parameters once, a few us of FP64), then several samples a thread
+  const int64_t want = static_cast<int64_t>(8) * num_sms_current();
+  const int nper = static_cast<int>(
+      std::min<int64_t>(kVmfPer, std::max<int64_t>(1, ceil_div(static_cast<int64_t>(S) * B, want * kVmfThreads))));
+  const int64_t per = std::max<int64_t>(1, ceil_div(want, B));
+  dim3 grid(static_cast<unsigned>(std::min<int64_t>(ceil_div(S, kVmfThreads * nper), per)), static_cast<unsigned>(B));
+  vmf_sample_kernel<<<grid, kVmfThreads, 0, st>>>(O, B, S, K, nper, seed, C, status);
   count_launch();
   return cuda_check(cudaGetLastError(), "vmf_sample_kernel");
 }
