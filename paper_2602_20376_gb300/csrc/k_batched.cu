@@ -135,7 +135,7 @@ struct BShared {
 // every row it reads (r <= 4), or a part of them at a time on the staged rows
 // (their directions re-read, their FP64 sums in local memory).
 // Bound: FP32 FMAs and shared-memory reads, as score_fp32_kernel; 512 uneven
-// instances of up to 8192 directions: 11.1 ms, 15.3 with one candidate per thread
+// instances of up to 8192 directions: 11.0 ms, 15.3 with one candidate per thread
 // and scalar FMAs, 11.7 with two.
 template <int R, int KC>
 __device__ void b_score_item(const BProb& pb, int s0, BShared& sh, uint64_t* __restrict__ keys) {
@@ -424,6 +424,145 @@ __device__ void b_select_exact(const BProb& pb, const EnumBest* __restrict__ ebe
   }
 }
 
+// V^H z of a candidate as unit sums, K in {2, 3, 4, 6, 8}: omega^k = i^q (a + b
+// tau) with a, b in {-1, 0, 1} and q in {0, 1}, so that conj(V_i) omega^k adds
+// conj(V_i), turned or not, to A, B or both, V^H z = A + tau B, without products.
+// The sums are exact three-word FP32 (two-sums twice).  The decision is certified
+// in FP32 as in the re-scoring kernel, else taken in FP64.
+constexpr int kBWarps = kBSelThreads / 32;
+__device__ __forceinline__ bool b_unit_alphabet(int K) { return K == 2 || K == 3 || K == 4 || K == 6 || K == 8; }
+__device__ __forceinline__ float4 b_unit_entry(int K, int k) {  // {a, b, turned, -}
+  if (K == 8) {
+    const float m = k < 4 ? 1.f : -1.f;
+    return make_float4(k & 1 ? 0.f : m, k & 1 ? m : 0.f, static_cast<float>((k >> 1) & 1), 0.f);
+  }
+  if (K == 2 || K == 4) {
+    const int q = K == 2 ? 2 * k : k;
+    return make_float4(q < 2 ? 1.f : -1.f, 0.f, static_cast<float>(q & 1), 0.f);
+  }
+  const int t = K == 3 ? 2 * k : k;  // powers of tau = exp(i pi / 3): 1, tau, tau - 1, -1, -tau, 1 - tau
+  const float a = t == 0 || t == 5 ? 1.f : (t == 2 || t == 3 ? -1.f : 0.f);
+  const float b = t == 1 || t == 2 ? 1.f : (t == 4 || t == 5 ? -1.f : 0.f);
+  return make_float4(a, b, 0.f, 0.f);
+}
+
+// The 2 r sums of candidate s over the rows of warp w of nw, to out; r <= R.
+template <int R>
+__device__ void b_unit_sums(const BProb& pb, int s, int w, int nw, const float4* __restrict__ unit, double* out) {
+  const BTable& tb = g_btab[pb.K];
+  const int K = pb.K, BK = K % 2 == 0 ? K / 2 : K, lane = threadIdx.x & 31;
+  float cr[R], ci[R], mx = 0.f;
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const float2 c = j < pb.r ? pb.C[static_cast<int64_t>(s) * pb.r + j] : make_float2(0.f, 0.f);
+    cr[j] = c.x;
+    ci[j] = c.y;
+    mx = fmaxf(mx, fabsf(c.x) + fabsf(c.y));
+  }
+  // the error of an FP32 boundary projection is below cb sum_j |V_ij|_1
+  const float cb = mx * (static_cast<float>(2 * R + 4) * 2.0f + 12.0f) * 5.9604644775390625e-08f;
+  f32x2 hi[2][R], lo[2][R], l3[2][R];
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+#pragma unroll
+    for (int j = 0; j < R; ++j) hi[g][j] = lo[g][j] = l3[g][j] = 0;
+  for (int64_t i = w * 32 + lane; i < pb.n; i += nw * 32) {
+    float2 v[R];
+    float x = 0.f, y = 0.f, ab = 0.f;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      v[j] = j < pb.r ? pb.V[i * pb.r + j] : make_float2(0.f, 0.f);
+      ab += fabsf(v[j].x) + fabsf(v[j].y);
+      x = fmaf(v[j].x, cr[j], x);
+      x = fmaf(-v[j].y, ci[j], x);
+      y = fmaf(v[j].x, ci[j], y);
+      y = fmaf(v[j].y, cr[j], y);
+    }
+    uint32_t sb = 0;
+    float pmin = INFINITY;
+    for (int m = 0; m < BK; ++m) {
+      const float p = fmaf(y, tb.bcos[m], -x * tb.bsin[m]);
+      sb |= (p > 0.0f ? 1u : 0u) << m;
+      pmin = fminf(pmin, fabsf(p));
+    }
+    int k;
+    if (pmin > ab * cb) {
+      if (K % 2 == 0) {
+        const int c = __popc(sb);
+        k = (sb & 1u) ? c : (c == 0 ? 0 : K - c);
+      } else {
+        const uint32_t t = sb & ~(sb >> 1) & ((1u << (K - 1)) - 1u);
+        k = t ? __ffs(t) : 0;
+      }
+    } else {
+      double xd = 0.0, yd = 0.0;
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        const double vr = v[j].x, vi = v[j].y, dr = cr[j], di = ci[j];
+        xd = fma(vr, dr, fma(-vi, di, xd));
+        yd = fma(vr, di, fma(vi, dr, yd));
+      }
+      k = decide_fp64(xd, yd, K, tb.bcos64, tb.bsin64);
+    }
+    const float4 u = unit[k];
+    const f32x2 ua = pack2(u.x, u.x), ub = pack2(u.y, u.y);
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const f32x2 vv = u.z != 0.f ? pack2(v[j].y, v[j].x) : pack2(v[j].x, -v[j].y);  // i conj(V_ij) or conj(V_ij)
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        const f32x2 e = add_unit(hi[g][j], vv, g ? ub : ua);
+        l3[g][j] = add2(l3[g][j], add_unit(lo[g][j], e, pack2(1.f, 1.f)));
+      }
+    }
+  }
+  // the lanes' sums in FP64; 16 values at a time, halved at every step
+  const double tr = K == 8 ? 0.70710678118654752440 : 0.5;
+  const double ti = K == 8 ? 0.70710678118654752440 : 0.86602540378443864676;
+  const bool both = K != 2 && K != 4;
+  double val[16];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    val[2 * j] = val[2 * j + 1] = 0.0;
+    if (j < R) {
+      double a[2][2];
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        a[g][0] = a[g][1] = 0.0;
+        if (g == 0 || both) {
+          float h0, h1, m0, m1, t0, t1;
+          unpack2(hi[g][j < R ? j : 0], h0, h1);
+          unpack2(lo[g][j < R ? j : 0], m0, m1);
+          unpack2(l3[g][j < R ? j : 0], t0, t1);
+          a[g][0] = static_cast<double>(h0) + (static_cast<double>(m0) + static_cast<double>(t0));
+          a[g][1] = static_cast<double>(h1) + (static_cast<double>(m1) + static_cast<double>(t1));
+        }
+      }
+      val[2 * j] = a[0][0];
+      val[2 * j + 1] = a[0][1];
+      if (both) {
+        val[2 * j] += tr * a[1][0] - ti * a[1][1];
+        val[2 * j + 1] += tr * a[1][1] + ti * a[1][0];
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 8, m = 16; k > 0; k >>= 1, m >>= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int q = 0; q < k; ++q) {
+      const double give = up ? val[q] : val[k + q], keep = up ? val[k + q] : val[q];
+      val[q] = keep + __shfl_xor_sync(0xffffffffu, give, m);
+    }
+  }
+  val[0] += __shfl_xor_sync(0xffffffffu, val[0], 1);
+  if ((lane & 1) == 0) out[lane >> 1] = val[0];
+}
+
+// One block per problem.  The keys are read once, into registers; the selected
+// candidates are re-scored side by side, the warps shared out among them (unit
+// alphabets), or one after the other in FP64.  512 instances, four candidates
+// each: 889 us with every candidate in FP64 by the whole block, now 303.
 __global__ void __launch_bounds__(kBSelThreads) batched_select_kernel(const BProb* __restrict__ probs,
                                                                    const uint64_t* __restrict__ keys, int top_m,
                                                                    const EnumBest* __restrict__ ebest,
@@ -439,35 +578,99 @@ __global__ void __launch_bounds__(kBSelThreads) batched_select_kernel(const BPro
     b_select_exact(pb, ebest, best_f, best_idx, status);
     return;
   }
+  __shared__ double part[kBWarps][16];
+  __shared__ float4 unit[8];
+  __shared__ int chosen[kBMaxTopM];
+  __shared__ double fq[kBMaxTopM];
   const uint64_t* kp = keys + pb.key_off;
   const int m = min(top_m, pb.S);
-  double bf = -1.0;
-  int bs = 0;
+  const bool fast = b_unit_alphabet(pb.K);
+  if (fast && threadIdx.x < pb.K) unit[threadIdx.x] = b_unit_entry(pb.K, threadIdx.x);
+  constexpr int kKeys = kBMaxS / kBSelThreads;
+  uint64_t key[kKeys];
+#pragma unroll
+  for (int q = 0; q < kKeys; ++q) {
+    const int s = threadIdx.x + q * kBSelThreads;
+    key[q] = s < pb.S ? kp[s] : 0ull;
+  }
+  int got = 0;
   uint64_t prev = ~0ull;
-  for (int q = 0; q < m; ++q) {
+  for (; got < m; ++got) {
     uint64_t v = 0;
-    for (int s = threadIdx.x; s < pb.S; s += kBSelThreads) {
-      const uint64_t k = kp[s];
-      if (k < prev && k > v) v = k;
-    }
+#pragma unroll
+    for (int q = 0; q < kKeys; ++q)
+      if (key[q] < prev && key[q] > v) v = key[q];
     const uint64_t kmax = b_block_max(v, redk);
     prev = kmax;
     const int s = static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(kmax & 0xFFFFFFFFull));
     if (kmax == 0 || s < 0 || s >= pb.S) break;  // no key left (block-uniform)
-    double f;
-    switch (pb.r) {
-      case 1: f = b_rescore<1>(pb, s, redd); break;
-      case 2: f = b_rescore<2>(pb, s, redd); break;
-      case 3: f = b_rescore<3>(pb, s, redd); break;
-      case 4: f = b_rescore<4>(pb, s, redd); break;
-      case 5: f = b_rescore<5>(pb, s, redd); break;
-      case 6: f = b_rescore<6>(pb, s, redd); break;
-      case 7: f = b_rescore<7>(pb, s, redd); break;
-      default: f = b_rescore<8>(pb, s, redd); break;
+    if (threadIdx.x == 0) chosen[got] = s;
+  }
+  __syncthreads();
+  double bf = -1.0;
+  int bs = 0;
+  if (fast) {
+    // warps per candidate; candidates q0 .. q0 + kBWarps / per - 1 at a time
+    const int per = got >= kBWarps ? 1 : (got >= 5 ? 1 : (got >= 3 ? 2 : (got == 2 ? 4 : 8)));
+    const int warp = threadIdx.x >> 5, at_once = kBWarps / per;
+    for (int q0 = 0; q0 < got; q0 += at_once) {
+      const int q = q0 + warp / per;
+      if (q < got) {
+        const int s = chosen[q];
+        if (pb.r <= 2)
+          b_unit_sums<2>(pb, s, warp % per, per, unit, part[warp]);
+        else if (pb.r <= 4)
+          b_unit_sums<4>(pb, s, warp % per, per, unit, part[warp]);
+        else
+          b_unit_sums<8>(pb, s, warp % per, per, unit, part[warp]);
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        for (int c = 0; c < at_once && q0 + c < got; ++c) {
+          double f = 0.0;
+          for (int j = 0; j < 2 * pb.r; ++j) {
+            double v = part[c * per][j];
+            for (int w = 1; w < per; ++w) v += part[c * per + w][j];
+            f += v * v;
+          }
+          fq[q0 + c] = f;
+        }
+      }
+      __syncthreads();
     }
-    if (f > bf || (f == bf && s < bs)) {
-      bf = f;
-      bs = s;
+    for (int q = 0; q < got; ++q) bf = fmax(bf, fq[q]);
+  }
+  // the best in FP64's own order: directions whose assignments are turns of one
+  // another have the same f, which only rounding tells apart, so values this
+  // close are taken again in FP64 as for the other alphabets
+  const double near = fast ? bf * (1.0 - 1e-10) : -1.0;
+  int close = 0;
+  for (int q = 0; q < got; ++q) {
+    if (!fast || fq[q] >= near) {
+      ++close;
+      bs = chosen[q];
+    }
+  }
+  if (!fast || close > 1) {
+    bf = -1.0;
+    for (int q = 0; q < got; ++q) {
+      if (fast && !(fq[q] >= near)) continue;
+      const int s = chosen[q];
+      double f;
+      switch (pb.r) {
+        case 1: f = b_rescore<1>(pb, s, redd); break;
+        case 2: f = b_rescore<2>(pb, s, redd); break;
+        case 3: f = b_rescore<3>(pb, s, redd); break;
+        case 4: f = b_rescore<4>(pb, s, redd); break;
+        case 5: f = b_rescore<5>(pb, s, redd); break;
+        case 6: f = b_rescore<6>(pb, s, redd); break;
+        case 7: f = b_rescore<7>(pb, s, redd); break;
+        default: f = b_rescore<8>(pb, s, redd); break;
+      }
+      if (f > bf || (f == bf && s < bs)) {
+        bf = f;
+        bs = s;
+      }
     }
   }
   if (threadIdx.x == 0) {

@@ -62,22 +62,8 @@ __device__ __forceinline__ void acc_dot2(float& hi, float& lo, float a, float bh
   lo += e4 + small;
 }
 
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
-
-// (hi, lo) += v m, m a pair of equal multipliers in {-1, 0, 1}: exact two-sum
-__device__ __forceinline__ void acc_unit(f32x2& hi, f32x2& lo, f32x2 v, f32x2 m) {
-  const f32x2 s = fma2(v, m, hi);
-  const f32x2 nb = add2(hi, neg2(s));  // minus the part of v m that reached s
-  const f32x2 t = add2(s, nb);
-  const f32x2 e = add2(add2(hi, neg2(t)), fma2(v, m, nb));
-  hi = s;
-  lo = add2(lo, e);
-}
+// (hi, lo) += v m, m a pair of multipliers in {-1, 0, 1}
+__device__ __forceinline__ void acc_unit(f32x2& hi, f32x2& lo, f32x2 v, f32x2 m) { lo = add2(lo, add_unit(hi, v, m)); }
 
 // omega^k = a + b tau
 struct RootAB {

@@ -38,6 +38,24 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   return r;
 }
 
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
+
+// hi += v m for a pair of multipliers in {-1, 0, 1}; returns the rounding error
+// (exact two-sum)
+__device__ __forceinline__ f32x2 add_unit(f32x2& hi, f32x2 v, f32x2 m) {
+  const f32x2 s = fma2(v, m, hi);
+  const f32x2 nb = add2(hi, neg2(s));  // minus the part of v m that reached s
+  const f32x2 t = add2(s, nb);
+  const f32x2 e = add2(add2(hi, neg2(t)), fma2(v, m, nb));
+  hi = s;
+  return e;
+}
+
 // Decision boundaries theta_m = pi(2m+1)/K in FP32, the first (B_K + 1) / 2 of
 // them: the others are mirror images (odd K: m and K-1-m share cos and have
 // opposite sin; even K: m and K/2-1-m share sin and have opposite cos).  The
