@@ -199,4 +199,91 @@ __device__ bool null_vector_fp64(double* H, int m, double* c) {
   return true;
 }
 
+// null_vector_fp64 for M rows with every index known at compile time, so that
+// H stays in registers: the same operations on the same operands in the same
+// order (same bits).  The pivot search compares magnitudes as integers, which
+// order like the absolute values (FP64 comparisons run on the FP64 unit).
+template <int M>
+__device__ __forceinline__ bool null_vector_fixed(double (&H)[M][M + 1], double (&c)[M + 1]) {
+  constexpr int NC = M + 1;
+  int colperm[NC];
+#pragma unroll
+  for (int j = 0; j < NC; ++j) colperm[j] = j;
+  auto mag = [](double v) { return __double_as_longlong(v) & 0x7fffffffffffffffll; };
+  long long sc = 0;
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int j = 0; j < NC; ++j) sc = max(sc, mag(H[i][j]));
+  if (sc == 0) return false;
+  const double scale = __longlong_as_double(sc);
+#pragma unroll
+  for (int k = 0; k < M; ++k) {
+    int pr = k, pc = k;
+    long long best = -1;
+#pragma unroll
+    for (int i = k; i < M; ++i)
+#pragma unroll
+      for (int j = k; j < NC; ++j) {
+        const long long v = mag(H[i][j]);
+        if (v > best) {
+          best = v;
+          pr = i;
+          pc = j;
+        }
+      }
+    if (__longlong_as_double(best) <= 1e-10 * scale) return false;
+#pragma unroll
+    for (int i = k + 1; i < M; ++i)
+      if (pr == i) {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          const double t = H[k][j];
+          H[k][j] = H[i][j];
+          H[i][j] = t;
+        }
+      }
+#pragma unroll
+    for (int j = k + 1; j < NC; ++j)
+      if (pc == j) {
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+          const double t = H[i][k];
+          H[i][k] = H[i][j];
+          H[i][j] = t;
+        }
+        const int t = colperm[k];
+        colperm[k] = colperm[j];
+        colperm[j] = t;
+      }
+#pragma unroll
+    for (int i = k + 1; i < M; ++i) {
+      const double f = H[i][k] / H[k][k];
+#pragma unroll
+      for (int j = k + 1; j < NC; ++j) H[i][j] -= f * H[k][j];
+    }
+  }
+  double y[NC];
+  y[M] = 1.0;
+#pragma unroll
+  for (int k = M - 1; k >= 0; --k) {
+    double t = H[k][M];
+#pragma unroll
+    for (int j = k + 1; j < M; ++j) t += H[k][j] * y[j];
+    y[k] = -t / H[k][k];
+  }
+  double nrm = 0.0;
+#pragma unroll
+  for (int j = 0; j < NC; ++j) nrm += y[j] * y[j];
+  nrm = 1.0 / sqrt(nrm);
+#pragma unroll
+  for (int j = 0; j < NC; ++j) {
+    const double v = y[j] * nrm;
+#pragma unroll
+    for (int q = 0; q < NC; ++q)
+      if (colperm[j] == q) c[q] = v;
+  }
+  return true;
+}
+
 }  // namespace lrq
