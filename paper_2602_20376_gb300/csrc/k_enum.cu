@@ -29,7 +29,7 @@
 // FP64 as the steps above say, the block's largest f_up first, so the result
 // (value, order of ties, error reports) is that of evaluating every vertex in
 // FP64.  n = 64, r = 2, K = 3 (1.16 * 10^6 sets): 42.4 ms when every vertex
-// was, 2.3 ms now.
+// was, 2.5 to 3.1 ms by instance now.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -40,7 +40,6 @@
 #include "enum_device.cuh"
 #include "lrq_device.cuh"
 #include "lrq_internal.h"
-#include "score_f32x2.cuh"
 
 namespace lrq {
 
@@ -51,10 +50,11 @@ constexpr int kEnumChunk = kEnumThreads * kEnumRanksPerThread;  // index sets pe
 constexpr int kEnumBlocks = 4096;                               // at most, per level
 constexpr double kEnumDefaultBudget = 1e12;
 
-// FP32 tables: omega^k and all K boundaries.
+// The FP32 copy of V (a power of two brings its largest component into
+// [1, 2)) and what the error bounds need.
 struct EnumF32 {
-  float zr[kMaxTcK], zi[kMaxTcK];
-  float bcos[kMaxTcK], bsin[kMaxTcK];
+  float zr[kMaxTcK], zi[kMaxTcK];      // omega^k
+  float bcos[kMaxTcK], bsin[kMaxTcK];  // all K boundaries
 };
 struct EnumScan {
   double scale;  // V32 = V scale
@@ -63,62 +63,19 @@ struct EnumScan {
   unsigned long long counts;
 };
 
-// The code of a sign pattern (decide_from_signs for any K <= 8).
-__device__ __forceinline__ int enum_code(uint32_t s, int K) {
+// decide_fp32 for any K <= 8
+__device__ __forceinline__ int enum_decide(float x, float y, int K, const EnumF32& tf) {
+  const int BK = (K % 2 == 0) ? K / 2 : K;
+  uint32_t s = 0;
+#pragma unroll
+  for (int m = 0; m < kMaxTcK; ++m)
+    if (m < BK) s |= (fmaf(y, tf.bcos[m], -x * tf.bsin[m]) > 0.0f ? 1u : 0u) << m;
   if (K % 2 == 0) {
     const int c = __popc(s);
     return (s & 1u) ? c : (c == 0 ? 0 : K - c);
   }
   const uint32_t t = s & ~(s >> 1) & ((1u << (K - 1)) - 1u);
   return t ? __ffs(t) : 0;
-}
-
-// Sign pattern [p_m > 0] of the boundary projections and the smallest |p_m|.
-template <int KT>
-__device__ __forceinline__ uint32_t enum_lines(float x, float y, int BK, const EnumF32& tf, float* pmin) {
-  uint32_t s = 0;
-  float mn = INFINITY;
-  if constexpr (KT > 0) {
-    constexpr int B = (KT % 2 == 0) ? KT / 2 : KT;
-#pragma unroll
-    for (int m = 0; m < (B + 1) / 2; ++m) {
-      const float c = boundary_cos<KT>(m), sn = boundary_sin<KT>(m);
-      const int mm = B - 1 - m;
-      float p, q;
-      if (sn == 0.f) {
-        p = q = -y;
-      } else if (c == 0.f) {
-        p = q = -x;
-      } else {
-        const float t = x * sn;
-        p = fmaf(y, c, -t);
-        q = KT % 2 == 1 ? fmaf(y, c, t) : fmaf(y, -c, -t);
-      }
-      if (p > 0.f) s |= 1u << m;
-      mn = fminf(mn, fabsf(p));
-      if (mm != m) {
-        if (q > 0.f) s |= 1u << mm;
-        mn = fminf(mn, fabsf(q));
-      }
-    }
-  } else {
-    for (int m = 0; m < BK; ++m) {
-      const float p = fmaf(y, tf.bcos[m], -x * tf.bsin[m]);
-      if (p > 0.f) s |= 1u << m;
-      mn = fminf(mn, fabsf(p));
-    }
-  }
-  *pmin = mn;
-  return s;
-}
-
-// w = V_i c in FP32 of a row staged as {re, re, im, im} per entry
-template <int D>
-__device__ __forceinline__ void enum_project(const ulonglong2* row, const Dir2<D>& dir, float* x, float* y) {
-  f32x2 w = 0;
-#pragma unroll
-  for (int j = 0; j < D; ++j) w = fma2(row[j].x, dir.a[j], fma2(row[j].y, dir.b[j], w));
-  unpack2(w, *x, *y);
 }
 
 // rank -> index set in the order of `unrank` (the largest index first, by
@@ -142,93 +99,90 @@ __device__ inline void enum_unrank(unsigned long long rank, int N, int m, int* i
 
 // Upper bound of |V^H z|^2 over the candidates of vertex (index set I, sign)
 // in the FP32 copy's scale, or INFINITY where FP32 cannot tell what the
-// candidates are.  `unc` counts the coordinates with a boundary projection
-// within its error bound, sum is V^H z with every coordinate's FP32 code.  A
-// coordinate of I near a boundary of its sector takes both codes, one with two
-// rows in I all K; any other coordinate has to be clear of every boundary.
-template <int D, int KT>
-__device__ __forceinline__ float enum_upper(const ulonglong2* V32, const float* rowb, int r, int K, int BK,
-                                            const EnumF32& tf, const int* I, const Dir2<D>& dir, bool neg, int unc,
-                                            const f32x2* sum, float esum) {
+// candidates are.  KT > 0: K known at compile time; RT: r known to be at most
+// RT.  `unc` counts the coordinates whose FP32 decision is not certain, S is
+// the sum with every coordinate's FP32 code.
+template <int D, int KT, int RT>
+__device__ __forceinline__ float enum_upper(const float2* __restrict__ V32, const float* __restrict__ rowb, int r,
+                                            int K, const EnumF32& tf, int BK, const int* I, const float* cr,
+                                            const float* ci, int sign, int unc, const float* sr, const float* si,
+                                            float esum) {
   constexpr int M = 2 * D - 1;
-  const uint32_t mask = (1u << BK) - 1u;
-  int nb = 0, bi[M], bk[M], bo[M], bc[M];  // row, code in `sum`, other code, options
+  // the coordinates of I that touch a boundary here: their options
+  int nb = 0, bi[M], bo[M][2], bc[M];
   int found = 0;
 #pragma unroll
   for (int t = 0; t < M; ++t) {
     const int g = I[t] / BK;
     if (t > 0 && I[t - 1] / BK == g) continue;  // handled with its first row
     const bool dbl = t + 1 < M && I[t + 1] / BK == g;
-    float x, y, pmin;
-    enum_project<D>(V32 + g * r, dir, &x, &y);
-    const uint32_t s = enum_lines<KT>(x, y, BK, tf, &pmin);
-    const float b = rowb[g];
-    if (b < 0.f) continue;  // a zero row: code 0, no contribution
-    found += pmin > b ? 0 : 1;
-    const int k = enum_code(neg ? mask ^ s : s, K);
-    const int ka = k == 0 ? K - 1 : k - 1;
-    if (neg) {
+    float x = 0.f, y = 0.f;
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      const float2 v = V32[g * r + j];
+      x = fmaf(v.x, cr[j], fmaf(-v.y, ci[j], x));
+      y = fmaf(v.x, ci[j], fmaf(v.y, cr[j], y));
+    }
+    if (sign < 0) {
       x = -x;
       y = -y;
     }
-    const bool na = !(fmaf(y, tf.bcos[ka], -x * tf.bsin[ka]) > b), nk = !(fmaf(y, tf.bcos[k], -x * tf.bsin[k]) < -b);
-    if (!dbl && !na && !nk) continue;  // the code is certain
-    if (!dbl && na && nk) return INFINITY;  // w too small for FP32
-    bi[nb] = g;
-    bk[nb] = k;
-    bo[nb] = na ? ka : (k + 1 == K ? 0 : k + 1);
-    bc[nb] = dbl ? K : 2;
-    ++nb;
+    const int k = KT > 0 ? decide_fp32<KT>(x, y, tf.bcos, tf.bsin) : enum_decide(x, y, K, tf);
+    const int ka = k == 0 ? K - 1 : k - 1;
+    const float pa = fmaf(y, tf.bcos[ka], -x * tf.bsin[ka]), pb = fmaf(y, tf.bcos[k], -x * tf.bsin[k]);
+    const float b = rowb[g];
+    const bool na = !(pa > b), nb_ = !(pb < -b);
+    found += (na || nb_) ? 1 : 0;
+    if (rowb[g] < 0.f) continue;  // a zero row: code 0, no contribution
+    if (dbl) {
+      bi[nb] = g;
+      bo[nb][0] = k;
+      bc[nb] = K;
+      ++nb;
+    } else if (na && nb_) {
+      return INFINITY;  // w too small for FP32
+    } else if (na || nb_) {
+      bi[nb] = g;
+      bo[nb][0] = k;
+      bo[nb][1] = na ? ka : (k + 1 == K ? 0 : k + 1);
+      bc[nb] = 2;
+      ++nb;
+    }
   }
   if (found != unc) return INFINITY;  // another coordinate is not certain
   int total = 1;
   for (int q = 0; q < nb; ++q) total *= bc[q];
   float best = 0.f;
   for (int ch = 0; ch < total; ++ch) {
-    f32x2 t[kEnumMaxD];
+    float tr[RT], ti[RT];
 #pragma unroll
-    for (int j = 0; j < kEnumMaxD; ++j) t[j] = sum[j];
+    for (int j = 0; j < RT; ++j) {
+      tr[j] = sr[j];
+      ti[j] = si[j];
+    }
     int rem = ch;
     for (int q = 0; q < nb; ++q) {
       const int o = rem % bc[q];
       rem /= bc[q];
-      const int k0 = bk[q], k1 = bc[q] > 2 || K == 2 ? o : (o ? bo[q] : k0);
+      const int k0 = bo[q][0], k1 = bc[q] == 2 ? bo[q][o] : o;
       if (k1 == k0) continue;
       const float dzr = tf.zr[k1] - tf.zr[k0], dzi = tf.zi[k1] - tf.zi[k0];
-      const f32x2 za = pack2(dzr, dzi), zb = pack2(dzi, -dzr);
 #pragma unroll
-      for (int j = 0; j < kEnumMaxD; ++j)
-        if (j < r) t[j] = fma2(V32[bi[q] * r + j].x, za, fma2(V32[bi[q] * r + j].y, zb, t[j]));
+      for (int j = 0; j < RT; ++j) {
+        if (j < r) {
+          const float2 v = V32[bi[q] * r + j];
+          tr[j] += v.x * dzr + v.y * dzi;
+          ti[j] += v.x * dzi - v.y * dzr;
+        }
+      }
     }
     float f = 0.f;
 #pragma unroll
-    for (int j = 0; j < kEnumMaxD; ++j) {
-      float re, im;
-      unpack2(t[j], re, im);
-      f = fmaf(re, re, fmaf(im, im, f));
-    }
+    for (int j = 0; j < RT; ++j) f = fmaf(tr[j], tr[j], fmaf(ti[j], ti[j], f));
     best = fmaxf(best, f);
   }
   const float a = sqrtf(best) * 1.00001f + esum;
   return a * a * 1.00001f;
-}
-
-// The best candidate of one vertex in FP64 (f = -1 when its rows are
-// dependent).
-__device__ __forceinline__ EnumBest enum_vertex_fp64(const double2* __restrict__ V, int n, int r,
-                                                     const double* __restrict__ rown, int d, unsigned long long rk,
-                                                     int sign, const EnumTables& tb, int32_t* status) {
-  const EnumV64 va{V, r, rown};
-  const int m = 2 * d - 1;
-  EnumBest best;
-  best.f = -1.0;
-  int I[kEnumMaxRows];
-  enum_unrank(rk, n * tb.BK, m, I);
-  double H[kEnumMaxRows * 2 * kEnumMaxD], ct[2 * kEnumMaxD];
-  build_rows(va, r, d, I, m, tb, H);
-  if (null_vector_fp64<kEnumMaxRows>(H, m, ct))
-    eval_vertex(va, n, r, d, I, m, ct, sign, tb, best, rk, -1, nullptr, nullptr, status);
-  return best;
 }
 
 template <int D, int KT>
@@ -244,36 +198,16 @@ __global__ void __launch_bounds__(kEnumThreads) enum_kernel(const double2* __res
   extern __shared__ __align__(16) uint8_t enum_smem[];
   float* lf = reinterpret_cast<float*>(enum_smem);                        // f_up of the vertices passed on
   int* lid = reinterpret_cast<int*>(lf + 2 * kEnumChunk);                 // 2 * set + (sign < 0)
-  float4* V4 = reinterpret_cast<float4*>(lid + 2 * kEnumChunk);           // n x r, {re, re, im, im}
-  float* rowb = reinterpret_cast<float*>(V4 + static_cast<size_t>(n) * r);  // bound of |p_m|'s error; -1: zero row
-  const ulonglong2* V32 = reinterpret_cast<const ulonglong2*>(V4);
-  // per sign pattern {zr, zi, zi, -zr}: of w, and of -w (the pattern's complement)
-  __shared__ float4 zt[2][1 << 7];
-  __shared__ EnumF32 st;
-  __shared__ EnumTables stb;
-  if (threadIdx.x == 0) stb = tb;
+  float2* V32 = reinterpret_cast<float2*>(lid + 2 * kEnumChunk);          // n x r
+  float* rowb = reinterpret_cast<float*>(V32 + static_cast<size_t>(n) * r);  // bound of |p_m|'s error; -1: zero row
   __shared__ EnumBest sb[kEnumThreads];
   __shared__ int lcount;
   __shared__ float wmax[kEnumThreads / 32];
-  for (int t = threadIdx.x; t < n * r; t += kEnumThreads) {
-    const float2 v = V32g[t];
-    V4[t] = make_float4(v.x, v.x, v.y, v.y);
-  }
+  for (int t = threadIdx.x; t < n * r; t += kEnumThreads) V32[t] = V32g[t];
   for (int t = threadIdx.x; t < n; t += kEnumThreads) rowb[t] = rowbg[t];
   const EnumV64 va{V, r, rown};
   const int K = KT > 0 ? KT : tb.K, BK = KT > 0 ? (KT % 2 == 0 ? KT / 2 : KT) : tb.BK;
   const int N = n * BK;
-  for (int t = threadIdx.x; t < 1 << BK; t += kEnumThreads) {
-    const int k = enum_code(t, K);
-    zt[0][t] = make_float4(tf.zr[k], tf.zi[k], tf.zi[k], -tf.zr[k]);
-    zt[1][((1 << BK) - 1) ^ t] = zt[0][t];
-  }
-  if (threadIdx.x < kMaxTcK) {
-    st.zr[threadIdx.x] = tf.zr[threadIdx.x];
-    st.zi[threadIdx.x] = tf.zi[threadIdx.x];
-    st.bcos[threadIdx.x] = tf.bcos[threadIdx.x];
-    st.bsin[threadIdx.x] = tf.bsin[threadIdx.x];
-  }
   const float esum = scan->esum;
   const double scale = scan->scale;
   // the best value so far in the FP32 copy's scale, rounded down
@@ -313,43 +247,58 @@ __global__ void __launch_bounds__(kEnumThreads) enum_kernel(const double2* __res
           H[t][D + j] = c * vr + s * vi;  // Re(rho V_ij)
         }
       }
-      bool full;
-      if constexpr (D <= 2)
-        full = null_vector_fixed<M>(H, ct);
-      else  // too many rows for registers
-        full = null_vector_fp64<M>(&H[0][0], M, ct);
-      if (!full) continue;
+      if (!null_vector_fixed<M>(H, ct)) continue;
       ++nfull;
-      Dir2<D> dir;
+      float cr[D], ci[D];
 #pragma unroll
-      for (int j = 0; j < D; ++j) dir.set(j, make_float2(static_cast<float>(ct[j]), static_cast<float>(ct[D + j])));
+      for (int j = 0; j < D; ++j) {
+        cr[j] = static_cast<float>(ct[j]);
+        ci[j] = static_cast<float>(ct[D + j]);
+      }
       // both signs at once: -c has -w, so every boundary's side changes
-      f32x2 sum[2][kEnumMaxD];
-      int unc = 0;
+      float sr[2][kEnumMaxD], si[2][kEnumMaxD];
+      int unc[2] = {0, 0};
 #pragma unroll
-      for (int j = 0; j < kEnumMaxD; ++j) sum[0][j] = sum[1][j] = 0;
-#pragma unroll 2
+      for (int j = 0; j < kEnumMaxD; ++j) sr[0][j] = si[0][j] = sr[1][j] = si[1][j] = 0.f;
       for (int i = 0; i < n; ++i) {
-        ulonglong2 v[kEnumMaxD];
+        float vx[kEnumMaxD], vy[kEnumMaxD], x = 0.f, y = 0.f;
 #pragma unroll
-        for (int j = 0; j < kEnumMaxD; ++j)
-          if (j < D || j < r) v[j] = V32[i * r + j];
-        float x, y, pmin;
-        enum_project<D>(v, dir, &x, &y);
-        const uint32_t sg = enum_lines<KT>(x, y, BK, st, &pmin);
-        unc += pmin > rowb[i] ? 0 : 1;
+        for (int j = 0; j < kEnumMaxD; ++j) {
+          vx[j] = vy[j] = 0.f;
+          if (j < D || j < r) {
+            const float2 v = V32[i * r + j];
+            vx[j] = v.x;
+            vy[j] = v.y;
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          x = fmaf(vx[j], cr[j], fmaf(-vy[j], ci[j], x));
+          y = fmaf(vx[j], ci[j], fmaf(vy[j], cr[j], y));
+        }
+        const float b = rowb[i];
 #pragma unroll
         for (int sgn = 0; sgn < 2; ++sgn) {
-          const ulonglong2 z = reinterpret_cast<const ulonglong2*>(zt[sgn])[sg];
+          const float xs = sgn ? -x : x, ys = sgn ? -y : y;
+          const int k = KT > 0 ? decide_fp32<KT>(xs, ys, tf.bcos, tf.bsin) : enum_decide(xs, ys, K, tf);
+          const int ka = k == 0 ? K - 1 : k - 1;
+          const float pa = fmaf(ys, tf.bcos[ka], -xs * tf.bsin[ka]), pb = fmaf(ys, tf.bcos[k], -xs * tf.bsin[k]);
+          unc[sgn] += (pa > b && pb < -b) ? 0 : 1;
+          const float zr = tf.zr[k], zi = tf.zi[k];
 #pragma unroll
-          for (int j = 0; j < kEnumMaxD; ++j)
-            if (j < D || j < r) sum[sgn][j] = fma2(v[j].x, z.x, fma2(v[j].y, z.y, sum[sgn][j]));
+          for (int j = 0; j < kEnumMaxD; ++j) {
+            if (j < D || j < r) {
+              sr[sgn][j] = fmaf(vx[j], zr, fmaf(vy[j], zi, sr[sgn][j]));
+              si[sgn][j] = fmaf(vx[j], zi, fmaf(-vy[j], zr, si[sgn][j]));
+            }
+          }
         }
       }
       const float b32 = best32();
 #pragma unroll
       for (int sgn = 0; sgn < 2; ++sgn) {
-        const float up = enum_upper<D, KT>(V32, rowb, r, K, BK, st, I, dir, sgn == 1, unc, sum[sgn], esum);
+        const float up = enum_upper<D, KT, kEnumMaxD>(V32, rowb, r, K, tf, BK, I, cr, ci, sgn ? -1 : 1, unc[sgn],
+                                                      sr[sgn], si[sgn], esum);
         if (!(up < b32)) {
           const int at = atomicAdd(&lcount, 1);
           lf[at] = up;
@@ -373,9 +322,16 @@ __global__ void __launch_bounds__(kEnumThreads) enum_kernel(const double2* __res
       for (int q = threadIdx.x; q < count; q += kEnumThreads) {
         const float up = lf[q];
         const bool first = up == mx;
-        if (up < b32 || (pass == 0 ? !first : first)) continue;
+        if (pass == 0 ? !first : (first || up < b32)) continue;
         const unsigned long long rk = c0 + static_cast<unsigned>(lid[q] >> 1);
-        const EnumBest mine = enum_vertex_fp64(V, n, r, rown, D, rk, (lid[q] & 1) ? -1 : 1, stb, status);
+        int J[kEnumMaxRows];
+        enum_unrank(rk, N, M, J);
+        double H[kEnumMaxRows * 2 * kEnumMaxD], ct[2 * kEnumMaxD];
+        build_rows(va, r, D, J, M, tb, H);
+        if (!null_vector_fp64<kEnumMaxRows>(H, M, ct)) continue;
+        EnumBest mine;
+        mine.f = -1.0;
+        eval_vertex(va, n, r, D, J, M, ct, (lid[q] & 1) ? -1 : 1, tb, mine, rk, -1, nullptr, nullptr, status);
         if (mine.f >= 0.0 && enum_better(mine, best)) best = mine;  // the list is not in rank order
         if (best.f >= 0.0)
           atomicMax(&scan->best, static_cast<unsigned long long>(__double_as_longlong(best.f)));
@@ -626,8 +582,8 @@ int enum_launch(const EnumLaunch& a, const EnumTables& tb, const EnumF32& tf, in
     per *= 2;
   const unsigned long long sets = static_cast<unsigned long long>(kEnumThreads) * per;
   const int blocks = static_cast<int>(std::min<unsigned long long>((a.total + sets - 1) / sets, kEnumBlocks));
-  const size_t smem = 2 * static_cast<size_t>(kEnumChunk) * 8 + static_cast<size_t>(a.n) * (a.r * 16 + 4);
-  if (smem > 36 * 1024) {
+  const size_t smem = 2 * static_cast<size_t>(kEnumChunk) * 8 + static_cast<size_t>(a.n) * (a.r * 8 + 4);
+  if (smem > 40 * 1024) {
     const int e = cuda_check(cudaFuncSetAttribute(enum_kernel<D, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   static_cast<int>(smem)),
                              "enumeration shared memory");
@@ -654,8 +610,8 @@ int enum_launch_level(const EnumLaunch& a, const EnumTables& tb, const EnumF32& 
   switch (d) {
     case 1: return enum_launch_k<1>(a, tb, tf, nbest);
     case 2: return enum_launch_k<2>(a, tb, tf, nbest);
-    case 3: return enum_launch<3, 0>(a, tb, tf, nbest);
-    default: return enum_launch<4, 0>(a, tb, tf, nbest);
+    case 3: return enum_launch_k<3>(a, tb, tf, nbest);
+    default: return enum_launch_k<4>(a, tb, tf, nbest);
   }
 }
 }  // namespace
