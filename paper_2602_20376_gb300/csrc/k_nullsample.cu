@@ -38,7 +38,7 @@ struct NsTables {
 // RT = r for r <= 4, so that the rows, the matrix (up to 7 x 8) and the
 // elimination have fixed indexes and stay in registers; 0 takes any rank, with
 // the matrix in local memory.  Bound: FP64 (16 cycles of an SM a warp
-// instruction).  10^5 directions, r = 3: 385 us, 490 with the matrix in local
+// instruction).  2^17 directions, r = 3: 385 us, 490 with the matrix in local
 // memory.
 template <int RT>
 __global__ void __launch_bounds__(kNsThreads) null_sample_kernel(const float2* __restrict__ V, int64_t n, int rd,

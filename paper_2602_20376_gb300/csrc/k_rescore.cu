@@ -89,14 +89,17 @@ struct RsLattice {
 // once per candidate.  RM is the largest rank the instance handles (4 or 8):
 // it sizes the per-thread accumulators.
 // Bound: FP32 issue and pipe (K = 3, r = 4: about 100 instructions and 136
-// pipe cycles an evaluation).  m = 64, n = 2^20, r = 4, K = 3: 500 us; 673 with
-// multiplied accumulation, FP32 scalars and a bound per evaluation (316
-// instructions).
-constexpr int kRsCpw = 2;                              // candidates per warp
+// pipe cycles an evaluation).  One candidate a warp, so that the registers leave
+// three blocks an SM: with two a warp and two blocks the exact sums' chains of
+// dependent instructions left 41% of the issue slots empty.  m = 64, n = 2^20,
+// r = 4, K = 3: 477 us, 490 with two a warp; 673 with multiplied accumulation,
+// FP32 scalars and a bound per evaluation (316 instructions).  m = 16, n = 3000:
+// 7.3 us (11.1); r = 6, K = 8, m = 32, n = 50021: 33 us (45).
+constexpr int kRsCpw = 1;                              // candidates per warp
 constexpr int kRsCpb = kRsCpw * (kRsThreads / 32);     // candidates per block
 constexpr int kRsTile = 256;                           // rows staged at a time
 constexpr int kRsFlush = 256 * 32 / kRsTile;           // tiles between FP64 flushes (256 rows per lane)
-static_assert(kRsCpw * 16 == 32 && 2 * kMaxRank <= 16, "one lane per (candidate, component) total");
+static_assert(kRsCpw * 16 <= 32 && 2 * kMaxRank <= 16, "one lane per (candidate, component) total");
 
 // (hi, lo) + (hi', lo') in double-float
 __device__ __forceinline__ void add_pair(float& hi, float& lo, float h2, float l2) {
@@ -109,7 +112,7 @@ __device__ __forceinline__ void add_pair(float& hi, float& lo, float h2, float l
 // Sums N double-float values over the warp, halving the values at every step:
 // lane l ends with the total of value l >> (5 - log2 N).  In double-float
 // because FP64 instructions take a warp 16 cycles of its SM: sums in FP64 cost
-// 11 us of the 21 that m = 64, n = 20000, r = 4, K = 3 took, double-float sums leave 11 us.
+// 10 us of the 21 that m = 16, n = 3000, r = 4, K = 3 took.
 template <int N>
 __device__ __forceinline__ void rs_warp_sums(float (&h)[N], float (&l)[N]) {
   const int lane = threadIdx.x & 31;
@@ -131,7 +134,7 @@ __device__ __forceinline__ void rs_warp_sums(float (&h)[N], float (&l)[N]) {
 }
 
 template <int K, int RM>
-__global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 2 : 1) rescore_partial_kernel(
+__global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_kernel(
     const float2* __restrict__ V, int64_t n, int r, const float2* __restrict__ C, int64_t S,
     const int64_t* __restrict__ idx, int m, int nchunk, int64_t rows_per_chunk, const __grid_constant__ RescoreTables tab,
     double* __restrict__ part, uint8_t* __restrict__ z_out, unsigned* __restrict__ done, int32_t* status) {
@@ -370,7 +373,7 @@ __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 2 : 1) rescore_partial_k
       const double tr = K == 4 ? 0.0 : 0.5, ti = K == 4 ? 1.0 : 0.86602540378443864676;
       out += tr * tot[1] + ((j & 1) ? ti : -ti) * other;
     }
-    if (j < 2 * r && act[q]) part[(static_cast<int64_t>(tc[q]) * nchunk + chunk) * (2 * kMaxRank) + j] = out;
+    if (q < kRsCpw && j < 2 * r && act[q < kRsCpw ? q : 0]) part[(static_cast<int64_t>(tc[q]) * nchunk + chunk) * (2 * kMaxRank) + j] = out;
   }
 }
 

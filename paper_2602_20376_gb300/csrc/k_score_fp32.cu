@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kVScanThreads) v_scan_kernel(const float2* __r
 }
 
 // At most one block per SM; few rows a thread while that spreads them over more
-// SMs (n = 20000, r = 4: 4.4 us, 15.1 with 2048 rows a block).
+// SMs (n = 3000, r = 4: 4.4 us, 15.1 with 2048 rows a block).
 int v_scan_blocks(int64_t n) {
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kVScanMaxBlocks, ceil_div(n, kVScanThreads))));
 }

@@ -206,12 +206,15 @@ int plan_rescore(int64_t n, int r, int m, RescorePlan* p) {
   p->n = n;
   p->r = r;
   p->m = m;
-  // blocks of (candidates x coordinate chunk): about four per SM, at most
-  // 65536 rows per chunk (which bounds the scratch: m x nchunk x 2 kMaxRank
-  // doubles), at least one staged tile of 256 rows per chunk
+  // blocks of (candidates x coordinate chunk): six per SM, two rounds of the
+  // three that run at a time, with at most the chunks (and scratch: m x nchunk x
+  // 2 kMaxRank doubles) that four blocks of 16 candidates per SM would have; at
+  // most 65536 rows per chunk, at least one staged tile of 256
   const int64_t max_rows = int64_t(65536);
   const int64_t bx = rescore_blocks_x(m);
-  int64_t nchunk = std::max<int64_t>(ceil_div(int64_t(4) * num_sms_current(), bx), ceil_div(n, max_rows));
+  const int64_t sms = num_sms_current();
+  int64_t nchunk = std::max<int64_t>(std::min<int64_t>(std::max<int64_t>(1, 6 * sms / bx), ceil_div(4 * sms, ceil_div(m, 16))),
+                                     ceil_div(n, max_rows));
   nchunk = std::max<int64_t>(1, std::min<int64_t>(nchunk, std::max<int64_t>(1, ceil_div(n, 256))));
   nchunk = std::min<int64_t>(nchunk, 65535);  // grid y limit; longer chunks are fine (periodic FP64 flushes)
   p->rows_per_chunk = ceil_div(n, nchunk);
