@@ -365,7 +365,8 @@ int lrq_graph_destroy(void* graph_exec);
  *   tol      : residual tolerance ||Q y - theta y|| <= tol ||T|| for every
  *              wanted Ritz pair (<= 0 selects 1e-10).
  *   max_iter : Krylov dimension cap per run (0 selects min(500, n); at most
- *              4096).  Workspace grows as n * (max_iter + 2r + 9) scalars.
+ *              4096).  Workspace grows as n * (max_iter + 2r + 9) scalars;
+ *              a dense Q with 1024 <= n <= 32768 adds 14 bytes an entry.
  *   seed     : start vectors are Philox4x32-10 Gaussians keyed by seed.
  *   V_out    : n x r complex128 (device) or NULL.
  *   V32_out  : n x r complex64 (device, V rounded to nearest) or NULL; the
