@@ -14,8 +14,9 @@
 // The uniforms' 54-bit integers 2 x + 1 (u = (2 x + 1) 2^-54) are taken apart
 // exactly.  Errors against extended precision over 2 * 10^7 draws (with many
 // near 0 and 1): -ln u below 2^-39 relative, sine and cosine below 2^-45
-// absolute; so a component rounded to FP32 is the rounded 64-bit one but for
-// about one in 10^5, which differs by its last bit.
+// absolute.  A direction's component that lies this close to the middle of two
+// FP32 numbers (about one in 5000) is drawn again in FP64, so that every
+// component is the rounded 64-bit one.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -257,6 +258,16 @@ LRQ_HD df32 df_recip(df32 x) {
   return df_fast_sum(r, df_mul(r, e));
 }
 
+// Whether rounding h + l (h the nearest FP32 number) may depend on an error of
+// 2^-37 of it plus 2^-43 (above a component's: g within 2^-38, sine and cosine
+// 2^-45).
+__device__ __forceinline__ bool df_near_midpoint(df32 x) {
+  const uint32_t b = __float_as_uint(x.h) & 0x7fffffffu;
+  if ((b & 0x7fffffu) == 0u || b < (24u << 23)) return true;  // a power of two (half the spacing below), tiny
+  const float half = __uint_as_float((b & 0x7f800000u) - (24u << 23));
+  return half - fabsf(x.l) <= fmaf(fabsf(x.h), 0x1p-37f, 0x1p-43f);
+}
+
 // The directions of a block of 256 threads (lrq_sample_directions' draws): a
 // thread per component, 256 / r candidates a block, ||Z||^2 = sum_j -ln u1_j
 // exchanged through shared memory.  s: the block's first candidate.
@@ -289,7 +300,23 @@ __device__ __forceinline__ void sphere_block(uint64_t seed, int64_t s_first, int
   df_sincos(U2, GaussTab(), &sn, &cs);
   const df32 g = df_times(df_sqrt(L), df_recip(df_sqrt(N)));
   const df32 re = df_times(g, cs), im = df_times(g, sn);
-  C[s * r + j] = make_float2(re.h, im.h);
+  float2 out = make_float2(re.h, im.h);
+  if (df_near_midpoint(re) || df_near_midpoint(im)) {
+    double a = 0.0, b = 0.0, nrm2 = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < r; ++k) {
+      double zr, zi;
+      sphere_component(seed, s, k, &zr, &zi);
+      nrm2 += zr * zr + zi * zi;
+      if (k == j) {
+        a = zr;
+        b = zi;
+      }
+    }
+    const double inv = 1.0 / sqrt(nrm2);
+    out = make_float2(static_cast<float>(a * inv), static_cast<float>(b * inv));
+  }
+  C[s * r + j] = out;
 }
 
 }  // namespace lrq

@@ -17,7 +17,8 @@
 namespace lrq {
 
 // Uniform directions on the complex unit sphere (gauss_df32.cuh).  Bound:
-// issue slots, about 250 instructions a component.  S = 2^14, r = 4: 3.2 us, 26
+// issue slots, about 250 instructions a component, and the few drawn again in
+// FP64 (3.2 us without them).  S = 2^14, r = 4: 14.7 us, 26
 // in FP64 (two lanes an SM).
 __global__ void __launch_bounds__(kSphereThreads) sample_directions_kernel(uint64_t seed, int64_t S, int r,
                                                                            float2* __restrict__ C) {
