@@ -11,7 +11,7 @@
 // coordinates sorted by (phi_i, i).
 //
 // GPU steps: per-coordinate key (FP64), a stable sort of (key, index) pairs
-// (radix, eight 8-bit digits; bitonic in one block for small n), the
+// (a bitonic network, or radix passes over eight 8-bit digits), the
 // increments conj(q_i) w^{k_i} (w - 1) in sorted order, an FP64 prefix scan
 // giving q^H z for every state, and the argmax (ties to the earliest state).
 // With a CSR graph the state at which coordinate i advances changes the cut by
@@ -32,6 +32,13 @@ namespace lrq {
 
 constexpr int kR1Threads = 256;
 constexpr int kR1Local = 2048;  // elements sorted per block in shared memory
+// Up to here the sort is the bitonic network, radix passes above.  A radix pass
+// costs three launches whatever n is, and below some 10^5 pairs they do little
+// but wait; the network's launches grow with log^2 n (1 up to 2048 pairs, 4 at
+// 4096, 28 at 2^17).  Whole sweep with a graph, network / radix passes: n = 3000
+// 186 / 315 us, 16384 230 / 345, 65536 304 / 357, 80000 346 / 365, 131072 359 /
+// 378; at 2^18 the network would take 37 launches over twice the pairs.
+constexpr int64_t kR1Bitonic = 1 << 17;
 constexpr int kR1Scan = 2048;   // elements per block in the scans (8 a thread)
 constexpr int kR1BaseBlocks = 1024;  // blocks that leave a partial of the base sum (at most)
 // radix sort: a block takes kR1Tile consecutive pairs, a warp 32 at a time of
@@ -127,22 +134,26 @@ __device__ __forceinline__ bool r1_less(uint64_t ka, uint32_t ia, uint64_t kb, u
   return ka < kb || (ka == kb && ia < ib);
 }
 
-// n <= kR1Local: one block sorts the padded pairs by a bitonic network in
-// shared memory
-__global__ void __launch_bounds__(kR1Local / 2) r1_sort_local(uint64_t* __restrict__ key, uint32_t* __restrict__ idx) {
+// n <= kR1Bitonic: a bitonic network over the pairs, padded to a power of two.
+// Stages with partner distance below kR1Local run in shared memory: a block
+// owns kR1Local consecutive pairs and takes the merge sizes k_first..k_last (all
+// up to kR1Local in the first launch, then the tail of one size each).
+__global__ void __launch_bounds__(kR1Local / 2) r1_sort_local(uint64_t* __restrict__ key, uint32_t* __restrict__ idx,
+                                                              int64_t k_first, int64_t k_last) {
   __shared__ uint64_t sk[kR1Local];
   __shared__ uint32_t si[kR1Local];
+  const int64_t base = static_cast<int64_t>(blockIdx.x) * kR1Local;
   for (int t = threadIdx.x; t < kR1Local; t += blockDim.x) {
-    sk[t] = key[t];
-    si[t] = idx[t];
+    sk[t] = key[base + t];
+    si[t] = idx[base + t];
   }
   __syncthreads();
-  for (int k = 2; k <= kR1Local; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
+  for (int64_t k = k_first; k <= k_last; k <<= 1) {
+    for (int j = static_cast<int>(min(k >> 1, static_cast<int64_t>(kR1Local / 2))); j > 0; j >>= 1) {
       const int t = threadIdx.x;
       const int a = (t / j) * 2 * j + (t % j);
       const int b = a + j;
-      const bool up = (a & k) == 0;
+      const bool up = ((base + a) & k) == 0;
       const bool sw = up ? r1_less(sk[b], si[b], sk[a], si[a]) : r1_less(sk[a], si[a], sk[b], si[b]);
       if (sw) {
         const uint64_t tk = sk[a];
@@ -156,8 +167,26 @@ __global__ void __launch_bounds__(kR1Local / 2) r1_sort_local(uint64_t* __restri
     }
   }
   for (int t = threadIdx.x; t < kR1Local; t += blockDim.x) {
-    key[t] = sk[t];
-    idx[t] = si[t];
+    key[base + t] = sk[t];
+    idx[base + t] = si[t];
+  }
+}
+
+// one stage (merge size k, partner distance j >= kR1Local) in global memory, a
+// thread per pair of pairs
+__global__ void __launch_bounds__(kR1Threads) r1_sort_global(uint64_t* __restrict__ key, uint32_t* __restrict__ idx,
+                                                             int64_t npad, int64_t k, int64_t j) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * kR1Threads + threadIdx.x;
+  if (t >= npad / 2) return;
+  const int64_t a = (t / j) * 2 * j + (t % j), b = a + j;
+  const bool up = (a & k) == 0;
+  const uint64_t ka = key[a], kb = key[b];
+  const uint32_t ia = idx[a], ib = idx[b];
+  if (up ? r1_less(kb, ib, ka, ia) : r1_less(ka, ia, kb, ib)) {
+    key[a] = kb;
+    key[b] = ka;
+    idx[a] = ib;
+    idx[b] = ia;
   }
 }
 
@@ -165,8 +194,8 @@ __global__ void __launch_bounds__(kR1Local / 2) r1_sort_local(uint64_t* __restri
 // the 64-bit keys, three launches each; every pass keeps the order of equal
 // digits, so equal keys stay in index order.  The pairs (12 MB at n = 10^6)
 // stay in L2; a pass is bound by launch latency and its reads and writes.
-// The bitonic network it takes the place of ran 55 launches over 2^20 padded
-// pairs: 503 us at n = 10^6; now 213 (scatter 15, counts 10, offsets 2 a pass).
+// n = 10^6: 213 us (scatter 15, counts 10, offsets 2 a pass); the network's 55
+// launches over 2^20 padded pairs took 503.
 //
 // r1_hist_kernel: counts[digit][block]
 __global__ void __launch_bounds__(kR1SortThreads) r1_hist_kernel(const uint64_t* __restrict__ key, int64_t n,
@@ -643,7 +672,11 @@ struct R1Layout {
 R1Layout r1_layout(int64_t n) {
   R1Layout l;
   l.n = n;
-  l.npad = std::max<int64_t>(n, kR1Local);
+  l.npad = n;
+  if (n <= kR1Bitonic) {
+    l.npad = kR1Local;
+    while (l.npad < n) l.npad <<= 1;
+  }
   l.nscan_blocks = ceil_div(n, kR1Scan);
   l.nscan_blocks_diff = ceil_div(n + 1, kR1Scan);
   l.nsort_blocks = ceil_div(n, kR1Tile);
@@ -731,14 +764,22 @@ int launch_rank1(const double2* q, int64_t n, int K, uint8_t* z_out, double* f_o
   }
   int e = cuda_check(cudaMemsetAsync(counter, 0, sizeof(unsigned), st), "memset counter");
   if (e) return e;
-  const bool local = n <= kR1Local;
-  const int64_t nkeys = local ? kR1Local : n;
-  const int nbase = static_cast<int>(std::min<int64_t>(kR1BaseBlocks, ceil_div(nkeys, kR1Threads)));
-  r1_prep_kernel<<<nbase, kR1Threads, 0, st>>>(q, n, nkeys, K, tb, key, idx, code0, base, counter, s0, status);
+  const int nbase = static_cast<int>(std::min<int64_t>(kR1BaseBlocks, ceil_div(L.npad, kR1Threads)));
+  r1_prep_kernel<<<nbase, kR1Threads, 0, st>>>(q, n, L.npad, K, tb, key, idx, code0, base, counter, s0, status);
   count_launch();
-  if (local) {
-    r1_sort_local<<<1, kR1Local / 2, 0, st>>>(key, idx);
+  if (n <= kR1Bitonic) {
+    const unsigned lb = static_cast<unsigned>(L.npad / kR1Local);
+    r1_sort_local<<<lb, kR1Local / 2, 0, st>>>(key, idx, 2, kR1Local);
     count_launch();
+    for (int64_t k = 2 * kR1Local; k <= L.npad; k <<= 1) {
+      for (int64_t j = k >> 1; j >= kR1Local; j >>= 1) {
+        r1_sort_global<<<static_cast<unsigned>(ceil_div(L.npad / 2, kR1Threads)), kR1Threads, 0, st>>>(key, idx, L.npad,
+                                                                                                      k, j);
+        count_launch();
+      }
+      r1_sort_local<<<lb, kR1Local / 2, 0, st>>>(key, idx, k, k);
+      count_launch();
+    }
   } else {
     if ((e = cuda_check(cudaFuncSetAttribute(r1_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              kR1SortSmem),
