@@ -19,6 +19,11 @@
 // over the n marks and gains (later rounds).  n = 10^6, 6.65 * 10^6 entries,
 // 16 rounds: gains 264 us (33 the first round), moves 174; 972 and 293 with
 // 8 lanes a row and every vertex in every round.
+// A graph of up to kGrSmall vertices leaves SMs without rows either way, and a
+// round is one chain of dependent reads: there 8 lanes share a row and every
+// vertex is taken in every round, without marks.  Whole call, that form / a
+// thread a row with marks: n = 1000 258 / 301 us, 5000 290 / 295, 20000 302 /
+// 327, 32768 315 / 331; at 50000 the first takes 346, the second 327.
 // Rounds are issued in batches of kGrBatch; each round's move count
 // lands in a device ring, the next round returns at once when it is zero, and
 // the host reads the ring once per batch.
@@ -45,6 +50,7 @@ __device__ __forceinline__ bool gr_row(const int32_t* __restrict__ rowptr, int64
 }
 
 constexpr int kGrRowMax = 64;  // at most 255: label counts of a thread are bytes
+constexpr int64_t kGrSmall = 40960;
 
 __device__ __forceinline__ void gr_store(int64_t i, int zi, int K, const int* cnt, int32_t* __restrict__ gain,
                                          uint8_t* __restrict__ best) {
@@ -65,7 +71,9 @@ __device__ __forceinline__ void gr_store(int64_t i, int zi, int K, const int* cn
 }
 
 // gain and target label (0 gain when no move helps) of every marked vertex;
-// prev NULL: the first round, every vertex
+// prev NULL: the first round, every vertex.  LR lanes a row; LR > 1 takes every
+// vertex and leaves the marks alone.
+template <int LR>
 __global__ void __launch_bounds__(kGrThreads) gr_gain_kernel(const int32_t* __restrict__ rowptr,
                                                              const int32_t* __restrict__ colidx, int64_t n,
                                                              int64_t nnz, int K, const uint8_t* __restrict__ z,
@@ -73,12 +81,14 @@ __global__ void __launch_bounds__(kGrThreads) gr_gain_kernel(const int32_t* __re
                                                              uint8_t* __restrict__ dirty,
                                                              const unsigned long long* prev, int32_t* status) {
   if (prev && *prev == 0ull) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * kGrThreads;
-  for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * kGrThreads + (threadIdx.x & ~31); i0 < n; i0 += stride) {
-    const int64_t i = i0 + lane;  // warp-uniform trips
-    const bool todo = i < n && (!prev || dirty[i]);
-    if (i < n && (todo || !prev)) dirty[i] = 0;
+  constexpr int RW = 32 / LR;  // rows a warp
+  const int lane = threadIdx.x & 31, sub = lane % LR;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * (kGrThreads / LR);
+  for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * (kGrThreads / LR) + (threadIdx.x >> 5) * RW; i0 < n;
+       i0 += stride) {
+    const int64_t i = i0 + lane / LR;  // warp-uniform trips
+    const bool todo = i < n && (LR > 1 || !prev || dirty[i]);
+    if (LR == 1 && i < n && (todo || !prev)) dirty[i] = 0;
     int zi = 0;
     int64_t e0 = 0, e1 = 0;
     bool ok = todo;
@@ -92,13 +102,14 @@ __global__ void __launch_bounds__(kGrThreads) gr_gain_kernel(const int32_t* __re
       }
     }
     const bool big = ok && e1 - e0 > kGrRowMax;
+    unsigned long long packed = 0;  // eight counts of a byte each
     if (ok && !big) {
-      unsigned long long packed = 0;  // eight counts of a byte each
-      for (int64_t e = e0; e < e1; e += 4) {
-        int32_t j[4];
-        int zj[4];
+      constexpr int U = LR == 1 ? 4 : 1;  // gathers in flight
+      for (int64_t e = e0 + sub; e < e1; e += U * LR) {
+        int32_t j[U];
+        int zj[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
           j[u] = e + u < e1 ? colidx[e + u] : static_cast<int32_t>(i);
           if (j[u] < 0 || j[u] >= n) {
             dev_fail(status, LRQ_EINVAL);
@@ -107,17 +118,21 @@ __global__ void __launch_bounds__(kGrThreads) gr_gain_kernel(const int32_t* __re
           zj[u] = j[u] != i ? z[j[u]] : kGrMaxK;
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < U; ++u)
           if (zj[u] < kGrMaxK) packed += 1ull << (8 * zj[u]);
       }
+    }
+#pragma unroll
+    for (int q = LR / 2; q > 0; q >>= 1) packed += __shfl_xor_sync(0xffffffffu, packed, q);
+    if (ok && !big && sub == 0) {
       int cnt[kGrMaxK];
 #pragma unroll
       for (int c = 0; c < kGrMaxK; ++c) cnt[c] = static_cast<int>((packed >> (8 * c)) & 0xff);
       gr_store(i, zi, K, cnt, gain, best);
     }
-    for (unsigned m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
+    for (unsigned m = __ballot_sync(0xffffffffu, big && sub == 0); m; m &= m - 1) {
       const int src = __ffs(m) - 1;
-      const int64_t ib = i0 + src, b0 = __shfl_sync(0xffffffffu, e0, src), b1 = __shfl_sync(0xffffffffu, e1, src);
+      const int64_t ib = i0 + src / LR, b0 = __shfl_sync(0xffffffffu, e0, src), b1 = __shfl_sync(0xffffffffu, e1, src);
       int cnt[kGrMaxK];
 #pragma unroll
       for (int c = 0; c < kGrMaxK; ++c) cnt[c] = 0;
@@ -142,8 +157,9 @@ __global__ void __launch_bounds__(kGrThreads) gr_gain_kernel(const int32_t* __re
   }
 }
 
-// move every gaining vertex that no gaining neighbour outranks, and mark it
-// and its neighbours
+// move every gaining vertex that no gaining neighbour outranks, and (LR = 1)
+// mark it and its neighbours
+template <int LR>
 __global__ void __launch_bounds__(kGrThreads) gr_move_kernel(const int32_t* __restrict__ rowptr,
                                                              const int32_t* __restrict__ colidx, int64_t n,
                                                              int64_t nnz, const int32_t* __restrict__ gain,
@@ -152,56 +168,67 @@ __global__ void __launch_bounds__(kGrThreads) gr_move_kernel(const int32_t* __re
                                                              const unsigned long long* prev,
                                                              unsigned long long* moved) {
   if (prev && *prev == 0ull) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * kGrThreads;
+  constexpr int RW = 32 / LR;
+  const int lane = threadIdx.x & 31, sub = lane % LR;
+  const unsigned row_lanes = ((1u << LR) - 1u) << (lane - sub);
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * (kGrThreads / LR);
   unsigned mine = 0;
-  for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * kGrThreads + (threadIdx.x & ~31); i0 < n; i0 += stride) {
-    const int64_t i = i0 + lane;
+  for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * (kGrThreads / LR) + (threadIdx.x >> 5) * RW; i0 < n;
+       i0 += stride) {
+    const int64_t i = i0 + lane / LR;
     const int gi = i < n ? gain[i] : 0;
     int64_t e0 = 0, e1 = 0;
     const bool act = gi > 0 && gr_row(rowptr, i, nnz, &e0, &e1);
     const bool big = act && e1 - e0 > kGrRowMax;
-    if (act && !big) {
-      bool blocked = false;
-      for (int64_t e = e0; e < e1 && !blocked; e += 4) {
+    bool blocked = !act || big;
+    if (!blocked) {
+      constexpr int U = LR == 1 ? 4 : 1;
+      for (int64_t e = e0 + sub; e < e1 && !blocked; e += U * LR) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
           const int32_t j = e + u < e1 ? colidx[e + u] : -1;
           if (j < 0 || j >= n || j == i) continue;
           const int gj = gain[j];
           blocked |= gj > gi || (gj == gi && j < i);
         }
       }
-      if (!blocked) {
+    }
+    if (LR > 1) blocked = (__ballot_sync(0xffffffffu, blocked) & row_lanes) != 0u;  // a row's lanes agree
+    if (!blocked) {
+      if (sub == 0) {
         z[i] = best[i];
+        ++mine;
+      }
+      if (LR == 1) {
         dirty[i] = 1;
         for (int64_t e = e0; e < e1; ++e) {
           const int32_t j = colidx[e];
           if (j >= 0 && j < n) dirty[j] = 1;
         }
-        ++mine;
       }
     }
-    for (unsigned m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
+    for (unsigned m = __ballot_sync(0xffffffffu, big && sub == 0); m; m &= m - 1) {
       const int src = __ffs(m) - 1;
-      const int64_t ib = i0 + src, b0 = __shfl_sync(0xffffffffu, e0, src), b1 = __shfl_sync(0xffffffffu, e1, src);
+      const int64_t ib = i0 + src / LR, b0 = __shfl_sync(0xffffffffu, e0, src), b1 = __shfl_sync(0xffffffffu, e1, src);
       const int gb = __shfl_sync(0xffffffffu, gi, src);
-      bool blocked = false;
-      for (int64_t e = b0 + lane; e < b1 && !blocked; e += 32) {
+      bool out = false;
+      for (int64_t e = b0 + lane; e < b1 && !out; e += 32) {
         const int32_t j = colidx[e];
         if (j < 0 || j >= n || j == ib) continue;
         const int gj = gain[j];
-        blocked = gj > gb || (gj == gb && j < ib);
+        out = gj > gb || (gj == gb && j < ib);
       }
-      if (__any_sync(0xffffffffu, blocked)) continue;
+      if (__any_sync(0xffffffffu, out)) continue;
       if (lane == src) {
         z[ib] = best[ib];
-        dirty[ib] = 1;
+        if (LR == 1) dirty[ib] = 1;
         ++mine;
       }
-      for (int64_t e = b0 + lane; e < b1; e += 32) {
-        const int32_t j = colidx[e];
-        if (j >= 0 && j < n) dirty[j] = 1;
+      if (LR == 1) {
+        for (int64_t e = b0 + lane; e < b1; e += 32) {
+          const int32_t j = colidx[e];
+          if (j >= 0 && j < n) dirty[j] = 1;
+        }
       }
     }
   }
@@ -226,7 +253,11 @@ int launch_greedy(const int32_t* rowptr, const int32_t* colidx, int64_t n, int64
   base += align_up(static_cast<size_t>(n), 256);
   unsigned long long* ring = reinterpret_cast<unsigned long long*>(base);
 
-  const int blocks = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, kGrThreads), 152 * 8)));
+  const int lanes = n <= kGrSmall ? 8 : 1;
+  const auto gr_gain = lanes == 8 ? gr_gain_kernel<8> : gr_gain_kernel<1>;
+  const auto gr_move = lanes == 8 ? gr_move_kernel<8> : gr_move_kernel<1>;
+  const int blocks =
+      static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(ceil_div(n * lanes, kGrThreads), 152 * 8)));
   int64_t launched = 0, rounds = 0, moves = 0;
   bool converged = false;
   int e = LRQ_OK;
@@ -238,8 +269,8 @@ int launch_greedy(const int32_t* rowptr, const int32_t* colidx, int64_t n, int64
     for (int t = 0; t < nr; ++t) {
       const unsigned long long* prev =
           (b == 0 && t == 0) ? nullptr : (t == 0 ? ring + ((b - 1) & 1) * kGrBatch + (kGrBatch - 1) : slot + t - 1);
-      gr_gain_kernel<<<blocks, kGrThreads, 0, st>>>(rowptr, colidx, n, nnz, K, z, gain, best, dirty, prev, status);
-      gr_move_kernel<<<blocks, kGrThreads, 0, st>>>(rowptr, colidx, n, nnz, gain, best, z, dirty, prev, slot + t);
+      gr_gain<<<blocks, kGrThreads, 0, st>>>(rowptr, colidx, n, nnz, K, z, gain, best, dirty, prev, status);
+      gr_move<<<blocks, kGrThreads, 0, st>>>(rowptr, colidx, n, nnz, gain, best, z, dirty, prev, slot + t);
       count_launch(2);
     }
     if ((e = cuda_check(cudaGetLastError(), "greedy kernels"))) return e;
@@ -261,7 +292,7 @@ int launch_greedy(const int32_t* rowptr, const int32_t* colidx, int64_t n, int64
     launched += nr;
   }
   if (max_rounds == 0) {  // no round ran: validate labels and graph before the cut reads them
-    gr_gain_kernel<<<blocks, kGrThreads, 0, st>>>(rowptr, colidx, n, nnz, K, z, gain, best, dirty, nullptr, status);
+    gr_gain<<<blocks, kGrThreads, 0, st>>>(rowptr, colidx, n, nnz, K, z, gain, best, dirty, nullptr, status);
     count_launch();
     int32_t hs = 0;
     if ((e = cuda_check(cudaGetLastError(), "greedy gain kernel"))) return e;
