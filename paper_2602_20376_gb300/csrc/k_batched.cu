@@ -5,9 +5,10 @@
 // Work decomposition: an item is (problem p, a tile of T consecutive
 // candidates); it scores those T directions against all n_p coordinates, so
 // items are independent and need no cross-item reduction.  A block of 64
-// threads holds T candidates (four per thread) x (256 / T) row groups; the row
-// groups split the coordinates of each shared-memory stage and are combined in
-// FP64 at the end of the item.  Items are sorted by cost (n_p T) longest first
+// threads holds T candidates (four per thread) x (256 / T) row groups, or of
+// 256 threads where the items are few (one per thread, b_slots_per_thread); the
+// row groups split the coordinates of each shared-memory stage and are combined
+// in FP64 at the end of the item.  Items are sorted by cost (n_p T) longest first
 // and pulled by the persistent blocks from an atomic counter.
 //
 // Per problem the launch sequence is: input checks, direction sampling
@@ -35,6 +36,7 @@
 #include <tuple>
 #include <vector>
 
+#include "batched_score.cuh"
 #include "enum_device.cuh"
 #include "gauss_df32.cuh"
 #include "lrq_device.cuh"
@@ -43,44 +45,11 @@
 
 namespace lrq {
 
-constexpr int kBThreads = 64;
-constexpr int kBSlots = 256;      // candidate x row group slots of a block, four per thread
-constexpr int kBPerThread = kBSlots / kBThreads;
 constexpr int kBSelThreads = 256; // selection kernel
-constexpr int kBRows = 128;       // V rows per shared-memory stage
 constexpr int kBMaxS = 8192;      // candidates per problem
 constexpr int kBMaxTopM = 16;
 constexpr int kBTiles[3] = {64, 128, 256};
-constexpr int kBEnumRanksPerThread = 16;
-constexpr int kBEnumChunk = kBThreads * kBEnumRanksPerThread;  // index sets per exact work item
 constexpr double kBEnumBudget = 1e10;                            // r n^(2r+1) of one exact problem
-
-struct BProb {
-  const float2* V;
-  const float2* C;  // directions: the caller's, or the workspace slot when drawn
-  int64_t n;
-  int r, K, S, tile;
-  int gen;          // 1: draw C from seed (+ epoch)
-  int exact;        // 1: solved exactly by vertex enumeration (S = 0)
-  uint64_t seed;
-  int64_t key_off;  // offset of the problem's selection keys
-  int64_t eb_off;   // exact: offset of its chunk results
-  int nchunks;      // exact: work items
-  int pad;
-  unsigned long long lvl_total[kEnumMaxD];  // exact: index sets of level d at [d - 1]
-};
-
-struct BItem {
-  int p;
-  int s0;
-};
-
-struct BTable {
-  float bcos[8], bsin[8];
-  float zr[kMaxK], zi[kMaxK];
-  double bcos64[8], bsin64[8];
-  double zr64[kMaxK], zi64[kMaxK];
-};
 
 // decision tables for K = 0..64 (entries below 2 unused), filled once per device
 static __device__ BTable g_btab[kMaxK + 1];
@@ -110,230 +79,6 @@ __global__ void batched_check_kernel(const BProb* __restrict__ probs, int32_t* s
        t += static_cast<int64_t>(gridDim.x) * blockDim.x)
     bad |= !isfinite(t < nv ? v[t] : c[t - nv]);
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) dev_fail(status, LRQ_EINVAL);
-}
-
-// ---------------------------------------------------------------------------
-// persistent scoring kernel
-// ---------------------------------------------------------------------------
-// The slots' FP64 sums: while a thread takes its four slots at once (r <= 4,
-// where the first 24 KB hold sums and staged rows) they stay in shared memory
-// over the stages; for larger r they take the staged rows' place at the end.
-struct BShared {
-  union {
-    struct {
-      double sums[kBSlots * 8];             // r <= 4: [2 r][slot]
-      float4 vs[kBRows * 4];                // {re, re, im, im} per entry (score_f32x2.cuh)
-    } small;
-    float4 vs[kBRows * kMaxRank];
-    double comb[kBSlots * 2 * kMaxRank];    // [slot][2 r]
-  };
-  float2 zt[kMaxK];                         // z table: 16 sign patterns at most, or a code each
-  int next;
-};
-
-// A thread scores candidates s0 + cl + q T / 4, q < 4, on row group g: all on
-// every row it reads (r <= 4), or a part of them at a time on the staged rows
-// (their directions re-read, their FP64 sums in local memory).
-// Bound: FP32 FMAs and shared-memory reads, as score_fp32_kernel; 512 uneven
-// instances of up to 8192 directions: 11.0 ms, 15.3 with one candidate per thread
-// and scalar FMAs, 11.7 with two.
-template <int R, int KC>
-__device__ void b_score_item(const BProb& pb, int s0, BShared& sh, uint64_t* __restrict__ keys) {
-  constexpr int P = R <= 4 ? kBPerThread : (R <= 6 ? 2 : 1);  // candidates at once
-  constexpr bool kShared = P == kBPerThread;
-  const int T = pb.tile, H = T / kBPerThread, RS = kBSlots / T;
-  const int tid = threadIdx.x, cl = tid % H, g = tid / H;
-  const BTable& tb = g_btab[pb.K];
-  float4* const vs = kShared ? sh.small.vs : sh.vs;
-  Dir2<R> d[P];
-  auto load_dirs = [&](int q0) {
-#pragma unroll
-    for (int q = 0; q < P; ++q) {
-      const int s = s0 + cl + (q0 + q) * H;
-#pragma unroll
-      for (int j = 0; j < R; ++j)
-        d[q].set(j, s < pb.S ? pb.C[static_cast<int64_t>(s) * R + j] : make_float2(0.f, 0.f));
-    }
-  };
-  double acc64[kShared ? 1 : kBPerThread][2 * R];
-  auto slot = [&](int q) { return g * T + cl + q * H; };
-  if constexpr (kShared) {
-    load_dirs(0);
-#pragma unroll
-    for (int q = 0; q < P; ++q)
-#pragma unroll
-      for (int j = 0; j < 2 * R; ++j) sh.small.sums[j * kBSlots + slot(q)] = 0.0;
-  } else {
-    for (int q = 0; q < kBPerThread; ++q)
-#pragma unroll
-      for (int j = 0; j < 2 * R; ++j) acc64[q][j] = 0.0;
-  }
-  fill_ztable<KC>(sh.zt, tb.zr, tb.zi, pb.K);
-  for (int64_t b0 = 0; b0 < pb.n; b0 += kBRows) {
-    const int rows = static_cast<int>(min(static_cast<int64_t>(kBRows), pb.n - b0));
-    __syncthreads();
-#pragma unroll 4
-    for (int t = tid; t < rows * R; t += kBThreads) {
-      const float2 v = pb.V[b0 * R + t];
-      vs[t] = make_float4(v.x, v.x, v.y, v.y);
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int q0 = 0; q0 < kBPerThread; q0 += P) {
-      if constexpr (!kShared) load_dirs(q0);
-      f32x2 acc[P][R];
-#pragma unroll
-      for (int q = 0; q < P; ++q)
-#pragma unroll
-        for (int j = 0; j < R; ++j) acc[q][j] = 0;
-#pragma unroll 1
-      for (int i = g; i < rows; i += RS) {
-        ulonglong2 v[R];
-#pragma unroll
-        for (int j = 0; j < R; ++j) v[j] = reinterpret_cast<const ulonglong2*>(vs)[i * R + j];
-#pragma unroll
-        for (int q = 0; q < P; ++q)
-          score_row<KC, R, false>(v, d[q], sh.zt, pb.K, tb.bcos, tb.bsin, acc[q]);
-      }
-#pragma unroll
-      for (int q = 0; q < P; ++q)
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-          float re, im;
-          unpack2(acc[q][j], re, im);
-          if constexpr (kShared) {
-            sh.small.sums[2 * j * kBSlots + slot(q)] += static_cast<double>(re);
-            sh.small.sums[(2 * j + 1) * kBSlots + slot(q)] += static_cast<double>(im);
-          } else {
-            acc64[q0 + q][2 * j] += static_cast<double>(re);
-            acc64[q0 + q][2 * j + 1] += static_cast<double>(im);
-          }
-        }
-    }
-  }
-  __syncthreads();
-  if constexpr (!kShared) {
-    for (int q = 0; q < kBPerThread; ++q)
-#pragma unroll
-      for (int j = 0; j < 2 * R; ++j) sh.comb[slot(q) * (2 * R) + j] = acc64[q][j];
-    __syncthreads();
-  }
-  for (int c = tid; c < T; c += kBThreads) {
-    const int s = s0 + c;
-    if (s >= pb.S) break;
-    double f = 0.0;
-#pragma unroll
-    for (int j = 0; j < 2 * R; ++j) {
-      double v = 0.0;
-      for (int gg = 0; gg < RS; ++gg)
-        v += kShared ? sh.small.sums[j * kBSlots + gg * T + c] : sh.comb[(gg * T + c) * (2 * R) + j];
-      f += v * v;
-    }
-    const uint32_t fb = __float_as_uint(static_cast<float>(f));
-    keys[pb.key_off + s] = (static_cast<uint64_t>(fb) << 32) | static_cast<uint64_t>(0xFFFFFFFFu - static_cast<uint32_t>(s));
-  }
-}
-
-template <int R>
-__device__ __forceinline__ void b_dispatch_k(const BProb& pb, int s0, BShared& sh, uint64_t* keys) {
-  switch (pb.K) {
-    case 2: b_score_item<R, 2>(pb, s0, sh, keys); break;
-    case 3: b_score_item<R, 3>(pb, s0, sh, keys); break;
-    case 4: b_score_item<R, 4>(pb, s0, sh, keys); break;
-    case 8: b_score_item<R, 8>(pb, s0, sh, keys); break;
-    default: b_score_item<R, 0>(pb, s0, sh, keys); break;
-  }
-}
-
-// One exact work item: index sets [chunk kBEnumChunk, (chunk + 1) kBEnumChunk)
-// of the problem's levels d = r..1 taken in turn, kBEnumRanksPerThread
-// consecutive ranks per thread; the block's best candidate (the solver's
-// order) goes to ebest[eb_off + chunk].  Kept out of line so that the
-// scoring path keeps its registers.
-__device__ __noinline__ void b_enum_item(const BProb& pb, int chunk, BShared& sh, EnumBest* __restrict__ ebest,
-                                         int32_t* status) {
-  const EnumTables& tb = g_etab[pb.K];
-  const EnumV32 va{pb.V, pb.r};
-  const int n = static_cast<int>(pb.n);
-  const int N = n * tb.BK;
-  unsigned long long total = 0;
-  for (int d = 1; d <= pb.r; ++d) total += pb.lvl_total[d - 1];
-  EnumBest best;
-  best.f = -1.0;
-  best.level = 0;
-  best.sign = 1;
-  best.rank = 0;
-  best.choice = 0;
-  unsigned long long q = static_cast<unsigned long long>(chunk) * kBEnumChunk +
-                         static_cast<unsigned long long>(threadIdx.x) * kBEnumRanksPerThread;
-  const unsigned long long qend = min(total, q + kBEnumRanksPerThread);
-  while (q < qend) {
-    int d = pb.r;
-    unsigned long long base = 0;
-    while (d >= 1 && q >= base + pb.lvl_total[d - 1]) {
-      base += pb.lvl_total[d - 1];
-      --d;
-    }
-    if (d < 1) break;
-    const int m = 2 * d - 1;
-    const unsigned long long l0 = q - base;
-    const unsigned long long l1 = min(qend - base, pb.lvl_total[d - 1]);
-    int I[kEnumMaxRows];
-    unrank(l0, N, m, I);
-    for (unsigned long long lr = l0; lr < l1; ++lr) {
-      if (lr > l0) next_comb(N, m, I);
-      if (!valid_set(I, m, tb.BK)) continue;
-      double H[kEnumMaxRows * 2 * kEnumMaxD];
-      build_rows(va, pb.r, d, I, m, tb, H);
-      double ct[2 * kEnumMaxD];
-      if (!null_vector_fp64<kEnumMaxRows>(H, m, ct)) continue;
-      eval_vertex(va, n, pb.r, d, I, m, ct, +1, tb, best, lr, -1, nullptr, nullptr, status);
-      eval_vertex(va, n, pb.r, d, I, m, ct, -1, tb, best, lr, -1, nullptr, nullptr, status);
-    }
-    q = base + l1;
-  }
-  EnumBest* sb = reinterpret_cast<EnumBest*>(sh.comb);  // kBThreads entries
-  __syncthreads();
-  sb[threadIdx.x] = best;
-  __syncthreads();
-  for (int h = kBThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h && enum_better(sb[threadIdx.x + h], sb[threadIdx.x])) sb[threadIdx.x] = sb[threadIdx.x + h];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) ebest[pb.eb_off + chunk] = sb[0];
-  __syncthreads();
-}
-
-__global__ void __launch_bounds__(kBThreads, 6) batched_score_kernel(const BProb* __restrict__ probs,
-                                                                  const BItem* __restrict__ items, int nitems,
-                                                                  int* __restrict__ counter,
-                                                                  uint64_t* __restrict__ keys,
-                                                                  EnumBest* __restrict__ ebest,
-                                                                  int32_t* status) {
-  __shared__ BShared sh;
-  for (;;) {
-    if (threadIdx.x == 0) sh.next = atomicAdd(counter, 1);
-    __syncthreads();
-    const int it = sh.next;
-    __syncthreads();
-    if (it >= nitems) break;
-    const BItem w = items[it];
-    const BProb pb = probs[w.p];
-    if (pb.exact) {
-      b_enum_item(pb, w.s0, sh, ebest, status);
-      continue;
-    }
-    switch (pb.r) {
-      case 1: b_dispatch_k<1>(pb, w.s0, sh, keys); break;
-      case 2: b_dispatch_k<2>(pb, w.s0, sh, keys); break;
-      case 3: b_dispatch_k<3>(pb, w.s0, sh, keys); break;
-      case 4: b_dispatch_k<4>(pb, w.s0, sh, keys); break;
-      case 5: b_dispatch_k<5>(pb, w.s0, sh, keys); break;
-      case 6: b_dispatch_k<6>(pb, w.s0, sh, keys); break;
-      case 7: b_dispatch_k<7>(pb, w.s0, sh, keys); break;
-      default: b_dispatch_k<8>(pb, w.s0, sh, keys); break;
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -688,12 +433,15 @@ struct lrq_batched_plan_impl {
   std::vector<int> tile;
   int top_m = 0;
   int device = 0;
-  int grid = 0;
+  int grid_wide = 0, grid = 0;  // resident blocks of batched_score_kernel<1> and <4>
   int64_t nkeys = 0, ncgen = 0;
   size_t off_probs = 0, off_items = 0, off_counter = 0, off_epoch = 0, off_keys = 0, off_C = 0, off_ebest = 0,
          total = 0;
   int64_t nebest = 0;
   int nitems = 0;
+  int per_thread = 4;     // slots per thread of the scoring kernel
+  const BTable* btab = nullptr;  // the device's decision tables, from prepare on
+  const EnumTables* etab = nullptr;
   int sample_blocks = 0;  // of the problem with most directions to draw
   bool prepared = false;
   const void* prepared_ws = nullptr;
@@ -794,10 +542,29 @@ void layout(lrq_batched_plan_impl* pl) {
   pl->total = cur;
 }
 
+// Slots per thread of the scoring kernel: four (fewest instructions an
+// evaluation) once the items' cost fills the resident blocks a good deal longer
+// than the longest item takes in one of them; below that the longest items, or
+// the last of them, are the launch's time, and a block of 256 threads takes
+// about half of it.  Measured with one / four slots a thread, by total over
+// longest item (four slots: 912 resident blocks): 26 126 / 176 us, 163 971 /
+// 2260, 330 179 / 250, 651 1849 / 2313, 892 773 / 730, 934 814 / 815, 1024 equal
+// items 364 / 352 (r = 4, K = 3) and 638 / 800 (r = 8), 1216 3858 / 3428, 4863
+// 14308 / 11794.
+// One slot also where most of the work is of a kind that gains nothing from four:
+// exact items (FP64 out of local memory; a unit of their cost takes about 24 times
+// a scoring item's; 64 with n = 24: 31.4 / 40.7 ms), K > 8 (the angle; 200 of
+// K = 11: 3494 / 3838 us) and K = 5, 6, 7 (b_dispatch_k; 200 of K = 5: 1965 /
+// 2501 us).
+// Either form adds the same numbers in the same order.
+int b_slots_per_thread(const lrq_batched_plan_impl* pl, double scoring, double other, double longest) {
+  return other > scoring || scoring + other < 1.25 * longest * pl->grid ? 1 : 4;
+}
+
 // Device descriptors and the item list for the problems in `subset` (all
 // when empty), with the plan's current tiles.
-int upload(lrq_batched_plan_impl* pl, uint8_t* ws, const std::vector<int>& subset, cudaStream_t st,
-           int* nitems_out) {
+int upload(lrq_batched_plan_impl* pl, uint8_t* ws, const std::vector<int>& subset, cudaStream_t st, int* nitems_out,
+           int* per_thread_out) {
   const int P = static_cast<int>(pl->probs.size());
   std::vector<BProb> hp(P);
   int64_t key_off = 0, c_off = 0, eb_off = 0;
@@ -863,10 +630,19 @@ int upload(lrq_batched_plan_impl* pl, uint8_t* ws, const std::vector<int>& subse
     return e;
   if ((e = cuda_check(cudaStreamSynchronize(st), "upload sync"))) return e;  // host vectors end here
   *nitems_out = static_cast<int>(items.size());
+  double scoring = 0.0, other = 0.0;
+  for (const BItem& it : items) {
+    const BProb& b = hp[it.p];
+    if (b.exact)
+      other += 24.0 * cost(it);
+    else
+      (b.K <= 4 || b.K == 8 ? scoring : other) += cost(it);
+  }
+  *per_thread_out = b_slots_per_thread(pl, scoring, other, items.empty() ? 0.0 : cost(items[0]));
   return LRQ_OK;
 }
 
-int launch_sequence(const lrq_batched_plan_impl* pl, uint8_t* ws, int nitems, bool sample, bool select,
+int launch_sequence(const lrq_batched_plan_impl* pl, uint8_t* ws, int nitems, int per_thread, bool sample, bool select,
                     double* best_f, int64_t* best_idx, int32_t* status, cudaStream_t st) {
   const int P = static_cast<int>(pl->probs.size());
   const BProb* probs = reinterpret_cast<const BProb*>(ws + pl->off_probs);
@@ -885,8 +661,12 @@ int launch_sequence(const lrq_batched_plan_impl* pl, uint8_t* ws, int nitems, bo
   if (e) return e;
   timing_start(st);
   EnumBest* ebest = reinterpret_cast<EnumBest*>(ws + pl->off_ebest);
-  batched_score_kernel<<<pl->grid, kBThreads, 0, st>>>(probs, reinterpret_cast<const BItem*>(ws + pl->off_items),
-                                                       nitems, counter, keys, ebest, status);
+  const BItem* items = reinterpret_cast<const BItem*>(ws + pl->off_items);
+  if (per_thread == 1)
+    launch_batched_wide(pl->grid_wide, st, probs, items, nitems, counter, pl->btab, pl->etab, keys, ebest, status);
+  else
+    batched_score_kernel<4><<<pl->grid, kBSlots / 4, 0, st>>>(probs, items, nitems, counter, pl->btab, pl->etab, keys,
+                                                              ebest, status);
   timing_stop(st);
   count_launch();
   if (select) {
@@ -947,14 +727,15 @@ int lrq_batched_plan_create(const lrq_problem* problems, int P, int top_m, lrq_b
       pl->tile[p] = it != g_tile_cache.end() ? it->second : 128;
     }
   }
-  int blocks_per_sm = 1;
-  if ((e = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, batched_score_kernel,
-                                                                    kBThreads, 0),
-                      "occupancy query"))) {
+  int per_sm = 1, per_sm_wide = 1;
+  if ((e = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_score_kernel<4>, kBSlots / 4, 0),
+                      "occupancy query")) ||
+      (e = batched_wide_blocks_per_sm(&per_sm_wide))) {
     delete pl;
     return e;
   }
-  pl->grid = std::max(1, blocks_per_sm) * num_sms_current();
+  pl->grid = std::max(1, per_sm) * num_sms_current();
+  pl->grid_wide = std::max(1, per_sm_wide) * num_sms_current();
   layout(pl);
   *plan_out = pl;
   return LRQ_OK;
@@ -975,9 +756,15 @@ int lrq_batched_prepare(lrq_batched_plan* plan, void* ws, size_t ws_bytes, void*
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int e = ensure_tables(plan->device);
   if (e) return e;
+  void *bt = nullptr, *et = nullptr;
+  if ((e = cuda_check(cudaGetSymbolAddress(&bt, g_btab), "decision tables")) ||
+      (e = cuda_check(cudaGetSymbolAddress(&et, g_etab), "enumeration tables")))
+    return e;
+  plan->btab = static_cast<const BTable*>(bt);
+  plan->etab = static_cast<const EnumTables*>(et);
   uint8_t* w = static_cast<uint8_t*>(ws);
   if ((e = cuda_check(cudaMemsetAsync(w + plan->off_epoch, 0, sizeof(int64_t), st), "reset epoch"))) return e;
-  if ((e = upload(plan, w, {}, st, &plan->nitems))) return e;
+  if ((e = upload(plan, w, {}, st, &plan->nitems, &plan->per_thread))) return e;
   plan->prepared = true;
   plan->prepared_ws = ws;
   return LRQ_OK;
@@ -988,7 +775,7 @@ int lrq_sample_score_batched(const lrq_batched_plan* plan, void* ws, size_t ws_b
   if (!plan || !best_f_out || !best_idx_out || !dev_status) return fail(LRQ_EINVAL, "NULL pointer argument");
   if (!plan->prepared || plan->prepared_ws != ws || ws_bytes < plan->total)
     return fail(LRQ_EINVAL, "call lrq_batched_prepare with this workspace first");
-  return launch_sequence(plan, static_cast<uint8_t*>(ws), plan->nitems, true, true, best_f_out, best_idx_out,
+  return launch_sequence(plan, static_cast<uint8_t*>(ws), plan->nitems, plan->per_thread, true, true, best_f_out, best_idx_out,
                          dev_status, static_cast<cudaStream_t>(stream));
 }
 
@@ -1000,7 +787,7 @@ int lrq_batched_autotune(lrq_batched_plan* plan, void* ws, size_t ws_bytes, int3
   uint8_t* w = static_cast<uint8_t*>(ws);
   const int P = static_cast<int>(plan->probs.size());
   // directions once (the timed runs score them again and again)
-  int e = launch_sequence(plan, w, 0, true, false, nullptr, nullptr, dev_status, st);
+  int e = launch_sequence(plan, w, 0, plan->per_thread, true, false, nullptr, nullptr, dev_status, st);
   if (e) return e;
   if ((e = cuda_check(cudaMemsetAsync(w + plan->off_epoch, 0, sizeof(int64_t), st), "reset epoch"))) return e;
   std::map<std::tuple<int, int, int>, std::vector<int>> classes;
@@ -1018,12 +805,12 @@ int lrq_batched_autotune(lrq_batched_plan* plan, void* ws, size_t ws_bytes, int3
     int best_tile = 128;
     for (int ti = 0; ti < 3; ++ti) {
       for (int p : kv.second) plan->tile[p] = kBTiles[ti];
-      int nit = 0;
-      if ((e = upload(plan, w, kv.second, st, &nit))) break;
+      int nit = 0, per_thread = 4;
+      if ((e = upload(plan, w, kv.second, st, &nit, &per_thread))) break;
       float ms = 0.f;
       for (int rep = 0; rep < 3 && !e; ++rep) {
         cudaEventRecord(t0, st);
-        e = launch_sequence(plan, w, nit, false, false, nullptr, nullptr, dev_status, st);
+        e = launch_sequence(plan, w, nit, per_thread, false, false, nullptr, nullptr, dev_status, st);
         cudaEventRecord(t1, st);
         if (!e) e = cuda_check(cudaEventSynchronize(t1), "autotune sync");
         float x = 0.f;
@@ -1045,7 +832,7 @@ int lrq_batched_autotune(lrq_batched_plan* plan, void* ws, size_t ws_bytes, int3
   cudaEventDestroy(t0);
   cudaEventDestroy(t1);
   if (e) return e;
-  return upload(plan, w, {}, st, &plan->nitems);
+  return upload(plan, w, {}, st, &plan->nitems, &plan->per_thread);
 }
 
 int lrq_batched_tile(const lrq_batched_plan* plan, int p) {

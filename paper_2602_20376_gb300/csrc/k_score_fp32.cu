@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(Fp32Shape<R>::kThreads) score_fp32_kernel(cons
   __shared__ float2 zt[ZTable<K>::kEntries];
   fill_ztable<K>(zt, tab.zr, tab.zi, Kdyn);
 
+  const float none[kAnyLines] = {};  // the boundaries of kAnyK8, not used here
   const int64_t s0 = static_cast<int64_t>(blockIdx.x) * kFp32Block + threadIdx.x;
   Dir2<R> d[kFp32Cpt];
   double acc64[kFp32Cpt][2 * R];
@@ -241,7 +242,7 @@ __global__ void __launch_bounds__(Fp32Shape<R>::kThreads) score_fp32_kernel(cons
 #pragma unroll
       for (int j = 0; j < R; ++j) v[j] = reinterpret_cast<const ulonglong2*>(vs)[i * R + j];
 #pragma unroll
-      for (int q = 0; q < kFp32Cpt; ++q) score_row<K, R, true>(v, d[q], zt, Kdyn, nullptr, nullptr, acc[q]);
+      for (int q = 0; q < kFp32Cpt; ++q) score_row<K, R, true>(v, d[q], zt, Kdyn, none, none, acc[q]);
     }
 #pragma unroll
     for (int q = 0; q < kFp32Cpt; ++q)

@@ -195,15 +195,19 @@ __device__ __forceinline__ uint32_t pattern_of(int k) {
   }
 }
 
-// entries of the z table (sign patterns; codes for K > 8) and its filling by
-// a block's threads
+// K as a template argument: 2..8, kAnyK8 for an alphabet of at most 8 known at
+// run time, 0 for larger ones.
+constexpr int kAnyK8 = -1;
+
+// entries of the z table (sign patterns; codes where K is known at run time only)
+// and its filling by a block's threads
 template <int K>
 struct ZTable {
-  static constexpr int kEntries = K == 0 ? kMaxK : 1 << ((K % 2 == 0) ? K / 2 : K);
+  static constexpr int kEntries = K <= 0 ? kMaxK : 1 << ((K % 2 == 0) ? K / 2 : K);
 };
 template <int K>
 __device__ __forceinline__ void fill_ztable(float2* zt, const float* zr, const float* zi, int Kdyn) {
-  const int count = K == 0 ? Kdyn : ZTable<K>::kEntries;
+  const int count = K <= 0 ? Kdyn : ZTable<K>::kEntries;
   for (int t = threadIdx.x; t < count; t += blockDim.x) {
     int k = t;
     if constexpr (K > 0) k = decide_from_signs<K>(static_cast<uint32_t>(t));
@@ -221,14 +225,25 @@ struct Dir2 {
   }
 };
 
-// K known at run time only: the sign rule of decide_fp32 for K <= 8 (bc, bs:
-// its boundaries), the angle above.
-__device__ __forceinline__ int decide_any(float x, float y, int K, const float* bc, const float* bs) {
-  if (K > 8) return decide_fp32_generic(x, y, K);
-  const int BK = (K % 2 == 0) ? K / 2 : K;
+// The sign rule of decide_fp32 for K <= 8 known at run time.  bc, bs: the first
+// (B_K + 1) / 2 boundaries (the others are their mirror images, as above), in
+// registers: read from memory line by line they took the batched kernel twice
+// its time at K = 5.
+constexpr int kAnyLines = 4;
+__device__ __forceinline__ int decide_any8(float x, float y, int K, const float (&bc)[kAnyLines],
+                                           const float (&bs)[kAnyLines]) {
+  const bool odd = K % 2 == 1;
+  const int BK = odd ? K : K / 2;
   uint32_t sb = 0;
-  for (int m = 0; m < BK; ++m) sb |= (fmaf(y, bc[m], -x * bs[m]) > 0.0f ? 1u : 0u) << m;
-  if (K % 2 == 0) {
+#pragma unroll
+  for (int m = 0; m < kAnyLines; ++m) {
+    if (2 * m < BK) {
+      const float t = x * bs[m], q = fmaf(y, bc[m], t);
+      if (fmaf(y, bc[m], -t) > 0.f) sb |= 1u << m;
+      if ((odd ? q : -q) > 0.f) sb |= 1u << (BK - 1 - m);
+    }
+  }
+  if (!odd) {
     const int c = __popc(sb);
     return (sb & 1u) ? c : (c == 0 ? 0 : K - c);
   }
@@ -237,10 +252,11 @@ __device__ __forceinline__ int decide_any(float x, float y, int K, const float* 
 }
 
 // acc[j] += conj(V_ij) z_i for one candidate; v: the row's {re, re, im, im}.
-// K = 0: any alphabet, Kdyn.  VFIRST: the order of the two products of w (each caller's own).
+// bc, bs: kAnyK8's boundaries.  VFIRST: the order of the two products of w (each caller's own).
 template <int K, int R, bool VFIRST>
 __device__ __forceinline__ void score_row(const ulonglong2 (&v)[R], const Dir2<R>& d, const float2* zt, int Kdyn,
-                                          const float* bc, const float* bs, f32x2 (&acc)[R]) {
+                                          const float (&bc)[kAnyLines], const float (&bs)[kAnyLines],
+                                          f32x2 (&acc)[R]) {
   f32x2 w = 0;  // {0, 0}
 #pragma unroll
   for (int j = 0; j < R; ++j) {
@@ -258,7 +274,7 @@ __device__ __forceinline__ void score_row(const ulonglong2 (&v)[R], const Dir2<R
   if constexpr (K > 0)
     off = sign_offset<K>(x, y);
   else
-    off = 8u * static_cast<uint32_t>(decide_any(x, y, Kdyn, bc, bs));
+    off = 8u * static_cast<uint32_t>(K == 0 ? decide_fp32_generic(x, y, Kdyn) : decide_any8(x, y, Kdyn, bc, bs));
   const float2 z = *reinterpret_cast<const float2*>(reinterpret_cast<const char*>(zt) + off);
   const f32x2 za = pack2(z.x, z.y), zb = pack2(z.y, -z.x);
 #pragma unroll
