@@ -202,7 +202,9 @@ __device__ bool null_vector_fp64(double* H, int m, double* c) {
 // null_vector_fp64 for M rows with every index known at compile time, so that
 // H stays in registers: the same operations on the same operands in the same
 // order (same bits).  The pivot search compares magnitudes as integers, which
-// order like the absolute values (FP64 comparisons run on the FP64 unit).
+// order like the absolute values (FP64 comparisons run on the FP64 unit).  A row
+// with an infinity or a NaN in it is rejected, as there: NaN entries are never
+// pivots and a null vector of M rows needs M pivot columns.
 template <int M>
 __device__ __forceinline__ bool null_vector_fixed(double (&H)[M][M + 1], double (&c)[M + 1]) {
   constexpr int NC = M + 1;
@@ -215,7 +217,7 @@ __device__ __forceinline__ bool null_vector_fixed(double (&H)[M][M + 1], double 
   for (int i = 0; i < M; ++i)
 #pragma unroll
     for (int j = 0; j < NC; ++j) sc = max(sc, mag(H[i][j]));
-  if (sc == 0) return false;
+  if (sc == 0 || sc >= 0x7ff0000000000000ll) return false;
   const double scale = __longlong_as_double(sc);
 #pragma unroll
   for (int k = 0; k < M; ++k) {
