@@ -204,8 +204,9 @@ __device__ void b_unit_sums(const BProb& pb, int s, int w, int nw, const float4*
     ci[j] = c.y;
     mx = fmaxf(mx, fabsf(c.x) + fabsf(c.y));
   }
-  // the error of an FP32 boundary projection is below cb sum_j |V_ij|_1
-  const float cb = mx * (static_cast<float>(2 * R + 4) * 2.0f + 12.0f) * 5.9604644775390625e-08f;
+  // the error of an FP32 boundary projection is below cb sum_j |V_ij|_1 + 2^-140
+  // where nothing overflows (fp32_row_bound, fp32_dir_bound)
+  const float cb = fp32_dir_bound(mx, R);
   f32x2 hi[2][R], lo[2][R], l3[2][R];
 #pragma unroll
   for (int g = 0; g < 2; ++g)
@@ -231,7 +232,7 @@ __device__ void b_unit_sums(const BProb& pb, int s, int w, int nw, const float4*
       pmin = fminf(pmin, fabsf(p));
     }
     int k;
-    if (pmin > ab * cb) {
+    if (pmin > fp32_proj_bound(fp32_row_bound(ab), cb)) {
       if (K % 2 == 0) {
         const int c = __popc(sb);
         k = (sb & 1u) ? c : (c == 0 ? 0 : K - c);
@@ -354,6 +355,7 @@ __global__ void __launch_bounds__(kBSelThreads) batched_select_kernel(const BPro
   __syncthreads();
   double bf = -1.0;
   int bs = 0;
+  bool all64 = !fast;
   if (fast) {
     // warps per candidate; candidates q0 .. q0 + kBWarps / per - 1 at a time
     const int per = got >= kBWarps ? 1 : (got >= 5 ? 1 : (got >= 3 ? 2 : (got == 2 ? 4 : 8)));
@@ -383,23 +385,26 @@ __global__ void __launch_bounds__(kBSelThreads) batched_select_kernel(const BPro
       }
       __syncthreads();
     }
-    for (int q = 0; q < got; ++q) bf = fmax(bf, fq[q]);
+    for (int q = 0; q < got; ++q) {
+      bf = fmax(bf, fq[q]);
+      all64 |= !isfinite(fq[q]);  // FP32 sums of entries around 10^38 overflow
+    }
   }
   // the best in FP64's own order: directions whose assignments are turns of one
   // another have the same f, which only rounding tells apart, so values this
   // close are taken again in FP64 as for the other alphabets
-  const double near = fast ? bf * (1.0 - 1e-10) : -1.0;
+  const double near = all64 ? -1.0 : bf * (1.0 - 1e-10);
   int close = 0;
   for (int q = 0; q < got; ++q) {
-    if (!fast || fq[q] >= near) {
+    if (all64 || fq[q] >= near) {
       ++close;
       bs = chosen[q];
     }
   }
-  if (!fast || close > 1) {
+  if (all64 || close > 1) {
     bf = -1.0;
     for (int q = 0; q < got; ++q) {
-      if (fast && !(fq[q] >= near)) continue;
+      if (!all64 && !(fq[q] >= near)) continue;
       const int s = chosen[q];
       double f;
       switch (pb.r) {

@@ -205,11 +205,6 @@ __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_k
     ok[q] = act[q] && s >= 0 && s < S;
     if (act[q] && !ok[q] && lane == 0 && chunk == 0) dev_fail(status, LRQ_EINVAL);
   }
-  // The error of an FP32 boundary projection is below gamma sum_j |V_ij|_1
-  // |c_j|_1 (|x|_1 = |Re| + |Im|), gamma = (2 r + 4) 2 u + 8 u with u = 2^-24;
-  // |c_j|_1 is replaced by its largest value (cb, rounded up), so that the
-  // bound is one product per evaluation.
-  const float u = 5.9604644775390625e-08f;
   float cr[kRsCpw][RM], ci[kRsCpw][RM], cb[kRsCpw];
 #pragma unroll
   for (int q = 0; q < kRsCpw; ++q) {
@@ -221,7 +216,7 @@ __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_k
       ci[q][j] = c.y;
       mx = fmaxf(mx, fabsf(c.x) + fabsf(c.y));
     }
-    cb[q] = mx * (static_cast<float>(2 * r + 4) * 2.0f + 12.0f) * u;
+    cb[q] = fp32_dir_bound(mx, r);  // the certificate's (score_f32x2.cuh)
   }
   f32x2 hi[kRsCpw][NACC][RM], lo[kRsCpw][NACC][RM];
 #pragma unroll
@@ -282,7 +277,7 @@ __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_k
         bad |= !isfinite(v.x) || !isfinite(v.y);
         ab += fabsf(v.x) + fabsf(v.y);
       }
-      rowabs[row] = ab;
+      rowabs[row] = fp32_row_bound(ab);
     }
     __syncthreads();
     for (int ro = lane; ro < rows; ro += 32) {
@@ -302,7 +297,7 @@ __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_k
           y = fmaf(v[j].x, ci[q][j], y);
           y = fmaf(v[j].y, cr[q][j], y);
         }
-        const float bound = ab * cb[q];
+        const float bound = fp32_proj_bound(ab, cb[q]);
         // certify: every boundary projection (K > 8: those of the sector's two
         // boundaries) is farther from zero than its error
         bool sure;

@@ -183,6 +183,20 @@ __device__ __forceinline__ uint32_t sign_lines(float x, float y, float* pmin) {
   return bits;
 }
 
+// Certificate of an FP32 decision.  The error of a boundary projection is below
+// gamma sum_j |V_ij|_1 |c_j|_1 (|x|_1 = |Re| + |Im|), gamma = (2 r + 4) 2 u + 8 u
+// with u = 2^-24, plus a few roundings of 2^-150 where products underflow;
+// |c_j|_1 is replaced by its largest value, so that the bound of an evaluation is
+// one FMA: fp32_proj_bound(fp32_row_bound(sum_j |V_ij|_1), fp32_dir_bound(max
+// |c_j|_1, r)).  Rows and directions whose products could overflow (sums or
+// components above 2^62), and directions too small for the product to hold the
+// bound, get an infinite one.
+__device__ __forceinline__ float fp32_row_bound(float ab) { return ab < 0x1p62f ? ab : INFINITY; }
+__device__ __forceinline__ float fp32_dir_bound(float mx, int r) {
+  return mx < 0x1p62f && mx > 0x1p-100f ? mx * (static_cast<float>(2 * r + 4) * 2.0f + 12.0f) * 5.9604644775390625e-08f : INFINITY;
+}
+__device__ __forceinline__ float fp32_proj_bound(float row, float dir) { return fmaf(row, dir, 0x1p-140f); }
+
 // A sign pattern whose code is k.
 template <int K>
 __device__ __forceinline__ uint32_t pattern_of(int k) {
