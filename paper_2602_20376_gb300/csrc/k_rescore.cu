@@ -298,8 +298,8 @@ __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_k
           y = fmaf(v[j].y, cr[q][j], y);
         }
         const float bound = fp32_proj_bound(ab, cb[q]);
-        // certify: every boundary projection (K > 8: those of the sector's two
-        // boundaries) is farther from zero than its error
+        // certify: every boundary projection (K > 8, and odd K at second sight:
+        // those of the sector's two boundaries) is farther from zero than its error
         bool sure;
         uint32_t s = 0;
         int k = 0;
@@ -311,6 +311,14 @@ __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_k
           k = decide_fp32_generic(x, y, Kr);
           const int ma = (k == 0) ? Kr - 1 : k - 1;
           sure = fmaf(y, sbc[ma], -x * sbs[ma]) > bound && fmaf(y, sbc[k], -x * sbs[k]) < -bound;
+        }
+        if constexpr (K > 0 && K % 2 == 1) {
+          // an odd alphabet's boundary is half of its line: w close to the other
+          // half is certain by its sector's own two boundaries
+          if (!sure) {
+            const int kk = scode[s], ma = kk == 0 ? K - 1 : kk - 1;
+            sure = fmaf(y, sbc[ma], -x * sbs[ma]) > bound && fmaf(y, sbc[kk], -x * sbs[kk]) < -bound;
+          }
         }
         if (!sure) {
           double xd = 0.0, yd = 0.0;
