@@ -40,6 +40,7 @@
 #include <utility>
 #include <vector>
 
+#include "lanczos_host.h"
 #include "lrq_device.cuh"
 #include "lrq_internal.h"
 
@@ -1407,6 +1408,8 @@ struct LzRun {
     double tn = 0.0;
     int e;
     if ((e = prepare())) return e;
+    auto wait = [this]() { cudaStreamSynchronize(st); };
+    HostCopies<decltype(wait)> copies(wait);
     while (L < n) {
       if (!verify && L >= r) verify = true;
       const int p_want = verify ? 1 : static_cast<int>(std::min<int64_t>(r - L, n - L));
@@ -1425,8 +1428,8 @@ struct LzRun {
       }
       const int q = verify ? 1 : hc.nvalid;
       if (L + q > p.lmax) return fail(LRQ_ENOCONV, "lrq_truncate: more repeated eigenvalues than locking slots");
-      if ((e = cuda_check(cudaMemcpyAsync(X(), x.data(), static_cast<size_t>(q) * hc.J * sizeof(double),
-                                          cudaMemcpyHostToDevice, st),
+      if ((e = cuda_check(cudaMemcpyAsync(X(), copies.keep(std::move(x)),
+                                          static_cast<size_t>(q) * hc.J * sizeof(double), cudaMemcpyHostToDevice, st),
                           "copy eigenvectors of T")))
         return e;
       lz_launch_ritz<T>(q, lz_rows_grid(n), st, U(), n, L, hc.J, X(), Y());
@@ -1444,7 +1447,7 @@ struct LzRun {
     LzOutput o;
     std::memset(&o, 0, sizeof(o));
     o.r = r;
-    double lam_host[kLzWant];
+    std::vector<double> lam_host(r);
     for (int j = 0; j < r; ++j) {
       if (j < static_cast<int>(order.size())) {
         o.col[j] = order[j];
@@ -1459,7 +1462,8 @@ struct LzRun {
       lz_output<T><<<lz_rows_grid(n), kLzThreads, 0, st>>>(U(), n, o, V, V32);
       count_launch();
     }
-    if ((e = cuda_check(cudaMemcpyAsync(lambda_out, lam_host, r * sizeof(double), cudaMemcpyHostToDevice, st),
+    if ((e = cuda_check(cudaMemcpyAsync(lambda_out, copies.keep(std::move(lam_host)), r * sizeof(double),
+                                        cudaMemcpyHostToDevice, st),
                         "copy eigenvalues")))
       return e;
     if ((e = cuda_check(cudaStreamSynchronize(st), "lanczos sync"))) return e;
