@@ -737,13 +737,13 @@ __device__ void lz_finish(double nrm2, const T* __restrict__ h1, const T* __rest
 //
 // After the three-term step w is orthogonal to every stored vector up to
 // rounding, so h is of rounding size and the correction sum_c U_c h[c] needs
-// no more than FP32: with sum |h_c| <= 2^-30 ||w|| (checked here, ||w|| from
-// lz_threeterm; h is taken relative to the power of two below ||w||, so that
-// the operator's scale does not matter), its relative error of 2^-22 moves w
-// by less than 2^-52 ||w||, within the rounding of w itself.  U is then read through lz_to_float and the
-// kernel is bound by HBM instead of FP64 (n = 10^6, 80 vectors: 121 us, 206 in
-// FP64).  Larger h (a start vector against
-// locked vectors, a vector close to the span) takes the FP64 sum.
+// no more than FP32 where sum |h_c| <= lz_fp32_gate(nc) ||w|| (checked here, ||w||
+// from lz_threeterm; h is taken relative to the power of two below ||w||, so
+// that the operator's scale does not matter): its error then moves w by less
+// than 2^-52 ||w||, within the rounding of w itself.  U is then read through
+// lz_to_float and the kernel is bound by HBM instead of FP64 (n = 10^6, 80
+// vectors: 121 us, 206 in FP64).  Larger h (a start vector against locked
+// vectors, a vector close to the span) takes the FP64 sum.
 template <int SL, typename T>
 __global__ void __launch_bounds__(kLzThreads) lz_update(const T* __restrict__ U, int64_t n, int nc,
                                                         const T* __restrict__ h, T* __restrict__ w,
@@ -786,7 +786,7 @@ __global__ void __launch_bounds__(kLzThreads) lz_update(const T* __restrict__ U,
   if (scale > 0.0) {
     float t = 0.f;
     for (int k = 0; k < kLzThreads / 32; ++k) t += fred[k];
-    f32 = t <= 0x1p-30f;
+    f32 = t <= lz_fp32_gate(nc);
   }
   const int slice = SL == 1 ? 0 : warp;
   constexpr int TILE = kLzThreads / SL;

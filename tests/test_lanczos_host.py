@@ -6,6 +6,7 @@ import re
 import shutil
 import subprocess
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -64,3 +65,42 @@ def test_every_copy_from_the_host_is_kept():
     text = open(os.path.join(CSRC, "k_lanczos.cu")).read()
     calls = re.findall(r"cudaMemcpyAsync\(([^;]*?)cudaMemcpyHostToDevice", text, re.S)
     assert calls and all("copies.keep(" in c for c in calls)
+
+
+@pytest.mark.parametrize("nc", [1, 8, 156, 500, 4096])
+@pytest.mark.parametrize("cplx", [False, True])
+def test_fp32_correction_moves_w_by_a_rounding(tmp_path, nc, cplx):
+    """The FP32 chain of lz_update at the largest h its gate lets through, on the
+    entries of random unit vectors: below 2^-52 ||w|| (||w|| = 1)."""
+    body = '#include <cstdio>\n#include "lanczos_host.h"\nint main() { std::printf("%%a", lrq::lz_fp32_gate(%d)); }'
+    gate = float.fromhex(_run(tmp_path, body % nc)[0])
+    n, f32 = 2048, np.float32
+    g = np.random.Generator(np.random.PCG64(nc))
+
+    def cut(x):  # to FP32, towards zero
+        y = x.astype(f32)
+        return np.where(np.abs(y.astype(np.float64)) > np.abs(x), np.nextafter(y, f32(0)), y)
+
+    def fma(a, b, c):  # the product of two FP32 numbers is exact in FP64, the sum rounds to FP32 after one of 2^-53
+        return (a.astype(np.float64) * np.float64(b) + c.astype(np.float64)).astype(f32)
+
+    parts = 2 if cplx else 1
+    h = g.standard_normal((nc, parts))
+    h *= gate / np.abs(h).sum()  # sum |Re h_c| + |Im h_c| at the gate
+    exact, t = np.zeros((n, parts)), np.zeros((n, parts), f32)
+    for c in range(nc):
+        u = g.standard_normal((n, parts))
+        u /= np.linalg.norm(u)
+        uf, hf = cut(u), cut(h[c])
+        if cplx:
+            exact += np.stack([u[:, 0] * h[c, 0] - u[:, 1] * h[c, 1], u[:, 0] * h[c, 1] + u[:, 1] * h[c, 0]], 1)
+            re = fma(uf[:, 0], hf[0], fma(-uf[:, 1], hf[1], t[:, 0]))
+            im = fma(uf[:, 0], hf[1], fma(uf[:, 1], hf[0], t[:, 1]))
+            t = np.stack([re, im], 1)
+        else:
+            exact += u * h[c]
+            t = fma(uf, hf[0], t)
+    assert np.linalg.norm(t - exact) <= 2.0 ** -52
+    # and with every rounding against it
+    roundings = (2 if cplx else 1) * nc + 12
+    assert roundings * 2.0 ** -24 * gate <= 2.0 ** -52
