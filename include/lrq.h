@@ -366,7 +366,10 @@ int lrq_graph_destroy(void* graph_exec);
  *              wanted Ritz pair (<= 0 selects 1e-10).
  *   max_iter : Krylov dimension cap per run (0 selects min(500, n); at most
  *              4096).  Workspace grows as n * (max_iter + 2r + 9) scalars;
- *              a dense Q with 1024 <= n <= 32768 adds 14 bytes an entry.
+ *              a dense Q with 1024 <= n <= 32768 adds 14 bytes an entry
+ *              (rows padded to 4, columns to 128) for the operator in fixed
+ *              point.  A workspace smaller by 14 n^2 bytes or less is accepted
+ *              too: the operator then runs in FP64 from Q itself.
  *   seed     : start vectors are Philox4x32-10 Gaussians keyed by seed.
  *   V_out    : n x r complex128 (device) or NULL.
  *   V32_out  : n x r complex64 (device, V rounded to nearest) or NULL; the

@@ -341,9 +341,12 @@ __global__ void __launch_bounds__(kLzMvThreads) lz_matvec_dense(
 constexpr int kLzQDigits = 7, kLzXDigits = 8;
 constexpr int kLzFixThreads = 256;  // laying out
 constexpr int kLzFixRows = 4;       // rows a warp
-// Smaller matrices leave SMs without rows; the sums of 8 digit pairs of 2 n
-// products of at most 2^14, times 2^24, have to stay below 2^63, and the digits
-// take as much memory as Q.
+// Smaller matrices leave SMs without rows; above, the sums of 8 digit pairs of 2 n
+// products of at most 2^14, times 2^24, would leave 63 bits.  The digits take
+// nearly as much memory as Q: a workspace without room for them gets the FP64
+// operator.  Truncations with the digits / in FP64, r = 4: n = 1024 13.3 / 14.4 ms
+// (252 steps), 2048 21.3 / 25.2 (316), 4096 37.2 / 68.3 (364), 200 steps at 8192
+// 54 / 109, 16384 154 / 441, 32768 615 / 1599.
 constexpr int64_t kLzFixMin = 1024, kLzFixMax = 32768;
 
 struct LzFixed {
@@ -1179,6 +1182,7 @@ struct LzPlan {
   size_t esz;
   size_t off_U, off_w, off_Y, off_part, off_h1, off_h2, off_npart, off_alpha, off_beta, off_state, off_X, off_deg,
       off_snap, off_count, off_two, off_qdig, off_xdig, off_rowexp, total;
+  size_t plain;  // bytes without the dense operator's digits, which come last
 };
 
 size_t lz_take(size_t& cur, size_t bytes) {
@@ -1218,6 +1222,7 @@ void lz_plan(int64_t n, int r, int maxit, bool cplx, LzPlan* p) {
   // arrival counters: matvec, three-term step, update, then one per vector group of lz_dots
   p->off_count = lz_take(cur, (3 + static_cast<size_t>(ceil_div(p->cap, kLzGroup))) * sizeof(unsigned));
   p->off_two = lz_take(cur, 2 * static_cast<size_t>(kLzMaxBlocks) * p->esz);  // the operator's block sums
+  p->plain = cur;
   const bool fixed = cplx && lz_use_fixed(n);  // the dense operator's digits
   const LzFixed f = lz_fixed(n);
   p->off_qdig = lz_take(cur, fixed ? f.qbytes : 0);
@@ -1231,7 +1236,7 @@ int lz_rows_grid(int64_t rows) { return static_cast<int>(std::max<int64_t>(1, st
 template <typename T>
 struct LzRun {
   // operator
-  bool dense;
+  bool fixed;  // dense, from the digits
   const double2* Q;
   int64_t ld;
   const int32_t* rowptr;
@@ -1266,7 +1271,7 @@ struct LzRun {
   unsigned* counter(int i) const { return reinterpret_cast<unsigned*>(ws + p.off_count) + i; }
   T* two() const { return reinterpret_cast<T*>(ws + p.off_two); }
   uint4* qdig() const { return reinterpret_cast<uint4*>(ws + p.off_qdig); }
-  uint8_t* xdig() const { return dense && lz_use_fixed(n) ? ws + p.off_xdig : nullptr; }
+  uint8_t* xdig() const { return fixed ? ws + p.off_xdig : nullptr; }
   int32_t* rowexp() const { return reinterpret_cast<int32_t*>(ws + p.off_rowexp); }
 
   // y = Q x, h1()[0] = uprev^H y (uprev may be NULL), h1()[1] = x^H y
@@ -1488,7 +1493,7 @@ int LzRun<double>::prepare() const {
 
 template <>
 int LzRun<double2>::prepare() const {
-  if (!lz_use_fixed(n)) {
+  if (!fixed) {
     lz_check_dense<<<lz_rows_grid(n * n), kLzThreads, 0, st>>>(Q, n, ld, status);
     count_launch();
     return LRQ_OK;
@@ -1506,7 +1511,7 @@ int LzRun<double2>::prepare() const {
 
 template <>
 void LzRun<double2>::matvec(const double2* x, double2* y, const double2* uprev) const {
-  if (lz_use_fixed(n)) {  // x is the column that scale() wrote last: its digits are in xdig()
+  if (fixed) {  // x is the column that scale() wrote last: its digits are in xdig()
     const LzFixed f = lz_fixed(n);
     const int blocks = static_cast<int>(std::min<int64_t>(f.units, kLzMaxBlocks));
     lz_matvec_fixed<<<blocks, 32, 0, st>>>(qdig(), rowexp(), n, static_cast<int>(f.units), static_cast<int>(f.steps),
@@ -1546,10 +1551,11 @@ int truncate_check(const lrq_matrix* Q, int r, int max_iter) {
   return LRQ_OK;
 }
 
-size_t truncate_workspace_bytes(const lrq_matrix* Q, int r, int max_iter) {
+size_t truncate_workspace_bytes(const lrq_matrix* Q, int r, int max_iter, size_t* least) {
   LzPlan p;
   const int it = static_cast<int>(std::min<int64_t>(max_iter > 0 ? max_iter : kLzDefaultIter, Q->n));
   lz_plan(Q->n, r, it, Q->kind == LRQ_MATRIX_DENSE_C128, &p);
+  if (least) *least = p.plain;
   return p.total;
 }
 
@@ -1572,7 +1578,8 @@ struct LzSide {
 }  // namespace
 
 int launch_truncate(const lrq_matrix* Q, int r, double tol, int max_iter, uint64_t seed, double2* V, float2* V32,
-                    double* lambda_out, int64_t* iters_out, void* ws, int32_t* status, cudaStream_t st) {
+                    double* lambda_out, int64_t* iters_out, void* ws, size_t ws_bytes, int32_t* status,
+                    cudaStream_t st) {
   const int it = static_cast<int>(std::min<int64_t>(max_iter > 0 ? max_iter : kLzDefaultIter, Q->n));
   const double t = tol > 0.0 ? tol : 1e-10;
   LzSide sd;
@@ -1580,7 +1587,6 @@ int launch_truncate(const lrq_matrix* Q, int r, double tol, int max_iter, uint64
   if (e) return e;
   if (Q->kind == LRQ_MATRIX_DENSE_C128) {
     LzRun<double2> R;
-    R.dense = true;
     R.Q = static_cast<const double2*>(Q->values);
     R.ld = Q->ld;
     R.rowptr = nullptr;
@@ -1591,6 +1597,7 @@ int launch_truncate(const lrq_matrix* Q, int r, double tol, int max_iter, uint64
     R.tol = t;
     R.seed = seed;
     lz_plan(Q->n, r, it, true, &R.p);
+    R.fixed = lz_use_fixed(R.n) && ws_bytes >= R.p.total;  // the caller may leave no room for the digits
     R.ws = static_cast<uint8_t*>(ws);
     R.status = status;
     R.st = st;
@@ -1599,7 +1606,7 @@ int launch_truncate(const lrq_matrix* Q, int r, double tol, int max_iter, uint64
     return R.solve(r, lambda_out, V, V32, iters_out);
   }
   LzRun<double> R;
-  R.dense = false;
+  R.fixed = false;
   R.Q = nullptr;
   R.ld = 0;
   R.rowptr = Q->rowptr;

@@ -498,9 +498,11 @@ int lrq_truncate(const lrq_matrix* Q, int r, double tol, int max_iter, uint64_t 
   if (e) return e;
   if (!lambda_out || !dev_status) return fail(LRQ_EINVAL, "NULL pointer argument");
   if (!(tol < 1.0) || tol != tol) return fail(LRQ_EINVAL, "tol must be below 1");
-  if ((e = check_ws(ws, ws_bytes, truncate_workspace_bytes(Q, r, max_iter)))) return e;
+  size_t least = 0;
+  truncate_workspace_bytes(Q, r, max_iter, &least);
+  if ((e = check_ws(ws, ws_bytes, least))) return e;
   return launch_truncate(Q, r, tol, max_iter, seed, static_cast<double2*>(V_out), static_cast<float2*>(V32_out),
-                         lambda_out, iters_out, ws, dev_status, static_cast<cudaStream_t>(stream));
+                         lambda_out, iters_out, ws, ws_bytes, dev_status, static_cast<cudaStream_t>(stream));
 }
 
 int lrq_proposal_num_features(int r) { return (r >= 1 && r <= kMaxRank) ? 5 * r + 4 : -1; }

@@ -124,9 +124,10 @@ int launch_cut_count(const int32_t* rowptr, const int32_t* colidx, int64_t n, co
                      int64_t* cut_out, cudaStream_t st);
 // spectral truncation (FP64 Lanczos)
 int truncate_check(const lrq_matrix* Q, int r, int max_iter);
-size_t truncate_workspace_bytes(const lrq_matrix* Q, int r, int max_iter);
+size_t truncate_workspace_bytes(const lrq_matrix* Q, int r, int max_iter, size_t* least = nullptr);
 int launch_truncate(const lrq_matrix* Q, int r, double tol, int max_iter, uint64_t seed, double2* V, float2* V32,
-                    double* lambda_out, int64_t* iters_out, void* ws, int32_t* status, cudaStream_t st);
+                    double* lambda_out, int64_t* iters_out, void* ws, size_t ws_bytes, int32_t* status,
+                    cudaStream_t st);
 // learned proposal
 int64_t proposal_num_params(int F);
 int launch_features(const float2* V, int B, int64_t n, int r, const double* lambda, float2* Vg, float* feat,

@@ -576,7 +576,13 @@ def truncate(Q: LrqMatrix, r, tol=0.0, max_iter=0, seed=0, want_c128=True, want_
              stream=None):
     """Top-r spectral truncation; keep the tensors behind Q alive meanwhile."""
     n = Q.n
-    ws = workspace(lrq_truncate_workspace_size(Q, r, max_iter), device)
+    need = lrq_truncate_workspace_size(Q, r, max_iter)
+    try:
+        ws = workspace(need, device)
+    except torch.cuda.OutOfMemoryError:
+        if Q.kind != LRQ_MATRIX_DENSE_C128 or not 1024 <= n <= 32768:
+            raise
+        ws = workspace(need - 14 * n * n, device)  # without the operator's digits
     dev_status = torch.zeros(1, dtype=torch.int32, device=device)
     V = torch.empty((n, r), dtype=torch.complex128, device=device) if want_c128 else None
     V32 = torch.empty((n, r), dtype=torch.complex64, device=device) if want_c64 else None
