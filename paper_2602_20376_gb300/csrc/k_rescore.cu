@@ -13,14 +13,17 @@
 //    the FP64 decision.  Otherwise w and the decision are recomputed in FP64
 //    (rare: the angle must be within ~1e-6 of a boundary).
 //  * conj(V_i) omega^k is accumulated in double-float form; a warp's (hi, lo)
-//    pairs are added in double-float, the warps' in FP64, both by fixed trees.
-//    For K in {2, 3, 4, 6}
-//    the roots of unity are omega^k = a + b tau with a, b in {-1, 0, 1}
+//    pairs and the warps' sums are added by fixed trees.
+//    For K in {2, 3, 4, 6} the roots of unity are omega^k = a + b tau with a, b in {-1, 0, 1}
 //    (tau = i for K = 4, exp(i pi / 3) for K = 3 and 6), so the sums A = sum a
 //    conj(V_i) and B = sum b conj(V_i) need no products: a sum's exact step
 //    (two-sum, a or b folded into its FMAs) is 7 packed FP32 instructions for
-//    both components, and V^H z = A + tau B is formed in FP64 at the end.  Other
-//    alphabets multiply (exact products by FMA residuals).
+//    both components, a warp's pairs are added in double-float, and V^H z = A +
+//    tau B is formed in FP64 at the end.  Other alphabets multiply (exact products
+//    by FMA residuals) and add a warp's pairs in three words.  Errors of f against
+//    extended precision, n = 300 to 200003, the largest: K = 2, 3, 4, 6 6.9e-16
+//    (1.4e-15 by products with FP64 sums over the warp), K = 5, 7, 8, 9, 16
+//    1.7e-15 (as with FP64 over the warp; 5.1e-15 with double-float).
 // The input check of V runs on the rows as they are staged.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -133,6 +136,43 @@ __device__ __forceinline__ void rs_warp_sums(float (&h)[N], float (&l)[N]) {
   }
 }
 
+// (h, m, l) += (h', m', l') in three words: exact but for l's roundings.
+__device__ __forceinline__ void add_triple(float& h, float& m, float& l, float h2, float m2, float l2) {
+  float e, f, g, t;
+  two_sum(h, h2, h, e);
+  two_sum(m, m2, t, f);
+  two_sum(t, e, m, g);
+  l += l2 + (f + g);
+}
+
+// The same with a third word (l: 0 on entry), exact to 2^-60 or so: products' (hi,
+// lo) pairs hold fewer bits than their FP64 sums, which double-float would lose
+// (f off by three times as much at n = 300).  In FP64 it took 20 us of the 52 of
+// r = 6, K = 8, m = 32, n = 50021 (a chunk is 220 rows there); 34 this way, 32 in
+// double-float.
+template <int N>
+__device__ __forceinline__ void rs_warp_sums3(float (&h)[N], float (&m)[N], float (&l)[N]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = N / 2, x = 16; x > 0; k >>= 1, x >>= 1) {
+    if (k > 0) {
+      const bool up = lane & x;
+#pragma unroll
+      for (int q = 0; q < (k > 0 ? k : 1); ++q) {
+        const float gh = up ? h[q] : h[k + q], gm = up ? m[q] : m[k + q], gl = up ? l[q] : l[k + q];
+        h[q] = up ? h[k + q] : h[q];
+        m[q] = up ? m[k + q] : m[q];
+        l[q] = up ? l[k + q] : l[q];
+        add_triple(h[q], m[q], l[q], __shfl_xor_sync(0xffffffffu, gh, x), __shfl_xor_sync(0xffffffffu, gm, x),
+                   x == 16 ? 0.f : __shfl_xor_sync(0xffffffffu, gl, x));
+      }
+    } else {
+      add_triple(h[0], m[0], l[0], __shfl_xor_sync(0xffffffffu, h[0], x), __shfl_xor_sync(0xffffffffu, m[0], x),
+                 __shfl_xor_sync(0xffffffffu, l[0], x));
+    }
+  }
+}
+
 template <int K, int RM>
 __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_kernel(
     const float2* __restrict__ V, int64_t n, int r, const float2* __restrict__ C, int64_t S,
@@ -226,9 +266,8 @@ __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_k
 #pragma unroll
       for (int j = 0; j < RM; ++j) hi[q][g][j] = lo[q][g][j] = 0;
   // Every kRsFlush tiles (at most 256 rows per lane, which bounds the error
-  // of the FP32 low parts) the lanes' (hi, lo) pairs are added in double-float
-  // over the warp and the FP64 total of component j of candidate q is kept by lane
-  // q * 16 + j.
+  // of the FP32 low parts) the lanes' (hi, lo) pairs are added over the warp
+  // and the FP64 total of component j of candidate q is kept by lane q * 16 + j.
   double tot[NACC];
 #pragma unroll
   for (int g = 0; g < NACC; ++g) tot[g] = 0.0;
@@ -244,11 +283,22 @@ __global__ void __launch_bounds__(kRsThreads, RM <= 4 ? 3 : 2) rescore_partial_k
           unpack2(lo[q][g][j], l[2 * j], l[2 * j + 1]);
           hi[q][g][j] = lo[q][g][j] = 0;
         }
-        rs_warp_sums(h, l);
         // value i ends in lane 32 / (2 RM) i; lane q * 16 + j takes it from there
         const int from = (32 / (2 * RM)) * (lane & 15) & 31;
-        const double mine = static_cast<double>(__shfl_sync(0xffffffffu, h[0], from)) +
-                            static_cast<double>(__shfl_sync(0xffffffffu, l[0], from));
+        double mine;
+        if constexpr (LAT) {
+          rs_warp_sums(h, l);
+          mine = static_cast<double>(__shfl_sync(0xffffffffu, h[0], from)) +
+                 static_cast<double>(__shfl_sync(0xffffffffu, l[0], from));
+        } else {
+          float t[2 * RM];
+#pragma unroll
+          for (int j = 0; j < 2 * RM; ++j) t[j] = 0.f;
+          rs_warp_sums3(h, l, t);
+          mine = static_cast<double>(__shfl_sync(0xffffffffu, h[0], from)) +
+                 (static_cast<double>(__shfl_sync(0xffffffffu, l[0], from)) +
+                  static_cast<double>(__shfl_sync(0xffffffffu, t[0], from)));
+        }
         if ((lane >> 4) == q) tot[g] += mine;
       }
     }
