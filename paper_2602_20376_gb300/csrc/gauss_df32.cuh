@@ -258,14 +258,17 @@ LRQ_HD df32 df_recip(df32 x) {
   return df_fast_sum(r, df_mul(r, e));
 }
 
-// Whether rounding h + l (h the nearest FP32 number) may depend on an error of
-// 2^-37 of it plus 2^-43 (above a component's: g within 2^-38, sine and cosine
-// 2^-45).
-__device__ __forceinline__ bool df_near_midpoint(df32 x) {
+// Whether rounding h + l (h the nearest FP32 number) may depend on an error of err.
+__device__ __forceinline__ bool df_near_midpoint(df32 x, float err) {
   const uint32_t b = __float_as_uint(x.h) & 0x7fffffffu;
   if ((b & 0x7fffffu) == 0u || b < (24u << 23)) return true;  // a power of two (half the spacing below), tiny
   const float half = __uint_as_float((b & 0x7f800000u) - (24u << 23));
-  return half - fabsf(x.l) <= fmaf(fabsf(x.h), 0x1p-37f, 0x1p-43f);
+  return half - fabsf(x.l) <= err;
+}
+// The same for a direction's component: 2^-37 of it plus 2^-43 are above its error
+// (g within 2^-38, sine and cosine 2^-45).
+__device__ __forceinline__ bool df_near_midpoint(df32 x) {
+  return df_near_midpoint(x, fmaf(fabsf(x.h), 0x1p-37f, 0x1p-43f));
 }
 
 // The directions of a block of 256 threads (lrq_sample_directions' draws): a

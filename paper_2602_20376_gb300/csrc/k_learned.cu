@@ -46,7 +46,8 @@ __device__ __forceinline__ df32 df_from(double x) {
 // norms and column moduli; then the gauge-fixed copy and the central moments
 // of all r + 1 populations at once (q = 0: a_i = ||V_i||^2 n / total, q = 1 + j:
 // b_ij = |V_ij|^2 n / lambda_j).  Bound: FP64 (about 60 warp instructions of 16
-// cycles per 32 rows at r = 4); the gauge product is double-float.  One block
+// cycles per 32 rows at r = 4); the gauge product is double-float, in FP64 where
+// its rounding to FP32 could depend on that.  One block
 // per instance with eleven passes took 247 us at B = 16, n = 4096; 77 now.
 constexpr int kFeatThreads = 256;
 constexpr int kFeatSums = 3 * (kMaxRank + 1);
@@ -58,6 +59,7 @@ struct FeatShared {
   long long row[kMaxRank];
   long long wbest[kFeatThreads / 32][kMaxRank], wrow[kFeatThreads / 32][kMaxRank];
   df32 ph_re[kMaxRank], ph_im[kMaxRank];
+  double ph_re64[kMaxRank], ph_im64[kMaxRank];
 };
 
 // the cluster's sums of `count` values per thread, in a fixed order
@@ -172,8 +174,10 @@ __global__ void __launch_bounds__(kFeatThreads) features_kernel(const float2* __
     const float2 a = Vb[min(row, static_cast<long long>(n - 1)) * r + j];
     const double am = sqrt(static_cast<double>(a.x) * a.x + static_cast<double>(a.y) * a.y);
     // multiply the column by |a| / a = conj(a) / |a|
-    sh.ph_re[j] = df_from(am > 0.0 ? a.x / am : 1.0);
-    sh.ph_im[j] = df_from(am > 0.0 ? -a.y / am : 0.0);
+    sh.ph_re64[j] = am > 0.0 ? a.x / am : 1.0;
+    sh.ph_im64[j] = am > 0.0 ? -a.y / am : 0.0;
+    sh.ph_re[j] = df_from(sh.ph_re64[j]);
+    sh.ph_im[j] = df_from(sh.ph_im64[j]);
   }
   feat_sums(cluster, sh, acc, r + 1);  // its barriers also publish the phases
   double mean[kMaxRank + 1];
@@ -198,7 +202,16 @@ __global__ void __launch_bounds__(kFeatThreads) features_kernel(const float2* __
         const df32 pr = sh.ph_re[j], pi = sh.ph_im[j];
         const df32 x = df_times(df32{v.x, 0.f}, pr), y = df_times(df32{v.y, 0.f}, pi);
         const df32 z = df_times(df32{v.x, 0.f}, pi), w = df_times(df32{v.y, 0.f}, pr);
-        Vo[i * r + j] = make_float2(df_sum(x, df32{-y.h, -y.l}).h, df_sum(z, w).h);
+        const df32 re = df_sum(x, df32{-y.h, -y.l}), im = df_sum(z, w);
+        float2 o = make_float2(re.h, im.h);
+        // each product and sum is off by less than 2^-45 of the terms: where that
+        // could turn the rounding (one entry in 10^5), in FP64
+        const float err = 0x1p-43f * (fabsf(v.x) + fabsf(v.y));
+        if (df_near_midpoint(re, err) || df_near_midpoint(im, err)) {
+          o.x = static_cast<float>(v.x * sh.ph_re64[j] - v.y * sh.ph_im64[j]);
+          o.y = static_cast<float>(v.x * sh.ph_im64[j] + v.y * sh.ph_re64[j]);
+        }
+        Vo[i * r + j] = o;
         const double m2 = feat_mod2(v);
         a += m2;
         moments(1 + j, m2);
@@ -532,7 +545,9 @@ __global__ void __launch_bounds__(kNllThreads) vmf_nll_kernel(const float* __res
 // The test runs in FP32 with a margin; inside the margin (about one try in
 // 10^4) it is repeated in FP64 as first written, so every draw is accepted or
 // not as in FP64.  Logs, Gaussians and the vectors are double-float
-// (gauss_df32.cuh): FP64 runs at 1/64 of the FP32 rate and took about 800
+// (gauss_df32.cuh): a component is within 2^-40 of FP64's before it is rounded to
+// FP32 (of 960000 components 8 differ from numpy's FP64 rounding, 9 when all of it
+// ran in FP64).  FP64 runs at 1/64 of the FP32 rate and took about 800
 // instructions a sample (16 x 65520 draws: 2298 us, 361 with one sample a thread
 // at a time).  A warp's tries run until its unluckiest lane is done, about four
 // times where the mean is 1.5, so a thread takes kVmfPer samples through the
