@@ -273,12 +273,18 @@ __device__ __forceinline__ bool df_near_midpoint(df32 x) {
 
 // The directions of a block of 256 threads (lrq_sample_directions' draws): a
 // thread per component, 256 / r candidates a block, ||Z||^2 = sum_j -ln u1_j
-// exchanged through shared memory.  s: the block's first candidate.
+// exchanged through shared memory.  A candidate with a component near a midpoint
+// is drawn again in FP64 by its r threads side by side (one thread doing it alone
+// for its component took 5.2 ms for 300000 directions of r = 64, 0.8 so, and 14.7
+// us for 2^14 of r = 4, 6.8 so).  s_first: the block's first candidate; every
+// thread of the block calls it.
 constexpr int kSphereThreads = 256;
 __host__ __device__ inline int sphere_per_block(int r) { return kSphereThreads / r; }
 
 __device__ __forceinline__ void sphere_block(uint64_t seed, int64_t s_first, int64_t S, int r, float2* __restrict__ C) {
   __shared__ df32 nl[kSphereThreads];
+  __shared__ double nd[kSphereThreads];
+  __shared__ uint8_t again[kSphereThreads];  // by candidate
   const int per = sphere_per_block(r);
   const int c = threadIdx.x / r, j = threadIdx.x - c * r;
   const int64_t s = s_first + c;
@@ -295,31 +301,37 @@ __device__ __forceinline__ void sphere_block(uint64_t seed, int64_t s_first, int
     L = df_neg_log(U1, GaussTab());
   }
   nl[threadIdx.x] = L;
+  again[threadIdx.x] = 0;
   __syncthreads();
-  if (!act) return;
-  df32 N = nl[c * r];
-  for (int k = 1; k < r; ++k) N = df_sum(N, nl[c * r + k]);
-  df32 sn, cs;
-  df_sincos(U2, GaussTab(), &sn, &cs);
-  const df32 g = df_times(df_sqrt(L), df_recip(df_sqrt(N)));
-  const df32 re = df_times(g, cs), im = df_times(g, sn);
-  float2 out = make_float2(re.h, im.h);
-  if (df_near_midpoint(re) || df_near_midpoint(im)) {
-    double a = 0.0, b = 0.0, nrm2 = 0.0;
-#pragma unroll 1
-    for (int k = 0; k < r; ++k) {
-      double zr, zi;
-      sphere_component(seed, s, k, &zr, &zi);
-      nrm2 += zr * zr + zi * zi;
-      if (k == j) {
-        a = zr;
-        b = zi;
-      }
-    }
-    const double inv = 1.0 / sqrt(nrm2);
-    out = make_float2(static_cast<float>(a * inv), static_cast<float>(b * inv));
+  float2 out = make_float2(0.f, 0.f);
+  bool unsure = false;
+  if (act) {
+    df32 N = nl[c * r];
+    for (int k = 1; k < r; ++k) N = df_sum(N, nl[c * r + k]);
+    df32 sn, cs;
+    df_sincos(U2, GaussTab(), &sn, &cs);
+    const df32 g = df_times(df_sqrt(L), df_recip(df_sqrt(N)));
+    const df32 re = df_times(g, cs), im = df_times(g, sn);
+    out = make_float2(re.h, im.h);
+    unsure = df_near_midpoint(re) || df_near_midpoint(im);
+    if (unsure) again[c] = 1;
   }
-  C[s * r + j] = out;
+  if (__syncthreads_or(unsure)) {
+    double a = 0.0, b = 0.0;
+    const bool mine = act && again[c];
+    if (mine) {
+      sphere_component(seed, s, j, &a, &b);
+      nd[threadIdx.x] = a * a + b * b;
+    }
+    __syncthreads();
+    if (mine && unsure) {
+      double nrm2 = 0.0;
+      for (int k = 0; k < r; ++k) nrm2 += nd[c * r + k];
+      const double inv = 1.0 / sqrt(nrm2);
+      out = make_float2(static_cast<float>(a * inv), static_cast<float>(b * inv));
+    }
+  }
+  if (act) C[s * r + j] = out;
 }
 
 }  // namespace lrq
