@@ -17,9 +17,9 @@
 namespace lrq {
 
 // Uniform directions on the complex unit sphere (gauss_df32.cuh).  Bound:
-// issue slots, about 250 instructions a component, and the few drawn again in
-// FP64 (3.2 us without them).  S = 2^14, r = 4: 14.7 us, 26
-// in FP64 (two lanes an SM).
+// issue slots, about 250 instructions a component, and the candidates drawn again
+// in FP64 (3.2 us without them).  S = 2^14, r = 4: 6.8 us, 26 in FP64 (two lanes an
+// SM).
 __global__ void __launch_bounds__(kSphereThreads) sample_directions_kernel(uint64_t seed, int64_t S, int r,
                                                                            float2* __restrict__ C) {
   sphere_block(seed, static_cast<int64_t>(blockIdx.x) * sphere_per_block(r), S, r, C);
@@ -191,32 +191,32 @@ struct Fp32Tables {
 
 constexpr int kFp32Block = 256;    // candidates
 constexpr int kFp32Batch = 256;
-template <int R>
-struct Fp32Shape {
-  static constexpr int kCpt = R <= 5 ? 2 : 1;  // candidates per thread
-  static constexpr int kThreads = kFp32Block / kCpt;
-};
 
-template <int K, int R>
-__global__ void __launch_bounds__(Fp32Shape<R>::kThreads) score_fp32_kernel(const float2* __restrict__ V, int64_t n,
+template <int K, int R, int kFp32Cpt>  // kFp32Cpt: candidates per thread
+__global__ void __launch_bounds__(kFp32Block / kFp32Cpt) score_fp32_kernel(const float2* __restrict__ V, int64_t n,
                                                                   const float2* __restrict__ C, int64_t S,
                                                                   int64_t S_pad, int64_t rows_per_chunk, int Kdyn,
                                                                   const __grid_constant__ Fp32Tables tab,
                                                                   double* __restrict__ partial) {
-  constexpr int kFp32Cpt = Fp32Shape<R>::kCpt, kFp32Threads = Fp32Shape<R>::kThreads;
-  __shared__ __align__(16) float4 vs[kFp32Batch * R];
+  constexpr int kFp32Threads = kFp32Block / kFp32Cpt;
+  constexpr bool kScalar = K == 0;  // score_row_scalar
+  __shared__ __align__(16) float4 vs[kScalar ? kFp32Batch * R / 2 : kFp32Batch * R];
   __shared__ float2 zt[ZTable<K>::kEntries];
   fill_ztable<K>(zt, tab.zr, tab.zi, Kdyn);
 
   const float none[kAnyLines] = {};  // the boundaries of kAnyK8, not used here
   const int64_t s0 = static_cast<int64_t>(blockIdx.x) * kFp32Block + threadIdx.x;
   Dir2<R> d[kFp32Cpt];
+  float2 c[R];  // kScalar's
   double acc64[kFp32Cpt][2 * R];
 #pragma unroll
   for (int q = 0; q < kFp32Cpt; ++q) {
     const int64_t s = s0 + q * kFp32Threads;
 #pragma unroll
-    for (int j = 0; j < R; ++j) d[q].set(j, s < S ? C[s * R + j] : make_float2(0.f, 0.f));
+    for (int j = 0; j < R; ++j) {
+      c[j] = s < S ? C[s * R + j] : make_float2(0.f, 0.f);
+      d[q].set(j, c[j]);
+    }
 #pragma unroll
     for (int j = 0; j < 2 * R; ++j) acc64[q][j] = 0.0;
   }
@@ -229,30 +229,54 @@ __global__ void __launch_bounds__(Fp32Shape<R>::kThreads) score_fp32_kernel(cons
 #pragma unroll 4
     for (int t = threadIdx.x; t < rows * R; t += kFp32Threads) {
       const float2 v = V[b0 * R + t];
-      vs[t] = make_float4(v.x, v.x, v.y, v.y);
+      if constexpr (kScalar)
+        reinterpret_cast<float2*>(vs)[t] = v;
+      else
+        vs[t] = make_float4(v.x, v.x, v.y, v.y);
     }
     __syncthreads();
-    f32x2 acc[kFp32Cpt][R];
+    if constexpr (kScalar) {
+      static_assert(kFp32Cpt == 1, "one candidate a thread");
+      float2 acc[R];
 #pragma unroll
-    for (int q = 0; q < kFp32Cpt; ++q)
+      for (int j = 0; j < R; ++j) acc[j] = make_float2(0.f, 0.f);
+      // four rows unrolled keep more angles in flight (n = 2000, r = 3: 73 us, 81 rolled);
+      // at r = 4 the registers for it cost a block an SM (269 us, 261 with two)
+#pragma unroll(R == 4 ? 2 : 4)
+      for (int i = 0; i < rows; ++i) {
+        float2 v[R];
 #pragma unroll
-      for (int j = 0; j < R; ++j) acc[q][j] = 0;
-    for (int i = 0; i < rows; ++i) {
-      ulonglong2 v[R];
-#pragma unroll
-      for (int j = 0; j < R; ++j) v[j] = reinterpret_cast<const ulonglong2*>(vs)[i * R + j];
-#pragma unroll
-      for (int q = 0; q < kFp32Cpt; ++q) score_row<K, R, true>(v, d[q], zt, Kdyn, none, none, acc[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < kFp32Cpt; ++q)
+        for (int j = 0; j < R; ++j) v[j] = reinterpret_cast<const float2*>(vs)[i * R + j];
+        score_row_scalar<R, true>(v, c, zt, Kdyn, acc);
+      }
 #pragma unroll
       for (int j = 0; j < R; ++j) {
-        float re, im;
-        unpack2(acc[q][j], re, im);
-        acc64[q][2 * j] += static_cast<double>(re);
-        acc64[q][2 * j + 1] += static_cast<double>(im);
+        acc64[0][2 * j] += static_cast<double>(acc[j].x);
+        acc64[0][2 * j + 1] += static_cast<double>(acc[j].y);
       }
+    } else {
+      f32x2 acc[kFp32Cpt][R];
+#pragma unroll
+      for (int q = 0; q < kFp32Cpt; ++q)
+#pragma unroll
+        for (int j = 0; j < R; ++j) acc[q][j] = 0;
+      for (int i = 0; i < rows; ++i) {
+        ulonglong2 v[R];
+#pragma unroll
+        for (int j = 0; j < R; ++j) v[j] = reinterpret_cast<const ulonglong2*>(vs)[i * R + j];
+#pragma unroll
+        for (int q = 0; q < kFp32Cpt; ++q) score_row<K, R, true>(v, d[q], zt, Kdyn, none, none, acc[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < kFp32Cpt; ++q)
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          float re, im;
+          unpack2(acc[q][j], re, im);
+          acc64[q][2 * j] += static_cast<double>(re);
+          acc64[q][2 * j + 1] += static_cast<double>(im);
+        }
+    }
   }
 #pragma unroll
   for (int q = 0; q < kFp32Cpt; ++q) {
@@ -265,16 +289,35 @@ __global__ void __launch_bounds__(Fp32Shape<R>::kThreads) score_fp32_kernel(cons
   }
 }
 
+// Two candidates a thread up to r = 5 and K = 8, once the blocks go round the chip
+// several times: below that a thread's chain of evaluations is the time.  Kernel
+// time with one / two: 4 blocks (K = 2, r = 1) 11 / 26 us, 160 (K = 8, r = 3) 34 / 42,
+// 320 (K = 2, r = 4) 42 / 46, 1024 (K = 8, r = 4) 118 / 116, 1185 (K = 2, r = 3) 601 /
+// 575.
+template <int K, int R>
+static void launch_fp32_one(const ScorePlan& p, dim3 grid, const Fp32Tables& tab, const float2* V, const float2* C,
+                            double* partial, cudaStream_t st) {
+  const int64_t S_pad = p.c_tiles * 128;
+  const int64_t blocks = static_cast<int64_t>(grid.x) * grid.y;
+  if constexpr (R <= 5 && K > 0) {
+    if (blocks >= 4 * static_cast<int64_t>(num_sms_current())) {
+      score_fp32_kernel<K, R, 2><<<grid, kFp32Block / 2, 0, st>>>(V, p.n, C, p.S, S_pad, p.fp32_rows_per_chunk, p.K, tab,
+                                                                  partial);
+      return;
+    }
+  }
+  score_fp32_kernel<K, R, 1><<<grid, kFp32Block, 0, st>>>(V, p.n, C, p.S, S_pad, p.fp32_rows_per_chunk, p.K, tab,
+                                                          partial);
+}
+
 template <int K>
 static int launch_fp32_r(const ScorePlan& p, const Fp32Tables& tab, const float2* V, const float2* C,
                          double* partial, cudaStream_t st) {
   dim3 grid(static_cast<unsigned>(ceil_div(p.S, kFp32Block)), static_cast<unsigned>(p.nsplit));
-  int64_t S_pad = p.c_tiles * 128;
   switch (p.r) {
-#define LRQ_FP32_CASE(RR)                                                                              \
-  case RR:                                                                                             \
-    score_fp32_kernel<K, RR><<<grid, Fp32Shape<RR>::kThreads, 0, st>>>(                                \
-        V, p.n, C, p.S, S_pad, p.fp32_rows_per_chunk, p.K, tab, partial);                              \
+#define LRQ_FP32_CASE(RR)                                       \
+  case RR:                                                      \
+    launch_fp32_one<K, RR>(p, grid, tab, V, C, partial, st);    \
     break;
     LRQ_FP32_CASE(1)
     LRQ_FP32_CASE(2)

@@ -298,4 +298,29 @@ __device__ __forceinline__ void score_row(const ulonglong2 (&v)[R], const Dir2<R
   }
 }
 
+// The same in scalar FMAs on the row's {re, im} (same operations and order), for K >
+// 8: the angle is most of an evaluation there and half the shared-memory reads count
+// for more than half the FMAs.
+template <int R, bool VFIRST>
+__device__ __forceinline__ void score_row_scalar(const float2 (&v)[R], const float2 (&c)[R], const float2* zt, int K,
+                                                 float2 (&acc)[R]) {
+  float x = 0.f, y = 0.f;
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    if constexpr (VFIRST) {
+      x = fmaf(-v[j].y, c[j].y, fmaf(v[j].x, c[j].x, x));
+      y = fmaf(v[j].y, c[j].x, fmaf(v[j].x, c[j].y, y));
+    } else {
+      x = fmaf(v[j].x, c[j].x, fmaf(-v[j].y, c[j].y, x));
+      y = fmaf(v[j].x, c[j].y, fmaf(v[j].y, c[j].x, y));
+    }
+  }
+  const float2 z = zt[decide_fp32_generic(x, y, K)];
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    acc[j].x = fmaf(v[j].x, z.x, fmaf(v[j].y, z.y, acc[j].x));
+    acc[j].y = fmaf(v[j].x, z.y, fmaf(-v[j].y, z.x, acc[j].y));
+  }
+}
+
 }  // namespace lrq
