@@ -139,17 +139,17 @@ __device__ __forceinline__ bool r1_less(uint64_t ka, uint32_t ia, uint64_t kb, u
 // owns kR1Local consecutive pairs and takes the merge sizes k_first..k_last (all
 // up to kR1Local in the first launch, then the tail of one size each).
 __global__ void __launch_bounds__(kR1Local / 2) r1_sort_local(uint64_t* __restrict__ key, uint32_t* __restrict__ idx,
-                                                              int64_t k_first, int64_t k_last) {
+                                                              int k_first, int k_last) {
   __shared__ uint64_t sk[kR1Local];
   __shared__ uint32_t si[kR1Local];
-  const int64_t base = static_cast<int64_t>(blockIdx.x) * kR1Local;
+  const int base = static_cast<int>(blockIdx.x) * kR1Local;  // below kR1Bitonic
   for (int t = threadIdx.x; t < kR1Local; t += blockDim.x) {
     sk[t] = key[base + t];
     si[t] = idx[base + t];
   }
   __syncthreads();
-  for (int64_t k = k_first; k <= k_last; k <<= 1) {
-    for (int j = static_cast<int>(min(k >> 1, static_cast<int64_t>(kR1Local / 2))); j > 0; j >>= 1) {
+  for (int k = k_first; k <= k_last; k <<= 1) {
+    for (int j = min(k >> 1, kR1Local / 2); j > 0; j >>= 1) {
       const int t = threadIdx.x;
       const int a = (t / j) * 2 * j + (t % j);
       const int b = a + j;
@@ -175,10 +175,10 @@ __global__ void __launch_bounds__(kR1Local / 2) r1_sort_local(uint64_t* __restri
 // one stage (merge size k, partner distance j >= kR1Local) in global memory, a
 // thread per pair of pairs
 __global__ void __launch_bounds__(kR1Threads) r1_sort_global(uint64_t* __restrict__ key, uint32_t* __restrict__ idx,
-                                                             int64_t npad, int64_t k, int64_t j) {
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * kR1Threads + threadIdx.x;
+                                                             int npad, int k, int j) {
+  const int t = static_cast<int>(blockIdx.x) * kR1Threads + threadIdx.x;
   if (t >= npad / 2) return;
-  const int64_t a = (t / j) * 2 * j + (t % j), b = a + j;
+  const int a = (t / j) * 2 * j + (t % j), b = a + j;
   const bool up = (a & k) == 0;
   const uint64_t ka = key[a], kb = key[b];
   const uint32_t ia = idx[a], ib = idx[b];
@@ -768,13 +768,13 @@ int launch_rank1(const double2* q, int64_t n, int K, uint8_t* z_out, double* f_o
   r1_prep_kernel<<<nbase, kR1Threads, 0, st>>>(q, n, L.npad, K, tb, key, idx, code0, base, counter, s0, status);
   count_launch();
   if (n <= kR1Bitonic) {
-    const unsigned lb = static_cast<unsigned>(L.npad / kR1Local);
+    const int npad = static_cast<int>(L.npad);
+    const unsigned lb = static_cast<unsigned>(npad / kR1Local);
     r1_sort_local<<<lb, kR1Local / 2, 0, st>>>(key, idx, 2, kR1Local);
     count_launch();
-    for (int64_t k = 2 * kR1Local; k <= L.npad; k <<= 1) {
-      for (int64_t j = k >> 1; j >= kR1Local; j >>= 1) {
-        r1_sort_global<<<static_cast<unsigned>(ceil_div(L.npad / 2, kR1Threads)), kR1Threads, 0, st>>>(key, idx, L.npad,
-                                                                                                      k, j);
+    for (int k = 2 * kR1Local; k <= npad; k <<= 1) {
+      for (int j = k >> 1; j >= kR1Local; j >>= 1) {
+        r1_sort_global<<<static_cast<unsigned>(ceil_div(npad / 2, kR1Threads)), kR1Threads, 0, st>>>(key, idx, npad, k, j);
         count_launch();
       }
       r1_sort_local<<<lb, kR1Local / 2, 0, st>>>(key, idx, k, k);
