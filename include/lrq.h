@@ -101,7 +101,9 @@ int lrq_abi_version(void);
  * and key (lo32(seed), hi32(seed)); output words (0,1) and (2,3) give two
  * 53-bit uniforms u1, u2 = (top 53 bits + 0.5) / 2^53, and
  * Z_j = sqrt(-ln u1) * exp(2 pi i u2) (Box-Muller, Re and Im ~ N(0, 1/2)).
- * The normalisation runs in FP64; the result is rounded once to complex64.
+ * Every component is the rounding to FP32 of the value computed in FP64
+ * (internally in pairs of FP32 numbers, in FP64 where the rounding could depend
+ * on that).
  *
  *   C_out : S x r complex64 (device), written.
  *   1 <= r <= 64, S >= 0 (S = 0 launches nothing).

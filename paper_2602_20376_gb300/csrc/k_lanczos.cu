@@ -328,13 +328,18 @@ __global__ void __launch_bounds__(kLzMvThreads) lz_matvec_dense(
 // ---------------------------------------------------------------------------
 // Four FP64 FMAs an entry keep the dense operator (141 us at n = 4096) well
 // above its bytes (40 us).  Here Q's entries are 55-bit integers relative to
-// their row's largest component (off by 2^-55 of it at most) and the unit
+// their row's largest component (off by 2^-54 of it at most) and the unit
 // vector's are 63-bit integers, both cut into signed bytes (seven and eight
 // base-256 digits d and j, the most significant first).  The digit products with
 // d + j <= 7 are summed exactly by 4-way byte dot products, by d + j; the others
 // are below 2^-59 of the largest product.  FP64 only joins a row's sums.
-// Against exact arithmetic the result is at least as close as that of FP64
-// FMAs, whose partial sums round at every entry.  Q's digits are laid out once
+// The error is bounded by the row: |y_i - (Q x)_i| is at most 2^-54 max_j |Q_ij|
+// ||x||_1 (the entries) plus 2^-57 n max_j |Q_ij| (x, the dropped digit pairs),
+// where FP64 FMAs, whose partial sums round at every entry, are off by some 2^-53
+// of them.  On rows of similar entries it is no larger (eigenvalues and residuals
+// of random Q agree with LAPACK's as well as in FP64); entries far below their
+// row's largest keep fewer bits, and such a row loses to FP64 where x is small at
+// its largest ones.  Lanczos needs the bound by ||Q||.  Q's digits are laid out once
 // per truncation (14 bytes an entry for 16), a vector's by the kernel that
 // normalises it.  (The 8-bit matrix instruction has the rate of the byte dot
 // products here and takes all 56 digit pairs: 91 us.)
