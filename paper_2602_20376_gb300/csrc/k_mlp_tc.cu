@@ -20,7 +20,9 @@
 // Bound: latency (at a batch of 64 a GEMM is under 1 us of loads and 0.1 of
 // MMAs); chunks of 64 along K with 64 scalar loads a thread, each chunk
 // waiting for its own loads and MMAs, took 21 us a GEMM, now 7.5.  BN = 32
-// while BN = 64 would leave most SMs without a tile.
+// while BN = 64 would leave SMs without a tile: the three layers forward with BN = 32 /
+// 64 take 36 / 41 us at a batch of 64, 39 / 45 at 2048, 47 / 46 at 4096 (128 tiles of
+// 64), 60 / 52 at 6000, 143 / 116 at 20000.
 // The wait is bounded (~1 s); if it runs out (never observed) the kernel
 // records the fault, writes NaN into its tile, waits (bounded) for its MMAs,
 // frees its tensor memory and returns.
