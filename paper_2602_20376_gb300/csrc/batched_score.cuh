@@ -1,7 +1,7 @@
 // batched_score.cuh -- the persistent scoring kernel of the batched launch
 // (k_batched.cu): its problem descriptors, work items and both forms' template.
-// The form with one slot a thread is compiled in k_batched_wide.cu, so that the
-// two compile side by side.
+// The forms, one and four slots a thread, are compiled in k_batched_wide.cu and
+// k_batched_four.cu, side by side.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -285,9 +285,24 @@ __global__ void __launch_bounds__(kBSlots / PT, PT == 4 ? 6 : 2) batched_score_k
   }
 }
 
-// The form with one slot a thread (k_batched_wide.cu).
-int batched_wide_blocks_per_sm(int* blocks);
-void launch_batched_wide(int grid, cudaStream_t st, const BProb* probs, const BItem* items, int nitems, int* counter,
-                         const BTable* btab, const EnumTables* etab, uint64_t* keys, EnumBest* ebest, int32_t* status);
+template <int PT>
+int batched_blocks_per_sm(int* blocks) {
+  return cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, batched_score_kernel<PT>, kBSlots / PT, 0),
+                    "occupancy query");
+}
+
+template <int PT>
+void launch_batched_score(int grid, cudaStream_t st, const BProb* probs, const BItem* items, int nitems, int* counter,
+                          const BTable* btab, const EnumTables* etab, uint64_t* keys, EnumBest* ebest,
+                          int32_t* status) {
+  batched_score_kernel<PT><<<grid, kBSlots / PT, 0, st>>>(probs, items, nitems, counter, btab, etab, keys, ebest, status);
+}
+
+#define LRQ_BATCHED_FORM(PREFIX, PT)                                                                                  \
+  PREFIX template int batched_blocks_per_sm<PT>(int*);                                                                \
+  PREFIX template void launch_batched_score<PT>(int, cudaStream_t, const BProb*, const BItem*, int, int*,             \
+                                                const BTable*, const EnumTables*, uint64_t*, EnumBest*, int32_t*);
+LRQ_BATCHED_FORM(extern, 1)
+LRQ_BATCHED_FORM(extern, 4)
 
 }  // namespace lrq

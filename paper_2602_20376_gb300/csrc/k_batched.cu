@@ -668,10 +668,9 @@ int launch_sequence(const lrq_batched_plan_impl* pl, uint8_t* ws, int nitems, in
   EnumBest* ebest = reinterpret_cast<EnumBest*>(ws + pl->off_ebest);
   const BItem* items = reinterpret_cast<const BItem*>(ws + pl->off_items);
   if (per_thread == 1)
-    launch_batched_wide(pl->grid_wide, st, probs, items, nitems, counter, pl->btab, pl->etab, keys, ebest, status);
+    launch_batched_score<1>(pl->grid_wide, st, probs, items, nitems, counter, pl->btab, pl->etab, keys, ebest, status);
   else
-    batched_score_kernel<4><<<pl->grid, kBSlots / 4, 0, st>>>(probs, items, nitems, counter, pl->btab, pl->etab, keys,
-                                                              ebest, status);
+    launch_batched_score<4>(pl->grid, st, probs, items, nitems, counter, pl->btab, pl->etab, keys, ebest, status);
   timing_stop(st);
   count_launch();
   if (select) {
@@ -733,9 +732,7 @@ int lrq_batched_plan_create(const lrq_problem* problems, int P, int top_m, lrq_b
     }
   }
   int per_sm = 1, per_sm_wide = 1;
-  if ((e = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_score_kernel<4>, kBSlots / 4, 0),
-                      "occupancy query")) ||
-      (e = batched_wide_blocks_per_sm(&per_sm_wide))) {
+  if ((e = batched_blocks_per_sm<4>(&per_sm)) || (e = batched_blocks_per_sm<1>(&per_sm_wide))) {
     delete pl;
     return e;
   }
